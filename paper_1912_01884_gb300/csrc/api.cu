@@ -491,9 +491,8 @@ int fhtdp_cnn_conv3x3_dgrad(const void *dz, int n, int h, int w, int dil, const 
     g_last_error[0] = 0;
     if (!dz || !wt || !wflip || !dx || n < 1 || !cnn_shape_ok(h, w, dil))
         return set_error(FHTDP_EINVAL, "conv3x3_dgrad: bad arguments");
-    int st = cnn_flip_transpose(wt, wflip, stream);
-    if (st) return st;
-    return cnn_conv3x3(dz, 32, n, h, w, dil, wflip, nullptr, 0, dx, stream);
+    // the kernel reads the weights flipped and transposed: the scratch stays unused
+    return cnn_conv3x3_tc(dz, n, h, w, dil, wt, nullptr, 0, dx, stream, true);
 }
 
 int fhtdp_cnn_relu_backward(const void *y, void *dy, long long count, cudaStream_t stream) {

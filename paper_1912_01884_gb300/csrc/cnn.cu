@@ -144,17 +144,6 @@ __global__ void relu_backward_kernel(const __nv_bfloat16 *__restrict__ Y,
         if (!(__bfloat162float(Y[i]) > 0.0f)) dY[i] = __float2bfloat16(0.0f);
 }
 
-// Weights of the data gradient: W'[tap'][co][ci] = W[8 - tap'][ci][co].
-__global__ void flip_transpose_kernel(const __nv_bfloat16 *__restrict__ Wt,
-                                      __nv_bfloat16 *__restrict__ Wf) {
-    for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < 9 * kC * kC;
-         i += blockDim.x * gridDim.x) {
-        const int tap = i / (kC * kC), r = i % (kC * kC);
-        const int co = r / kC, ci = r % kC;
-        Wf[i] = Wt[((size_t)(8 - tap) * kC + ci) * kC + co];
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Weight and bias gradients: dW[tap][ci][co] += sum_p X(p + off(tap))[ci] *
 // dZ(p)[co], db[co] += sum_p dZ(p)[co].  Persistent CTAs loop over row
@@ -410,11 +399,6 @@ int cnn_relu_backward(const void *Y, void *dY, long long count, cudaStream_t str
     relu_backward_kernel<<<grid_1d(count, 256), 256, 0, stream>>>(
         (const __nv_bfloat16 *)Y, (__nv_bfloat16 *)dY, count);
     return launched("relu_backward_kernel");
-}
-
-int cnn_flip_transpose(const void *Wt, void *Wf, cudaStream_t stream) {
-    flip_transpose_kernel<<<36, 256, 0, stream>>>((const __nv_bfloat16 *)Wt, (__nv_bfloat16 *)Wf);
-    return launched("flip_transpose_kernel");
 }
 
 int cnn_wgrad(const void *X, int cin, int N, int H, int W, int dil, const void *dZ, float *dW,

@@ -10,7 +10,6 @@ int cnn_downsample4(const uint8_t *img, int N, int H, int W, void *out, cudaStre
 int cnn_conv3x3(const void *X, int cin, int N, int H, int W, int dil, const void *Wt,
                 const float *bias, int relu, void *Y, cudaStream_t stream);
 int cnn_relu_backward(const void *Y, void *dY, long long count, cudaStream_t stream);
-int cnn_flip_transpose(const void *Wt, void *Wf, cudaStream_t stream);
 int cnn_wgrad(const void *X, int cin, int N, int H, int W, int dil, const void *dZ, float *dW,
               float *db, cudaStream_t stream);
 int cnn_band_head(const void *L, int N, int H, int W, int bands, const int32_t *labels,
@@ -24,7 +23,8 @@ int cnn_to_bf16(const float *src, void *dst, int count, cudaStream_t stream);
 // The 32-channel layers on tcgen05 (conv_tc.cu); cnn_tc_status reads (and
 // with `clear` resets) their device status, synchronising.
 int cnn_conv3x3_tc(const void *X, int N, int H, int W, int dil, const void *Wt,
-                   const float *bias, int relu, void *Y, cudaStream_t stream);
+                   const float *bias, int relu, void *Y, cudaStream_t stream, bool flip = false,
+                   const void *mask = nullptr);
 int cnn_wgrad_tc(const void *X, int N, int H, int W, int dil, const void *dZ, float *dW,
                  float *db, cudaStream_t stream);
 int cnn_tc_status(int clear);

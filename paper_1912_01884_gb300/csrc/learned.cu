@@ -251,7 +251,6 @@ int fhtdp_cnn_backward(const void *params, const int32_t *labels, int n, int h, 
     const char *P = (const char *)params;
     char *W = (char *)ws;
     const int ho = h / 4, wo = w / 4;
-    const long long cnt = (long long)n * ho * wo * kC;
     int st = cuda_status(cudaMemsetAsync(W + c.loss, 0, 4, stream), "cudaMemsetAsync");
     // the head's gradient (mean cross-entropy over images and bands)
     if (!st)
@@ -270,10 +269,10 @@ int fhtdp_cnn_backward(const void *params, const int32_t *labels, int n, int h, 
                            dw + (size_t)taps_rows(l) * kC, stream);
         if (l == 0 || st) break;
         // input gradient: the forward of the flipped and transposed weights,
-        // then the ReLU of the layer below
-        if (!st) st = cnn_flip_transpose(P + o.w16, W + c.wflip, stream);
-        if (!st) st = cnn_conv3x3(dz, kC, n, ho, wo, kDil[l], W + c.wflip, nullptr, 0, dx, stream);
-        if (!st) st = cnn_relu_backward(W + c.act[l - 1], dx, cnt, stream);
+        // masked by the ReLU of the layer below
+        if (!st)
+            st = cnn_conv3x3_tc(dz, n, ho, wo, kDil[l], P + o.w16, nullptr, 0, dx, stream, true,
+                                W + c.act[l - 1]);
         std::swap(dz, dx);
     }
     if (!st && loss)
