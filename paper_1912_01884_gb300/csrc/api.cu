@@ -37,6 +37,20 @@ int cuda_status(cudaError_t err, const char *what) {
     return set_error(FHTDP_ECUDA, "%s: %s", what, cudaGetErrorString(err));
 }
 
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000,
+                                             cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            return (PFN_cuTensorMapEncodeTiled_v12000)ptr;
+        cudaGetLastError();
+        return (PFN_cuTensorMapEncodeTiled_v12000) nullptr;
+    }();
+    return fn;
+}
+
 bool make_shape(int h, int w, int k, Shape *out) {
     if (h < 1 || w < 1 || k < 1 || h % k != 0) return false;
     int n = h / k;

@@ -7,131 +7,153 @@
 // Layout: activations NHWC bf16 ([N][H][W][C], C = 32; the input has C = 1),
 // weights bf16 [tap][ci][co] with tap = ky*3 + kx (layer 1: [16][32], taps
 // 9..15 zero), FP32 master weights and FP32 accumulation.  The 3x3 dilated
-// convolutions ("same" zero padding) run as implicit GEMMs on the tensor
-// cores: the 32-channel layers (forward and data gradient) with tcgen05.mma
-// (conv_tc.cu), the single-channel first layer and the weight gradient with
-// bf16 WMMA 16x16x16 tiles: a CTA takes 64 pixels of one image row and all
-// 32 output channels; K = 9 taps x 32 input channels.
-#include <mma.h>
-
+// convolutions ("same" zero padding) of 32 channels run on tcgen05.mma
+// (conv_tc.cu).  The single-channel first layer (9 products a value) is bound
+// by its 64 bytes a pixel of output: one warp MMA step in registers forward,
+// plain FP32 multiply-adds for its weight gradient.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "cnn.cuh"
 
 namespace fhtdp {
 namespace {
 
-using namespace nvcuda;
-
 constexpr int kC = 32;        // channels
-constexpr int kSeg = 64;      // pixels of a row per CTA
+constexpr int kSeg = 64;      // row widths are multiples of it
 constexpr int kMaxDil = 8;
 
 // ---------------------------------------------------------------------------
+// Eight bf16 values at p as four words; `wide` when p is 16-byte aligned.
+__device__ __forceinline__ uint4 ld8(const __nv_bfloat16 *p, bool wide) {
+    if (wide) return __ldg((const uint4 *)p);
+    const unsigned short *q = (const unsigned short *)p;
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = __ldg(q + 2 * i) | (uint32_t)__ldg(q + 2 * i + 1) << 16;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ void st8(__nv_bfloat16 *p, const uint32_t (&w)[4], bool wide) {
+    if (wide) {
+        *(uint4 *)p = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+        unsigned short *q = (unsigned short *)p;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] = (unsigned short)(i & 1 ? w[i / 2] >> 16 : w[i / 2]);
+    }
+}
+
 // 4x4 mean pool of uint8 images, scaled to [0, 1]: [N][H][W] -> [N][H/4][W/4].
-__global__ void downsample4_kernel(const uint8_t *__restrict__ img, long long n_img_stride,
-                                   int H, int W, __nv_bfloat16 *__restrict__ out) {
-    const int Ho = H / 4, Wo = W / 4;
-    const long long total = (long long)gridDim.y * Ho * Wo;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)Ho * Wo;
+// A thread makes V = 4 neighbouring values from four 16-byte loads (rows
+// 16-byte aligned, W a multiple of 16), or V = 1 from four 4-byte loads.
+template <int V>
+__global__ void downsample4_kernel(const uint8_t *__restrict__ img, int H, int W, long long total,
+                                   __nv_bfloat16 *__restrict__ out) {
+    const int Wv = W / (4 * V);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
-        const int n = blockIdx.y;
-        const int yo = (int)(i / Wo), xo = (int)(i % Wo);
-        const uint8_t *p = img + n * n_img_stride + (size_t)(4 * yo) * W + 4 * xo;
-        unsigned s = 0;
+        const long long row = i / Wv;   // output row over all images
+        const int xv = (int)(i - row * Wv);
+        const uint8_t *p = img + row * 4 * W + (size_t)xv * 4 * V;
+        unsigned s[V] = {};
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const uint32_t v = *(const uint32_t *)(p + (size_t)r * W);
-            s += (v & 255u) + ((v >> 8) & 255u) + ((v >> 16) & 255u) + (v >> 24);
+            uint32_t v[V];
+            if constexpr (V == 4) {
+                const uint4 q = __ldg((const uint4 *)(p + (size_t)r * W));
+                v[0] = q.x;
+                v[1] = q.y;
+                v[2] = q.z;
+                v[3] = q.w;
+            } else {
+                v[0] = __ldg((const uint32_t *)(p + (size_t)r * W));
+            }
+#pragma unroll
+            for (int k = 0; k < V; ++k) s[k] = __dp4a(v[k], 0x01010101u, s[k]);
         }
-        out[(size_t)n * Ho * Wo + i] = __float2bfloat16((float)s * (1.0f / (16.0f * 255.0f)));
+        __nv_bfloat16 *dst = out + row * (W / 4) + (size_t)xv * V;
+        if constexpr (V == 4) {
+            __nv_bfloat162 o[2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                (k & 1 ? o[k / 2].y : o[k / 2].x) =
+                    __float2bfloat16((float)s[k] * (1.0f / (16.0f * 255.0f)));
+            *(uint2 *)dst = make_uint2(*(const uint32_t *)&o[0], *(const uint32_t *)&o[1]);
+        } else {
+            dst[0] = __float2bfloat16((float)s[0] * (1.0f / (16.0f * 255.0f)));
+        }
     }
-    (void)total;
 }
 
 // ---------------------------------------------------------------------------
-// Rows y-dil, y, y+dil of one image, columns [x0 - dil, x0 + kSeg + dil),
-// all channels, zero outside the image, into sx[3][kSeg + 2*kMaxDil][kC].
-__device__ void stage_rows(const __nv_bfloat16 *X, int cin, int H, int W, int n, int y, int x0,
-                           int dil, __nv_bfloat16 *sx) {
-    const int width = kSeg + 2 * dil;
-    const int per_px = cin;   // 32 or 1
-    for (int i = threadIdx.x; i < 3 * width * kC; i += blockDim.x) {
-        const int r = i / (width * kC);
-        const int rem = i - r * width * kC;
-        const int px = rem / kC, c = rem % kC;
-        const int yy = y + (r - 1) * dil, xx = x0 - dil + px;
-        __nv_bfloat16 v = __float2bfloat16(0.0f);
-        if (c < per_px && yy >= 0 && yy < H && xx >= 0 && xx < W)
-            v = X[(((size_t)n * H + yy) * W + xx) * per_px + c];
-        sx[((size_t)r * (kSeg + 2 * kMaxDil) + px) * kC + c] = v;
-    }
-}
-
-// One CTA: 64 output pixels x 32 output channels.  8 warps, warp w owns the
-// 16x16 output tile (pixels 16*(w/2).., channels 16*(w%2)..).  For cin = 32:
-// K = 9 taps x 32 channels; for cin = 1: an im2col tile of the 9 taps
-// (padded to 16) and one K step.  out = act(sum + bias), bf16.
+// First layer: Y(p)[co] = act(sum over the nine taps of x(p + off) * w[tap][co]
+// + bias[co]), one input channel.  A warp takes 16 pixels of a row and one
+// m16n8k16 step per eight output channels: A = pixels x taps (taps 9..15 are
+// zero), B = the weights, kept in registers.  Column 2 t + e of step j stands
+// for channel 8 t + 2 j + e, so that a thread ends up with eight consecutive
+// channels of a pixel and a warp stores 512 contiguous bytes.
 template <bool kRelu>
-__global__ void __launch_bounds__(256) conv3x3_kernel(const __nv_bfloat16 *__restrict__ X,
-                                                      int cin, int H, int W, int dil,
-                                                      const __nv_bfloat16 *__restrict__ Wt,
-                                                      const float *__restrict__ bias,
-                                                      __nv_bfloat16 *__restrict__ Y) {
-    __shared__ __align__(128) __nv_bfloat16 sx[3 * (kSeg + 2 * kMaxDil) * kC];
-    __shared__ __align__(128) __nv_bfloat16 sw[9 * kC * kC];
-    __shared__ __align__(128) float so[kSeg * kC];
-    const int segs = W / kSeg;
-    const int n = blockIdx.x / (H * segs);
-    const int rem = blockIdx.x % (H * segs);
-    const int y = rem / segs, x0 = (rem % segs) * kSeg;
-    const int warp = threadIdx.x >> 5;
-    const int pb = warp >> 1, cb = warp & 1;
-    wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc;
-    wmma::fill_fragment(acc, 0.0f);
-    if (cin == kC) {
-        for (int i = threadIdx.x; i < 9 * kC * kC; i += blockDim.x) sw[i] = Wt[i];
-        stage_rows(X, cin, H, W, n, y, x0, dil, sx);
-        __syncthreads();
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ky = tap / 3, kx = tap % 3;
-            for (int c0 = 0; c0 < kC; c0 += 16) {
-                wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, wmma::row_major> a;
-                wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::row_major> b;
-                const __nv_bfloat16 *ap =
-                    sx + ((size_t)ky * (kSeg + 2 * kMaxDil) + 16 * pb + kx * dil) * kC + c0;
-                wmma::load_matrix_sync(a, ap, kC);
-                wmma::load_matrix_sync(b, sw + ((size_t)tap * kC + c0) * kC + 16 * cb, kC);
-                wmma::mma_sync(acc, a, b, acc);
-            }
-        }
-    } else {
-        // im2col of the single input channel: sx as [kSeg][16] (k = tap).
-        __nv_bfloat16 *col = sx;
-        for (int i = threadIdx.x; i < 16 * kC; i += blockDim.x) sw[i] = Wt[i];
-        for (int i = threadIdx.x; i < kSeg * 16; i += blockDim.x) {
-            const int p = i / 16, k = i % 16;
-            __nv_bfloat16 v = __float2bfloat16(0.0f);
-            if (k < 9) {
-                const int yy = y + (k / 3 - 1) * dil, xx = x0 + p + (k % 3 - 1) * dil;
-                if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = X[((size_t)n * H + yy) * W + xx];
-            }
-            col[i] = v;
-        }
-        __syncthreads();
-        wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, wmma::row_major> a;
-        wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::row_major> b;
-        wmma::load_matrix_sync(a, col + 16 * pb * 16, 16);
-        wmma::load_matrix_sync(b, sw + 16 * cb, kC);
-        wmma::mma_sync(acc, a, b, acc);
+__global__ void __launch_bounds__(256) conv3x3_first_kernel(
+    const __nv_bfloat16 *__restrict__ X, int H, int W, int dil, unsigned tiles,
+    const __nv_bfloat16 *__restrict__ Wt, const float *__restrict__ bias,
+    __nv_bfloat16 *__restrict__ Y, bool wide) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const unsigned short *xs = (const unsigned short *)X, *ws = (const unsigned short *)Wt;
+    uint32_t b0[4], b1[4];
+    float bs[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int co = 8 * (g >> 1) + 2 * j + (g & 1);
+        b0[j] = ws[2 * t * kC + co] | (uint32_t)ws[(2 * t + 1) * kC + co] << 16;
+        b1[j] = t == 0 ? ws[8 * kC + co] : 0;
     }
-    wmma::store_matrix_sync(so + (16 * pb) * kC + 16 * cb, acc, kC, wmma::mem_row_major);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kSeg * kC; i += blockDim.x) {
-        const int p = i / kC, c = i % kC;
-        float v = so[i] + (bias ? bias[c] : 0.0f);
-        if (kRelu) v = v > 0.0f ? v : 0.0f;
-        Y[(((size_t)n * H + y) * W + x0 + p) * kC + c] = __float2bfloat16(v);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) bs[c] = bias ? bias[8 * t + c] : 0.0f;
+    // the thread's taps: 2 t, 2 t + 1 and (t = 0) 8
+    const int dy[3] = {(2 * t / 3 - 1) * dil, ((2 * t + 1) / 3 - 1) * dil, dil};
+    const int dx[3] = {(2 * t % 3 - 1) * dil, ((2 * t + 1) % 3 - 1) * dil, dil};
+    const unsigned per_row = W / 16, step = gridDim.x * (blockDim.x / 32);
+    for (unsigned u = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); u < tiles; u += step) {
+        const unsigned r = u / per_row;   // row over all images
+        const long long row = r;
+        const int x0 = (int)(u - r * per_row) * 16, y = (int)(r % (unsigned)H);
+        uint32_t a[4];
+#pragma unroll
+        for (int hi = 0; hi < 2; ++hi) {   // pixels g and g + 8
+            uint32_t v[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int yy = y + dy[k], xx = x0 + g + 8 * hi + dx[k];
+                v[k] = (k < 2 || t == 0) && yy >= 0 && yy < H && xx >= 0 && xx < W
+                           ? __ldg(xs + (row + dy[k]) * W + xx)
+                           : 0;
+            }
+            a[hi] = v[0] | v[1] << 16;
+            a[2 + hi] = v[2];
+        }
+        uint32_t lo[4], hi[4];   // channels 8 t + 2 j, + 1 of pixels g and g + 8
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float c[4];
+            asm volatile(
+                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, "
+                "{%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+                : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0[j]), "r"(b1[j]), "f"(0.0f));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                c[k] += bs[2 * j + (k & 1)];
+                if (kRelu) c[k] = fmaxf(c[k], 0.0f);
+            }
+            const __nv_bfloat162 l = __floats2bfloat162_rn(c[0], c[1]);
+            const __nv_bfloat162 h = __floats2bfloat162_rn(c[2], c[3]);
+            lo[j] = *(const uint32_t *)&l;
+            hi[j] = *(const uint32_t *)&h;
+        }
+        __nv_bfloat16 *dst = Y + ((size_t)row * W + x0 + g) * kC + 8 * t;
+        st8(dst, lo, wide);
+        st8(dst + 8 * kC, hi, wide);
     }
 }
 
@@ -145,93 +167,113 @@ __global__ void relu_backward_kernel(const __nv_bfloat16 *__restrict__ Y,
 }
 
 // ---------------------------------------------------------------------------
-// Weight and bias gradients: dW[tap][ci][co] += sum_p X(p + off(tap))[ci] *
-// dZ(p)[co], db[co] += sum_p dZ(p)[co].  Persistent CTAs loop over row
-// segments and keep their partial sums in tensor-core accumulators; one
-// atomic flush per CTA.  8 warps share the 18 (tap, ci block) x 2 (co block)
-// output tiles of a 32-channel input (cin = 1: the 1 x 2 tiles of the
-// im2col form).
-__global__ void __launch_bounds__(256) conv3x3_wgrad_kernel(const __nv_bfloat16 *__restrict__ X,
-                                                            int cin, int N, int H, int W,
-                                                            int dil,
-                                                            const __nv_bfloat16 *__restrict__ dZ,
-                                                            float *__restrict__ dW,
-                                                            float *__restrict__ db) {
-    __shared__ __align__(128) __nv_bfloat16 sx[3 * (kSeg + 2 * kMaxDil) * kC];
-    __shared__ __align__(128) __nv_bfloat16 sz[kSeg * kC];
-    __shared__ __align__(128) float sacc[16 * 16 * 8];
-    const int warp = threadIdx.x >> 5;
-    const int tiles = cin == kC ? 36 : 2;
-    constexpr int kMaxTiles = 5;   // ceil(36 / 8)
-    wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc[kMaxTiles];
+// Weight and bias gradients of the first layer: dW[tap][co] = sum over pixels
+// p of x(p + off(tap)) * dZ(p)[co], db[co] = sum of dZ(p)[co].  A thread takes
+// eight channels of one pixel of a 64-pixel segment and goes down a chain of
+// rows: its nine inputs are three new ones a row and six kept, its 72 + 8 sums
+// stay in registers, the next row's loads are in flight; at the end the 64
+// pixels' sums are added in shared memory in a fixed order.
+constexpr int kW1Sums = 80;   // 9 taps and the bias, eight channels
+constexpr int kW1Part = 17 * kC;   // a row of `part`: 16 tap rows (9..15 zero) and the bias
+__global__ void __launch_bounds__(256, 2) wgrad_first_kernel(
+    const __nv_bfloat16 *__restrict__ X, int N, int H, int W, int dil,
+    const __nv_bfloat16 *__restrict__ dZ, float *__restrict__ dW, float *__restrict__ db,
+    float *__restrict__ part, bool wide) {
+    __shared__ float red[8][4][kW1Sums + 1];
+    const int c = threadIdx.x & 3, px = threadIdx.x >> 2;
+    const unsigned short *xs = (const unsigned short *)X;
+    float acc[kW1Sums];
 #pragma unroll
-    for (int t = 0; t < kMaxTiles; ++t) wmma::fill_fragment(acc[t], 0.0f);
-    float bsum = 0.0f;   // thread c < 32: bias gradient of channel c
-    const int segs = W / kSeg;
-    const long long units = (long long)N * H * segs;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-        const int n = (int)(u / (H * segs));
-        const int rem = (int)(u % (H * segs));
-        const int y = rem / segs, x0 = (rem % segs) * kSeg;
-        __syncthreads();
-        for (int i = threadIdx.x; i < kSeg * kC; i += blockDim.x)
-            sz[i] = dZ[(((size_t)n * H + y) * W + x0) * kC + i];
-        if (cin == kC) {
-            stage_rows(X, cin, H, W, n, y, x0, dil, sx);
-        } else {
-            for (int i = threadIdx.x; i < kSeg * 16; i += blockDim.x) {
-                const int p = i / 16, k = i % 16;
-                __nv_bfloat16 v = __float2bfloat16(0.0f);
-                if (k < 9) {
-                    const int yy = y + (k / 3 - 1) * dil, xx = x0 + p + (k % 3 - 1) * dil;
-                    if (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                        v = X[((size_t)n * H + yy) * W + xx];
-                }
-                sx[i] = v;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < kC)
-            for (int p = 0; p < kSeg; ++p) bsum += __bfloat162float(sz[p * kC + threadIdx.x]);
+    for (int k = 0; k < kW1Sums; ++k) acc[k] = 0.0f;
+    RowRange<kSeg> rr(N, H, W, dil);
+    while (rr.next()) {
+        const int x = rr.x0 + px;
+        const bool in0 = x >= dil, in2 = x + dil < W;
+        // the three inputs of chain row j at this pixel (zero outside the image)
+        auto inputs = [&](int j, uint32_t (&v)[3]) {
+            const int y = rr.row(j);
+            const unsigned short *p = xs + ((size_t)rr.n * H + (y >= 0 && y < H ? y : 0)) * W + x;
+            const bool in = y >= 0 && y < H;
+            v[0] = in && in0 ? __ldg(p - dil) : 0;
+            v[1] = in ? __ldg(p) : 0;
+            v[2] = in && in2 ? __ldg(p + dil) : 0;
+        };
+        auto dzs = [&](int j) {
+            return ld8(dZ + (((size_t)rr.n * H + rr.row(j)) * W + x) * kC + 8 * c, wide);
+        };
+        uint32_t v[3];
+        float xf[9];   // rows above, at and below
+        auto keep = [&](int at) {
 #pragma unroll
-        for (int t = 0; t < kMaxTiles; ++t) {
-            const int tile = warp + 8 * t;
-            if (tile >= tiles) break;
-            const int kb = tile >> 1, cb = tile & 1;   // kb: (tap, ci block) or 0
-            for (int p0 = 0; p0 < kSeg; p0 += 16) {
-                wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, wmma::col_major> a;
-                wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::row_major> b;
-                if (cin == kC) {
-                    const int tap = kb >> 1, c0 = 16 * (kb & 1);
-                    const int ky = tap / 3, kx = tap % 3;
-                    // A = X^T: rows = input channels, columns = pixels.
-                    wmma::load_matrix_sync(
-                        a, sx + ((size_t)ky * (kSeg + 2 * kMaxDil) + p0 + kx * dil) * kC + c0, kC);
-                } else {
-                    wmma::load_matrix_sync(a, sx + p0 * 16, 16);
-                }
-                wmma::load_matrix_sync(b, sz + p0 * kC + 16 * cb, kC);
-                wmma::mma_sync(acc[t], a, b, acc[t]);
+            for (int k = 0; k < 3; ++k) xf[3 * at + k] = __uint_as_float(v[k] << 16);
+        };
+        inputs(rr.i - 1, v);
+        keep(1);
+        inputs(rr.i, v);
+        keep(2);
+        inputs(rr.i + 1, v);
+        uint4 z = dzs(rr.i);
+        for (int o = 0; o < rr.L; ++o) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) xf[k] = xf[k + 3];
+            keep(2);
+            const uint32_t zw[4] = {z.x, z.y, z.z, z.w};
+            if (o + 1 < rr.L) {
+                inputs(rr.i + o + 2, v);
+                z = dzs(rr.i + o + 1);
             }
+            float f[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                f[e] = __uint_as_float(e & 1 ? zw[e / 2] & 0xffff0000u : zw[e / 2] << 16);
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[8 * k + e] = __fmaf_rn(xf[k], f[e], acc[8 * k + e]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[72 + e] += f[e];
         }
     }
-    // Flush: dW rows k = tap * 32 + ci (cin = 32) or k = tap (cin = 1).
-    float *st = sacc + warp * 256;
 #pragma unroll
-    for (int t = 0; t < kMaxTiles; ++t) {
-        const int tile = warp + 8 * t;
-        if (tile >= tiles) break;
-        const int kb = tile >> 1, cb = tile & 1;
-        wmma::store_matrix_sync(st, acc[t], 16, wmma::mem_row_major);
-        __syncwarp();
-        for (int i = threadIdx.x & 31; i < 256; i += 32) {
-            const int r = i / 16, c = i % 16;
-            const int k = 16 * kb + r;
-            atomicAdd(&dW[(size_t)k * kC + 16 * cb + c], st[i]);
-        }
-        __syncwarp();
+    for (int k = 0; k < kW1Sums; ++k) {
+        float v = acc[k];
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) < 4) red[threadIdx.x >> 5][c][k] = v;
     }
-    if (threadIdx.x < kC && db) atomicAdd(&db[threadIdx.x], bsum);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kW1Part; i += blockDim.x) {
+        const int row = i / kC, co = i % kC, k = row < 9 ? row : 9;   // tap, or 9: the bias
+        float v = 0.0f;
+        if (row < 9 || row == 16)
+            for (int w = 0; w < 8; ++w) v += red[w][co >> 3][8 * k + (co & 7)];
+        if (part)
+            part[(size_t)blockIdx.x * kW1Part + i] = v;
+        else if (row < 9)
+            atomicAdd(dW + i, v);
+        else if (row == 16 && db)
+            atomicAdd(db + co, v);
+    }
+}
+
+// out[i] = sum of part[r][i] over the rows r in a fixed order: 32 consecutive
+// values a block, 32 rows at a time.
+__global__ void __launch_bounds__(1024) sum_parts_kernel(const float *__restrict__ part, int rows,
+                                                         int stride, int count,
+                                                         float *__restrict__ out) {
+    __shared__ float red[32][33];
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane, w = threadIdx.x >> 5;
+    float v = 0.0f;
+    if (i < count) {
+#pragma unroll 10
+        for (int r = w; r < rows; r += 32) v += part[(size_t)r * stride + i];
+    }
+    red[w][lane] = v;
+    __syncthreads();
+    v = red[lane][w];   // value blockIdx.x * 32 + w
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0 && blockIdx.x * 32 + w < count) out[blockIdx.x * 32 + w] = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -240,6 +282,9 @@ __global__ void __launch_bounds__(256) conv3x3_wgrad_kernel(const __nv_bfloat16 
 // over the band), the softmax cross-entropy of the 32 pooled logits against
 // the label bin, its gradient dlogit = (softmax - onehot)[c] *
 // exp(logit - pooled[c]) * scale, and the predicted bin.
+// The sums run as eight chains a channel (position modulo 8, one warp each),
+// a value at a time without branches, the next values' loads in flight.  The
+// gradient pass takes 16 bytes a thread; the band comes from L2 then.
 __global__ void __launch_bounds__(256) band_head_kernel(const __nv_bfloat16 *__restrict__ L,
                                                         int H, int W, int bands,
                                                         const int32_t *__restrict__ labels,
@@ -247,27 +292,46 @@ __global__ void __launch_bounds__(256) band_head_kernel(const __nv_bfloat16 *__r
                                                         __nv_bfloat16 *__restrict__ dL,
                                                         float *__restrict__ loss,
                                                         int32_t *__restrict__ pred,
-                                                        float *__restrict__ conf) {
+                                                        float *__restrict__ conf, bool wide) {
     __shared__ float smax[8][kC], ssum[8][kC], pooled[kC], dpool[kC];
     const int n = blockIdx.x / bands, b = blockIdx.x % bands;
     const int rpb = H / bands;
-    const int c = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int positions = rpb * W;
-    const __nv_bfloat16 *base = L + ((size_t)n * H + (size_t)b * rpb) * W * kC;
-    float m = -INFINITY, s = 0.0f;
-    for (int pidx = part; pidx < positions; pidx += 8) {
-        const float v = __bfloat162float(base[(size_t)pidx * kC + c]);
-        if (v > m) {
-            s = s * __expf(m - v) + 1.0f;
-            m = v;
-        } else {
-            s += __expf(v - m);
+    const __nv_bfloat16 *band = L + ((size_t)n * H + (size_t)b * rpb) * W * kC;
+    {
+        const int c = threadIdx.x & 31, part = threadIdx.x >> 5;
+        const unsigned short *src = (const unsigned short *)band + c;
+        float m = -INFINITY, s = 0.0f;
+        auto take = [&](unsigned short bits) {
+            const float v = __uint_as_float((uint32_t)bits << 16);
+            const bool up = v > m;
+            const float e = __expf(up ? m - v : v - m);
+            s = up ? s * e + 1.0f : s + e;
+            m = up ? v : m;
+        };
+        constexpr int kB = 16;
+        int p = part;
+        unsigned short q[kB];
+        auto fetch = [&](int from) {
+#pragma unroll
+            for (int k = 0; k < kB; ++k) q[k] = __ldg(src + (size_t)(from + 8 * k) * kC);
+        };
+        if (p + 8 * (kB - 1) < positions) fetch(p);
+        for (; p + 8 * (kB - 1) < positions; p += 8 * kB) {
+            unsigned short cur[kB];
+#pragma unroll
+            for (int k = 0; k < kB; ++k) cur[k] = q[k];
+            if (p + 8 * (2 * kB - 1) < positions) fetch(p + 8 * kB);
+#pragma unroll
+            for (int k = 0; k < kB; ++k) take(cur[k]);
         }
+        for (; p < positions; p += 8) take(__ldg(src + (size_t)p * kC));
+        smax[part][c] = m;
+        ssum[part][c] = s;
     }
-    smax[part][c] = m;
-    ssum[part][c] = s;
     __syncthreads();
     if (threadIdx.x < kC) {
+        const int c = threadIdx.x;
         float M = -INFINITY;
         for (int p = 0; p < 8; ++p) M = fmaxf(M, smax[p][c]);
         float S = 0.0f;
@@ -294,11 +358,31 @@ __global__ void __launch_bounds__(256) band_head_kernel(const __nv_bfloat16 *__r
     }
     __syncthreads();
     if (!dL) return;
-    __nv_bfloat16 *dbase = dL + ((size_t)n * H + (size_t)b * rpb) * W * kC;
-    const float pc = pooled[c], g = dpool[c] * scale;
-    for (int pidx = part; pidx < positions; pidx += 8) {
-        const float v = __bfloat162float(base[(size_t)pidx * kC + c]);
-        dbase[(size_t)pidx * kC + c] = __float2bfloat16(g * __expf(v - pc));
+    const int c8 = (threadIdx.x & 3) * 8;
+    const __nv_bfloat16 *base = band + c8;
+    __nv_bfloat16 *dbase = dL + (band - L) + c8;
+    float pc[8], g[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        pc[e] = pooled[c8 + e];
+        g[e] = dpool[c8 + e] * scale;
+    }
+#pragma unroll 4
+    for (int p = threadIdx.x >> 2; p < positions; p += 64) {
+        const uint4 q = ld8(base + (size_t)p * kC, wide);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            v[e] = __uint_as_float(e & 1 ? w[e / 2] & 0xffff0000u : w[e / 2] << 16);
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(g[e] * __expf(v[e] - pc[e]),
+                                                           g[e + 1] * __expf(v[e + 1] - pc[e + 1]));
+            o[e / 2] = *(const uint32_t *)&h;
+        }
+        st8(dbase + (size_t)p * kC, o, wide);
     }
 }
 
@@ -317,6 +401,25 @@ __global__ void adam_kernel(float *__restrict__ p, float *__restrict__ m, float 
         const float pi = p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
         p[i] = pi;
         if (wb) wb[i] = __float2bfloat16(pi);
+    }
+}
+
+// The same step on up to eight tensors, one block row each.
+struct AdamTensors {
+    AdamTensor t[8];
+};
+__global__ void adam_all_kernel(const __grid_constant__ AdamTensors a, float lr, float b1, float b2,
+                                float eps, float c1, float c2) {
+    const AdamTensor &t = a.t[blockIdx.y];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < t.count; i += gridDim.x * blockDim.x) {
+        const float gi = t.g[i];
+        const float mi = b1 * t.m[i] + (1.0f - b1) * gi;
+        const float vi = b2 * t.v[i] + (1.0f - b2) * gi * gi;
+        t.m[i] = mi;
+        t.v[i] = vi;
+        const float pi = t.p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+        t.p[i] = pi;
+        if (t.wb) ((__nv_bfloat16 *)t.wb)[i] = __float2bfloat16(pi);
     }
 }
 
@@ -372,27 +475,28 @@ bool cnn_shape_ok(int H, int W, int dil) {
 }
 
 int cnn_downsample4(const uint8_t *img, int N, int H, int W, void *out, cudaStream_t stream) {
-    dim3 grid(grid_1d((long long)(H / 4) * (W / 4), 256), N);
-    downsample4_kernel<<<grid, 256, 0, stream>>>(img, (long long)H * W, H, W,
-                                                 (__nv_bfloat16 *)out);
+    const bool wide = W % 16 == 0 && (uintptr_t)img % 16 == 0 && (uintptr_t)out % 8 == 0;
+    const long long total = (long long)N * (H / 4) * (W / (wide ? 16 : 4));
+    if (wide)
+        downsample4_kernel<4><<<grid_1d(total, 256), 256, 0, stream>>>(img, H, W, total,
+                                                                     (__nv_bfloat16 *)out);
+    else
+        downsample4_kernel<1><<<grid_1d(total, 256), 256, 0, stream>>>(img, H, W, total,
+                                                                     (__nv_bfloat16 *)out);
     return launched("downsample4_kernel");
 }
 
 int cnn_conv3x3(const void *X, int cin, int N, int H, int W, int dil, const void *Wt,
                 const float *bias, int relu, void *Y, cudaStream_t stream) {
-    // 32 input channels: the tcgen05 kernel; the single-channel first layer
-    // (1/32 of the work) keeps the WMMA one
     if (cin == kC) return cnn_conv3x3_tc(X, N, H, W, dil, Wt, bias, relu, Y, stream);
-    const long long blocks = (long long)N * H * (W / kSeg);
-    if (relu)
-        conv3x3_kernel<true><<<(unsigned)blocks, 256, 0, stream>>>(
-            (const __nv_bfloat16 *)X, cin, H, W, dil, (const __nv_bfloat16 *)Wt, bias,
-            (__nv_bfloat16 *)Y);
-    else
-        conv3x3_kernel<false><<<(unsigned)blocks, 256, 0, stream>>>(
-            (const __nv_bfloat16 *)X, cin, H, W, dil, (const __nv_bfloat16 *)Wt, bias,
-            (__nv_bfloat16 *)Y);
-    return launched("conv3x3_kernel");
+    // (a GPU's memory holds fewer than 2^31 tiles' outputs of 1 KB)
+    const long long tiles = (long long)N * H * (W / 16);
+    const int grid = (int)std::min<long long>((tiles + 7) / 8, 152 * 8);
+    auto kern = relu ? conv3x3_first_kernel<true> : conv3x3_first_kernel<false>;
+    kern<<<grid, 256, 0, stream>>>((const __nv_bfloat16 *)X, H, W, dil, (unsigned)tiles,
+                                   (const __nv_bfloat16 *)Wt, bias, (__nv_bfloat16 *)Y,
+                                   (uintptr_t)Y % 16 == 0);
+    return launched("conv3x3_first_kernel");
 }
 
 int cnn_relu_backward(const void *Y, void *dY, long long count, cudaStream_t stream) {
@@ -402,18 +506,30 @@ int cnn_relu_backward(const void *Y, void *dY, long long count, cudaStream_t str
 }
 
 int cnn_wgrad(const void *X, int cin, int N, int H, int W, int dil, const void *dZ, float *dW,
-              float *db, cudaStream_t stream) {
-    if (cin == kC) return cnn_wgrad_tc(X, N, H, W, dil, dZ, dW, db, stream);
-    conv3x3_wgrad_kernel<<<2 * 152, 256, 0, stream>>>((const __nv_bfloat16 *)X, cin, N, H, W, dil,
-                                                      (const __nv_bfloat16 *)dZ, dW, db);
-    return launched("conv3x3_wgrad_kernel");
+              float *db, cudaStream_t stream, float *part) {
+    if (cin == kC) return cnn_wgrad_tc(X, N, H, W, dil, dZ, dW, db, stream, part);
+    const int grid = (int)std::min<long long>((long long)N * H * (W / kSeg), kWgradParts);
+    wgrad_first_kernel<<<grid, 256, 0, stream>>>((const __nv_bfloat16 *)X, N, H, W, dil,
+                                                 (const __nv_bfloat16 *)dZ, dW, db, part,
+                                                 (uintptr_t)dZ % 16 == 0);
+    int st = launched("wgrad_first_kernel");
+    if (!st && part) st = cnn_sum_parts(part, grid, kW1Part, kW1Part, dW, stream);
+    return st;
+}
+
+int cnn_sum_parts(const float *part, int rows, int stride, int count, float *out,
+                  cudaStream_t stream) {
+    sum_parts_kernel<<<(count + 31) / 32, 1024, 0, stream>>>(part, rows, stride, count, out);
+    return launched("sum_parts_kernel");
 }
 
 int cnn_band_head(const void *L, int N, int H, int W, int bands, const int32_t *labels,
                   float scale, void *dL, float *loss, int32_t *pred, cudaStream_t stream,
                   float *conf) {
+    const bool wide = ((uintptr_t)L | (uintptr_t)dL) % 16 == 0;
     band_head_kernel<<<N * bands, 256, 0, stream>>>((const __nv_bfloat16 *)L, H, W, bands, labels,
-                                                     scale, (__nv_bfloat16 *)dL, loss, pred, conf);
+                                                     scale, (__nv_bfloat16 *)dL, loss, pred, conf,
+                                                     wide);
     return launched("band_head_kernel");
 }
 
@@ -423,6 +539,22 @@ int cnn_adam(float *p, float *m, float *v, const float *g, int count, float lr, 
     adam_kernel<<<grid_1d(count, 256), 256, 0, stream>>>(p, m, v, g, count, lr, b1, b2, eps, c1,
                                                         c2, (__nv_bfloat16 *)wb);
     return launched("adam_kernel");
+}
+
+int cnn_adam_all(const AdamTensor *t, int tensors, float lr, float b1, float b2, float eps, int step,
+                 cudaStream_t stream) {
+    const float c1 = 1.0f / (1.0f - powf(b1, (float)step));
+    const float c2 = 1.0f / (1.0f - powf(b2, (float)step));
+    AdamTensors a{};
+    int most = 1;
+    if (tensors < 1 || tensors > 8) return set_error(FHTDP_EINVAL, "adam: 1..8 tensors");
+    for (int i = 0; i < tensors; ++i) {
+        a.t[i] = t[i];
+        most = std::max(most, t[i].count);
+    }
+    adam_all_kernel<<<dim3(grid_1d(most, 256), tensors), 256, 0, stream>>>(a, lr, b1, b2, eps, c1,
+                                                                           c2);
+    return launched("adam_all_kernel");
 }
 
 int cnn_bin_windows(const int32_t *pred, int count, int n, int margin, int32_t *win,

@@ -4,6 +4,8 @@
 #include <cstddef>
 #include <cstdint>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include "fhtdp.h"
@@ -59,6 +61,9 @@ void clear_error();
 int launched(const char *what);
 int cuda_status(cudaError_t err, const char *what);
 bool make_shape(int h, int w, int k, Shape *out);
+// cuTensorMapEncodeTiled through the runtime's driver entry point (no
+// link-time dependency on the driver library); null if there is none.
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 // Kernels launched by the API layer.
 template <typename In, typename Acc>

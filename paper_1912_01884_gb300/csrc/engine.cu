@@ -32,9 +32,6 @@
 #include <type_traits>
 #include <vector>
 
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
 #include "engine.cuh"
 
 namespace fhtdp {
@@ -3009,25 +3006,6 @@ RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve 
     L.total = L.data_off + d;
     L.items = items;
     return L;
-}
-
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no
-// link-time dependency on the driver library).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000,
-                                             cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)ptr;
-        else
-            cudaGetLastError();
-    }
-    return fn;
 }
 
 // 2-D uint8 tensor map of an image, box of 128 columns x n rows, zero fill

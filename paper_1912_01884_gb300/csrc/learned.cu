@@ -60,10 +60,10 @@ size_t param_bytes() {
 }
 
 // CNN workspace for n images of h x w pixels (low-resolution ho x wo): the
-// input, the four layer outputs, two gradient buffers, the flipped weights,
-// the FP32 gradients of every layer and the loss.
+// input, the four layer outputs, two gradient buffers, the FP32 gradients of
+// every layer, the loss and the CTAs' sums of a weight gradient.
 struct CnnWs {
-    size_t x0, act[kLayers], g0, g1, wflip, grads[kLayers], loss, total;
+    size_t x0, act[kLayers], g0, g1, grads[kLayers], loss, part, total;
 };
 CnnWs cnn_ws(int n, int h, int w) {
     const size_t px = (size_t)n * (h / 4) * (w / 4);
@@ -79,14 +79,15 @@ CnnWs cnn_ws(int n, int h, int w) {
     o = align256(o + px * kC * 2);
     c.g1 = o;
     o = align256(o + px * kC * 2);
-    c.wflip = o;
-    o = align256(o + 9 * kC * kC * 2);
+    o = align256(o + 9 * kC * kC * 2);   // unused: the gradients keep their place
     for (int l = 0; l < kLayers; ++l) {
         c.grads[l] = o;
         o = align256(o + ((size_t)taps_rows(l) * kC + kC) * 4);
     }
     c.loss = o;
     o = align256(o + 4);
+    c.part = o;
+    o = align256(o + (size_t)kWgradParts * kWgradPart * 4);
     c.total = o;
     return c;
 }
@@ -261,12 +262,9 @@ int fhtdp_cnn_backward(const void *params, const int32_t *labels, int n, int h, 
     for (int l = kLayers - 1; l >= 0 && !st; --l) {
         const LayerOff o = layer_off(l);
         float *dw = (float *)(W + c.grads[l]);
-        st = cuda_status(cudaMemsetAsync(dw, 0, ((size_t)taps_rows(l) * kC + kC) * 4, stream),
-                         "cudaMemsetAsync");
         const void *xin = l == 0 ? (const void *)(W + c.x0) : (const void *)(W + c.act[l - 1]);
-        if (!st)
-            st = cnn_wgrad(xin, l == 0 ? 1 : kC, n, ho, wo, kDil[l], dz, dw,
-                           dw + (size_t)taps_rows(l) * kC, stream);
+        st = cnn_wgrad(xin, l == 0 ? 1 : kC, n, ho, wo, kDil[l], dz, dw,
+                       dw + (size_t)taps_rows(l) * kC, stream, (float *)(W + c.part));
         if (l == 0 || st) break;
         // input gradient: the forward of the flipped and transposed weights,
         // masked by the ReLU of the layer below
@@ -288,18 +286,17 @@ int fhtdp_cnn_step(void *params, const void *ws, int n, int h, int w, float lr, 
     const CnnWs c = cnn_ws(n, h, w);
     char *P = (char *)params;
     const char *W = (const char *)ws;
-    int st = FHTDP_OK;
-    for (int l = 0; l < kLayers && !st; ++l) {
+    AdamTensor t[2 * kLayers];
+    for (int l = 0; l < kLayers; ++l) {
         const LayerOff o = layer_off(l);
         const int nw = taps_rows(l) * kC;
         const float *g = (const float *)(W + c.grads[l]);
-        st = cnn_adam((float *)(P + o.w), (float *)(P + o.mw), (float *)(P + o.vw), g, nw, lr,
-                      0.9f, 0.999f, 1e-8f, step, P + o.w16, stream);
-        if (!st)
-            st = cnn_adam((float *)(P + o.b), (float *)(P + o.mb), (float *)(P + o.vb), g + nw,
-                          kC, lr, 0.9f, 0.999f, 1e-8f, step, nullptr, stream);
+        t[2 * l] = AdamTensor{(float *)(P + o.w), (float *)(P + o.mw), (float *)(P + o.vw), g,
+                              P + o.w16, nw};
+        t[2 * l + 1] = AdamTensor{(float *)(P + o.b), (float *)(P + o.mb), (float *)(P + o.vb),
+                                  g + nw, nullptr, kC};
     }
-    return st;
+    return cnn_adam_all(t, 2 * kLayers, lr, 0.9f, 0.999f, 1e-8f, step, stream);
 }
 
 int fhtdp_learned_plan_create(const fhtdp_image *images, int count, int window_half,
