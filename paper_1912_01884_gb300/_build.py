@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libfhtdp.so")
 
-SOURCES = ["api.cu", "fht_stages.cu", "dp_basic.cu", "angle.cu", "queries.cu", "engine.cu",
+SOURCES = ["api.cu", "fht_stages.cu", "chain.cu", "angle.cu", "queries.cu", "engine.cu",
            "noalloc.cu", "cnn.cu", "conv_tc.cu", "learned.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--fmad=false", "-Xcompiler", "-fPIC",

@@ -7,6 +7,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "chain.cuh"
 #include "cnn.cuh"
 #include "engine.cuh"
 
@@ -105,7 +106,7 @@ size_t fhtdp_hough_bytes(int dtype, int h, int w, int k) {
 size_t fhtdp_fht_workspace_bytes(int dtype, int h, int w, int k) {
     Shape s;
     if (!valid_dtype(dtype) || !make_shape(h, w, k, &s)) return 0;
-    return s.log2n >= 2 ? hough_elems(s) * 4 : 0;
+    return s.log2n >= 2 ? hough_elems(s) * 4 : 0;   // (used by 256-row bands only)
 }
 
 int fhtdp_fht_bands(const void *img, int dtype, int h, int w, int pitch, int k, void *hough,
@@ -122,14 +123,14 @@ int fhtdp_fht_bands(const void *img, int dtype, int h, int w, int pitch, int k, 
                          ws ? ws_bytes : (size_t)0);
     switch (dtype) {
         case FHTDP_U8:
-            return launch_fht_stages<uint8_t, int32_t>((const uint8_t *)img, pitch, s,
-                                                       (int32_t *)hough, (int32_t *)ws, stream);
+            return launch_band_fht<uint8_t, int32_t>((const uint8_t *)img, pitch, s, s.W,
+                                                     (int32_t *)hough, (int32_t *)ws, s.W, stream);
         case FHTDP_I32:
-            return launch_fht_stages<int32_t, int32_t>((const int32_t *)img, pitch, s,
-                                                       (int32_t *)hough, (int32_t *)ws, stream);
+            return launch_band_fht<int32_t, int32_t>((const int32_t *)img, pitch, s, s.W,
+                                                     (int32_t *)hough, (int32_t *)ws, s.W, stream);
         default:
-            return launch_fht_stages<float, float>((const float *)img, pitch, s, (float *)hough,
-                                                   (float *)ws, stream);
+            return launch_band_fht<float, float>((const float *)img, pitch, s, s.W, (float *)hough,
+                                                 (float *)ws, s.W, stream);
     }
 }
 
@@ -140,8 +141,8 @@ int fhtdp_polyline_dp(void *hough, int dtype, int h, int w, int k, int B, cudaSt
     if (!make_shape(h, w, k, &s)) return bad_shape(h, w, k);
     if (B < 0) return set_error(FHTDP_EINVAL, "bend limit B=%d < 0", B);
     if (!hough) return set_error(FHTDP_EINVAL, "null hough pointer");
-    if (dtype == FHTDP_F32) return launch_dp_inplace<float>((float *)hough, s, B, stream);
-    return launch_dp_inplace<int32_t>((int32_t *)hough, s, B, stream);
+    if (dtype == FHTDP_F32) return launch_dp_window<float>((float *)hough, s, B, nullptr, stream);
+    return launch_dp_window<int32_t>((int32_t *)hough, s, B, nullptr, stream);
 }
 
 int fhtdp_backtrack(const void *V, int dtype, int h, int w, int k, int B, int32_t *x_out,
@@ -154,16 +155,16 @@ int fhtdp_backtrack(const void *V, int dtype, int h, int w, int k, int B, int32_
     if (!V || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null V or output pointer");
     if (dtype == FHTDP_F32)
-        return launch_backtrack<float>((const float *)V, s, B, x_out, d_out, (float *)score_out,
-                                       stream);
-    return launch_backtrack<int32_t>((const int32_t *)V, s, B, x_out, d_out,
+        return launch_backtrack<float>((const float *)V, s, B, nullptr, x_out, d_out,
+                                       (float *)score_out, stream);
+    return launch_backtrack<int32_t>((const int32_t *)V, s, B, nullptr, x_out, d_out,
                                      (int32_t *)score_out, stream);
 }
 
 size_t fhtdp_workspace_bytes(int dtype, int h, int w, int k, int B) {
     Shape s;
     if (!valid_dtype(dtype) || !make_shape(h, w, k, &s) || B < 0) return 0;
-    return engine_workspace_bytes(dtype, s, B);
+    return detect_workspace_bytes(dtype, s, B);
 }
 
 int fhtdp_detect_polyline(const void *img, int dtype, int h, int w, int pitch, int k, int B,
@@ -177,11 +178,11 @@ int fhtdp_detect_polyline(const void *img, int dtype, int h, int w, int pitch, i
     if (B < 0) return set_error(FHTDP_EINVAL, "bend limit B=%d < 0", B);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = engine_workspace_bytes(dtype, s, B);
+    size_t need = detect_least_bytes(dtype, s, B);
     if (!ws || ws_bytes < need)
         return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
                          ws ? ws_bytes : (size_t)0);
-    return engine_detect(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, ws_bytes, stream);
+    return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, ws_bytes, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -246,8 +247,8 @@ int fhtdp_polyline_dp_angle(void *hough, int dtype, int h, int w, int k, double 
     if (!hough) return set_error(FHTDP_EINVAL, "null hough pointer");
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
-    if (dtype == FHTDP_F32) return launch_dp_window<float>((float *)hough, s, t, stream);
-    return launch_dp_window<int32_t>((int32_t *)hough, s, t, stream);
+    if (dtype == FHTDP_F32) return launch_dp_window<float>((float *)hough, s, 0, &t, stream);
+    return launch_dp_window<int32_t>((int32_t *)hough, s, 0, &t, stream);
 }
 
 int fhtdp_backtrack_angle(const void *V, int dtype, int h, int w, int k, double gamma,
@@ -261,10 +262,10 @@ int fhtdp_backtrack_angle(const void *V, int dtype, int h, int w, int k, double 
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
     if (dtype == FHTDP_F32)
-        return launch_backtrack_angle<float>((const float *)V, s, t, x_out, d_out,
-                                             (float *)score_out, stream);
-    return launch_backtrack_angle<int32_t>((const int32_t *)V, s, t, x_out, d_out,
-                                           (int32_t *)score_out, stream);
+        return launch_backtrack<float>((const float *)V, s, 0, &t, x_out, d_out,
+                                       (float *)score_out, stream);
+    return launch_backtrack<int32_t>((const int32_t *)V, s, 0, &t, x_out, d_out,
+                                     (int32_t *)score_out, stream);
 }
 
 size_t fhtdp_angle_workspace_bytes(int dtype, int h, int w, int k, int r) {
@@ -291,7 +292,10 @@ int fhtdp_detect_polyline_angle(const void *img, int dtype, int h, int w, int pi
                          ws ? ws_bytes : (size_t)0);
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
-    return detect_angle(img, dtype, pitch, s, r, t, x_out, d_out, score_out, ws, stream);
+    ChainQuery q;
+    q.r = r;
+    q.table = &t;
+    return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
 }
 
 int fhtdp_detect_through_point_angle(const void *img, int dtype, int h, int w, int pitch, int k,
@@ -317,7 +321,11 @@ int fhtdp_detect_through_point_angle(const void *img, int dtype, int h, int w, i
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
     const PointMask pm{j, xp};
-    return detect_angle(img, dtype, pitch, s, r, t, x_out, d_out, score_out, ws, stream, &pm);
+    ChainQuery q;
+    q.r = r;
+    q.table = &t;
+    q.point = &pm;
+    return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -347,7 +355,10 @@ int fhtdp_detect_through_point(const void *img, int dtype, int h, int w, int pit
         return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
                          ws ? ws_bytes : (size_t)0);
     const PointMask pm{j, xp};
-    return detect_through(img, dtype, pitch, s, B, pm, x_out, d_out, score_out, ws, stream);
+    ChainQuery q;
+    q.B = B;
+    q.point = &pm;
+    return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -433,7 +444,7 @@ int fhtdp_transpose(const void *src, int dtype, int h, int w, int pitch, void *d
 size_t fhtdp_horizontal_workspace_bytes(int dtype, int h, int w, int k, int B) {
     Shape s;
     if (!valid_dtype(dtype) || !make_shape(w, h, k, &s) || B < 0) return 0;
-    return transposed_bytes(dtype, h, w) + engine_workspace_bytes(dtype, s, B);
+    return transposed_bytes(dtype, h, w) + detect_workspace_bytes(dtype, s, B);
 }
 
 int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, int pitch, int k,
@@ -452,7 +463,7 @@ int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, i
     if (!img || !y_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
     const size_t tb = transposed_bytes(dtype, h, w);
-    const size_t need = tb + engine_workspace_bytes(dtype, s, B);
+    const size_t need = tb + detect_least_bytes(dtype, s, B);
     if (!ws || ws_bytes < need)
         return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
                          ws ? ws_bytes : (size_t)0);
@@ -471,8 +482,8 @@ int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, i
             st = launch_transpose<float>((const float *)img, h, w, pitch, (float *)ws, tp, stream);
     }
     if (st) return st;
-    return engine_detect(ws, dtype, tp, s, B, y_out, d_out, score_out, (char *)ws + tb,
-                         ws_bytes - tb, stream);
+    return detect_one(ws, dtype, tp, s, B, y_out, d_out, score_out, (char *)ws + tb, ws_bytes - tb,
+                      stream);
 }
 
 // ---------------------------------------------------------------------------

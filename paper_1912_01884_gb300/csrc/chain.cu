@@ -1,0 +1,1079 @@
+// Band FHTs in one pass over the image, and the DP as a chain of column tiles
+// over the stored Hough rows: the path of single images, of the queries and of
+// the standalone calls.
+//
+// One image gives the fused engine (engine.cu) few tiles per band level, and
+// the levels depend on each other: 16 of 152 SMs work on a level of a 2048 x
+// 2048 image, about 15.6 us each.  Here the FHTs, which depend on nothing, run
+// first over the whole chip, and the DP items that remain are small: a tile of
+// 2048 / n columns (16 for bands of 128 rows), so that a level spreads over the
+// chip and the chain advances at the latency of one exchange through L2.
+// CHAIN_FIGURES
+#include <climits>
+#include <type_traits>
+#include <vector>
+
+#include "chain.cuh"
+#include "fht_smem.cuh"
+
+namespace fhtdp {
+namespace {
+
+// ---------------------------------------------------------------------------
+// Band FHT (Sec. 2.1): a block takes kFhtT columns of one sub-band of m <= 128
+// rows, builds the first three levels in registers from the image, merges the
+// rest in shared memory and writes the rows of both slope signs.  int32 and
+// float images run the signs one after the other, the "-" sign on the mirrored
+// strip; uint8 images both at once (fht_smem.cuh).  Bound by shared memory
+// (about 28 bytes a word and sign) and the stores of the rows.
+// FHT_FIGURES
+constexpr int kFhtT = 128, kFhtNT = 512;
+
+template <typename In, typename Acc>
+struct BandFht {
+    static constexpr bool kPacked = sizeof(In) == 1;
+    using Wd = typename std::conditional<kPacked, uint32_t, Acc>::type;
+    const FhtImg &im;
+    const In *base;     // first row of the sub-band
+    int x0, sign;
+    bool aligned;       // rows can be read four pixels at a time
+
+    // Pixel c of a row of the cyclic band: zero left of the image (the "-"
+    // strip never needs the columns it would wrap to: they are padding).
+    __device__ Acc px(const In *row, int c) const {
+        if (c >= im.W) c -= im.W;
+        return c >= 0 && c < im.w ? (Acc)row[c] : Acc(0);
+    }
+    // Pixels c .. c + 3, c a multiple of 4.
+    __device__ uint32_t quad8(const In *row, int c) const {
+        if (aligned && c >= 0 && c + 4 <= im.w) return __ldg((const uint32_t *)(row + c));
+        uint32_t v = 0;
+        for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
+        return v;
+    }
+    __device__ void quad32(const In *row, int c, Acc *v) const {
+        if (aligned && c >= 0 && c + 4 <= im.w) {
+            unpack4(__ldg((const uint4 *)(row + c)), v);
+            return;
+        }
+        for (int j = 0; j < 4; ++j) v[j] = px(row, c + j);
+    }
+    // Words u .. u + N - 1 (u a multiple of 4) of sub-band row y.
+    template <int N>
+    __device__ void words(int y, int u, Wd (&P)[N]) const {
+        constexpr int NW = (N + 3) / 4;
+        const In *row = base + (size_t)y * im.pitch;
+        if constexpr (kPacked) {
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                const uint32_t a = quad8(row, x0 + u + 4 * k);
+                const uint32_t b = quad8(row, x0 + kFhtT - 4 - u - 4 * k);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (4 * k + t < N)
+                        P[4 * k + t] = __byte_perm(a, b, t | (7 - t) << 8) & 0x00ff00ffu;
+            }
+        } else {
+            Acc q[4 * NW];
+#pragma unroll
+            for (int k = 0; k < NW; ++k)
+                quad32(row, sign == 0 ? x0 + u + 4 * k : x0 + kFhtT - 4 - u - 4 * k, q + 4 * k);
+#pragma unroll
+            for (int j = 0; j < N; ++j) P[j] = sign == 0 ? q[j] : q[(j & ~3) + 3 - (j & 3)];
+        }
+    }
+    // Levels 1 and 2 of rows y0 .. y0 + 3: o[s][j], shifts s < 4, words u + j.
+    template <int N>
+    __device__ void levels12(int y0, int u, Wd (&o)[4][N]) const {
+        Wd A[2][N], B[2][N + 2];
+        {
+            Wd p[N], q[N + 1];
+            words<N>(y0, u, p);
+            words<N + 1>(y0 + 1, u, q);
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                A[0][j] = p[j] + q[j];
+                A[1][j] = p[j] + q[j + 1];
+            }
+        }
+        {
+            Wd p[N + 2], q[N + 3];
+            words<N + 2>(y0 + 2, u, p);
+            words<N + 3>(y0 + 3, u, q);
+#pragma unroll
+            for (int j = 0; j < N + 2; ++j) {
+                B[0][j] = p[j] + q[j];
+                B[1][j] = p[j] + q[j + 1];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            o[0][j] = A[0][j] + B[0][j];
+            o[1][j] = A[0][j] + B[0][j + 1];
+            o[2][j] = A[1][j] + B[1][j + 1];
+            o[3][j] = A[1][j] + B[1][j + 2];
+        }
+    }
+    // Levels 1-3 in registers: a task is eight rows and four words.
+    __device__ void first_levels(Wd *F, int pitch) const {
+        const int C4 = (kFhtT + im.m - 8 + 3) / 4, tasks = (im.m / 8) * C4;
+        for (int t = threadIdx.x; t < tasks; t += kFhtNT) {
+            const int g = t / C4, u = 4 * (t - g * C4);
+            Wd lo[4][8], hi[4][4];
+            levels12<8>(8 * g + 4, u, lo);
+            levels12<4>(8 * g, u, hi);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                Wd v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = hi[s >> 1][j] + lo[s >> 1][((s + 1) >> 1) + j];
+                const int r = ((s & 1) << 2) | (s & 2) | (s >> 2);   // brev3(s)
+                *(uint4 *)&F[(size_t)(8 * g + r) * pitch + u] = pack4(v);
+            }
+        }
+    }
+};
+
+template <typename In, typename Acc>
+__global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_constant__ FhtImg one,
+                                                             const FhtImg *__restrict__ many,
+                                                             int count) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    using Tile = BandFht<In, Acc>;
+    using Wd = typename Tile::Wd;
+    int i = 0;
+    if (many) {   // the last image that starts at or before this block
+        int hi = count - 1;
+        while (i < hi) {
+            const int mid = (i + hi + 1) / 2;
+            if (many[mid].item0 <= (int)blockIdx.x) i = mid;
+            else hi = mid - 1;
+        }
+    }
+    const FhtImg &im = many ? many[i] : one;
+    const int item = blockIdx.x - (many ? im.item0 : 0);
+    const int sub = item / im.tiles, x0 = (item - sub * im.tiles) * kFhtT;
+    const int m = im.m, pitch = fht_pitch(m, kFhtT), per_band = im.n / m;
+    const int band = sub / per_band, j = sub - band * per_band;
+    Acc *rows = (Acc *)im.out + ((size_t)band * 2 * im.n + j * m) * im.opitch;
+    const bool vec = im.opitch % 4 == 0 && (uintptr_t)im.out % 16 == 0;
+    Wd *F = (Wd *)smem;
+    Tile t{im, (const In *)im.img + (size_t)sub * m * im.pitch, x0, 0,
+           (uintptr_t)im.img % (4 * sizeof(In)) == 0 && im.pitch % 4 == 0};
+    // four values of shift s, columns x .. x + 3
+    auto store = [&](int sign, int s, int x, const Acc *v) {
+        Acc *dst = rows + ((size_t)sign * im.n + s) * im.opitch + x;
+        if (vec && x + 4 <= im.wout) {
+            *(uint4 *)dst = pack4(v);
+        } else {
+            for (int e = 0; e < 4; ++e)
+                if (x + e < im.wout) dst[e] = v[e];
+        }
+    };
+    for (int sign = 0; sign < (Tile::kPacked ? 1 : 2); ++sign) {
+        t.sign = sign;
+        auto out = [&](int s, int u, const uint4 &q) {
+            Acc v[4];
+            if constexpr (Tile::kPacked) {
+                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = (Acc)(w[e] & 0xffffu);
+                store(0, s, x0 + u, v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = (Acc)(w[3 - e] >> 16);
+                store(1, s, x0 + kFhtT - 4 - u, v);
+            } else {
+                unpack4(q, v);
+                if (sign == 0) {
+                    store(0, s, x0 + u, v);
+                } else {
+                    const Acc r[4] = {v[3], v[2], v[1], v[0]};
+                    store(1, s, x0 + kFhtT - 4 - u, r);
+                }
+            }
+        };
+        int l = 0;   // levels merged
+        if (m >= 8) {
+            t.first_levels(F, pitch);
+            l = 3;
+        } else {
+            const int G = (kFhtT + m + 3) / 4;
+            for (int idx = threadIdx.x; idx < m * G; idx += kFhtNT) {
+                const int y = idx / G, u = 4 * (idx - y * G);
+                Wd v[4];
+                t.template words<4>(y, u, v);
+                *(uint4 *)&F[(size_t)y * pitch + u] = pack4(v);
+            }
+        }
+        __syncthreads();
+        if (l == im.log2m)   // bands of 8 rows: every level done
+            for (int idx = threadIdx.x; idx < m * (kFhtT / 4); idx += kFhtNT) {
+                const int s = idx / (kFhtT / 4), u = 4 * (idx % (kFhtT / 4));
+                out(s, u, *(const uint4 *)&F[(size_t)bit_reverse(s, l) * pitch + u]);
+            }
+        while (l < im.log2m) {
+            const int left = im.log2m - l;
+            if (left > 2) {
+                fht_two_levels<Wd, kFhtNT, false>(F, pitch, m, l, kFhtT, out);
+                l += 2;
+            } else if (left == 2) {
+                fht_two_levels<Wd, kFhtNT, true>(F, pitch, m, l, kFhtT, out);
+                l += 2;
+            } else {
+                fht_level<Wd, kFhtNT, true>(F, pitch, m, l + 1, kFhtT, out);
+                l += 1;
+            }
+            __syncthreads();
+        }
+        __syncthreads();   // F is rewritten for the other sign
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The DP chain (Sec. 2.2-2.3, Eqs. 3-4).  An item is one band b and `cols`
+// continuation columns xn: with V_{b+1}(xn, e) of all displacements e in
+// shared memory, it answers M(xn, d) = max of V_{b+1}(xn, e) over the window
+// of d, and adds it in place to the states that end in its columns,
+// V_b(xn - d, d) = H_b(xn - d, d) + M(xn, d): every state has one owner.  Items
+// come from a queue, band level by band level; an item waits for the tiles of
+// band b + 1 within n - 1 columns of its own (bounded acquire spins), so the
+// queue cannot deadlock: every item waits only for earlier ones, and a block
+// holds at most the item in work and the next one.
+//
+// A thread owns one column and runs of 16 displacements; its Hough values are
+// loaded before the wait, its window maxima come from one block pair of the van
+// Herk / Gil-Werman scheme per run.  States whose link leaves [0, vw), or that
+// the point mask excludes, are never stored as dead: every reader knows them by
+// their place (alive()).  Band 0 folds the lexicographic argmax; the last of
+// its tiles reads the polyline back (Eq. 5).
+// Bound by latency: one flag and one load round trip through L2 per band level.
+constexpr int kDpNT = 256;
+constexpr int kRun = 16;        // displacements of a thread's run
+constexpr int kPadB = 32;       // bend limits up to this read past the range unchecked
+
+struct ChainItem {
+    int image, band, tile, pad;
+};
+
+struct ChainArgs {
+    ChainImg one;
+    const ChainImg *many;      // several images (device), or null
+    const ChainItem *order;    // their queue
+    int items;
+    ChainCtl *ctl;
+    long long wait_cycles;
+    int skip_band, skip_tile;  // test hook: this tile of the first image never publishes
+    int band;                  // >= 0: one launch per band (no queue, no flags)
+    int store0;                // band 0's values are stored (needed after the run)
+    // With use_table the window of d is [tab.lo, tab.hi] instead of |e - d| <= B:
+    // answered from maxima of fixed half-width B0 (no longer than any window
+    // that an end of the range does not clip), wpad dead rows around V.
+    int use_table, B0, wpad;
+    WindowTable tab;
+};
+
+__device__ __forceinline__ int ld_acq(const int *p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_rel(int *p, int v) {
+    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+template <typename Acc>
+__device__ __forceinline__ Acc vmax(Acc a, Acc b) {
+    return a > b ? a : b;
+}
+template <>
+__device__ __forceinline__ float vmax(float a, float b) {
+    return fmaxf(a, b);
+}
+
+// Order-preserving 32-bit image of a value (negative zero counts as zero).
+__device__ __forceinline__ uint32_t vord(int32_t v) { return (uint32_t)v ^ 0x80000000u; }
+__device__ __forceinline__ uint32_t vord(float f) {
+    const uint32_t b = __float_as_uint(f == 0.0f ? 0.0f : f);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+template <typename Acc>
+__device__ __forceinline__ Acc vfrom(uint32_t o);
+template <>
+__device__ __forceinline__ int32_t vfrom<int32_t>(uint32_t o) {
+    return (int32_t)(o ^ 0x80000000u);
+}
+template <>
+__device__ __forceinline__ float vfrom<float>(uint32_t o) {
+    return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+}
+__device__ __forceinline__ int32_t ld_cg(const int32_t *p) { return __ldcg(p); }
+__device__ __forceinline__ float ld_cg(const float *p) { return __ldcg(p); }
+
+// State (x, e) of band b: both vertices inside and not excluded by the point.
+__device__ __forceinline__ bool alive(const ChainImg &im, int b, int x, int e) {
+    const int y = x + e;
+    if (x < 0 || x >= im.vw || y < 0 || y >= im.vw) return false;
+    return im.mask1 != b + 1 || (im.mask_end ? y : x) == im.mask_x;
+}
+template <typename Acc>
+__device__ __forceinline__ Acc *band_rows(const ChainImg &im, int b) {
+    return (Acc *)im.hv + (size_t)b * 2 * im.n * im.pitch;
+}
+// Place of state (x, d) in its band.
+__device__ __forceinline__ int state_at(const ChainImg &im, int x, int d) {
+    return (d < 0 ? im.n - d : d) * im.pitch + x;
+}
+
+// Window maxima of the NOUT displacements from c0 over [c - B, c + B], NOUT <=
+// 2B + 1, into M[at ..]: S[i] is the maximum over [c0 - B + i, c0 + B], G that
+// over [c0 + B + 1, c0 + B + i].  V(e) = v(e) must be readable (or dead) up to
+// c0 + B + NOUT.
+template <int NOUT, typename Acc, typename V>
+__device__ __forceinline__ void span_max(int c0, int B, Acc dead, V v, Acc *M) {
+    Acc run = dead;
+    int e = c0 + B;
+    const int stop = c0 - B + NOUT;
+#pragma unroll 1
+    for (; e - 7 >= stop; e -= 8) {
+        Acc k[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) k[i] = v(e - i);
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) k[i] = vmax(k[i], k[i + 1]);
+        run = vmax(run, vmax(vmax(k[0], k[2]), vmax(k[4], k[6])));
+    }
+#pragma unroll 1
+    for (; e >= stop; --e) run = vmax(run, v(e));
+#pragma unroll
+    for (int i = NOUT - 1; i >= 0; --i) {
+        run = vmax(run, v(c0 - B + i));
+        M[i] = run;
+    }
+    Acc G = dead;
+#pragma unroll
+    for (int i = 0; i + 1 < NOUT; ++i) {
+        G = vmax(G, v(c0 + B + 1 + i));
+        M[i + 1] = vmax(M[i + 1], G);
+    }
+}
+// The run of kRun displacements from c0 (those beyond hi are not read): one
+// block pair, or for windows shorter than the run four outputs or one at a time.
+template <typename Acc, typename V>
+__device__ __forceinline__ void run_max(int c0, int hi, int B, Acc dead, V v, Acc (&M)[kRun]) {
+    if (2 * B + 1 >= kRun) {
+        span_max<kRun, Acc>(c0, B, dead, v, M);
+    } else if (B >= 2) {
+#pragma unroll
+        for (int r = 0; r < kRun; r += 4)
+            if (c0 + r <= hi) span_max<4, Acc>(c0 + r, B, dead, v, M + r);
+    } else {
+#pragma unroll
+        for (int r = 0; r < kRun; ++r)
+            if (c0 + r <= hi) {
+                Acc m = v(c0 + r);
+                if (B) m = vmax(m, vmax(v(c0 + r - 1), v(c0 + r + 1)));
+                M[r] = m;
+            }
+    }
+}
+
+// One warp: the polyline from the argmax key (Eq. 5); every band's window is
+// scanned by the lanes, the smallest displacement of the largest value kept.
+// Key 0 (no admissible polyline): x = -1 everywhere and a dead score.
+template <typename Acc>
+__device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsigned long long key,
+                               int32_t *x_out, int32_t *d_out, Acc *score_out) {
+    const int lane = threadIdx.x & 31, n = im.n, D = 2 * n - 1;
+    if (key == 0) {
+        if (lane == 0) *score_out = Dead<Acc>::value();
+        for (int i = lane; i <= im.k; i += 32) x_out[i] = -1;
+        for (int i = lane; i < im.k; i += 32) d_out[i] = 0;
+        return;
+    }
+    const unsigned lin = 0xffffffffu - (unsigned)(key & 0xffffffffu);
+    int x = (int)(lin / D), d = (int)(lin % D) - (n - 1);
+    if (lane == 0) {
+        x_out[0] = x;
+        d_out[0] = d;
+        *score_out = vfrom<Acc>((uint32_t)(key >> 32));
+    }
+    for (int i = 1; i < im.k; ++i) {
+        x += d;
+        const int lo = args.use_table ? args.tab.lo[d + n - 1] : max(d - im.B, -(n - 1));
+        const int hi = args.use_table ? args.tab.hi[d + n - 1] : min(d + im.B, n - 1);
+        const Acc *V = band_rows<Acc>(im, i);
+        unsigned best = 0;     // order image of the value (0: none)
+        unsigned be = INT_MAX; // its displacement index
+        for (int e = lo + lane; e <= hi; e += 32) {
+            if (!alive(im, i, x, e)) continue;
+            const Acc v = ld_cg(V + state_at(im, x, e));
+            if (v == Dead<Acc>::value()) continue;
+            const unsigned o = vord(v);
+            if (o > best) {
+                best = o;
+                be = e + n - 1;
+            }
+        }
+        const unsigned top = __reduce_max_sync(0xffffffffu, best);
+        const unsigned at = __reduce_min_sync(0xffffffffu, best == top && top ? be : INT_MAX);
+        if (at >= (unsigned)D) {   // only with inconsistent values (a wait gave up)
+            if (lane == 0 && args.ctl) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
+            return;
+        }
+        d = (int)at - (n - 1);
+        if (lane == 0) {
+            x_out[i] = x;
+            d_out[i] = d;
+        }
+    }
+    if (lane == 0) x_out[im.k] = x + d;
+}
+
+template <typename Acc, int C>
+__device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char *smem,
+                           const ChainArgs &args) {
+    constexpr int Q = kDpNT / C;
+    const int n = im.n, D = 2 * n - 1, lo = -(n - 1), hi = n - 1, xn0 = tile * C;
+    const int u = threadIdx.x & (C - 1), q = threadIdx.x / C, xn = xn0 + u;
+    const bool last = band == im.k - 1;   // (only one-band images: V = H)
+    const int B = args.use_table ? args.B0 : im.B;
+    // dead rows around V: bend limits over kPadB check the range instead
+    const int wpad = args.use_table ? args.wpad : B <= kPadB ? B + kRun : 0;
+    const Acc dead = Dead<Acc>::value();
+    Acc *Vt = (Acc *)smem + wpad * C;     // V(e) at row e + n - 1
+    const Acc *Vb = last ? nullptr : band_rows<Acc>(im, band + 1);
+    Acc *Hb = band_rows<Acc>(im, band);
+    // this thread's Hough values (first run), in flight during the wait
+    Acc h[kRun];
+    auto load_h = [&](int c0) {
+#pragma unroll
+        for (int i = 0; i < kRun; ++i) {
+            const int d = c0 + i;
+            h[i] = d <= hi && alive(im, band, xn - d, d) ? ld_cg(Hb + state_at(im, xn - d, d))
+                                                         : Acc(0);
+        }
+    };
+    load_h(lo + kRun * q);
+    for (int i = threadIdx.x; i < 2 * wpad * C; i += kDpNT) {
+        const int r = i / C;
+        Vt[(r < wpad ? r - wpad : r - wpad + D) * C + (i & (C - 1))] = dead;
+    }
+    if (args.band >= 0) {
+        // one launch per band: this one began while the band below still ran
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    } else if (!last && threadIdx.x < 32) {
+        bool ok = true;
+        // bands below k - 1 are items; band k - 1 is complete (unless the test
+        // hook holds a tile of it back)
+        if (band + 1 < im.k - 1 || args.skip_band == band + 1) {
+            const int t0 = max(xn0 - (n - 1), 0) / C;
+            const int t1 = min(xn0 + C - 1 + n - 1, im.vw - 1) / C;
+            for (int t = t0 + (int)threadIdx.x; t <= t1 && ok; t += 32) {
+                if (band + 1 == im.k - 1 && t != args.skip_tile) continue;
+                const int *flag = im.flags + (size_t)(band + 1) * im.tiles + t;
+                const long long begin = clock64();
+                while (ld_acq(flag) == 0) {
+                    const long long spent = clock64() - begin;
+                    if (*(volatile int *)&args.ctl->status != FHTDP_OK ||
+                        spent > args.wait_cycles) {
+                        ok = false;
+                        break;
+                    }
+                    if (spent > 20000) __nanosleep(100);
+                }
+            }
+        }
+        if (!__all_sync(0xffffffffu, ok) && threadIdx.x == 0)
+            atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
+    }
+    if (!last) {
+        __syncthreads();
+        // V_{b+1} of these columns; the thread's own rows
+        for (int c0 = lo + kRun * q; c0 <= hi; c0 += kRun * Q) {
+            Acc v[kRun];
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                const int e = c0 + i;
+                v[i] = e <= hi && alive(im, band + 1, xn, e) ? ld_cg(Vb + state_at(im, xn, e))
+                                                             : dead;
+            }
+#pragma unroll
+            for (int i = 0; i < kRun; ++i)
+                if (c0 + i <= hi) Vt[(c0 + i + n - 1) * C + u] = v[i];
+        }
+        __syncthreads();
+    }
+    const Acc *col = Vt + (n - 1) * C + u;
+    auto vpad = [&](int e) -> Acc { return col[e * C]; };
+    unsigned long long best = 0;
+    const Acc *Mc = nullptr;
+    if (args.use_table && !last) {
+        // centred maxima over [p - B, p + B], p in [lo - B, hi + B]
+        Acc *mc = (Acc *)smem + (D + 2 * wpad) * C + u;   // row p - lo + B
+        const int NC = D + 2 * B;
+        for (int i0 = kRun * q; i0 < NC; i0 += kRun * Q) {
+            Acc M[kRun];
+            run_max<Acc>(i0 + lo - B, hi + B, B, dead, vpad, M);
+#pragma unroll
+            for (int i = 0; i < kRun; ++i)
+                if (i0 + i < NC) mc[(i0 + i) * C] = M[i];
+        }
+        __syncthreads();
+        Mc = mc;
+    }
+    for (int c0 = lo + kRun * q; c0 <= hi; c0 += kRun * Q) {
+        if (c0 != lo + kRun * q) load_h(c0);
+        Acc M[kRun];
+        if (last) {
+        } else if (args.use_table) {
+            const int L = 2 * B + 1;
+            auto mc = [&](int p) -> Acc { return Mc[(p - lo + B) * C]; };
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                if (c0 + i > hi) continue;
+                const int wl = args.tab.lo[c0 + i - lo], wh = args.tab.hi[c0 + i - lo];
+                Acc m = dead;
+                if (wh - wl + 1 >= L) {
+                    m = mc(wh - B);
+#pragma unroll 1
+                    for (int p = wl + B; p < wh - B; p += L) m = vmax(m, mc(p));
+                } else if (wh == hi) {   // clipped: the piece from the other end
+                    m = mc(wl + B);      // reaches only dead rows beyond the range
+                } else if (wl == lo) {
+                    m = mc(wh - B);
+                } else {   // not produced by the host's choice of B0; kept exact
+#pragma unroll 1
+                    for (int e = wl; e <= wh; ++e) m = vmax(m, vpad(e));
+                }
+                M[i] = m;
+            }
+        } else if (wpad) {
+            run_max<Acc>(c0, hi, B, dead, vpad, M);
+        } else {
+            // long windows (2B + 1 > 64): the part common to the run's windows
+            // inside the range, then one value more at either side
+            const int from = max(c0 + kRun - 1 - B, lo), to = min(c0 + B, hi);
+            Acc run = dead;
+#pragma unroll 4
+            for (int e = from; e <= to; ++e) run = vmax(run, vpad(e));
+#pragma unroll
+            for (int i = kRun - 1; i >= 0; --i) {   // down to c0 + i - B
+                const int e = c0 + i - B;
+                if (e >= lo && e < from) run = vmax(run, vpad(e));
+                M[i] = run;
+            }
+            Acc G = dead;
+#pragma unroll
+            for (int i = 1; i < kRun; ++i) {
+                const int e = c0 + i + B;
+                if (e <= hi) G = vmax(G, vpad(e));
+                M[i] = vmax(M[i], G);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kRun; ++i) {
+            const int d = c0 + i, x = xn - d;
+            if (d > hi || !alive(im, band, x, d)) continue;
+            const Acc v = last ? h[i] : M[i] == dead ? dead : h[i] + M[i];
+            if (band != 0 || args.store0) {
+                Hb[state_at(im, x, d)] = v;
+                if (args.band >= 0 && d == 0) Hb[n * im.pitch + x] = v;   // both copies of d = 0
+            }
+            if (band == 0 && v != dead) {
+                const unsigned long long k = ((unsigned long long)vord(v) << 32) |
+                                             (0xffffffffu - (unsigned)(x * D + d + n - 1));
+                best = best > k ? best : k;
+            }
+        }
+    }
+    if (band == 0 && args.band < 0) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+            best = best > other ? best : other;
+        }
+        if ((threadIdx.x & 31) == 0 && best) atomicMax(im.key, best);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            int finished = 0;
+            if (threadIdx.x == 0) {
+                __threadfence();
+                finished = atomicAdd(im.done, 1) == im.tiles - 1;
+            }
+            if (__shfl_sync(0xffffffffu, finished, 0)) {
+                __threadfence();
+                unsigned long long key = 0;
+                if (threadIdx.x == 0) key = atomicAdd(im.key, 0ull);
+                key = __shfl_sync(0xffffffffu, key, 0);
+                chain_readback<Acc>(im, args, key, im.x_out, im.d_out, (Acc *)im.score_out);
+            }
+        }
+    } else if (args.band < 0) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const ChainImg &first = args.many ? args.many[0] : args.one;
+            if (!(band == args.skip_band && tile == args.skip_tile && im.flags == first.flags)) {
+                __threadfence();
+                st_rel(im.flags + (size_t)band * im.tiles + tile, 1);
+            }
+        }
+    }
+    __syncthreads();   // shared memory is rewritten by the next item
+}
+
+// kC: the tile width when all images share it, or 0.
+template <typename Acc, int kC>
+__global__ void __launch_bounds__(kDpNT, 2) dp_chain_kernel(const __grid_constant__ ChainArgs args) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_next;
+    auto item = [&](const ChainImg &im, int band, int tile) {
+        if constexpr (kC != 0) {
+            chain_item<Acc, kC>(im, band, tile, smem, args);
+        } else {
+            switch (im.cols) {
+                case 16: chain_item<Acc, 16>(im, band, tile, smem, args); break;
+                case 32: chain_item<Acc, 32>(im, band, tile, smem, args); break;
+                case 64: chain_item<Acc, 64>(im, band, tile, smem, args); break;
+                case 128: chain_item<Acc, 128>(im, band, tile, smem, args); break;
+                default: chain_item<Acc, 256>(im, band, tile, smem, args); break;
+            }
+        }
+    };
+    if (args.band >= 0) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        item(args.one, args.band, blockIdx.x);
+        return;
+    }
+    if (threadIdx.x == 0) s_next = atomicAdd(&args.ctl->queue, 1);
+    __syncthreads();
+    int cur = s_next;
+    while (cur < args.items) {
+        __syncthreads();
+        // the next item, taken while this one is in work
+        if (threadIdx.x == kDpNT - 1) s_next = atomicAdd(&args.ctl->queue, 1);
+        if (args.many) {
+            const ChainItem it = args.order[cur];
+            item(args.many[it.image], it.band, it.tile);
+        } else {
+            const int lv = cur / args.one.tiles;
+            item(args.one, max(args.one.k - 2 - lv, 0), cur - lv * args.one.tiles);
+        }
+        cur = s_next;   // chain_item ends with a barrier
+    }
+}
+
+// fhtdp_polyline_dp stores dead states: every state of every band whose link
+// leaves [0, vw), and the padding columns.
+template <typename Acc>
+__global__ void dp_dead_kernel(Acc *hv, Shape s) {
+    const int row = blockIdx.x;   // [k][2][n]
+    const int r = row % (2 * s.n), d = r < s.n ? r : s.n - r;
+    Acc *v = hv + (size_t)row * s.W;
+    const int from = max(0, -d), to = min(s.vw, s.vw - d);   // live columns
+    for (int x = threadIdx.x; x < from; x += blockDim.x) v[x] = Dead<Acc>::value();
+    for (int x = max(to, from) + threadIdx.x; x < s.W; x += blockDim.x) v[x] = Dead<Acc>::value();
+}
+
+// The second of two different extreme polylines: the argmax of V_0 over the
+// columns at least sep from the optimum's top vertex (nothing when there is no
+// optimum), then its read-back by the last block.
+template <typename Acc>
+__global__ void __launch_bounds__(256) second_kernel(const __grid_constant__ ChainArgs args,
+                                                     int sep, unsigned long long *key2,
+                                                     int *done2, int32_t *x_out, int32_t *d_out,
+                                                     Acc *score_out) {
+    const ChainImg &im = args.one;
+    const int D = 2 * im.n - 1;
+    const unsigned long long k1 = *im.key;
+    const int x0 = (int)((0xffffffffu - (unsigned)(k1 & 0xffffffffu)) / D);
+    const Acc *V = band_rows<Acc>(im, 0);
+    unsigned long long best = 0;
+    if (k1 != 0)
+        for (int e = blockIdx.x; e < D; e += gridDim.x) {
+            const int d = e - (im.n - 1);
+#pragma unroll 4
+            for (int x = threadIdx.x; x < im.vw; x += blockDim.x) {
+                if (abs(x - x0) < sep || !alive(im, 0, x, d)) continue;
+                const Acc v = ld_cg(V + state_at(im, x, d));
+                if (v == Dead<Acc>::value()) continue;
+                const unsigned long long k = ((unsigned long long)vord(v) << 32) |
+                                             (0xffffffffu - (unsigned)(x * D + e));
+                best = best > k ? best : k;
+            }
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+        best = best > other ? best : other;
+    }
+    if ((threadIdx.x & 31) == 0 && best) atomicMax(key2, best);
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    int finished = 0;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        finished = atomicAdd(done2, 1) == (int)gridDim.x - 1;
+    }
+    if (!__shfl_sync(0xffffffffu, finished, 0)) return;
+    __threadfence();
+    unsigned long long key = 0;
+    if (threadIdx.x == 0) key = atomicAdd(key2, 0ull);
+    key = __shfl_sync(0xffffffffu, key, 0);
+    chain_readback<Acc>(im, args, key, x_out, d_out, score_out);
+}
+
+// fhtdp_backtrack has no workspace: one cluster of eight blocks finds the
+// argmax of V_0 (its dead states hold dead values), folded through distributed
+// shared memory, and its first warp reads the polyline back.
+constexpr int kBtBlocks = 8, kBtNT = 1024;
+template <typename Acc>
+__global__ void __cluster_dims__(kBtBlocks, 1, 1) __launch_bounds__(kBtNT)
+    backtrack_kernel(const __grid_constant__ ChainArgs args) {
+    __shared__ unsigned long long s_warp[kBtNT / 32], s_block[kBtBlocks];
+    const ChainImg &im = args.one;
+    const int D = 2 * im.n - 1;
+    // (the cluster barriers: every block runs before its shared memory is
+    // written from another, and the blocks' maxima are there before they are read)
+    auto cluster_sync = [] {
+        asm volatile("barrier.cluster.arrive;\n barrier.cluster.wait;" ::: "memory");
+    };
+    cluster_sync();
+    const Acc *V = band_rows<Acc>(im, 0);
+    unsigned long long best = 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int e = blockIdx.x * (kBtNT / 32) + warp; e < D; e += kBtBlocks * kBtNT / 32) {
+        const Acc *row = V + state_at(im, 0, e - (im.n - 1));
+#pragma unroll 8
+        for (int x = lane; x < im.vw; x += 32) {
+            const Acc v = ld_cg(row + x);
+            if (v == Dead<Acc>::value()) continue;
+            const unsigned long long k = ((unsigned long long)vord(v) << 32) |
+                                         (0xffffffffu - (unsigned)(x * D + e));
+            best = best > k ? best : k;
+        }
+    }
+    auto warp_max = [](unsigned long long k) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
+            k = k > other ? k : other;
+        }
+        return k;
+    };
+    best = warp_max(best);
+    if (lane == 0) s_warp[warp] = best;
+    __syncthreads();
+    if (warp == 0) {
+        best = warp_max(s_warp[lane]);
+        if (lane == 0) {
+            uint32_t slot;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                         : "=r"(slot)
+                         : "r"((uint32_t)__cvta_generic_to_shared(&s_block[blockIdx.x])));
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(slot), "l"(best) : "memory");
+        }
+    }
+    __syncthreads();
+    cluster_sync();
+    if (blockIdx.x == 0 && warp == 0)
+        chain_readback<Acc>(im, args, warp_max(lane < kBtBlocks ? s_block[lane] : 0ull), im.x_out,
+                            im.d_out, (Acc *)im.score_out);
+}
+
+// ---------------------------------------------------------------------------
+// Host side.
+int device_sms() {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 152;
+}
+
+// Columns of a DP item: 2048 / n, so that 256 threads cover its displacements
+// in runs of 16.
+int chain_cols(int n) { return n >= 128 ? 16 : n <= 8 ? 256 : 2048 / n; }
+
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+thread_local int g_skip_band = -1, g_skip_tile = -1;
+thread_local long long g_skip_wait = 0;
+
+size_t dp_smem(int n, int cols, int wpad, bool table) {
+    return (size_t)(2 * n - 1 + 2 * wpad) * cols * 4 * (table ? 2 : 1);
+}
+
+// The window table's cover: the shortest window that no end of the range clips
+// (else the shortest of all), made odd, is 2 B0 + 1.
+void chain_table(ChainArgs &a, const WindowTable &t) {
+    const int n = t.n, D = 2 * n - 1;
+    int L0 = D, L0c = D;
+    bool any = false;
+    for (int i = 0; i < D; ++i) {
+        const int len = t.hi[i] - t.lo[i] + 1;
+        L0c = len < L0c ? len : L0c;
+        if (t.lo[i] > -(n - 1) && t.hi[i] < n - 1) {
+            L0 = any && L0 < len ? L0 : len;
+            any = true;
+        }
+    }
+    if (!any) L0 = L0c;
+    if (L0 < 1) L0 = 1;
+    a.use_table = 1;
+    a.tab = t;
+    a.B0 = ((L0 % 2 ? L0 : L0 - 1) - 1) / 2;
+    a.wpad = 2 * a.B0 + kRun;
+}
+
+// Shared memory of one image's items.
+size_t item_smem(const ChainArgs &a, const ChainImg &im) {
+    const int wpad = a.use_table ? a.wpad : im.B <= kPadB ? im.B + kRun : 0;
+    return dp_smem(im.n, im.cols, wpad, a.use_table != 0);
+}
+
+template <typename Acc, int kC>
+int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cudaStream_t stream) {
+    auto kern = dp_chain_kernel<Acc, kC>;
+    int st = cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)smem),
+                         "cudaFuncSetAttribute");
+    if (st) return st;
+    if (a.band < 0) {
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kDpNT, smem);
+        const int most = device_sms() * (per_sm < 1 ? 1 : per_sm);
+        blocks = blocks < most ? blocks : most;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kDpNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    st = cuda_status(cudaLaunchKernelEx(&cfg, kern, a), "dp_chain_kernel");
+    if (st) return st;
+    return launched("dp_chain_kernel");
+}
+template <typename Acc>
+int launch_chain_cols(const ChainArgs &a, int cols, size_t smem, int blocks, bool dependent,
+                      cudaStream_t stream) {
+    switch (cols) {
+        case 16: return launch_chain<Acc, 16>(a, smem, blocks, dependent, stream);
+        case 32: return launch_chain<Acc, 32>(a, smem, blocks, dependent, stream);
+        case 64: return launch_chain<Acc, 64>(a, smem, blocks, dependent, stream);
+        case 128: return launch_chain<Acc, 128>(a, smem, blocks, dependent, stream);
+        default: return launch_chain<Acc, 256>(a, smem, blocks, dependent, stream);
+    }
+}
+
+FhtImg fht_img(const void *img, long long pitch, const Shape &s, int wout, void *out, int opitch) {
+    FhtImg f{};
+    f.img = img;
+    f.pitch = pitch;
+    f.w = s.w;
+    f.W = s.W;
+    f.wout = wout;
+    f.n = s.n;
+    f.m = s.n < 128 ? s.n : 128;
+    while ((1 << f.log2m) < f.m) ++f.log2m;
+    f.out = out;
+    f.opitch = opitch;
+    f.tiles = (wout + kFhtT - 1) / kFhtT;
+    f.subs = s.h / f.m;
+    return f;
+}
+
+size_t fht_smem_bytes(int m) { return (size_t)m * fht_pitch(m, kFhtT) * 4; }
+
+template <typename In, typename Acc>
+int launch_fht_img(const FhtImg &f, cudaStream_t stream) {
+    const size_t smem = fht_smem_bytes(f.m);
+    int st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<In, Acc>,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)smem),
+                         "cudaFuncSetAttribute");
+    if (st) return st;
+    fht_band_kernel<In, Acc><<<(unsigned)(f.tiles * f.subs), kFhtNT, smem, stream>>>(f, nullptr, 1);
+    return launched("fht_band_kernel");
+}
+
+}  // namespace
+
+// The Hough rows of an image, columns [0, wout) of rows `opitch` apart, into
+// hough; tmp (the same size) is needed for 256-row bands only, whose last level
+// is a pass of its own.
+template <typename In, typename Acc>
+int launch_band_fht(const In *img, long long pitch, const Shape &s, int wout, Acc *hough, Acc *tmp,
+                    int opitch, cudaStream_t stream) {
+    if (s.n == 1) return launch_fht_single_row<In, Acc>(img, pitch, s, wout, hough, opitch, stream);
+    Acc *first = s.n > 128 ? tmp : hough;
+    // the last level reads columns modulo W
+    int st = launch_fht_img<In, Acc>(fht_img(img, pitch, s, s.n > 128 ? s.W : wout, first, opitch),
+                                     stream);
+    if (!st && s.n > 128) st = launch_fht_last<Acc>(tmp, s, wout, hough, opitch, stream);
+    return st;
+}
+template int launch_band_fht<uint8_t, int32_t>(const uint8_t *, long long, const Shape &, int,
+                                               int32_t *, int32_t *, int, cudaStream_t);
+template int launch_band_fht<int32_t, int32_t>(const int32_t *, long long, const Shape &, int,
+                                               int32_t *, int32_t *, int, cudaStream_t);
+template int launch_band_fht<float, float>(const float *, long long, const Shape &, int, float *,
+                                           float *, int, cudaStream_t);
+
+template <typename Acc>
+int launch_dp_window(Acc *hv, const Shape &s, int B, const WindowTable *t, cudaStream_t stream) {
+    dp_dead_kernel<Acc><<<(unsigned)(s.k * 2 * s.n), 128, 0, stream>>>(hv, s);
+    int st = launched("dp_dead_kernel");
+    ChainArgs a{};
+    a.one.hv = hv;
+    a.one.n = s.n;
+    a.one.k = s.k;
+    a.one.vw = s.vw;
+    a.one.pitch = s.W;
+    a.one.B = B < 2 * s.n - 2 ? B : 2 * s.n - 2;
+    a.one.cols = chain_cols(s.n);
+    a.one.tiles = (s.vw + a.one.cols - 1) / a.one.cols;
+    a.skip_band = a.skip_tile = -1;
+    a.store0 = 1;
+    if (t) chain_table(a, *t);
+    const size_t smem = item_smem(a, a.one);
+    for (int b = s.k - 2; b >= 0 && !st; --b) {
+        a.band = b;
+        st = launch_chain_cols<Acc>(a, a.one.cols, smem, a.one.tiles, b != s.k - 2, stream);
+    }
+    return st;
+}
+template int launch_dp_window<int32_t>(int32_t *, const Shape &, int, const WindowTable *,
+                                       cudaStream_t);
+template int launch_dp_window<float>(float *, const Shape &, int, const WindowTable *,
+                                     cudaStream_t);
+
+template <typename Acc>
+int launch_backtrack(const Acc *V, const Shape &s, int B, const WindowTable *t, int32_t *x_out,
+                     int32_t *d_out, Acc *score_out, cudaStream_t stream) {
+    ChainArgs a{};
+    a.one.hv = const_cast<Acc *>(V);
+    a.one.n = s.n;
+    a.one.k = s.k;
+    a.one.vw = s.vw;
+    a.one.pitch = s.W;
+    a.one.B = B < 2 * s.n - 2 ? B : 2 * s.n - 2;
+    a.one.x_out = x_out;
+    a.one.d_out = d_out;
+    a.one.score_out = score_out;
+    if (t) chain_table(a, *t);
+    backtrack_kernel<Acc><<<kBtBlocks, kBtNT, 0, stream>>>(a);
+    return launched("backtrack_kernel");
+}
+template int launch_backtrack<int32_t>(const int32_t *, const Shape &, int, const WindowTable *,
+                                       int32_t *, int32_t *, int32_t *, cudaStream_t);
+template int launch_backtrack<float>(const float *, const Shape &, int, const WindowTable *,
+                                     int32_t *, int32_t *, float *, cudaStream_t);
+
+void chain_inject(int band, int tile, long long wait_cycles) {
+    g_skip_band = band;
+    g_skip_tile = tile;
+    g_skip_wait = wait_cycles;
+}
+
+ChainLayout chain_layout(const Shape &s, bool smooth) {
+    ChainLayout L{};
+    L.cols = chain_cols(s.n);
+    L.tiles = (s.vw + L.cols - 1) / L.cols;
+    // rows a multiple of 128 bytes apart, long enough for the cyclic width of
+    // 256-row bands
+    L.pitch = ((s.n > 128 ? s.W : s.vw) + 31) & ~31;
+    size_t o = sizeof(ChainCtl);
+    L.key = o;   // key, done; key, done of the second polyline
+    o += 256;
+    L.flags = o;
+    o = up256(o + (size_t)s.k * L.tiles * 4);
+    L.zero = o;
+    const size_t rows = up256((size_t)s.k * 2 * s.n * L.pitch * 4);
+    L.rows = o;
+    o += rows;
+    L.second = o;
+    if (s.n > 128) o += rows;
+    else if (smooth) o = up256(o + (size_t)s.h * s.w * 4);
+    L.total = o;
+    return L;
+}
+
+namespace {
+template <typename In, typename Acc>
+int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q, int32_t *x_out,
+                   int32_t *d_out, Acc *score_out, char *ws, cudaStream_t stream) {
+    const ChainLayout L = chain_layout(s, q.r > 0);
+    int st = cuda_status(cudaMemsetAsync(ws, 0, L.zero, stream), "cudaMemsetAsync");
+    Acc *rows = (Acc *)(ws + L.rows), *second = (Acc *)(ws + L.second);
+    if (st) return st;
+    if (q.r > 0) {
+        // the smoothed image: where the rows will be (256-row bands, whose
+        // first pass writes `second`), else in `second`
+        Acc *smooth = s.n > 128 ? rows : second;
+        st = launch_gauss_rows<In, Acc>(img, pitch, s.h, s.w, q.r, smooth, stream);
+        if (!st)
+            st = launch_band_fht<Acc, Acc>(smooth, s.w, s, s.vw, rows, second, L.pitch, stream);
+    } else {
+        st = launch_band_fht<In, Acc>(img, pitch, s, s.vw, rows, second, L.pitch, stream);
+    }
+    if (st) return st;
+    ChainArgs a{};
+    ChainImg &im = a.one;
+    im.hv = rows;
+    im.n = s.n;
+    im.k = s.k;
+    im.vw = s.vw;
+    im.pitch = L.pitch;
+    im.B = q.B < 2 * s.n - 2 ? q.B : 2 * s.n - 2;
+    im.cols = L.cols;
+    im.tiles = L.tiles;
+    im.flags = (int *)(ws + L.flags);
+    im.key = (unsigned long long *)(ws + L.key);
+    im.done = (int *)(ws + L.key + 8);
+    im.x_out = x_out;
+    im.d_out = d_out;
+    im.score_out = score_out;
+    if (q.point) {
+        im.mask1 = (q.point->j < s.k ? q.point->j : s.k - 1) + 1;
+        im.mask_x = q.point->xp;
+        im.mask_end = q.point->j == s.k ? 1 : 0;
+    }
+    a.items = L.tiles * (s.k > 1 ? s.k - 1 : 1);
+    a.ctl = (ChainCtl *)ws;
+    a.wait_cycles = 4000000000LL;   // about two seconds
+    a.skip_band = a.skip_tile = -1;
+    if (g_skip_band >= 0) {
+        a.skip_band = g_skip_band;
+        a.skip_tile = g_skip_tile;
+        a.wait_cycles = g_skip_wait;
+    }
+    g_skip_band = g_skip_tile = -1;
+    a.band = -1;
+    a.store0 = q.sep > 0;
+    if (q.table) chain_table(a, *q.table);
+    st = launch_chain_cols<Acc>(a, im.cols, item_smem(a, im), a.items, false, stream);
+    if (!st && q.sep > 0) {
+        const int D = 2 * s.n - 1;
+        second_kernel<Acc><<<D, 256, 0, stream>>>(
+            a, q.sep, (unsigned long long *)(ws + L.key + 16), (int *)(ws + L.key + 24),
+            x_out + s.k + 1, d_out + s.k, score_out + 1);
+        st = launched("second_kernel");
+    }
+    return st;
+}
+}  // namespace
+
+int chain_detect(const void *img, int dtype, int pitch, const Shape &s, const ChainQuery &q,
+                 int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream) {
+    if (dtype == FHTDP_U8)
+        return chain_detect_t<uint8_t, int32_t>((const uint8_t *)img, pitch, s, q, x_out, d_out,
+                                                (int32_t *)score_out, (char *)ws, stream);
+    if (dtype == FHTDP_I32)
+        return chain_detect_t<int32_t, int32_t>((const int32_t *)img, pitch, s, q, x_out, d_out,
+                                                (int32_t *)score_out, (char *)ws, stream);
+    return chain_detect_t<float, float>((const float *)img, pitch, s, q, x_out, d_out,
+                                        (float *)score_out, (char *)ws, stream);
+}
+
+}  // namespace fhtdp

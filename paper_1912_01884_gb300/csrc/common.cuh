@@ -47,8 +47,6 @@ struct WindowTable {
 };
 // Fills *t for bands of n rows; false if gamma is negative or not finite.
 bool make_angle_table(int n, double gamma, WindowTable *t);
-// The integer bend limit as a table (B >= 0).
-void make_bend_table(int n, int B, WindowTable *t);
 
 // Largest half-width of the row smoothing (binomial weights up to C(24, 12)).
 constexpr int kMaxGaussR = 12;
@@ -66,68 +64,48 @@ bool make_shape(int h, int w, int k, Shape *out);
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 // Kernels launched by the API layer.
+//
+// The Hough rows of an image (chain.cu): columns [0, wout) of [k][2][n] rows
+// `opitch` values apart; tmp (the same size) for 256-row bands only.
 template <typename In, typename Acc>
-int launch_fht_stages(const In *img, int pitch, const Shape &s, Acc *hough, Acc *tmp,
-                      cudaStream_t stream);
+int launch_band_fht(const In *img, long long pitch, const Shape &s, int wout, Acc *hough, Acc *tmp,
+                    int opitch, cudaStream_t stream);
+// Its passes of their own (fht_stages.cu): one-row bands, and the last level of
+// 256-row bands from the level of their 128-row halves.
+template <typename In, typename Acc>
+int launch_fht_single_row(const In *img, long long pitch, const Shape &s, int wout, Acc *out,
+                          int opitch, cudaStream_t stream);
+template <typename Acc>
+int launch_fht_last(const Acc *src, const Shape &s, int wout, Acc *dst, int opitch,
+                    cudaStream_t stream);
 // A point P = (xp, j*n) on the upper border of band j (j = k: the bottom
-// border) that the polyline must pass (Subproblems 2-3): the DP marks every
-// state whose vertex on that border is not xp dead.
+// border) that the polyline must pass (Subproblems 2-3): the DP treats every
+// state whose vertex on that border is not xp as dead.
 struct PointMask {
     int j, xp;
 };
+// The DP in place over Hough rows s.W apart, one launch per band, with the bend
+// limit B or (t non-null) a window table.
 template <typename Acc>
-int launch_dp_inplace(Acc *hv, const Shape &s, int B, cudaStream_t stream,
-                      const PointMask *pm = nullptr);
-// The read-back with a grid-wide argmax into *key (zero before the call).
+int launch_dp_window(Acc *hv, const Shape &s, int B, const WindowTable *t, cudaStream_t stream);
 template <typename Acc>
-int launch_backtrack_key(const Acc *V, const Shape &s, int B, unsigned long long *key,
-                         int32_t *x_out, int32_t *d_out, Acc *score_out, cudaStream_t stream);
-template <typename Acc>
-int launch_backtrack(const Acc *V, const Shape &s, int B, int32_t *x_out, int32_t *d_out,
-                     Acc *score_out, cudaStream_t stream);
+int launch_backtrack(const Acc *V, const Shape &s, int B, const WindowTable *t, int32_t *x_out,
+                     int32_t *d_out, Acc *score_out, cudaStream_t stream);
 
-// The main problem (Sec. 2.3): row smoothing into a dense [h][w] image
-// (int32 for integer images, float for float ones), the DP with bend-angle
-// windows, and its read-backs.
+// The main problem (Sec. 2.3), step 1: row smoothing into a dense [h][w] image
+// (int32 for integer images, float for float ones).
 template <typename In, typename Acc>
 int launch_gauss_rows(const In *img, int pitch, int h, int w, int r, Acc *out,
                       cudaStream_t stream);
-// The band FHTs of the smoothed image without storing it: the smoothing is
-// fused into the first level (bands of n >= 2 rows).
-template <typename In, typename Acc>
-int launch_fht_stages_gauss(const In *img, int pitch, const Shape &s, int r, Acc *hough, Acc *tmp,
-                            cudaStream_t stream);
-// The DP over any window table (int32 or float values), in place, with an
-// optional through-point restriction.
-template <typename Acc>
-int launch_dp_window(Acc *hv, const Shape &s, const WindowTable &t, cudaStream_t stream,
-                     const PointMask *pm = nullptr);
-template <typename Acc>
-int launch_backtrack_angle_key(const Acc *V, const Shape &s, const WindowTable &t,
-                               unsigned long long *key, int32_t *x_out, int32_t *d_out,
-                               Acc *score_out, cudaStream_t stream);
-template <typename Acc>
-int launch_backtrack_angle(const Acc *V, const Shape &s, const WindowTable &t, int32_t *x_out,
-                           int32_t *d_out, Acc *score_out, cudaStream_t stream);
 size_t angle_workspace_bytes(const Shape &s);
 size_t through_workspace_bytes(const Shape &s);
-// The method with vertices anywhere in [0, W) (s.vw = W): the standalone
-// FHT, DP and key read-back.
+// The method with vertices anywhere in [0, W) (s.vw = W).
 int detect_padded(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
                   int32_t *d_out, void *score_out, void *ws, cudaStream_t stream);
 // Two different extreme polylines: the optimum and the best one whose top
 // vertex is at least sep columns from the optimum's (outputs [2][...]).
 int detect_two(const void *img, int dtype, int pitch, const Shape &s, int B, int sep,
                int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream);
-// The argmax of V_0 over the columns at least sep from the top vertex that
-// key1 encodes (nothing when key1 is 0), into *key2 (zero before the call).
-template <typename Acc>
-int launch_argmax_apart(const Acc *V, const Shape &s, const unsigned long long *key1, int sep,
-                        unsigned long long *key2, cudaStream_t stream);
-// The read-back from an argmax key with the integer bend limit.
-template <typename Acc>
-int launch_readback_key(const Acc *V, const Shape &s, int B, const unsigned long long *key,
-                        int32_t *x_out, int32_t *d_out, Acc *score_out, cudaStream_t stream);
 // dst[x][y] = src[y][x] (Sec. 3, Fig. 7: mostly horizontal curves).
 template <typename T>
 int launch_transpose(const T *src, int h, int w, int pitch, T *dst, int dpitch,

@@ -32,6 +32,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "chain.cuh"
 #include "engine.cuh"
 
 namespace fhtdp {
@@ -3210,39 +3211,6 @@ LaunchArgs base_args(const RunLayout &L, char *ws, int count) {
     return args;
 }
 
-int run_fallback(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-                 int32_t *d_out, void *score_out, void *ws, cudaStream_t stream) {
-    // 256-row bands: the standalone FHT (two levels per pass), the in-place
-    // DP with per-column window maxima and the read-back from a grid-wide
-    // argmax.
-    int st = cuda_status(cudaMemsetAsync(ws, 0, sizeof(Ctl), stream), "cudaMemsetAsync");
-    if (st) return st;
-    size_t hough = (size_t)s.k * 2 * s.n * s.W;
-    char *base = (char *)ws + 256;
-    // The argmax key sits in the cleared control block, after its fields.
-    unsigned long long *key = (unsigned long long *)((char *)ws + 128);
-    static_assert(sizeof(Ctl) >= 136, "control block holds the argmax key");
-    if (dtype == FHTDP_F32) {
-        float *H = (float *)base, *tmp = H + hough;
-        st = launch_fht_stages<float, float>((const float *)img, pitch, s, H, tmp, stream);
-        if (!st) st = launch_dp_inplace<float>(H, s, B, stream);
-        if (!st)
-            st = launch_backtrack_key<float>(H, s, B, key, x_out, d_out, (float *)score_out,
-                                             stream);
-        return st;
-    }
-    int32_t *H = (int32_t *)base, *tmp = H + hough;
-    if (dtype == FHTDP_U8)
-        st = launch_fht_stages<uint8_t, int32_t>((const uint8_t *)img, pitch, s, H, tmp, stream);
-    else
-        st = launch_fht_stages<int32_t, int32_t>((const int32_t *)img, pitch, s, H, tmp, stream);
-    if (!st) st = launch_dp_inplace<int32_t>(H, s, B, stream);
-    if (!st)
-        st = launch_backtrack_key<int32_t>(H, s, B, key, x_out, d_out, (int32_t *)score_out,
-                                           stream);
-    return st;
-}
-
 ImgPlan single_plan(int dtype, const void *img, int pitch, const Shape &s, int B,
                     int32_t *x_out, int32_t *d_out, void *score_out) {
     ImgPlan p{};
@@ -3453,17 +3421,27 @@ std::vector<Item> queue_order(const std::vector<ImgPlan> &imgs, long long target
                 : queue_grouped(imgs, target);
 }
 
-size_t engine_workspace_bytes(int dtype, const Shape &s, int B) {
-    const size_t standalone = 256 + 2 * (size_t)s.k * 2 * s.n * s.W * 4;
-    if (s.n > kMaxBandFused) {
-        // Either path may run, depending on the image's alignment.
-        const int Bc = B < 2 * s.n - 2 ? B : 2 * s.n - 2;
-        if (dtype != FHTDP_U8 || Bc > 127) return standalone;
-        std::vector<ImgPlan> one{single_plan(dtype, nullptr, 16, s, B, nullptr, nullptr, nullptr)};
-        return std::max(standalone, plan_layout(one, false).total);
-    }
-    std::vector<ImgPlan> one{single_plan(dtype, nullptr, s.w, s, B, nullptr, nullptr, nullptr)};
+// The fused engine's workspace for one uint8 image (0 when it does not take
+// the image, whatever its alignment).
+static size_t engine_one_bytes(int dtype, const Shape &s, int B) {
+    const int Bc = B < 2 * s.n - 2 ? B : 2 * s.n - 2;
+    if (dtype != FHTDP_U8 || (s.n > kMaxBandFused && Bc > 127)) return 0;
+    std::vector<ImgPlan> one{single_plan(dtype, nullptr, s.n > kMaxBandFused ? 16 : s.w, s, B,
+                                         nullptr, nullptr, nullptr)};
     return plan_layout(one, false).total;
+}
+
+size_t detect_workspace_bytes(int dtype, const Shape &s, int B) {
+    return std::max(chain_layout(s, false).total, engine_one_bytes(dtype, s, B));
+}
+
+// uint8 images with bands of at most 128 rows run on the engine where the
+// workspace is too small for the chain.
+size_t detect_least_bytes(int dtype, const Shape &s, int B) {
+    const size_t chain = chain_layout(s, false).total;
+    return dtype == FHTDP_U8 && s.n <= kMaxBandFused
+               ? std::min(chain, engine_one_bytes(dtype, s, B))
+               : chain;
 }
 
 // The point of Subproblems 2-3 on an image's plan: the states of band j whose
@@ -3474,33 +3452,28 @@ void set_point(ImgPlan &p, int j, int xp) {
     p.mask_end = j == p.s.k ? 1 : 0;
 }
 
-// The fused engine masks the point's band in V after forming it, which band
-// 0 never stores: points on borders 1..k of uint8 images with at least two
-// bands of at most 128 rows.
-bool engine_takes_point(int dtype, const Shape &s, int j) {
-    return dtype == FHTDP_U8 && s.n <= kMaxBandFused && s.k >= 2 && j >= 1;
-}
-
-int engine_detect(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-                  int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream,
-                  const PointMask *pm) {
-    (void)ws_bytes;
-    std::vector<ImgPlan> one{single_plan(dtype, img, pitch, s, B, x_out, d_out, score_out)};
-    if (pm) {
-        if (!engine_takes_point(dtype, s, pm->j) || one[0].kind != 0)
-            return set_error(FHTDP_EINVAL, "the fused engine takes points on uint8 images only");
-        set_point(one[0], pm->j, pm->xp);
+// One image takes the chain (chain.cu): the engine's 128-column tiles leave
+// most of the chip idle on one image (2048 x 2048: CHAIN_VS_ENGINE).  The engine
+// needs a sixth of the workspace, and takes uint8 images whose workspace is
+// too small for the chain (the built-in scratch of the no-allocation call).
+int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
+               int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream) {
+    if (ws_bytes >= chain_layout(s, false).total) {
+        LaunchArgs hook{};
+        hook.skip_band = -1;
+        consume_injection(&hook);
+        if (hook.skip_band >= 0) chain_inject(hook.skip_band, hook.skip_tile, hook.wait_cycles);
+        ChainQuery q;
+        q.B = B;
+        return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
     }
-    if (s.n > kMaxBandFused && one[0].kind != 1)
-        return run_fallback(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, stream);
+    std::vector<ImgPlan> one{single_plan(dtype, img, pitch, s, B, x_out, d_out, score_out)};
     RunLayout L = plan_layout(one, false);
     char *base = (char *)ws;
     int st = cuda_status(cudaMemsetAsync(base, 0, L.zero_bytes, stream), "cudaMemsetAsync");
     if (st) return st;
     LaunchArgs args = base_args(L, base, 1);
     args.one = make_desc(one[0], L, base, dtype);
-    if (one[0].kind == 1 && (!args.one.use_tma || !args.one.use_mtma))
-        return set_error(FHTDP_ECUDA, "tensor maps of a 256-row-band image could not be encoded");
     args.many = nullptr;
     args.order = nullptr;
     return dispatch(dtype, L.max_h, args, L.max_n, L.multi_tile, stream);
@@ -3531,27 +3504,6 @@ void set_table(LaunchArgs &args, const WindowTable &t) {
     args.tab = t;
     args.B0 = (Lp - 1) / 2;
     args.wpad = std::max(kWPad, (2 * args.B0 + 16 + 1) & ~1);
-}
-
-// One int32 / float image with the bend-angle windows of table t (bands of 2
-// to 128 rows): the persistent engine with window-table DP items.
-int engine_detect_table(const void *img, int dtype, int pitch, const Shape &s,
-                        const WindowTable &t, int32_t *x_out, int32_t *d_out, void *score_out,
-                        void *ws, cudaStream_t stream) {
-    if (dtype == FHTDP_U8 || s.n < 2 || s.n > kMaxBandFused || t.n != s.n)
-        return set_error(FHTDP_EINVAL, "window-table engine: int32 / float, bands of 2..128 rows");
-    std::vector<ImgPlan> one{single_plan(dtype, img, pitch, s, 2 * s.n - 2, x_out, d_out,
-                                         score_out)};
-    RunLayout L = plan_layout(one, false);
-    char *base = (char *)ws;
-    int st = cuda_status(cudaMemsetAsync(base, 0, L.zero_bytes, stream), "cudaMemsetAsync");
-    if (st) return st;
-    LaunchArgs args = base_args(L, base, 1);
-    args.one = make_desc(one[0], L, base, dtype);
-    args.many = nullptr;
-    args.order = nullptr;
-    set_table(args, t);
-    return dispatch(dtype, L.max_h, args, L.max_n, false, stream);
 }
 
 int engine_status(const void *ws, cudaStream_t stream) {
@@ -3602,7 +3554,7 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
     // Scratch of the standalone path: up to kSideLanes lanes, each a stream
     // that runs its images one after the other on its own slice.
     size_t sep = 0;
-    for (auto &p : plan->separate) sep = std::max(sep, engine_workspace_bytes(dtype, p.s, p.io.B));
+    for (auto &p : plan->separate) sep = std::max(sep, chain_layout(p.s, false).total);
     plan->sep_bytes = align_up(sep, 256);
     plan->lanes = (int)std::min<size_t>(kSideLanes, plan->separate.size());
     plan->separate_off = align_up(plan->reserve, 256);
@@ -3690,9 +3642,11 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
         for (size_t i = 0; i < plan->separate.size() && !st; ++i) {
             const ImgPlan &p = plan->separate[i];
             const int l = (int)(i % plan->lanes);
-            st = run_fallback(p.io.img, plan->dtype, p.io.pitch, p.s, p.io.B, p.io.x_out,
-                              p.io.d_out, p.io.score_out,
-                              base + plan->separate_off + plan->sep_bytes * l, plan->side[l]);
+            ChainQuery q;
+            q.B = p.io.B;
+            st = chain_detect(p.io.img, plan->dtype, p.io.pitch, p.s, q, p.io.x_out, p.io.d_out,
+                              p.io.score_out, base + plan->separate_off + plan->sep_bytes * l,
+                              plan->side[l]);
         }
     }
     if (!plan->imgs.empty() && !st) {
@@ -3919,7 +3873,7 @@ int batch_points(BatchPlan *plan, void *ws, const int32_t *points, cudaStream_t 
         const ImgPlan &p = plan->imgs[i];
         if (j < 0) continue;
         if (j > p.s.k || xp < 0 || xp >= p.s.w || p.kind != 0 ||
-            !engine_takes_point(plan->dtype, p.s, j))
+            plan->dtype != FHTDP_U8 || p.s.n > kMaxBandFused || p.s.k < 2 || j < 1)
             return set_error(FHTDP_EINVAL,
                              "point %zu: border 1..k, column 0..w-1, uint8, 2+ bands of <= 128 rows",
                              i);

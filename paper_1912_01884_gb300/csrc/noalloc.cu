@@ -62,7 +62,7 @@ extern "C" int fhtdp_detect_polyline_noalloc(const void *img, int dtype, int h, 
     if (B < 0) return set_error(FHTDP_EINVAL, "bend limit B=%d < 0", B);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    const size_t need = engine_workspace_bytes(dtype, s, B);
+    const size_t need = detect_least_bytes(dtype, s, B);
     if (need > kNoallocScratchBytes)
         return set_error(FHTDP_EWORKSPACE,
                          "this image needs %zu bytes of scratch; the built-in scratch of "
@@ -72,8 +72,8 @@ extern "C" int fhtdp_detect_polyline_noalloc(const void *img, int dtype, int h, 
     void *ws = nullptr;
     int st = scratch_on_current_device(&ws);
     if (st) return st;
-    return engine_detect(img, dtype, pitch, s, B, x_out, d_out, score_out, ws,
-                         kNoallocScratchBytes, stream);
+    return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, kNoallocScratchBytes,
+                      stream);
 }
 
 // The status word of the last fhtdp_detect_polyline_noalloc run sits in the
