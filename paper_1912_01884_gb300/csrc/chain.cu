@@ -21,13 +21,13 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // Band FHT (Sec. 2.1): a block takes kFhtT columns of one sub-band of m <= 128
-// rows, builds the first three levels in registers from the image, merges the
+// rows, builds the first two levels in registers from the image, merges the
 // rest in shared memory and writes the rows of both slope signs.  int32 and
 // float images run the signs one after the other, the "-" sign on the mirrored
 // strip; uint8 images both at once (fht_smem.cuh).  Bound by shared memory
 // (about 28 bytes a word and sign) and the stores of the rows.
 // FHT_FIGURES
-constexpr int kFhtT = 128, kFhtNT = 512;
+constexpr int kFhtT = 128, kFhtNT = 1024;
 
 template <typename In, typename Acc>
 struct BandFht {
@@ -35,7 +35,7 @@ struct BandFht {
     using Wd = typename std::conditional<kPacked, uint32_t, Acc>::type;
     const FhtImg &im;
     const In *base;     // first row of the sub-band
-    int x0, sign;
+    int x0;
     bool aligned;       // rows can be read four pixels at a time
 
     // Pixel c of a row of the cyclic band: zero left of the image (the "-"
@@ -44,92 +44,99 @@ struct BandFht {
         if (c >= im.W) c -= im.W;
         return c >= 0 && c < im.w ? (Acc)row[c] : Acc(0);
     }
-    // Pixels c .. c + 3, c a multiple of 4.
+    // Pixels c .. c + 3, c a multiple of 4; kInside: all in the image and
+    // aligned.
+    template <bool kInside>
     __device__ uint32_t quad8(const In *row, int c) const {
-        if (aligned && c >= 0 && c + 4 <= im.w) return __ldg((const uint32_t *)(row + c));
+        if (kInside || (aligned && c >= 0 && c + 4 <= im.w))
+            return __ldg((const uint32_t *)(row + c));
         uint32_t v = 0;
+#pragma unroll 1
         for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
         return v;
     }
+    template <bool kInside>
     __device__ void quad32(const In *row, int c, Acc *v) const {
-        if (aligned && c >= 0 && c + 4 <= im.w) {
+        if (kInside || (aligned && c >= 0 && c + 4 <= im.w)) {
             unpack4(__ldg((const uint4 *)(row + c)), v);
             return;
         }
-        for (int j = 0; j < 4; ++j) v[j] = px(row, c + j);
+        v[0] = px(row, c);
+        v[1] = px(row, c + 1);
+        v[2] = px(row, c + 2);
+        v[3] = px(row, c + 3);
     }
-    // Words u .. u + N - 1 (u a multiple of 4) of sub-band row y.
-    template <int N>
+    // Words u .. u + N - 1 (u a multiple of 4) of sub-band row y; kSign 1: of
+    // the mirrored strip (packed words hold both).
+    template <bool kInside, int kSign, int N>
     __device__ void words(int y, int u, Wd (&P)[N]) const {
         constexpr int NW = (N + 3) / 4;
         const In *row = base + (size_t)y * im.pitch;
-        if constexpr (kPacked) {
 #pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                const uint32_t a = quad8(row, x0 + u + 4 * k);
-                const uint32_t b = quad8(row, x0 + kFhtT - 4 - u - 4 * k);
+        for (int k = 0; k < NW; ++k) {
+            const int cp = x0 + u + 4 * k, cm = x0 + kFhtT - 4 - u - 4 * k;
+            if constexpr (kPacked) {
+                const uint32_t a = quad8<kInside>(row, cp), b = quad8<kInside>(row, cm);
 #pragma unroll
                 for (int t = 0; t < 4; ++t)
                     if (4 * k + t < N)
                         P[4 * k + t] = __byte_perm(a, b, t | (7 - t) << 8) & 0x00ff00ffu;
+            } else {
+                Acc q[4];
+                quad32<kInside>(row, kSign == 0 ? cp : cm, q);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (4 * k + t < N) P[4 * k + t] = q[kSign == 0 ? t : 3 - t];
             }
-        } else {
-            Acc q[4 * NW];
-#pragma unroll
-            for (int k = 0; k < NW; ++k)
-                quad32(row, sign == 0 ? x0 + u + 4 * k : x0 + kFhtT - 4 - u - 4 * k, q + 4 * k);
-#pragma unroll
-            for (int j = 0; j < N; ++j) P[j] = sign == 0 ? q[j] : q[(j & ~3) + 3 - (j & 3)];
         }
     }
-    // Levels 1 and 2 of rows y0 .. y0 + 3: o[s][j], shifts s < 4, words u + j.
-    template <int N>
-    __device__ void levels12(int y0, int u, Wd (&o)[4][N]) const {
-        Wd A[2][N], B[2][N + 2];
-        {
-            Wd p[N], q[N + 1];
-            words<N>(y0, u, p);
-            words<N + 1>(y0 + 1, u, q);
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                A[0][j] = p[j] + q[j];
-                A[1][j] = p[j] + q[j + 1];
-            }
-        }
-        {
-            Wd p[N + 2], q[N + 3];
-            words<N + 2>(y0 + 2, u, p);
-            words<N + 3>(y0 + 3, u, q);
-#pragma unroll
-            for (int j = 0; j < N + 2; ++j) {
-                B[0][j] = p[j] + q[j];
-                B[1][j] = p[j] + q[j + 1];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            o[0][j] = A[0][j] + B[0][j];
-            o[1][j] = A[0][j] + B[0][j + 1];
-            o[2][j] = A[1][j] + B[1][j + 1];
-            o[3][j] = A[1][j] + B[1][j + 2];
-        }
-    }
-    // Levels 1-3 in registers: a task is eight rows and four words.
+    // Levels 1 and 2 in registers: a task is four rows and four words.
+    template <bool kInside, int kSign>
     __device__ void first_levels(Wd *F, int pitch) const {
-        const int C4 = (kFhtT + im.m - 8 + 3) / 4, tasks = (im.m / 8) * C4;
+        const int C4 = (kFhtT + im.m - 4 + 3) / 4, tasks = (im.m / 4) * C4;
         for (int t = threadIdx.x; t < tasks; t += kFhtNT) {
-            const int g = t / C4, u = 4 * (t - g * C4);
-            Wd lo[4][8], hi[4][4];
-            levels12<8>(8 * g + 4, u, lo);
-            levels12<4>(8 * g, u, hi);
+            const int g = t / C4, u = 4 * (t - g * C4), y0 = 4 * g;
+            Wd B[2][6];   // the lower pair's shifts 0 and 1
+            {
+                Wd p[6], q[7];
+                words<kInside, kSign>(y0 + 2, u, p);
+                words<kInside, kSign>(y0 + 3, u, q);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                Wd v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = hi[s >> 1][j] + lo[s >> 1][((s + 1) >> 1) + j];
-                const int r = ((s & 1) << 2) | (s & 2) | (s >> 2);   // brev3(s)
-                *(uint4 *)&F[(size_t)(8 * g + r) * pitch + u] = pack4(v);
+                for (int j = 0; j < 6; ++j) {
+                    B[0][j] = p[j] + q[j];
+                    B[1][j] = p[j] + q[j + 1];
+                }
             }
+            Wd p[4], q[5], o[4][4];
+            words<kInside, kSign>(y0, u, p);
+            words<kInside, kSign>(y0 + 1, u, q);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const Wd a0 = p[j] + q[j], a1 = p[j] + q[j + 1];
+                o[0][j] = a0 + B[0][j];
+                o[1][j] = a0 + B[0][j + 1];
+                o[2][j] = a1 + B[1][j + 1];
+                o[3][j] = a1 + B[1][j + 2];
+            }
+            Wd *row = F + (size_t)y0 * pitch + u;   // shift s to row brev2(s)
+            *(uint4 *)row = pack4(o[0]);
+            *(uint4 *)(row + 2 * pitch) = pack4(o[1]);
+            *(uint4 *)(row + pitch) = pack4(o[2]);
+            *(uint4 *)(row + 3 * pitch) = pack4(o[3]);
+        }
+    }
+    // The strip's 128-byte lines requested into L2 at once: the register levels
+    // would wait for DRAM task by task.
+    __device__ void prefetch() const {
+        const int lo = max(x0 - (im.m - 1), 0), hi = min(x0 + kFhtT + im.m - 1, im.w);
+        if (lo >= hi) return;
+        const int lines = ((hi - lo) * (int)sizeof(In) + 127) / 128 + 1;
+        for (int i = threadIdx.x; i < im.m * lines; i += kFhtNT) {
+            const int y = i / lines;
+            const uintptr_t a = (uintptr_t)(base + (size_t)y * im.pitch + lo);
+            const uintptr_t end = (uintptr_t)(base + (size_t)y * im.pitch + hi);
+            const uintptr_t line = (a & ~(uintptr_t)127) + (uintptr_t)(i - y * lines) * 128;
+            if (line < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
         }
     }
 };
@@ -158,8 +165,11 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
     Acc *rows = (Acc *)im.out + ((size_t)band * 2 * im.n + j * m) * im.opitch;
     const bool vec = im.opitch % 4 == 0 && (uintptr_t)im.out % 16 == 0;
     Wd *F = (Wd *)smem;
-    Tile t{im, (const In *)im.img + (size_t)sub * m * im.pitch, x0, 0,
-           (uintptr_t)im.img % (4 * sizeof(In)) == 0 && im.pitch % 4 == 0};
+    const Tile t{im, (const In *)im.img + (size_t)sub * m * im.pitch, x0,
+                 (uintptr_t)im.img % (4 * sizeof(In)) == 0 && im.pitch % 4 == 0};
+    t.prefetch();
+    // every column that a task reads (the widest: u + 8 past the strip's words)
+    const bool inside = t.aligned && x0 >= m + 8 && x0 + kFhtT + m + 8 <= im.w;
     // four values of shift s, columns x .. x + 3
     auto store = [&](int sign, int s, int x, const Acc *v) {
         Acc *dst = rows + ((size_t)sign * im.n + s) * im.opitch + x;
@@ -171,7 +181,6 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
         }
     };
     for (int sign = 0; sign < (Tile::kPacked ? 1 : 2); ++sign) {
-        t.sign = sign;
         auto out = [&](int s, int u, const uint4 &q) {
             Acc v[4];
             if constexpr (Tile::kPacked) {
@@ -193,20 +202,27 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
             }
         };
         int l = 0;   // levels merged
-        if (m >= 8) {
-            t.first_levels(F, pitch);
-            l = 3;
+        if (m >= 4) {
+            if (inside) {
+                if (Tile::kPacked || sign == 0) t.template first_levels<true, 0>(F, pitch);
+                else t.template first_levels<true, 1>(F, pitch);
+            } else {
+                if (Tile::kPacked || sign == 0) t.template first_levels<false, 0>(F, pitch);
+                else t.template first_levels<false, 1>(F, pitch);
+            }
+            l = 2;
         } else {
             const int G = (kFhtT + m + 3) / 4;
             for (int idx = threadIdx.x; idx < m * G; idx += kFhtNT) {
                 const int y = idx / G, u = 4 * (idx - y * G);
                 Wd v[4];
-                t.template words<4>(y, u, v);
+                if (sign == 0) t.template words<false, 0>(y, u, v);
+                else t.template words<false, 1>(y, u, v);
                 *(uint4 *)&F[(size_t)y * pitch + u] = pack4(v);
             }
         }
         __syncthreads();
-        if (l == im.log2m)   // bands of 8 rows: every level done
+        if (l == im.log2m)   // bands of 4 rows: every level done
             for (int idx = threadIdx.x; idx < m * (kFhtT / 4); idx += kFhtNT) {
                 const int s = idx / (kFhtT / 4), u = 4 * (idx % (kFhtT / 4));
                 out(s, u, *(const uint4 *)&F[(size_t)bit_reverse(s, l) * pitch + u]);
@@ -240,15 +256,15 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
 // queue cannot deadlock: every item waits only for earlier ones, and a block
 // holds at most the item in work and the next one.
 //
-// A thread owns one column and runs of 16 displacements; its Hough values are
+// A thread owns one column and runs of 8 displacements; its Hough values are
 // loaded before the wait, its window maxima come from one block pair of the van
 // Herk / Gil-Werman scheme per run.  States whose link leaves [0, vw), or that
 // the point mask excludes, are never stored as dead: every reader knows them by
 // their place (alive()).  Band 0 folds the lexicographic argmax; the last of
 // its tiles reads the polyline back (Eq. 5).
 // Bound by latency: one flag and one load round trip through L2 per band level.
-constexpr int kDpNT = 256;
-constexpr int kRun = 16;        // displacements of a thread's run
+constexpr int kDpNT = 512;
+constexpr int kRun = 8;         // displacements of a thread's run
 constexpr int kPadB = 32;       // bend limits up to this read past the range unchecked
 
 struct ChainItem {
@@ -319,9 +335,10 @@ template <typename Acc>
 __device__ __forceinline__ Acc *band_rows(const ChainImg &im, int b) {
     return (Acc *)im.hv + (size_t)b * 2 * im.n * im.pitch;
 }
-// Place of state (x, d) in its band.
+// Place of state (x, d) in its band; d = 0 is stored in both halves, and the
+// chain uses the copy in the "-" half.
 __device__ __forceinline__ int state_at(const ChainImg &im, int x, int d) {
-    return (d < 0 ? im.n - d : d) * im.pitch + x;
+    return (d <= 0 ? im.n - d : d) * im.pitch + x;
 }
 
 // Window maxima of the NOUT displacements from c0 over [c - B, c + B], NOUT <=
@@ -443,14 +460,31 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     Acc *Vt = (Acc *)smem + wpad * C;     // V(e) at row e + n - 1
     const Acc *Vb = last ? nullptr : band_rows<Acc>(im, band + 1);
     Acc *Hb = band_rows<Acc>(im, band);
+    // A run of kRun displacements lies in one half (bands of at least kRun
+    // rows), so its states are a fixed step apart: along a column for V, along a
+    // diagonal (fixed end column) for H.  Live states of an unmasked band: both
+    // vertices inside.
+    const bool in = xn < im.vw, whole = n >= kRun;
+    const bool mask_h = im.mask1 == band + 1, mask_v = im.mask1 == band + 2;
     // this thread's Hough values (first run), in flight during the wait
     Acc h[kRun];
     auto load_h = [&](int c0) {
+        if (whole && !mask_h) {
+            const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
+            const Acc *p = Hb + state_at(im, xn - c0, c0);
 #pragma unroll
-        for (int i = 0; i < kRun; ++i) {
-            const int d = c0 + i;
-            h[i] = d <= hi && alive(im, band, xn - d, d) ? ld_cg(Hb + state_at(im, xn - d, d))
-                                                         : Acc(0);
+            for (int i = 0; i < kRun; ++i) {
+                const bool ok = in && (unsigned)(xn - c0 - i) < (unsigned)im.vw && c0 + i <= hi;
+                h[i] = ok ? ld_cg(p + i * step) : Acc(0);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                const int d = c0 + i;
+                h[i] = d <= hi && alive(im, band, xn - d, d)
+                           ? ld_cg(Hb + state_at(im, xn - d, d))
+                           : Acc(0);
+            }
         }
     };
     load_h(lo + kRun * q);
@@ -491,11 +525,22 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         // V_{b+1} of these columns; the thread's own rows
         for (int c0 = lo + kRun * q; c0 <= hi; c0 += kRun * Q) {
             Acc v[kRun];
+            if (whole && !mask_v) {
+                const int step = c0 <= 0 ? -im.pitch : im.pitch;
+                const Acc *p = Vb + state_at(im, xn, c0);
 #pragma unroll
-            for (int i = 0; i < kRun; ++i) {
-                const int e = c0 + i;
-                v[i] = e <= hi && alive(im, band + 1, xn, e) ? ld_cg(Vb + state_at(im, xn, e))
-                                                             : dead;
+                for (int i = 0; i < kRun; ++i) {
+                    const bool ok =
+                        in && (unsigned)(xn + c0 + i) < (unsigned)im.vw && c0 + i <= hi;
+                    v[i] = ok ? ld_cg(p + i * step) : dead;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kRun; ++i) {
+                    const int e = c0 + i;
+                    v[i] = e <= hi && alive(im, band + 1, xn, e) ? ld_cg(Vb + state_at(im, xn, e))
+                                                                 : dead;
+                }
             }
 #pragma unroll
             for (int i = 0; i < kRun; ++i)
@@ -570,6 +615,15 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 M[i] = vmax(M[i], G);
             }
         }
+        if (whole && !mask_h && band != 0 && args.band < 0) {
+            const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
+            Acc *p = Hb + state_at(im, xn - c0, c0);
+#pragma unroll
+            for (int i = 0; i < kRun; ++i)
+                if (in && (unsigned)(xn - c0 - i) < (unsigned)im.vw && c0 + i <= hi)
+                    p[i * step] = M[i] == dead ? dead : h[i] + M[i];
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < kRun; ++i) {
             const int d = c0 + i, x = xn - d;
@@ -577,7 +631,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
             const Acc v = last ? h[i] : M[i] == dead ? dead : h[i] + M[i];
             if (band != 0 || args.store0) {
                 Hb[state_at(im, x, d)] = v;
-                if (args.band >= 0 && d == 0) Hb[n * im.pitch + x] = v;   // both copies of d = 0
+                if (args.band >= 0 && d == 0) Hb[x] = v;   // both copies of d = 0
             }
             if (band == 0 && v != dead) {
                 const unsigned long long k = ((unsigned long long)vord(v) << 32) |
@@ -786,8 +840,8 @@ int device_sms() {
     return v > 0 ? v : 152;
 }
 
-// Columns of a DP item: 2048 / n, so that 256 threads cover its displacements
-// in runs of 16.
+// Columns of a DP item: 2048 / n, so that 512 threads cover its displacements
+// in runs of 8.
 int chain_cols(int n) { return n >= 128 ? 16 : n <= 8 ? 256 : 2048 / n; }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
