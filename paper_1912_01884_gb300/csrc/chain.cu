@@ -20,14 +20,14 @@ namespace fhtdp {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Band FHT (Sec. 2.1): a block takes kFhtT columns of one sub-band of m <= 128
+// Band FHT (Sec. 2.1): a block takes T columns of one sub-band of m <= 128
 // rows, builds the first two levels in registers from the image, merges the
 // rest in shared memory and writes the rows of both slope signs.  int32 and
 // float images run the signs one after the other, the "-" sign on the mirrored
 // strip; uint8 images both at once (fht_smem.cuh).  Bound by shared memory
 // (about 28 bytes a word and sign) and the stores of the rows.
 // FHT_FIGURES
-constexpr int kFhtT = 128, kFhtNT = 1024;
+constexpr int kFhtNT = 1024;
 
 template <typename In, typename Acc>
 struct BandFht {
@@ -74,7 +74,7 @@ struct BandFht {
         const In *row = base + (size_t)y * im.pitch;
 #pragma unroll
         for (int k = 0; k < NW; ++k) {
-            const int cp = x0 + u + 4 * k, cm = x0 + kFhtT - 4 - u - 4 * k;
+            const int cp = x0 + u + 4 * k, cm = x0 + im.T - 4 - u - 4 * k;
             if constexpr (kPacked) {
                 const uint32_t a = quad8<kInside>(row, cp), b = quad8<kInside>(row, cm);
 #pragma unroll
@@ -93,7 +93,7 @@ struct BandFht {
     // Levels 1 and 2 in registers: a task is four rows and four words.
     template <bool kInside, int kSign>
     __device__ void first_levels(Wd *F, int pitch) const {
-        const int C4 = (kFhtT + im.m - 4 + 3) / 4, tasks = (im.m / 4) * C4;
+        const int C4 = (im.T + im.m - 4 + 3) / 4, tasks = (im.m / 4) * C4;
         for (int t = threadIdx.x; t < tasks; t += kFhtNT) {
             const int g = t / C4, u = 4 * (t - g * C4), y0 = 4 * g;
             Wd B[2][6];   // the lower pair's shifts 0 and 1
@@ -128,7 +128,7 @@ struct BandFht {
     // The strip's 128-byte lines requested into L2 at once: the register levels
     // would wait for DRAM task by task.
     __device__ void prefetch() const {
-        const int lo = max(x0 - (im.m - 1), 0), hi = min(x0 + kFhtT + im.m - 1, im.w);
+        const int lo = max(x0 - (im.m - 1), 0), hi = min(x0 + im.T + im.m - 1, im.w);
         if (lo >= hi) return;
         const int lines = ((hi - lo) * (int)sizeof(In) + 127) / 128 + 1;
         for (int i = threadIdx.x; i < im.m * lines; i += kFhtNT) {
@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
     }
     const FhtImg &im = many ? many[i] : one;
     const int item = blockIdx.x - (many ? im.item0 : 0);
-    const int sub = item / im.tiles, x0 = (item - sub * im.tiles) * kFhtT;
-    const int m = im.m, pitch = fht_pitch(m, kFhtT), per_band = im.n / m;
+    const int sub = item / im.tiles, T = im.T, x0 = (item - sub * im.tiles) * T;
+    const int m = im.m, pitch = fht_pitch(m, T), per_band = im.n / m;
     const int band = sub / per_band, j = sub - band * per_band;
     Acc *rows = (Acc *)im.out + ((size_t)band * 2 * im.n + j * m) * im.opitch;
     const bool vec = im.opitch % 4 == 0 && (uintptr_t)im.out % 16 == 0;
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
                  (uintptr_t)im.img % (4 * sizeof(In)) == 0 && im.pitch % 4 == 0};
     t.prefetch();
     // every column that a task reads (the widest: u + 8 past the strip's words)
-    const bool inside = t.aligned && x0 >= m + 8 && x0 + kFhtT + m + 8 <= im.w;
+    const bool inside = t.aligned && x0 >= m + 8 && x0 + T + m + 8 <= im.w;
     // four values of shift s, columns x .. x + 3
     auto store = [&](int sign, int s, int x, const Acc *v) {
         Acc *dst = rows + ((size_t)sign * im.n + s) * im.opitch + x;
@@ -190,14 +190,14 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
                 store(0, s, x0 + u, v);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = (Acc)(w[3 - e] >> 16);
-                store(1, s, x0 + kFhtT - 4 - u, v);
+                store(1, s, x0 + T - 4 - u, v);
             } else {
                 unpack4(q, v);
                 if (sign == 0) {
                     store(0, s, x0 + u, v);
                 } else {
                     const Acc r[4] = {v[3], v[2], v[1], v[0]};
-                    store(1, s, x0 + kFhtT - 4 - u, r);
+                    store(1, s, x0 + T - 4 - u, r);
                 }
             }
         };
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
             }
             l = 2;
         } else {
-            const int G = (kFhtT + m + 3) / 4;
+            const int G = (T + m + 3) / 4;
             for (int idx = threadIdx.x; idx < m * G; idx += kFhtNT) {
                 const int y = idx / G, u = 4 * (idx - y * G);
                 Wd v[4];
@@ -223,20 +223,20 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
         }
         __syncthreads();
         if (l == im.log2m)   // bands of 4 rows: every level done
-            for (int idx = threadIdx.x; idx < m * (kFhtT / 4); idx += kFhtNT) {
-                const int s = idx / (kFhtT / 4), u = 4 * (idx % (kFhtT / 4));
+            for (int idx = threadIdx.x; idx < m * (T / 4); idx += kFhtNT) {
+                const int s = idx / (T / 4), u = 4 * (idx % (T / 4));
                 out(s, u, *(const uint4 *)&F[(size_t)bit_reverse(s, l) * pitch + u]);
             }
         while (l < im.log2m) {
             const int left = im.log2m - l;
             if (left > 2) {
-                fht_two_levels<Wd, kFhtNT, false>(F, pitch, m, l, kFhtT, out);
+                fht_two_levels<Wd, kFhtNT, false>(F, pitch, m, l, T, out);
                 l += 2;
             } else if (left == 2) {
-                fht_two_levels<Wd, kFhtNT, true>(F, pitch, m, l, kFhtT, out);
+                fht_two_levels<Wd, kFhtNT, true>(F, pitch, m, l, T, out);
                 l += 2;
             } else {
-                fht_level<Wd, kFhtNT, true>(F, pitch, m, l + 1, kFhtT, out);
+                fht_level<Wd, kFhtNT, true>(F, pitch, m, l + 1, T, out);
                 l += 1;
             }
             __syncthreads();
@@ -288,11 +288,14 @@ struct ChainArgs {
     WindowTable tab;
 };
 
-__device__ __forceinline__ int ld_acq(const int *p) {
+// The flags are polled with relaxed loads, one fence after the last; a poll
+// reads nothing else (another load would double its round trip).
+__device__ __forceinline__ int ld_relaxed(const int *p) {
     int v;
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void st_rel(int *p, int v) {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -446,10 +449,14 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
     if (lane == 0) x_out[im.k] = x + d;
 }
 
+// Words between the rows of V: with 16 columns a warp holds two runs, eight
+// rows apart, and 18 words put them into different banks.
+__host__ __device__ constexpr int row_words(int cols) { return cols == 16 ? 18 : cols; }
+
 template <typename Acc, int C>
 __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char *smem,
                            const ChainArgs &args) {
-    constexpr int Q = kDpNT / C;
+    constexpr int Q = kDpNT / C, R = row_words(C);
     const int n = im.n, D = 2 * n - 1, lo = -(n - 1), hi = n - 1, xn0 = tile * C;
     const int u = threadIdx.x & (C - 1), q = threadIdx.x / C, xn = xn0 + u;
     const bool last = band == im.k - 1;   // (only one-band images: V = H)
@@ -457,7 +464,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     // dead rows around V: bend limits over kPadB check the range instead
     const int wpad = args.use_table ? args.wpad : B <= kPadB ? B + kRun : 0;
     const Acc dead = Dead<Acc>::value();
-    Acc *Vt = (Acc *)smem + wpad * C;     // V(e) at row e + n - 1
+    Acc *Vt = (Acc *)smem + wpad * R;     // V(e) at row e + n - 1
     const Acc *Vb = last ? nullptr : band_rows<Acc>(im, band + 1);
     Acc *Hb = band_rows<Acc>(im, band);
     // A run of kRun displacements lies in one half (bands of at least kRun
@@ -490,7 +497,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     load_h(lo + kRun * q);
     for (int i = threadIdx.x; i < 2 * wpad * C; i += kDpNT) {
         const int r = i / C;
-        Vt[(r < wpad ? r - wpad : r - wpad + D) * C + (i & (C - 1))] = dead;
+        Vt[(r < wpad ? r - wpad : r - wpad + D) * R + (i & (C - 1))] = dead;
     }
     if (args.band >= 0) {
         // one launch per band: this one began while the band below still ran
@@ -506,16 +513,17 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 if (band + 1 == im.k - 1 && t != args.skip_tile) continue;
                 const int *flag = im.flags + (size_t)(band + 1) * im.tiles + t;
                 const long long begin = clock64();
-                while (ld_acq(flag) == 0) {
+                while (ld_relaxed(flag) == 0) {
                     const long long spent = clock64() - begin;
-                    if (*(volatile int *)&args.ctl->status != FHTDP_OK ||
-                        spent > args.wait_cycles) {
+                    if (spent < 20000) continue;   // (about 10 us)
+                    if (ld_relaxed(&args.ctl->status) != FHTDP_OK || spent > args.wait_cycles) {
                         ok = false;
                         break;
                     }
-                    if (spent > 20000) __nanosleep(100);
+                    __nanosleep(100);
                 }
             }
+            fence_gpu();
         }
         if (!__all_sync(0xffffffffu, ok) && threadIdx.x == 0)
             atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
@@ -544,24 +552,24 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
             }
 #pragma unroll
             for (int i = 0; i < kRun; ++i)
-                if (c0 + i <= hi) Vt[(c0 + i + n - 1) * C + u] = v[i];
+                if (c0 + i <= hi) Vt[(c0 + i + n - 1) * R + u] = v[i];
         }
         __syncthreads();
     }
-    const Acc *col = Vt + (n - 1) * C + u;
-    auto vpad = [&](int e) -> Acc { return col[e * C]; };
+    const Acc *col = Vt + (n - 1) * R + u;
+    auto vpad = [&](int e) -> Acc { return col[e * R]; };
     unsigned long long best = 0;
     const Acc *Mc = nullptr;
     if (args.use_table && !last) {
         // centred maxima over [p - B, p + B], p in [lo - B, hi + B]
-        Acc *mc = (Acc *)smem + (D + 2 * wpad) * C + u;   // row p - lo + B
+        Acc *mc = (Acc *)smem + (D + 2 * wpad) * R + u;   // row p - lo + B
         const int NC = D + 2 * B;
         for (int i0 = kRun * q; i0 < NC; i0 += kRun * Q) {
             Acc M[kRun];
             run_max<Acc>(i0 + lo - B, hi + B, B, dead, vpad, M);
 #pragma unroll
             for (int i = 0; i < kRun; ++i)
-                if (i0 + i < NC) mc[(i0 + i) * C] = M[i];
+                if (i0 + i < NC) mc[(i0 + i) * R] = M[i];
         }
         __syncthreads();
         Mc = mc;
@@ -572,7 +580,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         if (last) {
         } else if (args.use_table) {
             const int L = 2 * B + 1;
-            auto mc = [&](int p) -> Acc { return Mc[(p - lo + B) * C]; };
+            auto mc = [&](int p) -> Acc { return Mc[(p - lo + B) * R]; };
 #pragma unroll
             for (int i = 0; i < kRun; ++i) {
                 if (c0 + i > hi) continue;
@@ -666,7 +674,6 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         if (threadIdx.x == 0) {
             const ChainImg &first = args.many ? args.many[0] : args.one;
             if (!(band == args.skip_band && tile == args.skip_tile && im.flags == first.flags)) {
-                __threadfence();
                 st_rel(im.flags + (size_t)band * im.tiles + tile, 1);
             }
         }
@@ -850,7 +857,7 @@ thread_local int g_skip_band = -1, g_skip_tile = -1;
 thread_local long long g_skip_wait = 0;
 
 size_t dp_smem(int n, int cols, int wpad, bool table) {
-    return (size_t)(2 * n - 1 + 2 * wpad) * cols * 4 * (table ? 2 : 1);
+    return (size_t)(2 * n - 1 + 2 * wpad) * row_words(cols) * 4 * (table ? 2 : 1);
 }
 
 // The window table's cover: the shortest window that no end of the range clips
@@ -920,6 +927,31 @@ int launch_chain_cols(const ChainArgs &a, int cols, size_t smem, int blocks, boo
     }
 }
 
+size_t fht_smem_bytes(int m, int T) { return (size_t)m * fht_pitch(m, T) * 4; }
+
+// Columns of an FHT block: a block's time grows as T + 0.8 m (the passes sweep
+// T + m - 4, T + m - 16, ... columns), and the last round of blocks may be nearly
+// empty, so the T (a multiple of 16, at most 256) of the least rounds x (T +
+// 0.8 m).  FHT_T_FIGURES
+int fht_columns(int m, int wout, int subs) {
+    const int sms = device_sms();
+    int best = 16;
+    double least = 1e30;
+    for (int T = 256; T >= 16; T -= 16) {
+        const size_t smem = fht_smem_bytes(m, T);
+        if (smem > 227 * 1024 - 1024) continue;
+        const int per_sm = smem <= 112 * 1024 ? 2 : 1;   // 1,024 threads a block
+        const long long blocks = (long long)((wout + T - 1) / T) * subs;
+        const long long rounds = (blocks + (long long)sms * per_sm - 1) / ((long long)sms * per_sm);
+        const double cost = (double)rounds * per_sm * (T + 0.8 * m);
+        if (cost < least) {
+            least = cost;
+            best = T;
+        }
+    }
+    return best;
+}
+
 FhtImg fht_img(const void *img, long long pitch, const Shape &s, int wout, void *out, int opitch) {
     FhtImg f{};
     f.img = img;
@@ -932,16 +964,15 @@ FhtImg fht_img(const void *img, long long pitch, const Shape &s, int wout, void 
     while ((1 << f.log2m) < f.m) ++f.log2m;
     f.out = out;
     f.opitch = opitch;
-    f.tiles = (wout + kFhtT - 1) / kFhtT;
     f.subs = s.h / f.m;
+    f.T = fht_columns(f.m, wout, f.subs);
+    f.tiles = (wout + f.T - 1) / f.T;
     return f;
 }
 
-size_t fht_smem_bytes(int m) { return (size_t)m * fht_pitch(m, kFhtT) * 4; }
-
 template <typename In, typename Acc>
 int launch_fht_img(const FhtImg &f, cudaStream_t stream) {
-    const size_t smem = fht_smem_bytes(f.m);
+    const size_t smem = fht_smem_bytes(f.m, f.T);
     int st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<In, Acc>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem),

@@ -35,7 +35,7 @@ struct FhtImg {
     int w, W, wout;      // image width, cyclic width w + n, columns to write
     int n, m, log2m;     // band height; sub-bands of m = min(n, 128) rows are merged
     void *out;           // [k][2][n][opitch], row j * m + s for sub-band j, shift s
-    int opitch, tiles, subs;
+    int opitch, T, tiles, subs;   // T columns a block (a multiple of 16)
     int item0;           // first block of this image in a launch of several
 };
 
