@@ -471,12 +471,21 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     // rows), so its states are a fixed step apart: along a column for V, along a
     // diagonal (fixed end column) for H.  Live states of an unmasked band: both
     // vertices inside.
+    // (Loads and stores under a condition cost a branch each, more than the
+    // rest of an element's work.)
     const bool in = xn < im.vw, whole = n >= kRun;
     const bool mask_h = im.mask1 == band + 1, mask_v = im.mask1 == band + 2;
+    const bool inner = whole && xn0 >= n && xn0 + C + n <= im.vw;   // every state is inside
     // this thread's Hough values (first run), in flight during the wait
     Acc h[kRun];
     auto load_h = [&](int c0) {
-        if (whole && !mask_h) {
+        if (inner && !mask_h) {
+            // (the last run's eighth row is a row of this band that is not used)
+            const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
+            const Acc *p = Hb + state_at(im, xn - c0, c0);
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) h[i] = ld_cg(p + i * step);
+        } else if (whole && !mask_h) {
             const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
             const Acc *p = Hb + state_at(im, xn - c0, c0);
 #pragma unroll
@@ -533,7 +542,12 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         // V_{b+1} of these columns; the thread's own rows
         for (int c0 = lo + kRun * q; c0 <= hi; c0 += kRun * Q) {
             Acc v[kRun];
-            if (whole && !mask_v) {
+            if (inner && !mask_v) {
+                const int step = c0 <= 0 ? -im.pitch : im.pitch;
+                const Acc *p = Vb + state_at(im, xn, c0);
+#pragma unroll
+                for (int i = 0; i < kRun; ++i) v[i] = ld_cg(p + i * step);
+            } else if (whole && !mask_v) {
                 const int step = c0 <= 0 ? -im.pitch : im.pitch;
                 const Acc *p = Vb + state_at(im, xn, c0);
 #pragma unroll
@@ -550,9 +564,16 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                                                                  : dead;
                 }
             }
+            Acc *dst = Vt + (c0 + n - 1) * R + u;
+            if (whole) {   // only the last run is one row short
 #pragma unroll
-            for (int i = 0; i < kRun; ++i)
-                if (c0 + i <= hi) Vt[(c0 + i + n - 1) * R + u] = v[i];
+                for (int i = 0; i + 1 < kRun; ++i) dst[i * R] = v[i];
+                if (c0 + kRun - 1 <= hi) dst[(kRun - 1) * R] = v[kRun - 1];
+            } else {
+#pragma unroll
+                for (int i = 0; i < kRun; ++i)
+                    if (c0 + i <= hi) dst[i * R] = v[i];
+            }
         }
         __syncthreads();
     }
@@ -622,6 +643,16 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 if (e <= hi) G = vmax(G, vpad(e));
                 M[i] = vmax(M[i], G);
             }
+        }
+        if (inner && !mask_h && band != 0 && args.band < 0) {
+            const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
+            Acc *p = Hb + state_at(im, xn - c0, c0);
+#pragma unroll
+            for (int i = 0; i + 1 < kRun; ++i) p[i * step] = M[i] == dead ? dead : h[i] + M[i];
+            if (c0 + kRun - 1 <= hi)
+                p[(kRun - 1) * step] =
+                    M[kRun - 1] == dead ? dead : h[kRun - 1] + M[kRun - 1];
+            continue;
         }
         if (whole && !mask_h && band != 0 && args.band < 0) {
             const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
