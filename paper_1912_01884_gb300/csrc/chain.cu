@@ -9,7 +9,9 @@
 // 2048 / n columns (16 for bands of 128 rows), so that a level spreads over the
 // chip and the chain advances at the latency of one exchange through L2.
 // CHAIN_FIGURES
+#include <algorithm>
 #include <climits>
+#include <new>
 #include <type_traits>
 #include <vector>
 
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
             }
         }
         __syncthreads();
-        if (l == im.log2m)   // bands of 4 rows: every level done
+        if (l == im.log2m)   // bands of 1 or 4 rows: every level done
             for (int idx = threadIdx.x; idx < m * (T / 4); idx += kFhtNT) {
                 const int s = idx / (T / 4), u = 4 * (idx % (T / 4));
                 out(s, u, *(const uint4 *)&F[(size_t)bit_reverse(s, l) * pitch + u]);
@@ -887,6 +889,17 @@ size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 thread_local int g_skip_band = -1, g_skip_tile = -1;
 thread_local long long g_skip_wait = 0;
 
+void take_injection(ChainArgs &a) {
+    a.wait_cycles = 4000000000LL;   // about two seconds
+    a.skip_band = a.skip_tile = -1;
+    if (g_skip_band >= 0) {
+        a.skip_band = g_skip_band;
+        a.skip_tile = g_skip_tile;
+        a.wait_cycles = g_skip_wait;
+    }
+    g_skip_band = g_skip_tile = -1;
+}
+
 size_t dp_smem(int n, int cols, int wpad, bool table) {
     return (size_t)(2 * n - 1 + 2 * wpad) * row_words(cols) * 4 * (table ? 2 : 1);
 }
@@ -950,6 +963,7 @@ template <typename Acc>
 int launch_chain_cols(const ChainArgs &a, int cols, size_t smem, int blocks, bool dependent,
                       cudaStream_t stream) {
     switch (cols) {
+        case 0: return launch_chain<Acc, 0>(a, smem, blocks, dependent, stream);
         case 16: return launch_chain<Acc, 16>(a, smem, blocks, dependent, stream);
         case 32: return launch_chain<Acc, 32>(a, smem, blocks, dependent, stream);
         case 64: return launch_chain<Acc, 64>(a, smem, blocks, dependent, stream);
@@ -1021,7 +1035,6 @@ int launch_fht_img(const FhtImg &f, cudaStream_t stream) {
 template <typename In, typename Acc>
 int launch_band_fht(const In *img, long long pitch, const Shape &s, int wout, Acc *hough, Acc *tmp,
                     int opitch, cudaStream_t stream) {
-    if (s.n == 1) return launch_fht_single_row<In, Acc>(img, pitch, s, wout, hough, opitch, stream);
     Acc *first = s.n > 128 ? tmp : hough;
     // the last level reads columns modulo W
     int st = launch_fht_img<In, Acc>(fht_img(img, pitch, s, s.n > 128 ? s.W : wout, first, opitch),
@@ -1157,14 +1170,7 @@ int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q
     }
     a.items = L.tiles * (s.k > 1 ? s.k - 1 : 1);
     a.ctl = (ChainCtl *)ws;
-    a.wait_cycles = 4000000000LL;   // about two seconds
-    a.skip_band = a.skip_tile = -1;
-    if (g_skip_band >= 0) {
-        a.skip_band = g_skip_band;
-        a.skip_tile = g_skip_tile;
-        a.wait_cycles = g_skip_wait;
-    }
-    g_skip_band = g_skip_tile = -1;
+    take_injection(a);
     a.band = -1;
     a.store0 = q.sep > 0;
     if (q.table) chain_table(a, *q.table);
@@ -1179,6 +1185,140 @@ int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q
     return st;
 }
 }  // namespace
+
+// ---------------------------------------------------------------------------
+// Batches.  Workspace: [head][flags, key and done of every image][FHT table]
+// [image table][queue][rows of every image]; the first two parts are cleared by
+// every run.
+struct ChainBatch {
+    int dtype;
+    std::vector<ChainImage> images;
+    std::vector<FhtImg> fht;         // as uploaded
+    std::vector<ChainImg> imgs;
+    std::vector<ChainItem> order;
+    std::vector<size_t> flags, keys, rows;   // offsets
+    size_t zero = 0, fht_off = 0, img_off = 0, order_off = 0, total = 0, fht_smem = 0;
+    int fht_blocks = 0, cols = 0;    // cols 0: several tile widths
+};
+
+ChainBatch *chain_batch_create(const std::vector<ChainImage> &images, int dtype) {
+    ChainBatch *b = new (std::nothrow) ChainBatch();
+    if (!b) return nullptr;
+    b->dtype = dtype;
+    b->images = images;
+    size_t o = sizeof(ChainCtl);
+    struct Level {
+        double when;
+        int image, lv;
+    };
+    std::vector<Level> levels;
+    for (const ChainImage &c : images) {
+        const int i = (int)b->imgs.size();
+        ChainImg im{};
+        im.n = c.s.n;
+        im.k = c.s.k;
+        im.vw = c.s.vw;
+        im.pitch = (c.s.vw + 31) & ~31;
+        im.B = c.B < 2 * c.s.n - 2 ? c.B : 2 * c.s.n - 2;
+        im.cols = chain_cols(c.s.n);
+        im.tiles = (c.s.vw + im.cols - 1) / im.cols;
+        im.x_out = c.x_out;
+        im.d_out = c.d_out;
+        im.score_out = c.score_out;
+        b->cols = i == 0 ? im.cols : b->cols == im.cols ? im.cols : 0;
+        b->keys.push_back(o);
+        o += 16;
+        b->flags.push_back(o);
+        o = (o + (size_t)im.k * im.tiles * 4 + 15) & ~(size_t)15;
+        FhtImg f = fht_img(c.img, c.pitch, c.s, c.s.vw, nullptr, im.pitch);
+        f.T = std::min(256, (c.s.vw + 15) & ~15);   // the least work a column
+        f.tiles = (c.s.vw + f.T - 1) / f.T;
+        f.item0 = b->fht_blocks;
+        b->fht_blocks += f.tiles * f.subs;
+        b->fht_smem = std::max(b->fht_smem, fht_smem_bytes(f.m, f.T));
+        b->imgs.push_back(im);
+        b->fht.push_back(f);
+        const int L = std::max(im.k - 1, 1);
+        for (int lv = 0; lv < L; ++lv) levels.push_back(Level{(lv + 0.5) / L, i, lv});
+    }
+    // Queue: every image's band levels in proportion to their number, so that
+    // all chains begin and end together and each level's wait is covered by the
+    // other images' items.
+    std::stable_sort(levels.begin(), levels.end(),
+                     [](const Level &x, const Level &y) { return x.when < y.when; });
+    for (const Level &l : levels) {
+        const ChainImg &im = b->imgs[l.image];
+        for (int t = 0; t < im.tiles; ++t)
+            b->order.push_back(ChainItem{l.image, std::max(im.k - 2 - l.lv, 0), t, 0});
+    }
+    b->zero = o = up256(o);
+    b->fht_off = o;
+    o = up256(o + b->fht.size() * sizeof(FhtImg));
+    b->img_off = o;
+    o = up256(o + b->imgs.size() * sizeof(ChainImg));
+    b->order_off = o;
+    o = up256(o + b->order.size() * sizeof(ChainItem));
+    for (const ChainImg &im : b->imgs) {
+        b->rows.push_back(o);
+        o = up256(o + (size_t)im.k * 2 * im.n * im.pitch * 4);
+    }
+    b->total = o;
+    return b;
+}
+void chain_batch_destroy(ChainBatch *b) { delete b; }
+size_t chain_batch_bytes(const ChainBatch *b) { return b->total; }
+long long chain_batch_items(const ChainBatch *b) { return (long long)b->order.size(); }
+
+int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream) {
+    char *W = (char *)ws;
+    for (size_t i = 0; i < b->imgs.size(); ++i) {
+        b->fht[i].out = b->imgs[i].hv = W + b->rows[i];
+        b->imgs[i].flags = (int *)(W + b->flags[i]);
+        b->imgs[i].key = (unsigned long long *)(W + b->keys[i]);
+        b->imgs[i].done = (int *)(W + b->keys[i] + 8);
+    }
+    auto put = [&](size_t off, const void *src, size_t bytes) {
+        return cuda_status(cudaMemcpyAsync(W + off, src, bytes, cudaMemcpyHostToDevice, stream),
+                           "cudaMemcpyAsync");
+    };
+    int st = put(b->fht_off, b->fht.data(), b->fht.size() * sizeof(FhtImg));
+    if (!st) st = put(b->img_off, b->imgs.data(), b->imgs.size() * sizeof(ChainImg));
+    if (!st) st = put(b->order_off, b->order.data(), b->order.size() * sizeof(ChainItem));
+    return st;
+}
+
+namespace {
+template <typename Acc>
+int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaStream_t stream) {
+    int st = cuda_status(cudaMemsetAsync(ws, 0, b->zero, stream), "cudaMemsetAsync");
+    if (!st)
+        st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<Acc, Acc>,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)b->fht_smem),
+                         "cudaFuncSetAttribute");
+    if (st) return st;
+    fht_band_kernel<Acc, Acc><<<(unsigned)b->fht_blocks, kFhtNT, b->fht_smem, stream>>>(
+        b->fht[0], (const FhtImg *)(ws + b->fht_off), (int)b->fht.size());
+    st = launched("fht_band_kernel");
+    if (st) return st;
+    ChainArgs a{};
+    a.many = (const ChainImg *)(ws + b->img_off);
+    a.order = (const ChainItem *)(ws + b->order_off);
+    a.items = (int)b->order.size();
+    a.ctl = (ChainCtl *)ws;
+    take_injection(a);
+    a.band = -1;
+    if (t) chain_table(a, *t);
+    size_t smem = 0;
+    for (const ChainImg &im : b->imgs) smem = std::max(smem, item_smem(a, im));
+    return launch_chain_cols<Acc>(a, b->cols, smem, a.items, false, stream);
+}
+}  // namespace
+
+int chain_batch_run(const ChainBatch *b, void *ws, const WindowTable *t, cudaStream_t stream) {
+    return b->dtype == FHTDP_F32 ? chain_batch_run_t<float>(b, (char *)ws, t, stream)
+                                 : chain_batch_run_t<int32_t>(b, (char *)ws, t, stream);
+}
 
 int chain_detect(const void *img, int dtype, int pitch, const Shape &s, const ChainQuery &q,
                  int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream) {

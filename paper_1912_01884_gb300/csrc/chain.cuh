@@ -1,6 +1,8 @@
 // Band FHT in one pass and the DP chain over stored Hough rows (chain.cu).
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace fhtdp {
@@ -58,7 +60,28 @@ struct ChainQuery {
 // least chain_layout().total bytes.
 int chain_detect(const void *img, int dtype, int pitch, const Shape &s, const ChainQuery &q,
                  int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream);
-// The next chain_detect of this thread never publishes tile `tile` of band
+
+// A batch of int32 or float images (bands of at most 128 rows): all their
+// FHTs in one launch, all their DP items in one more.
+struct ChainImage {
+    const void *img;
+    long long pitch;
+    Shape s;
+    int B;
+    int32_t *x_out, *d_out;
+    void *score_out;
+};
+struct ChainBatch;
+ChainBatch *chain_batch_create(const std::vector<ChainImage> &images, int dtype);
+void chain_batch_destroy(ChainBatch *b);
+size_t chain_batch_bytes(const ChainBatch *b);
+long long chain_batch_items(const ChainBatch *b);
+// The batch's tables for workspace ws (from host memory held by the batch).
+int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream);
+// t (optional): bend-angle windows for all images (one band height).
+int chain_batch_run(const ChainBatch *b, void *ws, const WindowTable *t, cudaStream_t stream);
+
+// The next chain run of this thread never publishes tile `tile` of band
 // `band`, and its waits give up after `wait_cycles` (band < 0: none).
 void chain_inject(int band, int tile, long long wait_cycles);
 

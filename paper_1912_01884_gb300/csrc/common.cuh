@@ -70,11 +70,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 template <typename In, typename Acc>
 int launch_band_fht(const In *img, long long pitch, const Shape &s, int wout, Acc *hough, Acc *tmp,
                     int opitch, cudaStream_t stream);
-// Its passes of their own (fht_stages.cu): one-row bands, and the last level of
-// 256-row bands from the level of their 128-row halves.
-template <typename In, typename Acc>
-int launch_fht_single_row(const In *img, long long pitch, const Shape &s, int wout, Acc *out,
-                          int opitch, cudaStream_t stream);
+// The last level of 256-row bands, from the level of their 128-row halves
+// (fht_stages.cu).
 template <typename Acc>
 int launch_fht_last(const Acc *src, const Shape &s, int wout, Acc *dst, int opitch,
                     cudaStream_t stream);

@@ -146,13 +146,6 @@ struct LaunchArgs {
     // Fault injection for tests (fhtdp_debug_inject): the tile (band, tile)
     // of the first image never publishes; -1 disables.
     int skip_band, skip_tile;
-    // int32 / float images, one image: with use_table the bend-angle windows
-    // of Sec. 2.3 (Eqs. 6-7) replace |e - d| <= B, e in [tab.lo[d + n - 1],
-    // tab.hi[d + n - 1]].  The DP items answer them from maxima of fixed
-    // half-width B0 (every window that no end of the displacement range
-    // clips is at least 2 B0 + 1 long), with wpad dead rows above and below V.
-    int use_table, B0, wpad;
-    WindowTable tab;
 };
 
 // ---------------------------------------------------------------------------
@@ -2207,507 +2200,6 @@ struct U8Ctl {
 };
 
 // ---------------------------------------------------------------------------
-// int32 / float images.  Two kinds of work items per band level: FHT items
-// compute a band's Hough values for 64 columns, both slope signs, and store
-// them to the image's hw rows; DP items of 16 columns bring their Hough rows
-// and their M tile by TMA, form V (Eqs. 3-4) as 64-bit window keys, compute
-// the bend-window maxima (Sec. 2.3) and publish.  Items are small (256 threads, at
-// most 102 KB of shared memory), two CTAs share an SM, and one band level of
-// an image spreads over many CTAs, so that the band chain of a single large
-// image advances quickly.  The float sums follow the same tree as the
-// oracle's float32 recursion (top half + bottom half at every level).
-constexpr int kWThreads = 256;
-constexpr int kWTileF = 64;    // FHT item columns
-constexpr int kWTileD = 16;    // DP item columns
-constexpr int kWPad = 48;      // dead rows above and below V in a DP item
-constexpr int kItemWideFht = 1, kItemWideDp = 3;
-
-template <typename In, typename Acc, typename Key>
-struct WideEngine {
-    using KO = KeyOps<Acc, Key>;
-    static constexpr int NT = kWThreads;
-
-    __host__ __device__ static int fpitch(int n) { return (kWTileF + n + 8 + 3) & ~3; }
-    __host__ __device__ static size_t fht_smem(int n) {
-        return (size_t)(n < 2 ? 2 : n) * fpitch(n) * 4;
-    }
-    // Hough rows [2][n][T] (each sign from a 128-byte boundary, as TMA
-    // destinations are), then V [wpad + D + wpad][T]: the M tile lands in its
-    // D middle rows and V is formed there in place; the pad rows hold dead
-    // values, so that the window reads past [-(n-1), n-1] unchecked.  With a
-    // window table, the centred maxima Mc [D + 2 wpad][T] follow.
-    __host__ __device__ static int dp_sign1(int n) { return (n * kWTileD + 31) & ~31; }
-    __host__ __device__ static size_t dp_mc_off(int n, int wpad) {
-        return (size_t)(2 * dp_sign1(n) + (2 * n - 1 + 2 * wpad) * kWTileD) * 4;
-    }
-    __host__ __device__ static size_t dp_smem(int n, int wpad, bool table) {
-        return dp_mc_off(n, wpad) + (table ? (size_t)(2 * n - 1 + 2 * wpad) * kWTileD * 4 : 0);
-    }
-    static size_t smem_bytes(int max_n, int wpad, bool table) {
-        return std::max(fht_smem(max_n), dp_smem(max_n, wpad, table));
-    }
-    __device__ static Acc *hw_row(const ImgDesc &im, int band, int sign, int s) {
-        return (Acc *)im.hw + (((size_t)band * 2 + sign) * im.n + s) * im.hwpitch;
-    }
-
-    // Pixels [c, c+4) of a row, zero outside [0, w); c is a multiple of 4.
-    __device__ static void load4(const In *row, int c, int w, bool aligned, Acc out[4]) {
-        if (aligned && c >= 0 && c + 4 <= w) {
-            const int4 v = __ldg((const int4 *)(row + c));
-            out[0] = from_bits<Acc>((uint32_t)v.x);
-            out[1] = from_bits<Acc>((uint32_t)v.y);
-            out[2] = from_bits<Acc>((uint32_t)v.z);
-            out[3] = from_bits<Acc>((uint32_t)v.w);
-            return;
-        }
-        for (int j = 0; j < 4; ++j) out[j] = (Acc)pix(row, c + j, w);
-    }
-
-    // N consecutive strip words of band row y from word u: sign 0 reads
-    // pixels x0 + u.., sign 1 the mirrored strip (word u = pixel x0 + 63 - u).
-    template <int N>
-    __device__ static void strip_words(const In *row, int w, bool aligned, int x0, int u,
-                                       int sign, Acc (&P)[N]) {
-        constexpr int NW = (N + 3) / 4;
-        Acc q[4 * NW];
-        if (sign == 0) {
-#pragma unroll
-            for (int k = 0; k < NW; ++k) load4(row, x0 + u + 4 * k, w, aligned, &q[4 * k]);
-#pragma unroll
-            for (int j = 0; j < N; ++j) P[j] = q[j];
-        } else {
-            // words u .. u + 4NW - 1 are pixels x0 + 63 - u down to x0 + 64 - u - 4NW
-            const int c = x0 + kWTileF - u - 4 * NW;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) load4(row, c + 4 * k, w, aligned, &q[4 * k]);
-#pragma unroll
-            for (int j = 0; j < N; ++j) P[j] = q[4 * NW - 1 - j];
-        }
-    }
-    // Levels 1 and 2 on four rows y0..y0+3 of a sub-band: out[s][u] (s < 4,
-    // u < W) from the rows' words u .. u + W + 2 (the recursion's sums, in
-    // its order).
-    template <int W>
-    __device__ static void levels12(const In *base, long long pitch, int w, bool aligned,
-                                    int x0, int u, int sign, int y0, Acc (&out)[4][W]) {
-        Acc A[2][W], Bq[2][W + 2];
-        {
-            Acc p0[W], p1[W + 1];
-            strip_words<W>(base + (size_t)y0 * pitch, w, aligned, x0, u, sign, p0);
-            strip_words<W + 1>(base + (size_t)(y0 + 1) * pitch, w, aligned, x0, u, sign, p1);
-#pragma unroll
-            for (int j = 0; j < W; ++j) {
-                A[0][j] = p0[j] + p1[j];
-                A[1][j] = p0[j] + p1[j + 1];
-            }
-        }
-        {
-            Acc p2[W + 2], p3[W + 3];
-            strip_words<W + 2>(base + (size_t)(y0 + 2) * pitch, w, aligned, x0, u, sign, p2);
-            strip_words<W + 3>(base + (size_t)(y0 + 3) * pitch, w, aligned, x0, u, sign, p3);
-#pragma unroll
-            for (int j = 0; j < W + 2; ++j) {
-                Bq[0][j] = p2[j] + p3[j];
-                Bq[1][j] = p2[j] + p3[j + 1];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            out[0][j] = A[0][j] + Bq[0][j];
-            out[1][j] = A[0][j] + Bq[0][j + 1];
-            out[2][j] = A[1][j] + Bq[1][j + 1];
-            out[3][j] = A[1][j] + Bq[1][j + 2];
-        }
-    }
-    // Levels 1-3 in registers straight from the image (n >= 8): a task is an
-    // 8-row sub-band g and the 4 words [4c, 4c + 4) of the level-3 width;
-    // shift s of the sub-band goes to row 8g + brev3(s) of F.
-    __device__ static void fht_regs8(Acc *F, int pitch, const ImgDesc &im, const In *base,
-                                     bool aligned, int x0, int sign) {
-        const int n = im.n, T = kWTileF;
-        const int C4 = (T + n - 8 + 3) / 4;
-        const int tasks = (n / 8) * C4;
-        for (int t = threadIdx.x; t < tasks; t += NT) {
-            const int g = t / C4, c = t - g * C4;
-            Acc B2[4][8], T2[4][4];
-            levels12<8>(base, im.pitch, im.w, aligned, x0, 4 * c, sign, 8 * g + 4, B2);
-            levels12<4>(base, im.pitch, im.w, aligned, x0, 4 * c, sign, 8 * g, T2);
-            Acc *row0 = F + (size_t)(8 * g) * pitch + 4 * c;
-#pragma unroll
-            for (int sh = 0; sh < 8; ++sh) {
-                const int h = sh >> 1, o = (sh + 1) >> 1;
-                const int r = ((sh & 1) << 2) | (sh & 2) | ((sh >> 2) & 1);
-                *(uint4 *)&row0[(size_t)r * pitch] =
-                    make_uint4(to_bits(T2[h][0] + B2[h][o + 0]), to_bits(T2[h][1] + B2[h][o + 1]),
-                               to_bits(T2[h][2] + B2[h][o + 2]), to_bits(T2[h][3] + B2[h][o + 3]));
-            }
-        }
-        csync<NT>();
-    }
-
-    // FHT item: the band's Hough values of columns [x0, x0 + 64), both signs,
-    // into hw.  Sign 0 ("+") runs on the strip as it is and its last level
-    // writes the rows of hw directly; sign 1 ("-") runs on the mirrored strip
-    // (word u = pixel x0 + 63 - u), and its rows, bit-reversed in F, are
-    // copied out mirrored back.
-    // The strip of an FHT item (columns [x0, x0 + T + n - 1) of the band's
-    // rows, clipped to the image) requested into L2, every 128-byte line at
-    // once, at the item's start: the register levels read the strip task by
-    // task, and their first reads would otherwise wait on DRAM one task
-    // after another.
-    __device__ static void prefetch_strip(const ImgDesc &im, int band, int ft) {
-        const int n = im.n, x0 = ft * kWTileF;
-        const In *base = (const In *)im.img + (size_t)band * n * im.pitch;
-        const int c_lo = x0, c_hi = min(x0 + kWTileF + n - 1, im.w);   // [c_lo, c_hi)
-        if (c_lo >= c_hi) return;
-        const size_t bytes = (size_t)(c_hi - c_lo) * sizeof(In);
-        const int lines = (int)((bytes + 127) / 128) + 1;
-        for (int i = threadIdx.x; i < n * lines; i += NT) {
-            const int y = i / lines, l = i - y * lines;
-            const uintptr_t a = (uintptr_t)(base + (size_t)y * im.pitch + c_lo);
-            const uintptr_t line = (a & ~(uintptr_t)127) + (uintptr_t)l * 128;
-            // only lines that hold a byte of the row's range
-            if (line < a + bytes) prefetch_l2((const void *)line);
-        }
-    }
-
-    __device__ static void fht_item(const ImgDesc &im, int band, int ft, unsigned char *smem) {
-        const int n = im.n, T = kWTileF, pitch = fpitch(n), x0 = ft * T;
-        Acc *F = (Acc *)smem;
-        const int G = (T + n - 1 + 3) / 4;
-        const In *base = (const In *)im.img + (size_t)band * n * im.pitch;
-        const bool aligned = ((uintptr_t)im.img % 16 == 0) && (im.pitch % 4 == 0);
-        constexpr int kLB = 8;
-        prefetch_strip(im, band, ft);
-        for (int sign = 0; sign < 2; ++sign) {
-            int first = 1;   // the first level left to merge in shared memory
-            if (n >= 8) {
-                fht_regs8(F, pitch, im, base, aligned, x0, sign);
-                first = 4;
-            } else
-            for (int b0 = threadIdx.x; b0 < n * G; b0 += kLB * NT) {
-                Acc v[kLB][4];
-#pragma unroll
-                for (int i = 0; i < kLB; ++i) {
-                    const int idx = b0 + i * NT;
-                    if (idx < n * G) {
-                        const int y = idx / G, u0 = 4 * (idx - y * G);
-                        load4(base + (size_t)y * im.pitch, sign == 0 ? x0 + u0 : x0 + T - 4 - u0,
-                              im.w, aligned, v[i]);
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < kLB; ++i) {
-                    const int idx = b0 + i * NT;
-                    if (idx < n * G) {
-                        const int y = idx / G, u0 = 4 * (idx - y * G);
-                        const bool fw = sign == 0;
-                        *(uint4 *)&F[(size_t)y * pitch + u0] =
-                            make_uint4(to_bits(fw ? v[i][0] : v[i][3]),
-                                       to_bits(fw ? v[i][1] : v[i][2]),
-                                       to_bits(fw ? v[i][2] : v[i][1]),
-                                       to_bits(fw ? v[i][3] : v[i][0]));
-                    }
-                }
-            }
-            csync<NT>();
-            if (sign == 0) {
-                if (!fht_merge<Acc, NT>(F, pitch, n, im.log2n, T, first,
-                                         hw_row(im, band, 0, 0) + x0, im.hwpitch)) {
-                    // no merge level (n = 1, or n = 8 done in registers): rows
-                    // brev(s) hold the shifts
-                    for (int idx = threadIdx.x; idx < n * T; idx += NT) {
-                        const int sh = idx / T, u = idx - sh * T;
-                        hw_row(im, band, 0, sh)[x0 + u] = F[(size_t)brev(sh, im.log2n) * pitch + u];
-                    }
-                }
-            } else {
-                fht_merge<Acc, NT>(F, pitch, n, im.log2n, T, first);
-                // shift s of the mirrored strip at word u: the left-moving sum
-                // from column x0 + 63 - u, in row brev(s) of F
-                for (int idx = threadIdx.x; idx < n * (T / 4); idx += NT) {
-                    const int sh = idx / (T / 4), u0 = 4 * (idx % (T / 4));
-                    const uint4 w4 =
-                        *(const uint4 *)&F[(size_t)brev(sh, im.log2n) * pitch + T - 4 - u0];
-                    *(uint4 *)(hw_row(im, band, 1, sh) + x0 + u0) =
-                        make_uint4(w4.w, w4.z, w4.y, w4.x);
-                }
-            }
-            csync<NT>();
-        }
-    }
-
-    // DP item: columns [x0, x0 + 16) of band `band`.
-    __device__ static void dp_item(const ImgDesc &im, int band, int tile, unsigned char *smem,
-                                   Pipe &pipe, const LaunchArgs &args) {
-        const int n = im.n, D = 2 * n - 1, T = kWTileD, x0 = tile * T;
-        const bool last = band == im.k - 1;
-        const int wpad = args.wpad;
-        Acc *Ht = (Acc *)smem;          // [2][n][T]: Hough rows of both signs
-        const int h1 = dp_sign1(n);     // offset of sign 1
-        Acc *Vt = Ht + 2 * h1;          // [wpad + D + wpad][T]: M tile, then V
-        Acc *Mt = Vt + wpad * T;        // row e + n - 1: displacement e
-        const Acc dead = Dead<Acc>::value();
-        if (threadIdx.x < 32) {
-            // M(x + d, d): band+1 tiles over [x0 - (n-1), x0 + T + n - 2] (lanes
-            // 0..30); the FHT item of these columns (lane 31)
-            const int lane = threadIdx.x;
-            const int t0 = (x0 - (n - 1)) >= 0 ? (x0 - (n - 1)) / T : -((n - 1 - x0 + T - 1) / T);
-            const int *flag = nullptr;
-            if (lane < 31) {
-                const int c = t0 + lane;
-                if (!last && c >= 0 && c < im.tiles && c * T <= x0 + T + n - 2)
-                    flag = im.flags + (size_t)(band + 1) * im.tiles + c;
-            } else {
-                flag = im.fflags + (size_t)band * im.ftiles + x0 / kWTileF;
-            }
-            bool ok = true;
-            if (flag) {
-                ok = wait_flag(flag, args.ctl, args.wait_cycles);
-                fence_acq_rel_gpu();
-            }
-            __syncwarp();
-            ok = __all_sync(0xffffffffu, ok);
-            if (lane == 0) {
-                if (!ok) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
-                fence_proxy_async_global();
-                fence_proxy_async_smem();
-                mbar_expect_tx(pipe.mbar, (uint32_t)((2 * n + (last ? 0 : D)) * T * 4));
-                tma_load_2d(Ht, &im.tmap, x0, band * 2 * n, pipe.mbar);
-                tma_load_2d(Ht + h1, &im.tmap, x0, (band * 2 + 1) * n, pipe.mbar);
-                if (!last) tma_load_2d(Mt, &im.mtmap, im.moff + x0, (band + 1) * D, pipe.mbar);
-            }
-        } else if (band != 0) {
-            // the dead pad rows (outside the copies' destinations)
-            for (int idx = threadIdx.x - 32; idx < 2 * wpad * (T / 4); idx += NT - 32) {
-                const int r = idx / (T / 4), u0 = 4 * (idx % (T / 4));
-                const int row = r < wpad ? r : r + D;
-                *(uint4 *)&Vt[row * T + u0] =
-                    make_uint4(to_bits(dead), to_bits(dead), to_bits(dead), to_bits(dead));
-            }
-        }
-        if (!mbar_wait(pipe.mbar, pipe.mphase, args.wait_cycles)) {
-            if (threadIdx.x == 0) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
-            mbar_wait(pipe.mbar, pipe.mphase, kDrainCycles);
-        }
-        pipe.mphase ^= 1u;
-        // V(x, e) = H(x, e) + M(x + e, e), dead outside the image (Eqs. 3-4),
-        // in place of the M tile.
-        unsigned long long best = 0;
-        for (int idx = threadIdx.x; idx < D * (T / 4); idx += NT) {
-            const int ei = idx / (T / 4), u0 = 4 * (idx % (T / 4));
-            const int e = ei - (n - 1), sh = e < 0 ? -e : e;
-            const uint4 h4 = *(const uint4 *)&Ht[(e < 0 ? h1 : 0) + sh * T + u0];
-            uint4 m4 = make_uint4(0, 0, 0, 0);
-            if (!last) m4 = *(const uint4 *)&Mt[ei * T + u0];
-            const uint32_t hb[4] = {h4.x, h4.y, h4.z, h4.w};
-            const uint32_t mb[4] = {m4.x, m4.y, m4.z, m4.w};
-            Acc v[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int x = x0 + u0 + j;
-                const bool ok = x < im.w && x + e >= 0 && x + e < im.w;
-                const Acc h = from_bits<Acc>(hb[j]), m = from_bits<Acc>(mb[j]);
-                v[j] = !ok ? dead : last ? h : (m == dead ? dead : h + m);
-            }
-            if (band == 0) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (v[j] != dead) {
-                        const unsigned long long k = argmax_key(ord32(v[j]), x0 + u0 + j, ei);
-                        best = best > k ? best : k;
-                    }
-            } else {
-                *(uint4 *)&Mt[ei * T + u0] =
-                    make_uint4(to_bits(v[0]), to_bits(v[1]), to_bits(v[2]), to_bits(v[3]));
-            }
-        }
-        if (band == 0) {
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-                best = best > other ? best : other;
-            }
-            if ((threadIdx.x & 31) == 0 && best) atomicMax(im.best, best);
-            csync<NT>();
-            if (threadIdx.x < 32) {
-                int is_last = 0;
-                if (threadIdx.x == 0) {
-                    __threadfence();
-                    is_last = atomicAdd(im.done, 1) == im.tiles - 1;
-                }
-                if (__shfl_sync(0xffffffffu, is_last, 0)) readback_values(im, args);
-            }
-            return;
-        }
-        csync<NT>();
-        // Window maxima (values only: the read-back recomputes the argmax),
-        // 16 threads per column, 16 displacements each.
-        const int u = threadIdx.x & (T - 1), q = threadIdx.x / T;
-        const int x = x0 + u;
-        const int lo = -(n - 1), hi = n - 1;
-        const int B = args.use_table ? args.B0 : im.B;
-        const Acc *col = Mt + (n - 1) * T + u;   // V(e) at col[e * T]
-        // Runs of NOUT outputs from c0 (count of them) of the maxima over
-        // [c - B, c + B], NOUT the largest power of two up to 16 that the
-        // window length L = 2B + 1 covers (one block pair per run).
-        auto maxima = [&](int c0, int count, auto vkey, auto emit) {
-            auto runs = [&](auto nout) {
-                constexpr int NOUT = decltype(nout)::value;
-                for (int r0 = 0; r0 < count; r0 += NOUT)
-                    window_span<NOUT, Acc>(c0 + r0, count - r0, B, dead, vkey,
-                                           [&](int i, Acc m) { emit(r0 + i, m); });
-            };
-            const int L = 2 * B + 1;
-            if (L >= 16) runs(std::integral_constant<int, 16>());
-            else if (L >= 8) runs(std::integral_constant<int, 8>());
-            else if (L >= 4) runs(std::integral_constant<int, 4>());
-            else if (L >= 2) runs(std::integral_constant<int, 2>());
-            else runs(std::integral_constant<int, 1>());
-        };
-        auto vpad = [&](int e) -> Acc { return col[e * T]; };   // dead pad rows outside
-        const int c0 = lo + 16 * q;
-        if (!args.use_table) {
-            if (x < im.w && c0 <= hi) {
-                Acc *mcol = mband(im, band) + (size_t)(c0 + n - 1) * im.mpitch + im.moff + x - c0;
-                const int count = min(16, hi - c0 + 1);
-                auto emit = [&](int i, Acc m) { mcol[(long long)i * (im.mpitch - 1)] = m; };
-                // A run reads V over [c - B, c + B + 16]: inside the pad rows
-                // when B + 16 <= wpad.
-                if (B + 16 <= wpad) maxima(c0, count, vpad, emit);
-                else
-                    maxima(c0, count,
-                           [&](int e) -> Acc { return (e < lo || e > hi) ? dead : col[e * T]; },
-                           emit);
-            }
-        } else {
-            // Bend-angle windows (Sec. 2.3): the centred maxima Mc(p) over
-            // [p - B0, p + B0] for p in [-(n-1) - B0, n-1 + B0] (they read V
-            // over [-(n-1) - 2 B0, n-1 + 2 B0 + 16], inside the pad rows),
-            // then each window [lo(c), hi(c)] as the maximum of the pieces
-            // that cover it: centres lo + B0, lo + B0 + L, ... and hi - B0.  A
-            // window shorter than L = 2 B0 + 1 is cut by an end of the range:
-            // the piece from its other end reaches only dead rows beyond it.
-            Acc *Mc = (Acc *)(smem + dp_mc_off(n, wpad)) + u;   // row p + (n-1) + B0
-            const int NC = D + 2 * B;
-            for (int i0 = 16 * q; i0 < NC; i0 += 16 * (NT / T))
-                maxima(i0 - (n - 1) - B, min(16, NC - i0), vpad,
-                       [&](int i, Acc m) { Mc[(size_t)(i0 + i) * T] = m; });
-            csync<NT>();
-            if (x < im.w && c0 <= hi) {
-                Acc *mcol = mband(im, band) + (size_t)(c0 + n - 1) * im.mpitch + im.moff + x - c0;
-                const int count = min(16, hi - c0 + 1);
-                const int L = 2 * B + 1;
-                auto mc = [&](int p) -> Acc { return Mc[(size_t)(p + n - 1 + B) * T]; };
-                for (int i = 0; i < count; ++i) {
-                    const int c = c0 + i;
-                    const int wl = args.tab.lo[c + n - 1], wh = args.tab.hi[c + n - 1];
-                    Acc m = dead;
-                    if (wh - wl + 1 >= L) {
-                        for (int p = wl + B; p < wh - B; p += L) m = kmax(m, mc(p));
-                        m = kmax(m, mc(wh - B));
-                    } else if (wh == hi) {
-                        m = mc(wl + B);
-                    } else if (wl == lo) {
-                        m = mc(wh - B);
-                    } else {   // not produced by the host's choice of B0; kept exact
-                        for (int e = wl; e <= wh; ++e) m = kmax(m, col[e * T]);
-                    }
-                    mcol[(long long)i * (im.mpitch - 1)] = m;
-                }
-            }
-        }
-        fence_acq_rel_gpu();
-        csync<NT>();
-        if (threadIdx.x == 0) {
-            const ImgDesc &first = args.many ? args.many[0] : args.one;
-            if (!(band == args.skip_band && tile == args.skip_tile && im.flags == first.flags))
-                st_release(im.flags + (size_t)band * im.tiles + tile, 1);
-        }
-    }
-
-    // The window maxima of band b: [D][mpitch], one array per band (the
-    // read-back recomputes each band's argmax from them and the Hough rows).
-    __device__ static Acc *mband(const ImgDesc &im, int band) {
-        return (Acc *)im.mbuf[0] + (size_t)band * (2 * im.n - 1) * im.mpitch;
-    }
-
-    // Eq. 5 by one warp, from the best top point: at band i the smallest e
-    // with |e - d_{i-1}| <= B maximising V_i(x_i, e) = H_i(x_i, e) +
-    // M_{i+1}(x_i + e, e), recomputed from the stored Hough rows and window
-    // maxima with the same additions as the DP item (lanes over e, then a
-    // warp maximum of (value, smallest e) keys).
-    __device__ static void readback_values(const ImgDesc &im, const LaunchArgs &args) {
-        const int lane = threadIdx.x & 31, n = im.n, D = 2 * n - 1;
-        const Acc dead = Dead<Acc>::value();
-        __threadfence();
-        unsigned long long key = 0;
-        if (lane == 0) key = atomicAdd(im.best, 0ull);
-        key = __shfl_sync(0xffffffffu, key, 0);
-        if (key == 0) {   // no admissible polyline
-            if (lane == 0) {
-                *(Acc *)im.score_out = dead;
-                for (int i = 0; i <= im.k; ++i) im.x_out[i] = -1;
-                for (int i = 0; i < im.k; ++i) im.d_out[i] = 0;
-            }
-            return;
-        }
-        const unsigned lin = 0xffffffffu - (unsigned)(key & 0xffffffffu);
-        int xx = (int)(lin >> 9), d = (int)(lin & 511) - (n - 1);
-        if (lane == 0) {
-            im.x_out[0] = xx;
-            im.d_out[0] = d;
-            *(Acc *)im.score_out = from_ord32<Acc>((uint32_t)(key >> 32));
-        }
-        for (int i = 1; i < im.k; ++i) {
-            xx += d;
-            // Only reachable with inconsistent DP data (a wait gave up): stop
-            // instead of reading outside the arrays.
-            if (xx < 0 || xx >= im.w || d < -(n - 1) || d > n - 1) {
-                if (lane == 0) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
-                return;
-            }
-            const int lo = args.use_table ? args.tab.lo[d + n - 1] : max(-(n - 1), d - im.B);
-            const int hi = args.use_table ? args.tab.hi[d + n - 1] : min(n - 1, d + im.B);
-            const Acc *mb = i + 1 < im.k ? mband(im, i + 1) : nullptr;
-            unsigned long long bk = 0;
-            for (int e = lo + lane; e <= hi; e += 32) {
-                const int sh = e < 0 ? -e : e;
-                Acc v = dead;   // the link must end inside the image (every band)
-                if (xx + e >= 0 && xx + e < im.w) {
-                    const Acc h =
-                        from_bits<Acc>(__ldcg((const uint32_t *)hw_row(im, i, e < 0, sh) + xx));
-                    v = h;
-                    if (mb) {
-                        // M_{i+1}(xx + e, e): row e + n - 1, skewed column moff + xx
-                        const Acc m = from_bits<Acc>(__ldcg(
-                            (const uint32_t *)mb + (size_t)(e + n - 1) * im.mpitch + im.moff + xx));
-                        v = m == dead ? dead : h + m;
-                    }
-                }
-                if (v != dead) {
-                    const unsigned long long k =
-                        ((unsigned long long)ord32(v) << 32) | (0xffffffffu - (unsigned)(e + n - 1));
-                    bk = bk > k ? bk : k;
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(0xffffffffu, bk, o);
-                bk = bk > other ? bk : other;
-            }
-            if (bk == 0) {   // inconsistent data, as above
-                if (lane == 0) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
-                return;
-            }
-            d = (int)(0xffffffffu - (unsigned)(bk & 0xffffffffu)) - (n - 1);
-            if (lane == 0) {
-                im.x_out[i] = xx;
-                im.d_out[i] = d;
-            }
-        }
-        if (lane == 0) im.x_out[im.k] = xx + d;
-    }
-};
-
 // The work items of an image whose bands need FHT items of their own (int32
 // / float images; the half-band items of 256-row uint8 bands), in queue
 // order, by band level: level 0 opens with the FHT items of band k-1; level
@@ -2772,55 +2264,6 @@ struct WideLevels {
         at(lo, item - start(lo), kind, band, tile);
     }
 };
-
-__device__ inline void decode_wide_one(const ImgDesc &im, long long item, int *kind, int *band,
-                                       int *tile) {
-    int fd;
-    WideLevels{im.k, im.ftiles, im.tiles}.decode(item, &fd, band, tile);
-    *kind = fd ? kItemWideDp : kItemWideFht;
-}
-
-template <typename In, typename Acc, typename Key>
-__global__ void __launch_bounds__(kWThreads, 2)
-    engine_kernel_wide(const __grid_constant__ LaunchArgs args) {
-    using P = WideEngine<In, Acc, Key>;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t s_mbar;
-    __shared__ long long s_item;
-    if (threadIdx.x == 0) {
-        mbar_init(&s_mbar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    Pipe pipe{nullptr, 0u, &s_mbar, 0u, nullptr};
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(&args.ctl->queue, 1);
-        csync<kWThreads>();
-        const long long item = s_item;
-        csync<kWThreads>();   // s_item is rewritten at the next item
-        if (item >= args.items) break;
-        const ImgDesc *im;
-        int kind, band, tile;
-        if (args.many) {
-            const Item it = args.order[item];
-            im = &args.many[it.image];
-            kind = (it.nflags >> 19) & 3;
-            band = it.band;
-            tile = it.tile;
-        } else {
-            im = &args.one;
-            decode_wide_one(args.one, item, &kind, &band, &tile);
-        }
-        if (kind == kItemWideFht) {
-            P::fht_item(*im, band, tile, smem_raw);
-            if (threadIdx.x == 0) {
-                fence_acq_rel_gpu();
-                st_release(im->fflags + (size_t)band * im->ftiles + tile, 1);
-            }
-        } else {
-            P::dp_item(*im, band, tile, smem_raw, pipe, args);
-        }
-    }
-}
 
 // The uint8 engine: four compute warpgroups (112 registers a thread) and a
 // control warp (32 registers; the rest of its warpgroup exits at once).  The
@@ -2951,14 +2394,6 @@ RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve 
             items += 2LL * p.s.k * p.ftiles;
             p.fflags = off;
             off = align_up(off + (size_t)p.s.k * 2 * p.ftiles * 4, 8);
-        } else if (p.kind == 2) {
-            p.moff = kMOff;
-            p.mpitch = (int)align_up((size_t)kMOff + p.s.w + kWTileD + 4, 32);
-            p.ftiles = (p.s.w + kWTileF - 1) / kWTileF;
-            p.hpitch = p.ftiles * kWTileF;
-            items += (long long)p.s.k * p.ftiles;
-            p.fflags = off;
-            off = align_up(off + (size_t)p.s.k * p.ftiles * 4, 8);
         } else {
             // Row reads of M go up to 4 words past the last tile's columns.
             p.moff = kMOff;
@@ -2983,13 +2418,7 @@ RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve 
     size_t d = 0;
     for (auto &p : imgs) {
         p.m0 = d;   // the two M buffers are adjacent: one tensor map covers both
-        if (p.kind == 2) {
-            // int32 / float images: one M array per band and no backpointers
-            // (the read-back recomputes each band's argmax)
-            p.m1 = d;
-            d = align_up(d + (size_t)p.s.k * p.s.D * p.mpitch * 4, 256);
-            p.bp = d;
-        } else {
+        {
             p.m1 = d + (size_t)p.s.D * p.mpitch * 4;
             d = align_up(p.m1 + (size_t)p.s.D * p.mpitch * 4, 256);
             p.bp = d;
@@ -2998,9 +2427,6 @@ RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve 
         if (p.kind == 1) {
             p.h256 = d;
             d = align_up(d + (size_t)p.s.k * 4 * 128 * p.hpitch * 2, 256);
-        } else if (p.kind == 2) {
-            p.h256 = d;   // the Hough rows, [k][2][n][hpitch] of 4 bytes
-            d = align_up(d + (size_t)p.s.k * 2 * p.s.n * p.hpitch * 4, 256);
         }
     }
     L.data_off = L.order_off + L.order_bytes;
@@ -3045,21 +2471,6 @@ bool encode_m_map(CUtensorMap *map, void *m0, int D, int mpitch, int bw, int bh,
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2-D tensor map of `rows` rows of `pitch` 4-byte values, box bw x bh (the
-// Hough rows of an int32 / float image).
-bool encode_rows_map(CUtensorMap *map, void *base, int pitch, int rows, int bw, int bh) {
-    if ((uintptr_t)base % 16 != 0 || pitch % 4 != 0 || bh > 256 || bw > 256) return false;
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)pitch, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)pitch * 4};
-    cuuint32_t box[2] = {(cuuint32_t)bw, (cuuint32_t)bh};
-    cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, 2, base, dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws, int dtype) {
     ImgDesc im{};
     im.use_tma = dtype == FHTDP_U8 &&
@@ -3068,11 +2479,6 @@ ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws, int dtype) {
     if (p.kind == 1)
         im.use_mtma = ws && encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch,
                                          kTile256, kMBox256);
-    else if (p.kind == 2)
-        im.use_mtma = ws && encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch,
-                                         kWTileD, p.s.D, p.s.k) &&
-                      encode_rows_map(&im.tmap, ws + L.data_off + p.h256, p.hpitch,
-                                      2 * p.s.k * p.s.n, kWTileD, p.s.n);
     else
         im.use_mtma = dtype == FHTDP_U8 && p.s.n <= kMaxBandFused && ws &&
                       encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch, kTile,
@@ -3112,11 +2518,6 @@ ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws, int dtype) {
         im.hpitch = p.hpitch;
         im.h256 = (uint16_t *)(data + p.h256);
         im.fflags = (int *)(ws + p.fflags);
-    } else if (p.kind == 2) {
-        im.ftiles = p.ftiles;
-        im.hwpitch = p.hpitch;
-        im.hw = data + p.h256;
-        im.fflags = (int *)(ws + p.fflags);
     }
     return im;
 }
@@ -3132,25 +2533,6 @@ int num_sms() {
         cached[dev] = v > 0 ? v : 1;
     }
     return cached[dev];
-}
-
-template <typename In, typename Acc>
-int launch_kernel_wide(const LaunchArgs &args, int max_n, cudaStream_t stream) {
-    using P = WideEngine<In, Acc, long long>;
-    const size_t smem = P::smem_bytes(max_n, args.wpad, args.use_table != 0);
-    auto kern = engine_kernel_wide<In, Acc, long long>;
-    int st = cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem),
-                         "cudaFuncSetAttribute");
-    if (st) return st;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWThreads, smem);
-    if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)num_sms() * per_sm;
-    if (grid > args.items) grid = args.items;
-    if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, kWThreads, smem, stream>>>(args);
-    return launched("engine_kernel_wide");
 }
 
 template <typename Key>
@@ -3169,19 +2551,11 @@ int launch_kernel_u8(const LaunchArgs &args, bool multi, cudaStream_t stream) {
 }
 
 // `multi`: the run holds items of more than one tile width.
-int dispatch(int dtype, int max_h, const LaunchArgs &args, int max_n, bool multi,
-             cudaStream_t stream) {
-    switch (dtype) {
-        case FHTDP_U8:
-            // 32-bit keys: values below 2^22, and dead keys (negative) that
-            // take on at most 512 * (255 h + k) over the bands stay negative.
-            if (256LL * max_h < (1LL << 22)) return launch_kernel_u8<int32_t>(args, multi, stream);
-            return launch_kernel_u8<long long>(args, multi, stream);
-        case FHTDP_I32:
-            return launch_kernel_wide<int32_t, int32_t>(args, max_n, stream);
-        default:
-            return launch_kernel_wide<float, float>(args, max_n, stream);
-    }
+int dispatch(int max_h, const LaunchArgs &args, bool multi, cudaStream_t stream) {
+    // 32-bit keys: values below 2^22, and dead keys (negative) that
+    // take on at most 512 * (255 h + k) over the bands stay negative.
+    if (256LL * max_h < (1LL << 22)) return launch_kernel_u8<int32_t>(args, multi, stream);
+    return launch_kernel_u8<long long>(args, multi, stream);
 }
 
 // Test hook state (per host thread), consumed by the next run.
@@ -3198,6 +2572,14 @@ void consume_injection(LaunchArgs *args) {
     g_inject_wait = 0;
 }
 
+// The chain takes this thread's injection for its next run.
+void hand_injection() {
+    if (g_inject_band < 0) return;
+    chain_inject(g_inject_band, g_inject_tile, g_inject_wait);
+    g_inject_band = g_inject_tile = -1;
+    g_inject_wait = 0;
+}
+
 LaunchArgs base_args(const RunLayout &L, char *ws, int count) {
     LaunchArgs args{};
     args.count = count;
@@ -3206,7 +2588,6 @@ LaunchArgs base_args(const RunLayout &L, char *ws, int count) {
     args.wait_cycles = 4000000000LL;   // about two seconds at GB300 clocks
     args.skip_band = -1;
     args.skip_tile = -1;
-    args.wpad = kWPad;
     consume_injection(&args);
     return args;
 }
@@ -3230,9 +2611,6 @@ ImgPlan single_plan(int dtype, const void *img, int pitch, const Shape &s, int B
     if (fused_256(dtype, s, p.B, img, pitch)) {
         p.kind = 1;
         p.T = kTile256;
-    } else if (dtype != FHTDP_U8 && s.n <= kMaxBandFused) {
-        p.kind = 2;   // FHT items and narrow DP items
-        p.T = kWTileD;
     }
     return p;
 }
@@ -3258,11 +2636,16 @@ struct BatchPlan {
     void *bound_ws = nullptr;
     long long target = 0;           // queue width (tiles per band level or step)
     int mode = 0;                   // queue schedule, see queue_order
+    // int32 / float images with bands of at most 128 rows run on the chain
+    // (chain.cu), in the place of the fused launch.
+    ChainBatch *chain = nullptr;
+    std::vector<ChainImage> chain_images;
     bool use_table = false;         // bend-angle windows (fhtdp_batch_angle)
     WindowTable tab{};
     size_t reserve = 0;             // bytes of the fused part for any tile-width choice
     size_t ws_total = 0;            // workspace bytes (the reserve and the side lanes)
     ~BatchPlan() {
+        if (chain) chain_batch_destroy(chain);
         for (cudaStream_t st : side) cudaStreamDestroy(st);
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
     }
@@ -3276,7 +2659,6 @@ struct BatchPlan {
 // band level also holds the half-band FHT items of the band above).
 long long level_weight(const ImgPlan &p) {
     if (p.kind == 1) return p.tiles + 2LL * p.ftiles;
-    if (p.kind == 2) return std::max(1LL, (long long)((p.tiles + 3) / 4 + (p.ftiles + 1) / 2));
     return p.tiles;
 }
 
@@ -3286,22 +2668,15 @@ long long level_weight(const ImgPlan &p) {
 // ready one level ahead.
 void push_level(std::vector<Item> &order, const ImgPlan &p, int i, int lv) {
     const int b = p.s.k - 1 - lv;
-    if (p.kind == 1 || p.kind == 2) {
-        // FHT items of a band: both halves' tiles (256-row bands) or its tiles
-        // (256-row bands: the halves of band b-1 in a block before the DP items
-        // of band b; their DP items wait mostly for those of band b+1)
-        const long long F = p.kind == 1 ? 2LL * p.ftiles : p.ftiles;
-        const WideLevels wl{p.s.k, F, p.tiles, p.kind == 1 ? 1 : kWAhead, p.kind != 1};
+    if (p.kind == 1) {
+        // both halves' tiles: the halves of band b-1 in a block before the DP
+        // items of band b (whose DP items wait mostly for those of band b+1)
+        const WideLevels wl{p.s.k, 2LL * p.ftiles, p.tiles, 1, false};
         const long long len = wl.start(lv + 1) - wl.start(lv);
         for (long long off = 0; off < len; ++off) {
-            int dp, band, tile;
+            int dp, band, tile, kind = kItemDp256;
             wl.at(lv, off, &dp, &band, &tile);
-            int kind;
-            if (p.kind == 2) {
-                kind = dp ? kItemWideDp : kItemWideFht;
-            } else if (dp) {
-                kind = kItemDp256;
-            } else {
+            if (!dp) {
                 kind = kItemHalf0 + tile / p.ftiles;
                 tile %= p.ftiles;
             }
@@ -3459,10 +2834,7 @@ void set_point(ImgPlan &p, int j, int xp) {
 int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
                int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream) {
     if (ws_bytes >= chain_layout(s, false).total) {
-        LaunchArgs hook{};
-        hook.skip_band = -1;
-        consume_injection(&hook);
-        if (hook.skip_band >= 0) chain_inject(hook.skip_band, hook.skip_tile, hook.wait_cycles);
+        hand_injection();
         ChainQuery q;
         q.B = B;
         return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
@@ -3476,34 +2848,7 @@ int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int
     args.one = make_desc(one[0], L, base, dtype);
     args.many = nullptr;
     args.order = nullptr;
-    return dispatch(dtype, L.max_h, args, L.max_n, L.multi_tile, stream);
-}
-
-// The window table's cover in the DP items: the shortest window that no end
-// of the range clips (else the shortest of all), made odd, is 2 B0 + 1; every
-// window at least as long is covered by pieces of that length, every shorter
-// one is clipped.  The centred maxima read V up to 2 B0 + 16 rows beyond the
-// range, so the dead pad holds that many rows (even, for the copies' 128-byte
-// alignment).
-void set_table(LaunchArgs &args, const WindowTable &t) {
-    const int n = t.n, D = 2 * n - 1;
-    int L0 = D, L0c = D;
-    bool any = false;
-    for (int i = 0; i < D; ++i) {
-        const int len = t.hi[i] - t.lo[i] + 1;
-        L0c = std::min(L0c, len);
-        if (t.lo[i] > -(n - 1) && t.hi[i] < n - 1) {
-            L0 = any ? std::min(L0, len) : len;
-            any = true;
-        }
-    }
-    if (!any) L0 = L0c;
-    if (L0 < 1) L0 = 1;
-    const int Lp = L0 % 2 ? L0 : L0 - 1;
-    args.use_table = 1;
-    args.tab = t;
-    args.B0 = (Lp - 1) / 2;
-    args.wpad = std::max(kWPad, (2 * args.B0 + 16 + 1) & ~1);
+    return dispatch(L.max_h, args, L.multi_tile, stream);
 }
 
 int engine_status(const void *ws, cudaStream_t stream) {
@@ -3543,11 +2888,21 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
         }
         if (s.n > kMaxBandFused && p.kind != 1)
             plan->separate.push_back(p);
-        else
+        else if (dtype == FHTDP_U8)
             plan->imgs.push_back(p);
+        else
+            plan->chain_images.push_back(ChainImage{io.img, io.pitch, s, io.B, io.x_out, io.d_out,
+                                                    io.score_out});
     }
     plan->L = plan_layout(plan->imgs, true);
-    {
+    if (!plan->chain_images.empty()) {
+        plan->chain = chain_batch_create(plan->chain_images, dtype);
+        if (!plan->chain) {
+            delete plan;
+            return set_error(FHTDP_EINVAL, "out of host memory");
+        }
+        plan->reserve = chain_batch_bytes(plan->chain);
+    } else {
         std::vector<ImgPlan> any = plan->imgs;
         plan->reserve = plan_layout(any, true, true, dtype).total;
     }
@@ -3591,10 +2946,13 @@ void set_nflags(BatchPlan *plan) {
 
 size_t batch_workspace_bytes(const BatchPlan *plan) { return plan ? plan->ws_total : 0; }
 
-long long batch_items(const BatchPlan *plan) { return plan ? plan->L.items : 0; }
+long long batch_items(const BatchPlan *plan) {
+    return !plan ? 0 : plan->chain ? chain_batch_items(plan->chain) : plan->L.items;
+}
 
 // The image table and the queue of the plan's current layout into `ws`.
 int upload_tables(BatchPlan *plan, void *ws, cudaStream_t stream) {
+    if (plan->chain) return chain_batch_upload(plan->chain, ws, stream);
     plan->staging.clear();
     for (auto &p : plan->imgs) {
         plan->staging.push_back(make_desc(p, plan->L, (char *)ws, plan->dtype));
@@ -3629,9 +2987,11 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
     if (ws != plan->bound_ws)
         return set_error(FHTDP_EINVAL, "workspace differs from the one given to fhtdp_batch_upload");
     char *base = (char *)ws;
-    int st = cuda_status(cudaMemsetAsync(base, 0, plan->L.zero_bytes, stream), "cudaMemsetAsync");
+    int st = FHTDP_OK;
+    if (!plan->chain)   // (the chain clears its own part)
+        st = cuda_status(cudaMemsetAsync(base, 0, plan->L.zero_bytes, stream), "cudaMemsetAsync");
     if (st) return st;
-    // Images with 256-row bands: the standalone kernels, spread over the
+    // Images outside the batch's launch (256-row bands): the chain, spread over the
     // plan's lanes (forked from and joined back into `stream` by events, so
     // the run stays one stream-ordered operation for the caller).
     if (plan->lanes) {
@@ -3653,8 +3013,11 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
         LaunchArgs args = base_args(plan->L, base, (int)plan->imgs.size());
         args.many = (const ImgDesc *)(base + plan->L.table_off);
         args.order = (const Item *)(base + plan->L.order_off);
-        if (plan->use_table) set_table(args, plan->tab);
-        st = dispatch(plan->dtype, plan->L.max_h, args, plan->L.max_n, plan->L.multi_tile, stream);
+        st = dispatch(plan->L.max_h, args, plan->L.multi_tile, stream);
+    }
+    if (plan->chain && !st) {
+        hand_injection();
+        st = chain_batch_run(plan->chain, base, plan->use_table ? &plan->tab : nullptr, stream);
     }
     // Join the lanes back (also after an error, so that `stream` never runs
     // ahead of work it forked).
@@ -3865,7 +3228,7 @@ int batch_points(BatchPlan *plan, void *ws, const int32_t *points, cudaStream_t 
     if (!plan || !points) return set_error(FHTDP_EINVAL, "null plan or points");
     if (ws != plan->bound_ws)
         return set_error(FHTDP_EINVAL, "workspace differs from the one given to fhtdp_batch_upload");
-    if (!plan->separate.empty())
+    if (!plan->separate.empty() || plan->chain)
         return set_error(FHTDP_EINVAL, "points: the batch has images outside the fused engine");
     // The images in the caller's order are the plan's images (none separate).
     for (size_t i = 0; i < plan->imgs.size(); ++i) {
@@ -3888,12 +3251,12 @@ int batch_points(BatchPlan *plan, void *ws, const int32_t *points, cudaStream_t 
 
 int batch_angle(BatchPlan *plan, double gamma) {
     if (!plan) return set_error(FHTDP_EINVAL, "null plan");
-    if (plan->dtype == FHTDP_U8 || !plan->separate.empty() || plan->imgs.empty())
+    if (!plan->chain || !plan->separate.empty())
         return set_error(FHTDP_EINVAL,
                          "bend-angle batches: int32 / float images with bands of 2..128 rows");
-    const int n = plan->imgs[0].s.n;
-    for (const ImgPlan &p : plan->imgs)
-        if (p.s.n != n || p.kind != 2 || n < 2)
+    const int n = plan->chain_images[0].s.n;
+    for (const ChainImage &c : plan->chain_images)
+        if (c.s.n != n || n < 2)
             return set_error(FHTDP_EINVAL,
                              "bend-angle batches: one band height of 2..128 rows for all images");
     WindowTable t;

@@ -1,5 +1,5 @@
-// Passes over whole images beside the band FHT of chain.cu: one-row bands, the
-// last dyadic level of 256-row bands, the row smoothing and the transpose.
+// Passes over whole images beside the band FHT of chain.cu: the last dyadic
+// level of 256-row bands, the row smoothing and the transpose.
 //
 // Sec. 2.1 (refs [10], [34]): the Hough image of a band is built bottom-up
 // over sub-bands of 1, 2, 4, ..., n rows.  Merging the top half A and the
@@ -19,19 +19,6 @@ namespace {
 
 __device__ __forceinline__ int wrap(int x, int W) {
     return x >= W ? x - W : (x < 0 ? x + W : x);
-}
-
-// n == 1: the band is a single row, and both "signs" are the padded row.
-template <typename In, typename Acc>
-__global__ void fht_single_row_kernel(const In *img, long long pitch, Shape s, int wout, Acc *out,
-                                      int opitch) {
-    const size_t total = (size_t)s.k * 2 * wout;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % wout);
-        const size_t row = i / wout;   // [band][sign]
-        out[row * opitch + x] = x < s.w ? (Acc)img[row / 2 * pitch + x] : Acc(0);
-    }
 }
 
 // The last level (sub-bands of n rows from those of n/2): a block writes one
@@ -61,12 +48,6 @@ GaussWeights binomial_weights(int r) {
     for (int j = 1; j <= 2 * r; ++j)   // row 2r of Pascal's triangle
         g.c[j] = (int32_t)((int64_t)g.c[j - 1] * (2 * r - j + 1) / j);
     return g;
-}
-
-int grid_for(size_t total) {
-    size_t blocks = (total + 255) / 256;
-    size_t cap = 152 * 16;
-    return (int)(blocks < cap ? (blocks ? blocks : 1) : cap);
 }
 
 // Main problem, step 1 (Sec. 2.3): every row convolved with the discrete
@@ -188,13 +169,6 @@ template int launch_gauss_rows<int32_t, int32_t>(const int32_t *, int, int, int,
 template int launch_gauss_rows<float, float>(const float *, int, int, int, int, float *,
                                              cudaStream_t);
 
-template <typename In, typename Acc>
-int launch_fht_single_row(const In *img, long long pitch, const Shape &s, int wout, Acc *out,
-                          int opitch, cudaStream_t stream) {
-    fht_single_row_kernel<In, Acc><<<grid_for((size_t)s.k * 2 * wout), 256, 0, stream>>>(
-        img, pitch, s, wout, out, opitch);
-    return launched("fht_single_row_kernel");
-}
 template <typename Acc>
 int launch_fht_last(const Acc *src, const Shape &s, int wout, Acc *dst, int opitch,
                     cudaStream_t stream) {
@@ -202,12 +176,6 @@ int launch_fht_last(const Acc *src, const Shape &s, int wout, Acc *dst, int opit
     return launched("fht_last_kernel");
 }
 
-template int launch_fht_single_row<uint8_t, int32_t>(const uint8_t *, long long, const Shape &,
-                                                     int, int32_t *, int, cudaStream_t);
-template int launch_fht_single_row<int32_t, int32_t>(const int32_t *, long long, const Shape &,
-                                                     int, int32_t *, int, cudaStream_t);
-template int launch_fht_single_row<float, float>(const float *, long long, const Shape &, int,
-                                                 float *, int, cudaStream_t);
 template int launch_fht_last<int32_t>(const int32_t *, const Shape &, int, int32_t *, int,
                                       cudaStream_t);
 template int launch_fht_last<float>(const float *, const Shape &, int, float *, int, cudaStream_t);
