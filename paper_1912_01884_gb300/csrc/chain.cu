@@ -259,8 +259,13 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
 // holds at most the item in work and the next one.
 //
 // A thread owns one column and runs of 8 displacements; its Hough values are
-// loaded before the wait, its window maxima come from one block pair of the van
-// Herk / Gil-Werman scheme per run.  States whose link leaves [0, vw), or that
+// loaded before the wait.  The window maxima are van Herk / Gil-Werman with the
+// runs as blocks: of its run of V_{b+1} a thread stores the maxima from every
+// value to the run's end (S) and from its start to every value (P), and a window
+// [a, z] is the largest of S(a), P(z) and the runs between (S of their first
+// values): two shared-memory reads an output and a few a run, whatever the
+// window's length, for the bend limit and for tables alike.  Windows that may
+// lie inside one run (shorter than 9) scan the values themselves.  States whose link leaves [0, vw), or that
 // the point mask excludes, are never stored as dead: every reader knows them by
 // their place (alive()).  Band 0 folds the lexicographic argmax; the last of
 // its tiles reads the polyline back (Eq. 5).
@@ -268,6 +273,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
 constexpr int kDpNT = 512;
 constexpr int kRun = 8;         // displacements of a thread's run
 constexpr int kPadB = 32;       // bend limits up to this read past the range unchecked
+constexpr int kMinLen = kRun + 1;   // windows from this length on span two runs
 
 struct ChainItem {
     int image, band, tile, pad;
@@ -283,10 +289,9 @@ struct ChainArgs {
     int skip_band, skip_tile;  // test hook: this tile of the first image never publishes
     int band;                  // >= 0: one launch per band (no queue, no flags)
     int store0;                // band 0's values are stored (needed after the run)
-    // With use_table the window of d is [tab.lo, tab.hi] instead of |e - d| <= B:
-    // answered from maxima of fixed half-width B0 (no longer than any window
-    // that an end of the range does not clip), wpad dead rows around V.
-    int use_table, B0, wpad;
+    // With use_table the window of d is [tab.lo, tab.hi] instead of |e - d| <= B;
+    // minlen: the shortest of them.
+    int use_table, minlen;
     WindowTable tab;
 };
 
@@ -327,6 +332,25 @@ template <>
 __device__ __forceinline__ float vfrom<float>(uint32_t o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
+// A load or store under a predicate: a condition in C++ costs a branch each,
+// more than the rest of an element's work.
+__device__ __forceinline__ uint32_t ld_if_bits(const void *p, bool ok, uint32_t other) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.cg.b32 %0, [%1];\n}\n"
+                 : "+r"(other)
+                 : "l"(p), "r"((uint32_t)ok));
+    return other;
+}
+template <typename Acc>
+__device__ __forceinline__ Acc ld_if(const Acc *p, bool ok, Acc other) {
+    return word_from<Acc>(ld_if_bits(p, ok, word_bits(other)));
+}
+template <typename Acc>
+__device__ __forceinline__ void st_if(Acc *p, bool ok, Acc v) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.global.b32 [%0], %1;\n}\n" ::"l"(
+                     p),
+                 "r"(word_bits(v)), "r"((uint32_t)ok)
+                 : "memory");
+}
 __device__ __forceinline__ int32_t ld_cg(const int32_t *p) { return __ldcg(p); }
 __device__ __forceinline__ float ld_cg(const float *p) { return __ldcg(p); }
 
@@ -344,59 +368,6 @@ __device__ __forceinline__ Acc *band_rows(const ChainImg &im, int b) {
 // chain uses the copy in the "-" half.
 __device__ __forceinline__ int state_at(const ChainImg &im, int x, int d) {
     return (d <= 0 ? im.n - d : d) * im.pitch + x;
-}
-
-// Window maxima of the NOUT displacements from c0 over [c - B, c + B], NOUT <=
-// 2B + 1, into M[at ..]: S[i] is the maximum over [c0 - B + i, c0 + B], G that
-// over [c0 + B + 1, c0 + B + i].  V(e) = v(e) must be readable (or dead) up to
-// c0 + B + NOUT.
-template <int NOUT, typename Acc, typename V>
-__device__ __forceinline__ void span_max(int c0, int B, Acc dead, V v, Acc *M) {
-    Acc run = dead;
-    int e = c0 + B;
-    const int stop = c0 - B + NOUT;
-#pragma unroll 1
-    for (; e - 7 >= stop; e -= 8) {
-        Acc k[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) k[i] = v(e - i);
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) k[i] = vmax(k[i], k[i + 1]);
-        run = vmax(run, vmax(vmax(k[0], k[2]), vmax(k[4], k[6])));
-    }
-#pragma unroll 1
-    for (; e >= stop; --e) run = vmax(run, v(e));
-#pragma unroll
-    for (int i = NOUT - 1; i >= 0; --i) {
-        run = vmax(run, v(c0 - B + i));
-        M[i] = run;
-    }
-    Acc G = dead;
-#pragma unroll
-    for (int i = 0; i + 1 < NOUT; ++i) {
-        G = vmax(G, v(c0 + B + 1 + i));
-        M[i + 1] = vmax(M[i + 1], G);
-    }
-}
-// The run of kRun displacements from c0 (those beyond hi are not read): one
-// block pair, or for windows shorter than the run four outputs or one at a time.
-template <typename Acc, typename V>
-__device__ __forceinline__ void run_max(int c0, int hi, int B, Acc dead, V v, Acc (&M)[kRun]) {
-    if (2 * B + 1 >= kRun) {
-        span_max<kRun, Acc>(c0, B, dead, v, M);
-    } else if (B >= 2) {
-#pragma unroll
-        for (int r = 0; r < kRun; r += 4)
-            if (c0 + r <= hi) span_max<4, Acc>(c0 + r, B, dead, v, M + r);
-    } else {
-#pragma unroll
-        for (int r = 0; r < kRun; ++r)
-            if (c0 + r <= hi) {
-                Acc m = v(c0 + r);
-                if (B) m = vmax(m, vmax(v(c0 + r - 1), v(c0 + r + 1)));
-                M[r] = m;
-            }
-    }
 }
 
 // One warp: the polyline from the argmax key (Eq. 5); every band's window is
@@ -455,26 +426,44 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
 // rows apart, and 18 words put them into different banks.
 __host__ __device__ constexpr int row_words(int cols) { return cols == 16 ? 18 : cols; }
 
-template <typename Acc, int C>
+// How an image's windows are answered: by scanning the values, from S and P with
+// dead rows around the range (bend limits up to kPadB), or from S and P with the
+// windows clipped to the range (tables, longer limits).
+enum { kScan, kPadded, kClipped };
+__host__ __device__ inline int window_mode(int use_table, int minlen, int B) {
+    if (use_table) return minlen >= kMinLen ? kClipped : kScan;
+    return 2 * B + 1 < kMinLen ? kScan : B <= kPadB ? kPadded : kClipped;
+}
+// Dead rows above and below the range, whole runs.
+__host__ __device__ inline int window_pad(int mode, int use_table, int B) {
+    if (mode == kScan && !use_table) return kRun;
+    return mode == kPadded ? (B + kRun - 1) / kRun * kRun : 0;
+}
+__host__ __device__ inline int range_rows(int n) {
+    return (2 * n - 1 + kRun - 1) / kRun * kRun;
+}
+
+// kC: the image's tile width, or 0 to take it from the image (a batch of several
+// widths: five copies of the code for one kernel spill).
+template <typename Acc, int kC>
 __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char *smem,
                            const ChainArgs &args) {
-    constexpr int Q = kDpNT / C, R = row_words(C);
+    const int C = kC ? kC : im.cols, lg = 31 - __clz(C);
+    const int Q = kDpNT >> lg, R = row_words(C);
     const int n = im.n, D = 2 * n - 1, lo = -(n - 1), hi = n - 1, xn0 = tile * C;
-    const int u = threadIdx.x & (C - 1), q = threadIdx.x / C, xn = xn0 + u;
+    const int u = threadIdx.x & (C - 1), q = threadIdx.x >> lg, xn = xn0 + u;
     const bool last = band == im.k - 1;   // (only one-band images: V = H)
-    const int B = args.use_table ? args.B0 : im.B;
-    // dead rows around V: bend limits over kPadB check the range instead
-    const int wpad = args.use_table ? args.wpad : B <= kPadB ? B + kRun : 0;
+    const int B = im.B, mode = window_mode(args.use_table, args.minlen, B);
+    const int pad = window_pad(mode, args.use_table, B), rows = range_rows(n);
     const Acc dead = Dead<Acc>::value();
-    Acc *Vt = (Acc *)smem + wpad * R;     // V(e) at row e + n - 1
+    // S (or the values), then P: row e - lo + pad of displacement e
+    Acc *S = (Acc *)smem, *P = S + (rows + 2 * pad) * R;
     const Acc *Vb = last ? nullptr : band_rows<Acc>(im, band + 1);
     Acc *Hb = band_rows<Acc>(im, band);
     // A run of kRun displacements lies in one half (bands of at least kRun
     // rows), so its states are a fixed step apart: along a column for V, along a
     // diagonal (fixed end column) for H.  Live states of an unmasked band: both
     // vertices inside.
-    // (Loads and stores under a condition cost a branch each, more than the
-    // rest of an element's work.)
     const bool in = xn < im.vw, whole = n >= kRun;
     const bool mask_h = im.mask1 == band + 1, mask_v = im.mask1 == band + 2;
     const bool inner = whole && xn0 >= n && xn0 + C + n <= im.vw;   // every state is inside
@@ -493,7 +482,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
 #pragma unroll
             for (int i = 0; i < kRun; ++i) {
                 const bool ok = in && (unsigned)(xn - c0 - i) < (unsigned)im.vw && c0 + i <= hi;
-                h[i] = ok ? ld_cg(p + i * step) : Acc(0);
+                h[i] = ld_if(p + i * step, ok, Acc(0));
             }
         } else {
 #pragma unroll
@@ -506,9 +495,10 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         }
     };
     load_h(lo + kRun * q);
-    for (int i = threadIdx.x; i < 2 * wpad * C; i += kDpNT) {
-        const int r = i / C;
-        Vt[(r < wpad ? r - wpad : r - wpad + D) * R + (i & (C - 1))] = dead;
+    for (int i = threadIdx.x; i < 2 * pad * C; i += kDpNT) {
+        const int r = i >> lg, at = (r < pad ? r : r + rows) * R + (i & (C - 1));
+        S[at] = dead;
+        if (mode == kPadded) P[at] = dead;
     }
     if (args.band >= 0) {
         // one launch per band: this one began while the band below still ran
@@ -518,8 +508,8 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         // bands below k - 1 are items; band k - 1 is complete (unless the test
         // hook holds a tile of it back)
         if (band + 1 < im.k - 1 || args.skip_band == band + 1) {
-            const int t0 = max(xn0 - (n - 1), 0) / C;
-            const int t1 = min(xn0 + C - 1 + n - 1, im.vw - 1) / C;
+            const int t0 = max(xn0 - (n - 1), 0) >> lg;
+            const int t1 = min(xn0 + C - 1 + n - 1, im.vw - 1) >> lg;
             for (int t = t0 + (int)threadIdx.x; t <= t1 && ok; t += 32) {
                 if (band + 1 == im.k - 1 && t != args.skip_tile) continue;
                 const int *flag = im.flags + (size_t)(band + 1) * im.tiles + t;
@@ -556,7 +546,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 for (int i = 0; i < kRun; ++i) {
                     const bool ok =
                         in && (unsigned)(xn + c0 + i) < (unsigned)im.vw && c0 + i <= hi;
-                    v[i] = ok ? ld_cg(p + i * step) : dead;
+                    v[i] = ld_if(p + i * step, ok, dead);
                 }
             } else {
 #pragma unroll
@@ -566,85 +556,93 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                                                                  : dead;
                 }
             }
-            Acc *dst = Vt + (c0 + n - 1) * R + u;
-            if (whole) {   // only the last run is one row short
-#pragma unroll
-                for (int i = 0; i + 1 < kRun; ++i) dst[i * R] = v[i];
-                if (c0 + kRun - 1 <= hi) dst[(kRun - 1) * R] = v[kRun - 1];
-            } else {
+            if (c0 + kRun - 1 > hi)   // the last run is short
 #pragma unroll
                 for (int i = 0; i < kRun; ++i)
-                    if (c0 + i <= hi) dst[i * R] = v[i];
+                    if (c0 + i > hi) v[i] = dead;
+            Acc *s = S + (c0 - lo + pad) * R + u, *p = P + (c0 - lo + pad) * R + u;
+            if (mode == kScan) {
+#pragma unroll
+                for (int i = 0; i < kRun; ++i) s[i * R] = v[i];
+            } else {
+                Acc run = v[0];
+                p[0] = run;
+#pragma unroll
+                for (int i = 1; i < kRun; ++i) p[i * R] = run = vmax(run, v[i]);
+                run = v[kRun - 1];
+                s[(kRun - 1) * R] = run;
+#pragma unroll
+                for (int i = kRun - 2; i >= 0; --i) s[i * R] = run = vmax(run, v[i]);
             }
         }
         __syncthreads();
     }
-    const Acc *col = Vt + (n - 1) * R + u;
-    auto vpad = [&](int e) -> Acc { return col[e * R]; };
+    const Acc *Su = S + u, *Pu = P + u;
     unsigned long long best = 0;
-    const Acc *Mc = nullptr;
-    if (args.use_table && !last) {
-        // centred maxima over [p - B, p + B], p in [lo - B, hi + B]
-        Acc *mc = (Acc *)smem + (D + 2 * wpad) * R + u;   // row p - lo + B
-        const int NC = D + 2 * B;
-        for (int i0 = kRun * q; i0 < NC; i0 += kRun * Q) {
-            Acc M[kRun];
-            run_max<Acc>(i0 + lo - B, hi + B, B, dead, vpad, M);
-#pragma unroll
-            for (int i = 0; i < kRun; ++i)
-                if (i0 + i < NC) mc[(i0 + i) * R] = M[i];
-        }
-        __syncthreads();
-        Mc = mc;
-    }
     for (int c0 = lo + kRun * q; c0 <= hi; c0 += kRun * Q) {
         if (c0 != lo + kRun * q) load_h(c0);
         Acc M[kRun];
+        const int r0 = c0 - lo + pad;   // the run's first row
+        auto run_of = [&](int j) -> Acc { return Su[j * kRun * R]; };   // maximum of run j
         if (last) {
-        } else if (args.use_table) {
-            const int L = 2 * B + 1;
-            auto mc = [&](int p) -> Acc { return Mc[(p - lo + B) * R]; };
+        } else if (mode == kPadded) {
+            // windows [r - B, r + B]: their first run is j0 or, from row 8 - ol
+            // on, j0 + 1; their last one z0 or, from row 8 - oz on, z0 + 1
+            const int j0 = (r0 - B) >> 3, z0 = (r0 + B) >> 3;
+            const int ol = (r0 - B) & 7, oz = (r0 + B) & 7;
+            Acc mid = dead;   // runs j0 + 2 .. z0 - 1
+#pragma unroll 1
+            for (int j = j0 + 2; j < z0; ++j) mid = vmax(mid, run_of(j));
+            const Acc x = run_of(j0 + 1), y = run_of(z0);
+            const Acc m00 = j0 + 1 < z0 ? vmax(mid, x) : dead;
+            const Acc m01 = j0 + 1 < z0 ? vmax(vmax(mid, x), y) : y;
+            const Acc m11 = j0 + 1 < z0 ? vmax(mid, y) : dead;
+            const Acc *a = Su + (r0 - B) * R, *z = Pu + (r0 + B) * R;
 #pragma unroll
             for (int i = 0; i < kRun; ++i) {
-                if (c0 + i > hi) continue;
-                const int wl = args.tab.lo[c0 + i - lo], wh = args.tab.hi[c0 + i - lo];
-                Acc m = dead;
-                if (wh - wl + 1 >= L) {
-                    m = mc(wh - B);
+                const bool la = i + ol >= kRun, lz = i + oz >= kRun;
+                const Acc between = la ? (lz ? m11 : mid) : (lz ? m01 : m00);
+                M[i] = vmax(vmax(a[i * R], z[i * R]), between);
+            }
+        } else if (mode == kClipped) {
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                const int c = min(c0 + i, hi);
+                const int a = (args.use_table ? args.tab.lo[c - lo] : max(c - B, lo)) - lo;
+                const int z = (args.use_table ? args.tab.hi[c - lo] : min(c + B, hi)) - lo;
+                Acc m = vmax(Su[a * R], Pu[z * R]);
 #pragma unroll 1
-                    for (int p = wl + B; p < wh - B; p += L) m = vmax(m, mc(p));
-                } else if (wh == hi) {   // clipped: the piece from the other end
-                    m = mc(wl + B);      // reaches only dead rows beyond the range
-                } else if (wl == lo) {
-                    m = mc(wh - B);
-                } else {   // not produced by the host's choice of B0; kept exact
-#pragma unroll 1
-                    for (int e = wl; e <= wh; ++e) m = vmax(m, vpad(e));
-                }
+                for (int j = (a >> 3) + 1; j < z >> 3; ++j) m = vmax(m, run_of(j));
                 M[i] = m;
             }
-        } else if (wpad) {
-            run_max<Acc>(c0, hi, B, dead, vpad, M);
+        } else if (args.use_table) {
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) {
+                const int c = min(c0 + i, hi);
+                const int a = args.tab.lo[c - lo] - lo, z = args.tab.hi[c - lo] - lo;
+                Acc m = dead;
+#pragma unroll 1
+                for (int r = a; r <= z; ++r) m = vmax(m, Su[r * R]);
+                M[i] = m;
+            }
         } else {
-            // long windows (2B + 1 > 64): the part common to the run's windows
-            // inside the range, then one value more at either side
-            const int from = max(c0 + kRun - 1 - B, lo), to = min(c0 + B, hi);
-            Acc run = dead;
-#pragma unroll 4
-            for (int e = from; e <= to; ++e) run = vmax(run, vpad(e));
+            // B <= 3: the run and three values either side, widened B times
+            Acc w[kRun + 6];
 #pragma unroll
-            for (int i = kRun - 1; i >= 0; --i) {   // down to c0 + i - B
-                const int e = c0 + i - B;
-                if (e >= lo && e < from) run = vmax(run, vpad(e));
-                M[i] = run;
-            }
-            Acc G = dead;
+            for (int i = 0; i < kRun + 6; ++i) w[i] = Su[(r0 - 3 + i) * R];
 #pragma unroll
-            for (int i = 1; i < kRun; ++i) {
-                const int e = c0 + i + B;
-                if (e <= hi) G = vmax(G, vpad(e));
-                M[i] = vmax(M[i], G);
-            }
+            for (int t = 1; t <= 3; ++t)
+                if (B >= t) {
+                    Acc before = w[t - 1];
+#pragma unroll
+                    for (int i = t; i < kRun + 6 - t; ++i) {
+                        const Acc here = w[i];
+                        w[i] = vmax(vmax(before, here), w[i + 1]);
+                        before = here;
+                    }
+                }
+#pragma unroll
+            for (int i = 0; i < kRun; ++i) M[i] = w[i + 3];
         }
         if (inner && !mask_h && band != 0 && args.band < 0) {
             const int step = c0 <= 0 ? -(im.pitch + 1) : im.pitch - 1;
@@ -661,8 +659,9 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
             Acc *p = Hb + state_at(im, xn - c0, c0);
 #pragma unroll
             for (int i = 0; i < kRun; ++i)
-                if (in && (unsigned)(xn - c0 - i) < (unsigned)im.vw && c0 + i <= hi)
-                    p[i * step] = M[i] == dead ? dead : h[i] + M[i];
+                st_if(p + i * step,
+                      in && (unsigned)(xn - c0 - i) < (unsigned)im.vw && c0 + i <= hi,
+                      M[i] == dead ? dead : h[i] + M[i]);
             continue;
         }
 #pragma unroll
@@ -720,17 +719,7 @@ __global__ void __launch_bounds__(kDpNT, 2) dp_chain_kernel(const __grid_constan
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
     auto item = [&](const ChainImg &im, int band, int tile) {
-        if constexpr (kC != 0) {
-            chain_item<Acc, kC>(im, band, tile, smem, args);
-        } else {
-            switch (im.cols) {
-                case 16: chain_item<Acc, 16>(im, band, tile, smem, args); break;
-                case 32: chain_item<Acc, 32>(im, band, tile, smem, args); break;
-                case 64: chain_item<Acc, 64>(im, band, tile, smem, args); break;
-                case 128: chain_item<Acc, 128>(im, band, tile, smem, args); break;
-                default: chain_item<Acc, 256>(im, band, tile, smem, args); break;
-            }
-        }
+        chain_item<Acc, kC>(im, band, tile, smem, args);
     };
     if (args.band >= 0) {
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -900,36 +889,21 @@ void take_injection(ChainArgs &a) {
     g_skip_band = g_skip_tile = -1;
 }
 
-size_t dp_smem(int n, int cols, int wpad, bool table) {
-    return (size_t)(2 * n - 1 + 2 * wpad) * row_words(cols) * 4 * (table ? 2 : 1);
-}
-
-// The window table's cover: the shortest window that no end of the range clips
-// (else the shortest of all), made odd, is 2 B0 + 1.
 void chain_table(ChainArgs &a, const WindowTable &t) {
-    const int n = t.n, D = 2 * n - 1;
-    int L0 = D, L0c = D;
-    bool any = false;
-    for (int i = 0; i < D; ++i) {
-        const int len = t.hi[i] - t.lo[i] + 1;
-        L0c = len < L0c ? len : L0c;
-        if (t.lo[i] > -(n - 1) && t.hi[i] < n - 1) {
-            L0 = any && L0 < len ? L0 : len;
-            any = true;
-        }
-    }
-    if (!any) L0 = L0c;
-    if (L0 < 1) L0 = 1;
     a.use_table = 1;
     a.tab = t;
-    a.B0 = ((L0 % 2 ? L0 : L0 - 1) - 1) / 2;
-    a.wpad = 2 * a.B0 + kRun;
+    a.minlen = 2 * t.n - 1;
+    for (int i = 0; i < 2 * t.n - 1; ++i) {
+        const int len = t.hi[i] - t.lo[i] + 1;
+        a.minlen = len < a.minlen ? len : a.minlen;
+    }
 }
 
 // Shared memory of one image's items.
 size_t item_smem(const ChainArgs &a, const ChainImg &im) {
-    const int wpad = a.use_table ? a.wpad : im.B <= kPadB ? im.B + kRun : 0;
-    return dp_smem(im.n, im.cols, wpad, a.use_table != 0);
+    const int mode = window_mode(a.use_table, a.minlen, im.B);
+    const int rows = range_rows(im.n) + 2 * window_pad(mode, a.use_table, im.B);
+    return (size_t)rows * row_words(im.cols) * 4 * 2;
 }
 
 template <typename Acc, int kC>
