@@ -21,6 +21,33 @@
 namespace fhtdp {
 namespace {
 
+// A load or store under a predicate: a condition in C++ costs a branch each,
+// more than the rest of an element's work.
+__device__ __forceinline__ uint32_t ld_nc_if(const void *p, bool ok) {   // through L1
+    uint32_t v = 0;
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.nc.b32 %0, [%1];\n}\n"
+                 : "+r"(v)
+                 : "l"(p), "r"((uint32_t)ok));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_if_bits(const void *p, bool ok, uint32_t other) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.cg.b32 %0, [%1];\n}\n"
+                 : "+r"(other)
+                 : "l"(p), "r"((uint32_t)ok));
+    return other;
+}
+template <typename Acc>
+__device__ __forceinline__ Acc ld_if(const Acc *p, bool ok, Acc other) {
+    return word_from<Acc>(ld_if_bits(p, ok, word_bits(other)));
+}
+template <typename Acc>
+__device__ __forceinline__ void st_if(Acc *p, bool ok, Acc v) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.global.b32 [%0], %1;\n}\n" ::"l"(
+                     p),
+                 "r"(word_bits(v)), "r"((uint32_t)ok)
+                 : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Band FHT (Sec. 2.1): a block takes T columns of one sub-band of m <= 128
 // rows, builds the first two levels in registers from the image, merges the
@@ -47,26 +74,52 @@ struct BandFht {
         return c >= 0 && c < im.w ? (Acc)row[c] : Acc(0);
     }
     // Pixels c .. c + 3, c a multiple of 4; kInside: all in the image and
-    // aligned.
+    // aligned.  Elsewhere a predicated load (one launch of one image waits for
+    // its edge blocks), or four in unaligned rows and where the four straddle
+    // the image's edge; columns past W (of the padding's outputs) wrap around.
+    __device__ bool inside4(int c) const { return aligned && c >= 0 && c + 4 <= im.w; }
     template <bool kInside>
     __device__ uint32_t quad8(const In *row, int c) const {
-        if (kInside || (aligned && c >= 0 && c + 4 <= im.w))
-            return __ldg((const uint32_t *)(row + c));
-        uint32_t v = 0;
-#pragma unroll 1
-        for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
+        if (kInside) return __ldg((const uint32_t *)(row + c));
+        const bool ok = inside4(c);
+        uint32_t v = ld_nc_if(row + c, ok);
+        if (!ok && c >= 0 && c < im.w) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                uint32_t b = 0;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.nc.u8 %0, [%1];\n}\n"
+                    : "+r"(b)
+                    : "l"(row + c + j), "r"((uint32_t)(c + j < im.w)));
+                v |= b << (8 * j);
+            }
+        } else if (c + 3 >= im.W) {
+            for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
+        }
         return v;
     }
     template <bool kInside>
     __device__ void quad32(const In *row, int c, Acc *v) const {
-        if (kInside || (aligned && c >= 0 && c + 4 <= im.w)) {
+        if (kInside) {
             unpack4(__ldg((const uint4 *)(row + c)), v);
             return;
         }
-        v[0] = px(row, c);
-        v[1] = px(row, c + 1);
-        v[2] = px(row, c + 2);
-        v[3] = px(row, c + 3);
+        const bool ok = inside4(c);
+        uint4 q = make_uint4(0, 0, 0, 0);
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n"
+            " @p ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];\n}\n"
+            : "+r"(q.x), "+r"(q.y), "+r"(q.z), "+r"(q.w)
+            : "l"(row + c), "r"((uint32_t)ok));
+        unpack4(q, v);
+        if (!ok && c >= 0 && c < im.w) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                v[j] = word_from<Acc>(ld_nc_if(row + c + j, c + j < im.w));
+        } else if (c + 3 >= im.W) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = px(row, c + j);
+        }
     }
     // Words u .. u + N - 1 (u a multiple of 4) of sub-band row y; kSign 1: of
     // the mirrored strip (packed words hold both).
@@ -331,25 +384,6 @@ __device__ __forceinline__ int32_t vfrom<int32_t>(uint32_t o) {
 template <>
 __device__ __forceinline__ float vfrom<float>(uint32_t o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
-}
-// A load or store under a predicate: a condition in C++ costs a branch each,
-// more than the rest of an element's work.
-__device__ __forceinline__ uint32_t ld_if_bits(const void *p, bool ok, uint32_t other) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p ld.global.cg.b32 %0, [%1];\n}\n"
-                 : "+r"(other)
-                 : "l"(p), "r"((uint32_t)ok));
-    return other;
-}
-template <typename Acc>
-__device__ __forceinline__ Acc ld_if(const Acc *p, bool ok, Acc other) {
-    return word_from<Acc>(ld_if_bits(p, ok, word_bits(other)));
-}
-template <typename Acc>
-__device__ __forceinline__ void st_if(Acc *p, bool ok, Acc v) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.global.b32 [%0], %1;\n}\n" ::"l"(
-                     p),
-                 "r"(word_bits(v)), "r"((uint32_t)ok)
-                 : "memory");
 }
 __device__ __forceinline__ int32_t ld_cg(const int32_t *p) { return __ldcg(p); }
 __device__ __forceinline__ float ld_cg(const float *p) { return __ldcg(p); }
