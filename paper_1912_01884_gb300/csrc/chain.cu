@@ -431,14 +431,21 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
         const Acc *V = band_rows<Acc>(im, i);
         unsigned best = 0;     // order image of the value (0: none)
         unsigned be = INT_MAX; // its displacement index
-        for (int e = lo + lane; e <= hi; e += 32) {
-            if (!alive(im, i, x, e)) continue;
-            const Acc v = ld_cg(V + state_at(im, x, e));
-            if (v == Dead<Acc>::value()) continue;
-            const unsigned o = vord(v);
-            if (o > best) {
-                best = o;
-                be = e + n - 1;
+        for (int e0 = lo + lane; e0 <= hi; e0 += 128) {   // four loads in flight
+            Acc v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int e = e0 + 32 * j;
+                v[j] = ld_if(V + state_at(im, x, e), e <= hi && alive(im, i, x, e),
+                             Dead<Acc>::value());
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned o = v[j] == Dead<Acc>::value() ? 0 : vord(v[j]);
+                if (o > best) {
+                    best = o;
+                    be = e0 + 32 * j + n - 1;
+                }
             }
         }
         const unsigned top = __reduce_max_sync(0xffffffffu, best);
