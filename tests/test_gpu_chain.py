@@ -1,0 +1,125 @@
+"""The chain (one-pass band FHT, DP tiles, read-back) at the edges of its rules:
+window modes, tile and block widths, edge columns, unaligned rows, batches of
+several tile widths.  Integer results and decisions equal the oracle's exactly,
+float Hough values bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import hough_from_oracle, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _img(h, w, dtype, seed):
+    rng = np.random.default_rng(seed)
+    if dtype == "u8":
+        return rng.integers(0, 256, (h, w)).astype(np.uint8)
+    if dtype == "i32":
+        return rng.integers(-3000, 3000, (h, w)).astype(np.int32)
+    return np.abs(rng.standard_normal((h, w))).astype(np.float32)
+
+
+def _detect(img, k, B):
+    return oracle.detect_f32(img, k, B) if img.dtype == np.float32 else oracle.detect(img, k, B)
+
+
+def _same(got, want):
+    x, d, s = (t.cpu().numpy() for t in got)
+    xo, do, so = want
+    assert list(x) == list(xo) and list(d) == list(do)
+    assert s.reshape(-1)[0] == s.dtype.type(so)
+
+
+# Scanned windows (B <= 3), padded ones (up to 32; not a multiple of the run of
+# 8, one run, several), clipped ones (33 and on), for the tile widths 256 .. 16.
+@pytest.mark.parametrize("n,B", [(1, 0), (2, 1), (4, 3), (4, 6), (8, 2), (8, 3), (8, 4), (8, 14),
+                                 (16, 7), (16, 8), (32, 9), (32, 31), (64, 16), (64, 32), (64, 33),
+                                 (128, 5), (128, 24), (128, 32), (128, 33), (128, 100), (128, 254),
+                                 (256, 3), (256, 32), (256, 40), (256, 510)])
+def test_detect_every_window_mode_matches_oracle(lib, n, B):
+    for dtype, w in (("u8", 333), ("i32", 260), ("f32", 301)):
+        k = 4 if n > 64 else 6
+        img = _img(k * n, w, dtype, 13 * n + B)
+        _same(lib.detect_polyline(to_device(img), k, B), _detect(img, k, B))
+
+
+# Shortest windows of 1 (scanned), 8 / 9 / 10 around the rule, and long ones.
+@pytest.mark.parametrize("n,gamma", [(8, 0.3), (32, 0.12), (32, 0.14), (32, 0.16), (64, 0.07),
+                                     (128, 0.02), (128, 0.035), (128, 0.04), (128, 0.5),
+                                     (256, 0.0175), (256, 0.3)])
+def test_angle_windows_around_the_run_length(lib, n, gamma):
+    k = 4
+    for dtype in ("u8", "f32"):
+        img = _img(k * n, 290, dtype, n)
+        want = (oracle.detect_angle_f32 if dtype == "f32" else oracle.detect_angle)(img, k, 1, gamma)
+        _same(lib.detect_polyline_angle(to_device(img), k, 1, gamma), want)
+
+
+# Widths at the edges of the FHT's columns (multiples of 16), rows that cannot
+# be read four pixels at a time, images narrower than a band.
+@pytest.mark.parametrize("n", [4, 8, 16, 128, 256])
+@pytest.mark.parametrize("w", [1, 15, 16, 17, 255, 256, 257, 512, 530])
+def test_fht_block_widths_match_oracle(lib, n, w):
+    for dtype in ("u8", "f32"):
+        img = _img(2 * n, w, dtype, n + w)
+        H = lib.fht_bands(to_device(img), 2).cpu().numpy()
+        if dtype == "f32":
+            want = hough_from_oracle(img, 2, float32=True)
+            assert np.array_equal(H.view(np.uint32), want.view(np.uint32))
+        else:
+            assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, 2))
+
+
+@pytest.mark.parametrize("dtype", ["i32", "f32"])
+def test_batch_of_every_band_height(lib, dtype):
+    shapes = [(256, 333, 128, 16), (512, 70, 128, 40), (256, 500, 64, 3), (320, 201, 32, 5),
+              (128, 640, 16, 2), (64, 300, 8, 4), (64, 19, 4, 1), (40, 33, 2, 2), (17, 50, 1, 0),
+              (512, 90, 256, 20)]
+    imgs = [_img(h, w, dtype, h + w) for h, w, n, B in shapes]
+    plan = lib.BatchPlan([to_device(im) for im in imgs], [h // n for h, w, n, B in shapes],
+                         [B for h, w, n, B in shapes])
+    for _ in range(2):   # the second run finds the first one's counters
+        plan.run()
+        plan.status()
+        for i, (h, w, n, B) in enumerate(shapes):
+            _same((plan.x[i], plan.d[i], plan.score[i]), _detect(imgs[i], h // n, B))
+
+
+def test_detect_runs_in_the_engine_workspace_too(lib):
+    """A uint8 image whose workspace is too small for the chain runs on the
+    fused engine, with the same results."""
+    import torch
+    img = _img(1024, 700, "u8", 5)
+    dimg = to_device(img)
+    need = lib.workspace_bytes(0, 1024, 700, 8, 12)
+    want = _detect(img, 8, 12)
+    for size in (need, need - 4096):
+        _same(lib.detect_polyline(dimg, 8, 12, ws=torch.empty(size, dtype=torch.uint8, device="cuda")),
+              want)
+
+
+@pytest.mark.parametrize("r", [0, 1, 4, 5])
+@pytest.mark.parametrize("w,pitch", [(1, 1), (7, 8), (64, 64), (130, 131), (1025, 1028)])
+def test_gauss_rows_edges(lib, r, w, pitch):
+    import torch
+    for dtype in ("u8", "i32", "f32"):
+        img = _img(5, w, dtype, w + r)
+        big = torch.zeros((5, pitch), dtype=to_device(img).dtype, device="cuda")
+        big[:, :w] = to_device(img)
+        got = lib.gauss_rows(big[:, :w], r).cpu().numpy()
+        want = (oracle.gauss_rows_f32 if dtype == "f32" else oracle.gauss_rows)(img, r)
+        assert np.array_equal(got, want)
+
+
+def test_missing_producer_of_a_middle_band_times_out(lib):
+    import torch
+    img = to_device(_img(512, 384, "f32", 3))
+    ws = torch.empty(lib.workspace_bytes(2, 512, 384, 4, 8), dtype=torch.uint8, device="cuda")
+    lib.lib().fhtdp_debug_inject(2, 5, 2_000_000)
+    lib.detect_polyline(img, 4, 8, ws=ws)
+    with pytest.raises(lib.FhtdpError) as e:
+        lib.workspace_status(ws)
+    assert e.value.code == 4
+    _same(lib.detect_polyline(img, 4, 8, ws=ws), _detect(img.cpu().numpy(), 4, 8))
+    lib.workspace_status(ws)
