@@ -82,7 +82,8 @@ def lane_images(seed: int, count: int, h: int = 1024, w: int = 1024, k: int = 16
         lo = -offs.min(1).values
         hi = (w - 1) - offs.max(1).values
         x0 = torch.randint(0, 1 << 30, (count,), generator=g, device=device)
-        x0 = lo + x0 % (hi - lo + 1)
+        # a curve wider than the image starts at its left edge and runs off it
+        x0 = lo + x0 % (hi - lo + 1).clamp(min=1)
         xs = x0[:, None] + offs                                            # [N, k+1]
         val = torch.randint(70, 141, (count,), generator=g, device=device).float()
         # column of every row: x_i + round(d_i * y / (n-1)), halves up
@@ -92,6 +93,7 @@ def lane_images(seed: int, count: int, h: int = 1024, w: int = 1024, k: int = 16
                                            rounding_mode="floor")
         else:
             cols = xs[:, band]
+        cols = cols.clamp(0, w - 1)   # a scatter outside would stop the device
         img.scatter_(2, cols[:, :, None], val[:, None, None].expand(count, h, 1))
     return img.to(torch.uint8)
 

@@ -97,3 +97,13 @@ def test_lane_images_follow_their_recipe_on_the_host():
             prev = np.flatnonzero(bright[n, r])
             for c in np.flatnonzero(bright[n, r + 1]):
                 assert np.abs(prev - c).min() <= 1, (n, r, c)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_lane_images_narrower_than_their_curves(seed):
+    """A curve that moves further than the image is wide starts at the left
+    edge and is clipped to the image (no column outside it is written)."""
+    a = learned.lane_images(seed, 8, h=512, w=16, k=8, B=10, device="cpu")
+    assert a.dtype == torch.uint8 and tuple(a.shape) == (8, 512, 16)
+    bright = a.numpy() >= 70
+    assert np.all(bright.sum(2) >= 1) and np.all(bright.sum(2) <= 2)
