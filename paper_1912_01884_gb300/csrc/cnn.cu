@@ -171,8 +171,13 @@ __global__ void relu_backward_kernel(const __nv_bfloat16 *__restrict__ Y,
 // p of x(p + off(tap)) * dZ(p)[co], db[co] = sum of dZ(p)[co].  A thread takes
 // eight channels of one pixel of a 64-pixel segment and goes down a chain of
 // rows: its nine inputs are three new ones a row and six kept, its 72 + 8 sums
-// stay in registers, the next row's loads are in flight; at the end the 64
-// pixels' sums are added in shared memory in a fixed order.
+// stay in registers.  Bound by the loads' latency at 16 warps an SM, so three
+// rows of dZ are in flight into a ring in shared memory (a slot belongs to one
+// thread: no barrier) and one row of inputs, which L2 holds; at the end the 64
+// pixels' sums are added in shared memory in a fixed order.  32 images of
+// 256 x 256: WMMA tiles with a copy of the inputs per tap 353 us, one row in
+// flight 95 us, this 84 us.
+constexpr int kW1Ring = 4;    // slots: a row of dZ read, three in flight
 constexpr int kW1Sums = 80;   // 9 taps and the bias, eight channels
 constexpr int kW1Part = 17 * kC;   // a row of `part`: 16 tap rows (9..15 zero) and the bias
 __global__ void __launch_bounds__(256, 2) wgrad_first_kernel(
@@ -180,6 +185,7 @@ __global__ void __launch_bounds__(256, 2) wgrad_first_kernel(
     const __nv_bfloat16 *__restrict__ dZ, float *__restrict__ dW, float *__restrict__ db,
     float *__restrict__ part, bool wide) {
     __shared__ float red[8][4][kW1Sums + 1];
+    __shared__ uint4 ring[kW1Ring][256];
     const int c = threadIdx.x & 3, px = threadIdx.x >> 2;
     const unsigned short *xs = (const unsigned short *)X;
     float acc[kW1Sums];
@@ -198,9 +204,24 @@ __global__ void __launch_bounds__(256, 2) wgrad_first_kernel(
             v[1] = in ? __ldg(p) : 0;
             v[2] = in && in2 ? __ldg(p + dil) : 0;
         };
-        auto dzs = [&](int j) {
-            return ld8(dZ + (((size_t)rr.n * H + rr.row(j)) * W + x) * kC + 8 * c, wide);
+        // dZ of chain row i + o into its slot of this thread's ring
+        auto dzs = [&](int o) {
+            if (o < rr.L) {
+                const __nv_bfloat16 *p =
+                    dZ + (((size_t)rr.n * H + rr.row(rr.i + o)) * W + x) * kC + 8 * c;
+                uint4 *slot = &ring[o % kW1Ring][threadIdx.x];
+                if (wide)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(slot)),
+                                 "l"(p)
+                                 : "memory");
+                else
+                    *slot = ld8(p, false);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
         };
+#pragma unroll
+        for (int o = 0; o < kW1Ring - 1; ++o) dzs(o);
         uint32_t v[3];
         float xf[9];   // rows above, at and below
         auto keep = [&](int at) {
@@ -212,16 +233,15 @@ __global__ void __launch_bounds__(256, 2) wgrad_first_kernel(
         inputs(rr.i, v);
         keep(2);
         inputs(rr.i + 1, v);
-        uint4 z = dzs(rr.i);
         for (int o = 0; o < rr.L; ++o) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) xf[k] = xf[k + 3];
             keep(2);
+            if (o + 1 < rr.L) inputs(rr.i + o + 2, v);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kW1Ring - 2) : "memory");
+            const uint4 z = ring[o % kW1Ring][threadIdx.x];
+            dzs(o + kW1Ring - 1);   // into the slot that the row before was read from
             const uint32_t zw[4] = {z.x, z.y, z.z, z.w};
-            if (o + 1 < rr.L) {
-                inputs(rr.i + o + 2, v);
-                z = dzs(rr.i + o + 1);
-            }
             float f[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e)
