@@ -1,6 +1,6 @@
 // Band FHTs in one pass over the image, and the DP as a chain of column tiles
-// over the stored Hough rows: the path of single images, of the queries and of
-// the standalone calls.
+// over the stored Hough rows: the path of single images, of the queries, of
+// int32 and float batches and of the calls that run one step of the method.
 //
 // One image gives the fused engine (engine.cu) few tiles per band level, and
 // the levels depend on each other: 16 of 152 SMs work on a level of a 2048 x
@@ -338,6 +338,7 @@ struct ChainArgs {
     const ChainItem *order;    // their queue
     int items;
     ChainCtl *ctl;
+    int *report;         // where a wait that gave up is noted as well (or null)
     long long wait_cycles;
     int skip_band, skip_tile;  // test hook: this tile of the first image never publishes
     int band;                  // >= 0: one launch per band (no queue, no flags)
@@ -347,6 +348,11 @@ struct ChainArgs {
     int use_table, minlen;
     WindowTable tab;
 };
+
+__device__ __forceinline__ void gave_up(const ChainArgs &a) {
+    atomicExch(&a.ctl->status, FHTDP_ETIMEOUT);
+    if (a.report) atomicExch(a.report, FHTDP_ETIMEOUT);
+}
 
 // The flags are polled with relaxed loads, one fence after the last; a poll
 // reads nothing else (another load would double its round trip).
@@ -451,7 +457,7 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
         const unsigned top = __reduce_max_sync(0xffffffffu, best);
         const unsigned at = __reduce_min_sync(0xffffffffu, best == top && top ? be : INT_MAX);
         if (at >= (unsigned)D) {   // only with inconsistent values (a wait gave up)
-            if (lane == 0 && args.ctl) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
+            if (lane == 0 && args.ctl) gave_up(args);
             return;
         }
         d = (int)at - (n - 1);
@@ -568,7 +574,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
             fence_gpu();
         }
         if (!__all_sync(0xffffffffu, ok) && threadIdx.x == 0)
-            atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
+            gave_up(args);
     }
     if (!last) {
         __syncthreads();
@@ -1120,13 +1126,14 @@ void chain_inject(int band, int tile, long long wait_cycles) {
     g_skip_wait = wait_cycles;
 }
 
-ChainLayout chain_layout(const Shape &s, bool smooth) {
+ChainLayout chain_layout(const Shape &s, bool smooth, bool tight) {
     ChainLayout L{};
     L.cols = chain_cols(s.n);
     L.tiles = (s.vw + L.cols - 1) / L.cols;
-    // rows a multiple of 128 bytes apart, long enough for the cyclic width of
-    // 256-row bands
-    L.pitch = ((s.n > 128 ? s.W : s.vw) + 31) & ~31;
+    // rows a multiple of 128 bytes apart; those of 256-row bands hold the cyclic
+    // width (tight: and no more, where the workspace is short)
+    L.pitch = s.n > 128 ? s.W : s.vw;
+    if (!tight || s.n <= 128) L.pitch = (L.pitch + 31) & ~31;
     size_t o = sizeof(ChainCtl);
     L.key = o;   // key, done; key, done of the second polyline
     o += 256;
@@ -1147,7 +1154,7 @@ namespace {
 template <typename In, typename Acc>
 int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q, int32_t *x_out,
                    int32_t *d_out, Acc *score_out, char *ws, cudaStream_t stream) {
-    const ChainLayout L = chain_layout(s, q.r > 0);
+    const ChainLayout L = chain_layout(s, q.r > 0, q.tight);
     int st = cuda_status(cudaMemsetAsync(ws, 0, L.zero, stream), "cudaMemsetAsync");
     Acc *rows = (Acc *)(ws + L.rows), *second = (Acc *)(ws + L.second);
     if (st) return st;
@@ -1185,6 +1192,7 @@ int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q
     }
     a.items = L.tiles * (s.k > 1 ? s.k - 1 : 1);
     a.ctl = (ChainCtl *)ws;
+    a.report = q.report;
     take_injection(a);
     a.band = -1;
     a.store0 = q.sep > 0;
@@ -1305,9 +1313,7 @@ int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream) {
 namespace {
 template <typename Acc>
 int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaStream_t stream) {
-    int st = cuda_status(cudaMemsetAsync(ws, 0, b->zero, stream), "cudaMemsetAsync");
-    if (!st)
-        st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<Acc, Acc>,
+    int st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<Acc, Acc>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)b->fht_smem),
                          "cudaFuncSetAttribute");
@@ -1329,6 +1335,10 @@ int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaS
     return launch_chain_cols<Acc>(a, b->cols, smem, a.items, false, stream);
 }
 }  // namespace
+
+int chain_batch_clear(const ChainBatch *b, void *ws, cudaStream_t stream) {
+    return cuda_status(cudaMemsetAsync(ws, 0, b->zero, stream), "cudaMemsetAsync");
+}
 
 int chain_batch_run(const ChainBatch *b, void *ws, const WindowTable *t, cudaStream_t stream) {
     return b->dtype == FHTDP_F32 ? chain_batch_run_t<float>(b, (char *)ws, t, stream)

@@ -47,7 +47,7 @@ struct ChainLayout {
     int pitch, cols, tiles;
 };
 // smooth: the image is smoothed first (angle queries, r > 0).
-ChainLayout chain_layout(const Shape &s, bool smooth);
+ChainLayout chain_layout(const Shape &s, bool smooth, bool tight = false);
 
 struct ChainQuery {
     int B = 0;                          // bend limit
@@ -55,6 +55,8 @@ struct ChainQuery {
     const PointMask *point = nullptr;
     int r = 0;                          // smoothing half-width
     int sep = 0;                        // > 0: also the second polyline
+    bool tight = false;                 // the layout of chain_layout(.., tight)
+    int *report = nullptr;              // a second place for the run's status
 };
 // FHT (after smoothing), DP and read-back of one image on workspace ws of at
 // least chain_layout().total bytes.
@@ -78,7 +80,9 @@ size_t chain_batch_bytes(const ChainBatch *b);
 long long chain_batch_items(const ChainBatch *b);
 // The batch's tables for workspace ws (from host memory held by the batch).
 int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream);
-// t (optional): bend-angle windows for all images (one band height).
+// A run: the clearing of its head, then the launches.  t (optional): bend-angle
+// windows for all images (one band height).
+int chain_batch_clear(const ChainBatch *b, void *ws, cudaStream_t stream);
 int chain_batch_run(const ChainBatch *b, void *ws, const WindowTable *t, cudaStream_t stream);
 
 // The next chain run of this thread never publishes tile `tile` of band

@@ -24,7 +24,8 @@
 // 32-bit word (two 16-bit lanes: sums of at most 128 uint8 pixels fit), so
 // one shared-memory access and one integer add serve both halves.  The "-"
 // half is computed on the mirrored strip, so both halves use the same
-// merge.  int32 and float images run the halves one after the other.
+// merge.  int32 and float images, and single images of every type, run on the
+// chain (chain.cu).
 #include <algorithm>
 #include <climits>
 #include <cstddef>
@@ -40,7 +41,6 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kTile = 128;             // output columns of one item
-constexpr int kQ = kThreads / kTile;   // threads sharing a column in the DP
 // The uint8 engine adds a fifth warpgroup whose first warp runs the control
 // of the work items (queue, dependency flags, copies, publication) so that
 // its waits stay off the compute warps' path; the other three warps exit.
@@ -95,13 +95,7 @@ struct ImgDesc {
     int hpitch;               // row pitch of h256 in elements
     uint16_t *h256;           // [k][2 halves][2 signs][128 shifts][hpitch], see h256_row
     int *fflags;              // [k][2][ftiles] publication flags of the half-band items
-                              // (int32 / float images: [k][ftiles], their FHT items)
     int moff;                 // column offset of the skewed M layout
-    // int32 / float images (kind 2): Hough rows of every band stored by the
-    // FHT items, [k][2 signs][n][hwpitch] of 4-byte values; `tmap` then
-    // describes them for the DP items' TMA copies (boxes of 32 x n).
-    void *hw;
-    int hwpitch;
     // Optional device flag: when it reads 0 at the launch, every item of the
     // image is skipped (the learned proposal's fallback run only redoes the
     // images that need the full DP).
@@ -151,32 +145,18 @@ struct LaunchArgs {
 // ---------------------------------------------------------------------------
 // Value <-> order-preserving integers.
 __device__ __forceinline__ uint32_t ord32(int32_t v) { return (uint32_t)v ^ 0x80000000u; }
-__device__ __forceinline__ uint32_t ord32(float f) {
-    uint32_t b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
 template <typename Acc>
 __device__ __forceinline__ Acc from_ord32(uint32_t o);
 template <>
 __device__ __forceinline__ int32_t from_ord32<int32_t>(uint32_t o) {
     return (int32_t)(o ^ 0x80000000u);
 }
-template <>
-__device__ __forceinline__ float from_ord32<float>(uint32_t o) {
-    return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
-}
 
 template <typename W>
 __device__ __forceinline__ W from_bits(uint32_t b);
 template <>
 __device__ __forceinline__ uint32_t from_bits<uint32_t>(uint32_t b) { return b; }
-template <>
-__device__ __forceinline__ int32_t from_bits<int32_t>(uint32_t b) { return (int32_t)b; }
-template <>
-__device__ __forceinline__ float from_bits<float>(uint32_t b) { return __uint_as_float(b); }
 __device__ __forceinline__ uint32_t to_bits(uint32_t v) { return v; }
-__device__ __forceinline__ uint32_t to_bits(int32_t v) { return (uint32_t)v; }
-__device__ __forceinline__ uint32_t to_bits(float v) { return __float_as_uint(v); }
 
 // Window keys: a value and its displacement index e + n - 1 (< 512) in one
 // integer whose maximum is the largest value with the smallest index.
@@ -206,7 +186,6 @@ template <typename T>
 __device__ __forceinline__ T kmax(T a, T b) {
     return a > b ? a : b;
 }
-__device__ __forceinline__ float kmax(float a, float b) { return fmaxf(a, b); }
 
 __device__ __forceinline__ int brev(int r, int bits) {
     return bits ? (int)(__brev((unsigned)r) >> (32 - bits)) : 0;
@@ -238,12 +217,6 @@ __device__ __forceinline__ void nb_sync(int id, int count) {
 
 // Bounded wait on a publication flag: gives up after `limit` cycles, or at
 // once when another wait of this launch has already given up.
-// A hint to bring the 128-byte line holding p into L2 (callers pass only
-// lines that hold bytes of their buffers).
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 __device__ bool wait_flag(const int *flag, const Ctl *ctl, long long limit) {
     long long t0 = clock64();
     while (ld_acquire(flag) == 0) {
@@ -324,49 +297,12 @@ constexpr int kItemHalf0 = 1;   // FHT of the top 128-row half of a 256-row band
 constexpr int kItemHalf1 = 2;   // FHT of the bottom half
 constexpr int kItemDp256 = 3;   // last FHT level + DP of a 64-column tile of a 256-row band
 
-struct NextItem {
-    long long item;
-    int prefetched;   // its strip copy has been issued on the strip barrier
-    int pad;
-    Item it;          // its order entry (batches), copied by cp.async
-};
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
-                 : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
 struct Pipe {
     uint64_t *bar;        // strip barrier
     uint32_t phase;       // parity of its next completion
     uint64_t *mbar;       // M tile barrier
     uint32_t mphase;      // parity of its next completion
-    NextItem *next;       // shared: the CTA's next item
 };
-
-// Thread 0: records the item taken from the queue and starts copying its
-// order entry (completed by cp_async_wait_all before anyone reads it).
-__device__ __forceinline__ void stage_next(const LaunchArgs &args, NextItem *next,
-                                           long long item) {
-    next->item = item;
-    next->prefetched = 0;
-    if (args.many && item < args.items) cp_async16(&next->it, &args.order[item]);
-}
-// The staged item (item < items).
-__device__ __forceinline__ void decode_staged(const LaunchArgs &args, const NextItem &nx,
-                                              const ImgDesc **imp, int *band, int *tile) {
-    if (args.many) {
-        *imp = &args.many[nx.it.image];
-        *band = nx.it.band;
-        *tile = nx.it.tile;
-    } else {
-        *imp = &args.one;
-        *band = args.one.k - 1 - (int)(nx.item / args.one.tiles);
-        *tile = (int)(nx.item % args.one.tiles);
-    }
-}
 
 __device__ __forceinline__ uint32_t pix_u8(const uint8_t *row, int col, int w) {
     return (col >= 0 && col < w) ? (uint32_t)row[col] : 0u;
@@ -758,42 +694,6 @@ __device__ __forceinline__ void window_span32(int c0, int count, int B, VGet vke
     }
 }
 
-// Window maxima of the NOUT displacements [c0, c0 + NOUT - 1] for windows
-// of L = 2B + 1 >= NOUT (any B beyond that), one block pair of the van Herk /
-// Gil-Werman scheme: S[i] (registers) is the maximum over [c0 - B + i, c0 + B]
-// and G that over [c0 + B + 1, c0 + B + i]; output i < count goes to emit(i, m).
-template <int NOUT, typename Key, typename VGet, typename Emit>
-__device__ __forceinline__ void window_span(int c0, int count, int B, Key dead, VGet vkey,
-                                            Emit emit) {
-    const int L = 2 * B + 1;
-    const int a = c0 - B;
-    Key run = dead;
-    int j = L - 1;
-    // the part of the block beyond the first NOUT values: 8 loads at a time
-    for (; j - 7 >= NOUT; j -= 8) {
-        Key k[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) k[i] = vkey(a + j - i);
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) k[i] = kmax(k[i], k[i + 1]);
-        run = kmax(run, kmax(kmax(k[0], k[2]), kmax(k[4], k[6])));
-    }
-    for (; j >= NOUT; --j) run = kmax(run, vkey(a + j));
-    Key S[NOUT];
-#pragma unroll
-    for (int jj = NOUT - 1; jj >= 0; --jj) {
-        run = kmax(run, vkey(a + jj));
-        S[jj] = run;
-    }
-    Key G = dead;
-#pragma unroll
-    for (int i = 0; i < NOUT; ++i) {
-        const Key m = kmax(S[i], G);
-        G = kmax(G, vkey(c0 + B + 1 + i));
-        if (i < count) emit(i, m);
-    }
-}
-
 // Two-pass version for any L: pass 1 stores the in-block suffix maxima
 // S(e), e in [c0-B, c1-B], through sput/sget; pass 2 runs the in-block prefix
 // maximum G(c+B) and combines.  Blocks are aligned at `a` (a <= c0 - B).
@@ -896,56 +796,6 @@ __device__ void finish_band0(unsigned long long best, const ImgDesc &im, const L
 
 __device__ __forceinline__ unsigned long long argmax_key(uint32_t ordv, int x, int eidx) {
     return ((unsigned long long)ordv << 32) | (0xffffffffu - (unsigned)(x * 512 + eidx));
-}
-
-// Waits for the three band+1 tiles whose window maxima a tile of `band` reads.
-// `after` runs on thread 0 once the flags are seen (or the wait gave up).
-
-// Lanes 0..2 of warp 0 poll the three flags at the same time (a flag already
-// seen set by peek_dep is not read again: the fence that follows makes that
-// read an acquisition); the warp barrier passes the acquisitions on to lane 0
-// and, through the CTA barrier, to every thread.
-template <typename After>
-__device__ void wait_deps(const ImgDesc &im, int band, int tile, const LaunchArgs &args,
-                          After after, int seen = 0) {
-    if (band >= im.k - 1) return;
-    if (threadIdx.x < 32) {
-        const int c = tile - 1 + (int)threadIdx.x;
-        bool ok = true;
-        if (threadIdx.x < 3 && c >= 0 && c < im.tiles) {
-            if (!seen)
-                ok = wait_flag(im.flags + (size_t)(band + 1) * im.tiles + c, args.ctl,
-                               args.wait_cycles);
-            fence_acq_rel_gpu();
-        }
-        __syncwarp();
-        ok = __all_sync(0xffffffffu, ok);
-        if (threadIdx.x == 0) {
-            if (!ok) atomicExch(&args.ctl->status, FHTDP_ETIMEOUT);
-            after();
-        }
-    }
-    csync();
-}
-__device__ void wait_deps(const ImgDesc &im, int band, int tile, const LaunchArgs &args) {
-    wait_deps(im, band, tile, args, [] {});
-}
-
-// `before` runs on thread 0 after the CTA barrier, before the flag.
-// Every warp fences its own M and bp stores as soon as it is done, so that
-// the release by thread 0 after the CTA barrier has little left to wait for.
-template <typename Before>
-__device__ void publish(const ImgDesc &im, int band, int tile, const LaunchArgs &args,
-                        Before before) {
-    fence_acq_rel_gpu();
-    csync();
-    if (threadIdx.x == 0) before();
-    const ImgDesc &first = args.many ? args.many[0] : args.one;
-    if (band == args.skip_band && tile == args.skip_tile && im.flags == first.flags) return;
-    if (threadIdx.x == 0) st_release(im.flags + (size_t)band * im.tiles + tile, 1);
-}
-__device__ void publish(const ImgDesc &im, int band, int tile, const LaunchArgs &args) {
-    publish(im, band, tile, args, [] {});
 }
 
 // Stores M_b(x, c) (skewed so that the consumer reads M(x + d, d) as row d,
@@ -1505,7 +1355,7 @@ struct U8Path {
     // Subproblems 2-3: the states of the point's band whose vertex on the
     // point's border is not mask_x become dead (their link's start x, or for
     // the image's bottom border its end x + e), in V once it is formed: the
-    // same restriction as the standalone point mask.
+    // same restriction as the band chain's.
     template <int T>
     __device__ static void mask_point(int32_t *Vn, const ImgDesc &im, int x0) {
         const int n = im.n, D = 2 * n - 1;
@@ -2200,23 +2050,16 @@ struct U8Ctl {
 };
 
 // ---------------------------------------------------------------------------
-// The work items of an image whose bands need FHT items of their own (int32
-// / float images; the half-band items of 256-row uint8 bands), in queue
-// order, by band level: level 0 opens with the FHT items of band k-1; level
-// lv (band b = k-1-lv) holds the DP items of band b and, spread evenly among
-// them (or in a block before them), the FHT items of band b - A (level 0: of
-// bands k-2 .. k-1-A).  An FHT
-// item takes several DP items' time, so it is queued A levels before the DP
-// items that read its rows, and spreading them keeps a level's DP items from
-// waiting behind a block of FHT items.  Every item still comes after all the
-// items it waits for.
-constexpr int kWAhead = 2;
-struct WideLevels {
+// The work items of an image with 256-row bands, in queue order, by band level:
+// level 0 opens with the half-band FHT items of band k-1; level lv (band b =
+// k-1-lv) holds the half-band items of band b - 1 and, after them, the DP items
+// of band b.  A half-band item is queued a level before the DP items that read
+// its rows, and every item comes after all the items it waits for.
+struct HalfLevels {
     int k;
-    long long F, P;   // FHT and DP items of one band
-    int A = kWAhead;  // levels between an FHT item and the DP items that read it
-    bool spread = true;   // false: a level's FHT items before its DP items
-    __host__ __device__ long long fht_in(int lv) const {   // FHT items spread in level lv
+    long long F, P;   // half-band and DP items of one band
+    static constexpr int A = 1;   // levels between a half-band item and its DP items
+    __host__ __device__ long long fht_in(int lv) const {   // half-band items in level lv
         if (lv == 0) return (long long)(A < k - 1 ? A : k - 1) * F;
         return k - 1 - lv - A >= 0 ? F : 0;
     }
@@ -2228,7 +2071,7 @@ struct WideLevels {
         if (full < 0) full = 0;
         return l0 + (long long)full * (F + P) + (long long)(lv - 1 - full) * P;
     }
-    // Item `off` of level lv: FHT item `tile` of `band` (kind 0), or DP item
+    // Item `off` of level lv: half-band item `tile` of `band` (kind 0), or DP item
     // `tile` of `band` (kind 1).
     __host__ __device__ void at(int lv, long long off, int *kind, int *band, int *tile) const {
         const int b = k - 1 - lv;
@@ -2241,27 +2084,16 @@ struct WideLevels {
             }
             off -= F;
         }
-        const long long Fl = fht_in(lv), S = Fl + P;
-        const long long c0 = spread ? off * Fl / S : (off < Fl ? off : Fl);
-        const long long c1 = spread ? (off + 1) * Fl / S : (off < Fl ? off + 1 : Fl);
-        if (c1 > c0) {   // the FHT item number c0 of the level
+        const long long Fl = fht_in(lv);
+        if (off < Fl) {
             *kind = 0;
-            *band = lv == 0 ? k - 2 - (int)(c0 / F) : b - A;
-            *tile = (int)(c0 % F);
+            *band = lv == 0 ? k - 2 - (int)(off / F) : b - A;
+            *tile = (int)(off % F);
         } else {
             *kind = 1;
             *band = b;
-            *tile = (int)(off - c0);
+            *tile = (int)(off - Fl);
         }
-    }
-    __host__ __device__ void decode(long long item, int *kind, int *band, int *tile) const {
-        int lo = 0, hi = k - 1;   // the last level that starts at or before item
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) / 2;
-            if (start(mid) <= item) lo = mid;
-            else hi = mid - 1;
-        }
-        at(lo, item - start(lo), kind, band, tile);
     }
 };
 
@@ -2283,7 +2115,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    Pipe pipe{&s_bar, 0u, &s_mbar, 0u, nullptr};
+    Pipe pipe{&s_bar, 0u, &s_mbar, 0u};
     if (threadIdx.x < kThreads) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 112;" ::: "memory");
         for (;;) {
@@ -2353,8 +2185,8 @@ int tiles_of(const Shape &s, int T) { return (s.w + T - 1) / T; }
 
 // uint8 images with 256-row bands run in the fused engine when their strips
 // can go through TMA (16-byte aligned rows) and the backpointer byte
-// identifies the argmax inside a window (B <= 127); the others take the
-// standalone kernels.
+// identifies the argmax inside a window (B <= 127); the others run one by one
+// on the band chain.
 bool fused_256(int dtype, const Shape &s, int B, const void *img, long long pitch) {
     return dtype == FHTDP_U8 && s.n == 256 && B <= 127 && (uintptr_t)img % 16 == 0 &&
            pitch % 16 == 0;
@@ -2452,17 +2284,14 @@ bool encode_strip_map(CUtensorMap *map, const void *img, int h, int w, long long
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2-D int32 tensor map of an image's adjacent M buffers ([arrays * D][mpitch]:
-// two ping-pong buffers, or one per band for int32 / float images), box of bw
-// columns x bh rows: for uint8 bands of at most 128 rows 128 x D (one copy
-// brings a tile's whole M_{b+1}), for 256-row bands 64 x 73 (seven), for
-// int32 / float images 16 x D.
-bool encode_m_map(CUtensorMap *map, void *m0, int D, int mpitch, int bw, int bh,
-                  int arrays = 2) {
+// 2-D int32 tensor map of an image's two adjacent M buffers ([2 D][mpitch]), box
+// of bw columns x bh rows: for bands of at most 128 rows 128 x D (one copy
+// brings a tile's whole M_{b+1}), for 256-row bands 64 x 73 (seven).
+bool encode_m_map(CUtensorMap *map, void *m0, int D, int mpitch, int bw, int bh) {
     if ((uintptr_t)m0 % 16 != 0 || mpitch % 4 != 0 || bh > 256 || bw > 256) return false;
     PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
     if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)mpitch, (cuuint64_t)arrays * D};
+    cuuint64_t dims[2] = {(cuuint64_t)mpitch, 2 * (cuuint64_t)D};
     cuuint64_t strides[1] = {(cuuint64_t)mpitch * 4};
     cuuint32_t box[2] = {(cuuint32_t)bw, (cuuint32_t)bh};
     cuuint32_t estr[2] = {1u, 1u};
@@ -2475,7 +2304,6 @@ ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws, int dtype) {
     ImgDesc im{};
     im.use_tma = dtype == FHTDP_U8 &&
                  encode_strip_map(&im.tmap, p.io.img, p.s.h, p.s.w, p.io.pitch, p.s.n);
-    // (int32 / float images: tmap describes their Hough rows, below)
     if (p.kind == 1)
         im.use_mtma = ws && encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch,
                                          kTile256, kMBox256);
@@ -2624,7 +2452,7 @@ constexpr int kSideLanes = 4;
 struct BatchPlan {
     int dtype;
     std::vector<ImgPlan> imgs;      // images of the fused launch
-    std::vector<ImgPlan> separate;  // 256-row bands: run with the standalone kernels
+    std::vector<ImgPlan> separate;  // 256-row bands: run one by one on the band chain
     size_t separate_off = 0;        // their scratch: `lanes` slices of sep_bytes
     size_t sep_bytes = 0;
     int lanes = 0;                  // streams the separate images are spread over
@@ -2671,7 +2499,7 @@ void push_level(std::vector<Item> &order, const ImgPlan &p, int i, int lv) {
     if (p.kind == 1) {
         // both halves' tiles: the halves of band b-1 in a block before the DP
         // items of band b (whose DP items wait mostly for those of band b+1)
-        const WideLevels wl{p.s.k, 2LL * p.ftiles, p.tiles, 1, false};
+        const HalfLevels wl{p.s.k, 2LL * p.ftiles, p.tiles};
         const long long len = wl.start(lv + 1) - wl.start(lv);
         for (long long off = 0; off < len; ++off) {
             int dp, band, tile, kind = kItemDp256;
@@ -2811,9 +2639,10 @@ size_t detect_workspace_bytes(int dtype, const Shape &s, int B) {
 }
 
 // uint8 images with bands of at most 128 rows run on the engine where the
-// workspace is too small for the chain.
+// workspace is too small for the chain, the others with rows that are not padded
+// to whole lines.
 size_t detect_least_bytes(int dtype, const Shape &s, int B) {
-    const size_t chain = chain_layout(s, false).total;
+    const size_t chain = chain_layout(s, false, true).total;
     return dtype == FHTDP_U8 && s.n <= kMaxBandFused
                ? std::min(chain, engine_one_bytes(dtype, s, B))
                : chain;
@@ -2828,14 +2657,17 @@ void set_point(ImgPlan &p, int j, int xp) {
 }
 
 // One image takes the chain (chain.cu): the engine's 128-column tiles leave
-// most of the chip idle on one image (2048 x 2048: CHAIN_VS_ENGINE).  The engine
-// needs a sixth of the workspace, and takes uint8 images whose workspace is
-// too small for the chain (the built-in scratch of the no-allocation call).
+// most of the chip idle on one image (2048 x 2048 uint8: 249 us, 115 on the
+// chain; 256 x 256: 67 and 34).  The engine needs a sixth of the workspace, and
+// takes uint8 images whose workspace is too small for the chain (the built-in
+// scratch of the no-allocation call).
 int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
                int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream) {
-    if (ws_bytes >= chain_layout(s, false).total) {
+    const bool room = ws_bytes >= chain_layout(s, false).total;
+    if (room || dtype != FHTDP_U8 || s.n > kMaxBandFused) {
         hand_injection();
         ChainQuery q;
+        q.tight = !room;
         q.B = B;
         return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
     }
@@ -2906,7 +2738,7 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
         std::vector<ImgPlan> any = plan->imgs;
         plan->reserve = plan_layout(any, true, true, dtype).total;
     }
-    // Scratch of the standalone path: up to kSideLanes lanes, each a stream
+    // Scratch of the images that run by themselves: up to kSideLanes lanes, each a stream
     // that runs its images one after the other on its own slice.
     size_t sep = 0;
     for (auto &p : plan->separate) sep = std::max(sep, chain_layout(p.s, false).total);
@@ -2987,14 +2819,16 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
     if (ws != plan->bound_ws)
         return set_error(FHTDP_EINVAL, "workspace differs from the one given to fhtdp_batch_upload");
     char *base = (char *)ws;
-    int st = FHTDP_OK;
-    if (!plan->chain)   // (the chain clears its own part)
-        st = cuda_status(cudaMemsetAsync(base, 0, plan->L.zero_bytes, stream), "cudaMemsetAsync");
+    int st = plan->chain
+                 ? chain_batch_clear(plan->chain, base, stream)
+                 : cuda_status(cudaMemsetAsync(base, 0, plan->L.zero_bytes, stream),
+                               "cudaMemsetAsync");
     if (st) return st;
     // Images outside the batch's launch (256-row bands): the chain, spread over the
     // plan's lanes (forked from and joined back into `stream` by events, so
     // the run stays one stream-ordered operation for the caller).
     if (plan->lanes) {
+        if (plan->imgs.empty() && !plan->chain) hand_injection();   // (test hook)
         st = cuda_status(cudaEventRecord(plan->ev[0], stream), "cudaEventRecord");
         for (int l = 0; l < plan->lanes && !st; ++l)
             st = cuda_status(cudaStreamWaitEvent(plan->side[l], plan->ev[0], 0),
@@ -3004,6 +2838,7 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
             const int l = (int)(i % plan->lanes);
             ChainQuery q;
             q.B = p.io.B;
+            q.report = (int *)(base + offsetof(Ctl, status));
             st = chain_detect(p.io.img, plan->dtype, p.io.pitch, p.s, q, p.io.x_out, p.io.d_out,
                               p.io.score_out, base + plan->separate_off + plan->sep_bytes * l,
                               plan->side[l]);

@@ -15,11 +15,12 @@ namespace fhtdp {
 namespace {
 
 constexpr size_t kNoallocScratchBytes = FHTDP_NOALLOC_SCRATCH_BYTES;
+constexpr size_t kNoallocHead = 4096;   // the control block and flags beside the arrays
 
 // The built-in scratch.  Every GPU on which this module is loaded holds it
 // until the process exits.  In host code its name is only a stand-in for the
 // device symbol; its device address comes from cudaGetSymbolAddress.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes + kNoallocHead];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -63,7 +64,7 @@ extern "C" int fhtdp_detect_polyline_noalloc(const void *img, int dtype, int h, 
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
     const size_t need = detect_least_bytes(dtype, s, B);
-    if (need > kNoallocScratchBytes)
+    if (need > kNoallocScratchBytes + kNoallocHead)
         return set_error(FHTDP_EWORKSPACE,
                          "this image needs %zu bytes of scratch; the built-in scratch of "
                          "fhtdp_detect_polyline_noalloc holds %zu bytes (use "
@@ -72,8 +73,8 @@ extern "C" int fhtdp_detect_polyline_noalloc(const void *img, int dtype, int h, 
     void *ws = nullptr;
     int st = scratch_on_current_device(&ws);
     if (st) return st;
-    return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, kNoallocScratchBytes,
-                      stream);
+    return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws,
+                      kNoallocScratchBytes + kNoallocHead, stream);
 }
 
 // The status word of the last fhtdp_detect_polyline_noalloc run sits in the

@@ -123,3 +123,42 @@ def test_missing_producer_of_a_middle_band_times_out(lib):
     assert e.value.code == 4
     _same(lib.detect_polyline(img, 4, 8, ws=ws), _detect(img.cpu().numpy(), 4, 8))
     lib.workspace_status(ws)
+
+
+@pytest.mark.parametrize("w", [197, 244, 255])
+def test_noalloc_takes_256_row_bands_up_to_its_scratch(lib, w):
+    """int32 rows of eight bands of 256 rows: 14.8, 16.4 and 16.7 of 16.8 MB, the
+    last two only with rows that are not padded to whole lines."""
+    import ctypes
+
+    import torch
+    img = _img(2048, w, "i32", w)
+    src = to_device(img)
+    x = torch.empty(9, dtype=torch.int32, device="cuda")
+    d = torch.empty(8, dtype=torch.int32, device="cuda")
+    s = torch.empty(1, dtype=torch.int32, device="cuda")
+    p = [ctypes.c_void_p(t.data_ptr()) for t in (src, x, d, s)]
+    rc = lib.lib().fhtdp_detect_polyline_noalloc(
+        p[0], 1, 2048, w, w, 8, 20, p[1], p[2], p[3],
+        ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0, lib.lib().fhtdp_last_error().decode()
+    _same((x, d, s), oracle.detect(img, 8, 20))
+
+
+def test_batch_status_reports_a_wait_of_a_256_row_image_that_gave_up(lib):
+    """Those images run by themselves beside the batch's launch: the plan's
+    status covers them."""
+    import torch
+    img = _img(1024, 300, "i32", 5)
+    plan = lib.BatchPlan([to_device(img)] * 2, [4, 4], [9, 9])
+    lib.lib().fhtdp_debug_inject(3, 1, 2_000_000)   # waits of about 1 ms
+    plan.run()
+    torch.cuda.synchronize()
+    with pytest.raises(lib.FhtdpError) as e:
+        plan.status()
+    assert e.value.code == 4
+    plan.run()
+    torch.cuda.synchronize()
+    assert plan.status() == 0
+    for i in range(2):
+        _same((plan.x[i], plan.d[i], plan.score[i]), oracle.detect(img, 4, 9))
