@@ -8,7 +8,10 @@
 // first over the whole chip, and the DP items that remain are small: a tile of
 // 2048 / n columns (16 for bands of 128 rows), so that a level spreads over the
 // chip and the chain advances at the latency of one exchange through L2.
-// CHAIN_FIGURES
+// Bound by that latency, about 5 us a level (poll, V_{b+1} from L2, windows in
+// shared memory, store, release).  One call on 2048 x 2048 uint8, n = 128, B =
+// 16: engine 249 us, chain 110 (FHT 34); 8192 x 8192 float, 64 bands: 1842 ->
+// 969; two polylines 281 -> 128; 24 ragged int32 images in a batch 1406 -> 629.
 #include <algorithm>
 #include <climits>
 #include <new>
@@ -55,7 +58,8 @@ __device__ __forceinline__ void st_if(Acc *p, bool ok, Acc v) {
 // float images run the signs one after the other, the "-" sign on the mirrored
 // strip; uint8 images both at once (fht_smem.cuh).  Bound by shared memory
 // (about 28 bytes a word and sign) and the stores of the rows.
-// FHT_FIGURES
+// 2048 x 2048 uint8, n = 128: four passes over the whole arrays 102 us, this 34
+// (three register levels and 768 threads: 43).
 constexpr int kFhtNT = 1024;
 
 template <typename In, typename Acc>
@@ -953,6 +957,24 @@ size_t item_smem(const ChainArgs &a, const ChainImg &im) {
     return (size_t)rows * row_words(im.cols) * 4 * 2;
 }
 
+// Blocks for one image whose band levels have t tiles.  A level can only use t,
+// and blocks that wait for the next one slow those that share their SM: t of
+// them, while there is an SM for each two (up to 2 t: the second takes the next
+// level's item and loads its Hough values early), and beyond one an SM a
+// multiple of half the SMs, so that the SMs are loaded evenly.  The whole chip (304)
+// against this rule, whole calls: 2048 x 2048 uint8, n = 128 (t = 128) 130 ->
+// 110 us and, from eight streams at once, 155 -> 91 us an image with the bend
+// angle; float, n = 128, t = 188: 172 -> 160, t = 282: 392 -> 351 (282 x 32 bands);
+// uint8, n = 64, t = 63: 193 -> 168 (t blocks: 173); n = 16, t = 4: 278 -> 270
+// (t blocks: 339).
+int one_image_blocks(int t) {
+    const int sms = device_sms();
+    if (2 * t <= sms) return 2 * t;
+    if (t <= sms) return t;
+    const int half = sms > 1 ? sms / 2 : 1;
+    return t / half * half;
+}
+
 template <typename Acc, int kC>
 int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cudaStream_t stream) {
     auto kern = dp_chain_kernel<Acc, kC>;
@@ -964,7 +986,8 @@ int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cu
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kDpNT, smem);
         const int most = device_sms() * (per_sm < 1 ? 1 : per_sm);
-        blocks = blocks < most ? blocks : most;
+        if (a.one.tiles) blocks = std::min(blocks, one_image_blocks(a.one.tiles));
+        blocks = std::min(blocks, most);
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
