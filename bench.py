@@ -97,11 +97,8 @@ EXTRAS = ("plain2048", "float8192")
 NCU_TRAFFIC_BYTES_PER_PIXEL = {
     "mixed": 15.0048e9 / 1064894464,     # engine_kernel_u8<int, 1>: 4.445 + 10.559 GB
     "plain2048": 1.2455e9 / 134217728,   # engine_kernel_u8<int, 0>: 0.216 + 1.030 GB
-    "float8192": 1.2905e9 / 67108864,    # engine_kernel_wide: 0.275 + 1.015 GB
+    "float8192": None,
 }
-# DRAM bytes of one dp_band_window_kernel band launch on the 2048x2048, k = 16
-# workloads (profiles/dp_band_window_kernel_angle2048.md).
-NCU_TRAFFIC_DP_WINDOW_LAUNCH = 4.14e6
 
 
 # The main problem's smoothing half-width and bend angle (the paper's
@@ -659,7 +656,7 @@ def roofline(bb, per_step_s):
     hbm, peak_kind = peaks()
     achieved = bb.alg / per_step_s / 1e9
     tpp = NCU_TRAFFIC_BYTES_PER_PIXEL.get(bb.name)
-    kern = ("engine_kernel (float images, one persistent launch per step)"
+    kern = ("fht_band_kernel<float> + dp_chain_kernel<float> (one launch of each per step)"
             if bb.tdt == bb.torch.float32 else
             "engine_kernel_u8 (one persistent launch per step%s)"
             % (", after one transpose_kernel per image" if bb.horizontal else ""))
@@ -756,11 +753,11 @@ ANGLE_LANES = 8   # streams over which one step spreads its images (4: -4 %, 2: 
 
 
 def run_standalone(args):
-    """The calls that run on the standalone kernels, on a batch of images per
-    step: the main problem (angle2048: smoothing + band FHT + bend-angle DP +
-    read-back, one fhtdp_detect_polyline_angle call of 24 launches per image)
-    or the through-point query (through2048: band FHT + DP with the point's
-    band masked + read-back, one fhtdp_detect_through_point call per image).
+    """The calls on one image, on a batch of images per step: the main problem
+    (angle2048: smoothing + band FHT + bend-angle DP with read-back, one
+    fhtdp_detect_polyline_angle call of 3 launches per image) or the
+    through-point query (through2048: band FHT + DP with the point's band
+    masked and read-back, one fhtdp_detect_through_point call per image).
     A step spreads the images over ANGLE_LANES streams, each with its own
     workspace, and is captured once as a CUDA graph that every timed step
     replays."""
@@ -951,8 +948,9 @@ def run_standalone(args):
         "engine": algorithmic_bytes(w, h, k, 1),
     }
     # The roofline kernel is the DP (the largest share of the launch list);
-    # "backtrack" here is the standalone one-block read-back, not the argmax
-    # + one-warp read-back that the detection calls run.
+    # "dp" and "backtrack" here are the public calls that leave the DP's state
+    # in the caller's array and read it back (a launch per band, one cluster),
+    # not the queue with its own read-back that the detection calls run.
     top = "dp_angle" if angle else ("engine" if name == "horizontal2048" else "dp")
     hbm, peak_kind = peaks()
     achieved = stage_bytes[top] / (stage_ms[top] / 1e3) / 1e9
@@ -976,13 +974,12 @@ def run_standalone(args):
                              % (host.numel() // 2**20, ">" if host.numel() > 129e6 else "<")},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm,
-                         "traffic": NCU_TRAFFIC_DP_WINDOW_LAUNCH * (k - 1)
-                                    if NCU_TRAFFIC_DP_WINDOW_LAUNCH and top != "engine" else None,
+                         "traffic": None,
                          "peak_kind": peak_kind,
-                         "kernel": ("engine_kernel_u8 (one image per launch, the transposed "
-                                    "image)" if top == "engine" else
-                                    "dp_band_window_kernel (the k-1 band launches of one image "
-                                    "and the last-band kernel, timed together)")},
+                         "kernel": ("fht_band_kernel + dp_chain_kernel (one call on the "
+                                    "transposed image)" if top == "engine" else
+                                    "dp_chain_kernel (the band launches of one image, timed "
+                                    "together)")},
             "stages_ms_one_image": stage_ms,
             "pipeline_frac_of_hbm": sum(algorithmic_bytes(h, w, k, 1) for _ in range(I))
                                     / (total_s / args.steps) / 1e9 / hbm,
@@ -1126,8 +1123,8 @@ def run_angle_batch(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": None, "peak_kind": peak_kind,
                          "algorithmic_bytes_per_launch": eng_bytes,
-                         "kernel": "engine_kernel_wide<int, int> (window-table DP items, one "
-                                   "launch per step; %.3f ms)" % eng_ms},
+                         "kernel": "fht_band_kernel<int> + dp_chain_kernel<int> (window-table "
+                                   "DP items, one launch of each per step; %.3f ms)" % eng_ms},
             "e2e": {"value": e2e_value, "unit": "Mpix/s", "h2d_bytes_per_step": host.numel(),
                     "d2h_bytes_per_step": (hx.numel() + hd.numel() + hs.numel()) * 4},
             "gpu_launches": int(launches_per_step * args.steps),

@@ -262,8 +262,8 @@ int fhtdp_detect_through_point(const void *img, int dtype, int h, int w, int pit
  * [0, w + h/k - 1]; Sec. 2.1 extends every band by n zero columns on the
  * right).  As fhtdp_detect_polyline, but every vertex may lie anywhere in
  * [0, W), W = w + n: the pixels a link covers right of the image count as
- * zero, so a curve that runs off the right edge can be followed.  Runs the
- * standalone kernels.  dtype any of the three; ws of at least
+ * zero, so a curve that runs off the right edge can be followed.  One launch
+ * of the FHT and one of the DP.  dtype any of the three; ws of at least
  * fhtdp_through_workspace_bytes() bytes.  Outputs as for fhtdp_backtrack.
  * ---------------------------------------------------------------------- */
 int fhtdp_detect_polyline_padded(const void *img, int dtype, int h, int w, int pitch, int k,
@@ -324,9 +324,10 @@ int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, i
 int fhtdp_cnn_downsample4(const uint8_t *img, int n, int h, int w, void *out, cudaStream_t stream);
 /* y = act(conv3x3_dil(x, wt) + bias), act = ReLU when relu != 0; cin 1 or 32,
  * cout 32, zero padding ("same").  32 input channels run on tcgen05.mma
- * (persistent CTAs over tiles of 128 pixels x 32 channels, K = 9 x 32, FP32
- * accumulators in tensor memory); a bounded wait for the MMAs that gives up
- * records FHTDP_ETIMEOUT for fhtdp_cnn_status. */
+ * (persistent CTAs down columns of 256 pixels, an input row meeting the nine
+ * taps of the three output rows that it feeds, FP32 accumulators in tensor
+ * memory); a bounded wait that gives up records FHTDP_ETIMEOUT for
+ * fhtdp_cnn_status. */
 int fhtdp_cnn_conv3x3(const void *x, int cin, int n, int h, int w, int dil, const void *wt,
                       const float *bias, int relu, void *y, cudaStream_t stream);
 /* Device status of the tensor-core convolutions since the last clear: 0, or
@@ -336,7 +337,8 @@ int fhtdp_cnn_conv3x3(const void *x, int cin, int n, int h, int w, int dil, cons
  * the status cannot be read. */
 int fhtdp_cnn_status(int clear);
 /* dx = gradient of a 32-channel layer's input from the gradient dz of its
- * pre-activation output; wflip is caller scratch of 9*32*32 bf16. */
+ * pre-activation output; wflip (9*32*32 bf16) must not be NULL but is not
+ * written: the kernel mirrors the taps as it loads them. */
 int fhtdp_cnn_conv3x3_dgrad(const void *dz, int n, int h, int w, int dil, const void *wt,
                             void *wflip, void *dx, cudaStream_t stream);
 /* dy *= (y > 0): the ReLU of a layer, in place, from its output y. */
@@ -382,12 +384,12 @@ int fhtdp_workspace_status(const void *ws, cudaStream_t stream);
 void fhtdp_debug_inject(int band, int tile, long long wait_cycles);
 
 /* ------------------------------------------------------------------------
- * Batches: many images of different h, w, k and B (one pixel type) in ONE
- * persistent kernel launch.  Work items (image, band, column tile) are taken
- * from a device-side queue, so the band chains of different images overlap
- * and the GPU stays busy; a run is one memset and one kernel launch and may
- * be captured in a CUDA graph.  Each image's result is the same as
- * fhtdp_detect_polyline's.
+ * Batches: many images of different h, w, k and B (one pixel type) in one
+ * persistent kernel launch (uint8) or two (int32 and float: the bands' FHTs,
+ * then the DP).  Work items (image, band, column tile) are taken from a
+ * device-side queue, so the band chains of different images overlap and the
+ * GPU stays busy; a run is a memset and these launches and may be captured in
+ * a CUDA graph.  Each image's result is the same as fhtdp_detect_polyline's.
  * ---------------------------------------------------------------------- */
 typedef struct fhtdp_image {
     const void *img;     /* device pixels [h][pitch] of the batch's dtype */
@@ -417,7 +419,8 @@ size_t fhtdp_batch_workspace_bytes(const fhtdp_batch_plan *plan);
  * image table into `ws` (from memory held by the plan; keep the plan alive
  * until the copy has run).  Call once per workspace, before the runs. */
 int fhtdp_batch_upload(fhtdp_batch_plan *plan, void *ws, size_t ws_bytes, cudaStream_t stream);
-/* Runs the whole batch on `stream`: one memset and one kernel launch. */
+/* Runs the whole batch on `stream`: a memset and one kernel launch (int32 and
+ * float images: two). */
 int fhtdp_batch_run(const fhtdp_batch_plan *plan, void *ws, cudaStream_t stream);
 /* Number of work items (image, band, column tile) of a run. */
 long long fhtdp_batch_items(const fhtdp_batch_plan *plan);
@@ -438,8 +441,9 @@ long long fhtdp_batch_items(const fhtdp_batch_plan *plan);
  *   3. the schedule again.
  * It uploads the chosen layout and queue, and writes the width to
  * *target_out (may be NULL); fhtdp_batch_choice reports the rest.  The
- * outputs are those of an ordinary run.  It synchronises `stream` (not for use
- * under stream capture).  The paper has no counterpart: this tunes the GPU
+ * outputs are those of an ordinary run.  Batches of int32 and float images
+ * have one schedule and nothing to tune: the call runs them and leaves the
+ * plan as it is.  It synchronises `stream` (not for use under stream capture).  The paper has no counterpart: this tunes the GPU
  * schedule of its method, not the method. */
 int fhtdp_batch_autotune(fhtdp_batch_plan *plan, void *ws, int reps, cudaStream_t stream,
                          long long *target_out);
@@ -465,8 +469,7 @@ int fhtdp_batch_configure(fhtdp_batch_plan *plan, void *ws, int n, int tile, int
  * fhtdp_backtrack_angle give.  The images are the rows already smoothed
  * (fhtdp_gauss_rows, step 1): int32 or float32, all of one band height n in
  * 2..128.  Host only (no device work); FHTDP_EINVAL otherwise.  All the
- * images' band chains then run in one persistent launch: the window maxima
- * come from maxima of a fixed half-width that cover every window. */
+ * images' band chains then run in one persistent launch after the FHTs'. */
 int fhtdp_batch_angle(fhtdp_batch_plan *plan, double gamma);
 /* Sec. 2.2-2.3, Subproblems 2-3: the plan's runs find, for image i, the best
  * polyline through the point (points[2i + 1], points[2i] n) on band border

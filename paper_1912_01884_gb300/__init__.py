@@ -301,13 +301,14 @@ def workspace_status(ws, stream=None) -> int:
 
 
 class BatchPlan:
-    """Many images of one pixel type in one persistent launch.
+    """Many images of one pixel type in one persistent launch (int32 and float: two).
 
     ``images`` are 2-D CUDA tensors, ``ks`` and ``Bs`` their band counts and
     bend limits.  Outputs ``x[i]``, ``d[i]``, ``score[i]`` are allocated here,
     or are the rows of ``out = (X, D, S)``; ``windows[i]`` (optional) is a
     device int32 [k][2] tensor of allowed displacements per band (pruned DP).
-    ``run()`` enqueues the whole batch (one memset, one kernel) and may be
+    ``run()`` enqueues the whole batch (a memset and one kernel, two for int32
+    and float images) and may be
     captured in a CUDA graph."""
 
     def __init__(self, images, ks, Bs, ws=None, stream=None, out=None, windows=None):

@@ -662,8 +662,13 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 const int a = (args.use_table ? args.tab.lo[c - lo] : max(c - B, lo)) - lo;
                 const int z = (args.use_table ? args.tab.hi[c - lo] : min(c + B, hi)) - lo;
                 Acc m = vmax(Su[a * R], Pu[z * R]);
+                const int e = (z >> 3) - 1;   // the last run inside
 #pragma unroll 1
-                for (int j = (a >> 3) + 1; j < z >> 3; ++j) m = vmax(m, run_of(j));
+                for (int j = (a >> 3) + 1; j <= e; j += 4) {   // four loads in flight
+                    const Acc x0 = run_of(j), x1 = run_of(min(j + 1, e));
+                    const Acc x2 = run_of(min(j + 2, e)), x3 = run_of(min(j + 3, e));
+                    m = vmax(vmax(m, vmax(x0, x1)), vmax(x2, x3));
+                }
                 M[i] = m;
             }
         } else if (args.use_table) {
@@ -672,8 +677,14 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 const int c = min(c0 + i, hi);
                 const int a = args.tab.lo[c - lo] - lo, z = args.tab.hi[c - lo] - lo;
                 Acc m = dead;
+                // four loads in flight (the last ones twice): 1120 x 603 float, n = 32,
+                // bends of 0.1 rad, whole call 232 -> 197 us
 #pragma unroll 1
-                for (int r = a; r <= z; ++r) m = vmax(m, Su[r * R]);
+                for (int r = a; r <= z; r += 4) {
+                    const Acc x0 = Su[r * R], x1 = Su[min(r + 1, z) * R];
+                    const Acc x2 = Su[min(r + 2, z) * R], x3 = Su[min(r + 3, z) * R];
+                    m = vmax(vmax(m, vmax(x0, x1)), vmax(x2, x3));
+                }
                 M[i] = m;
             }
         } else {
@@ -1021,7 +1032,7 @@ size_t fht_smem_bytes(int m, int T) { return (size_t)m * fht_pitch(m, T) * 4; }
 // Columns of an FHT block: a block's time grows as T + 0.8 m (the passes sweep
 // T + m - 4, T + m - 16, ... columns), and the last round of blocks may be nearly
 // empty, so the T (a multiple of 16, at most 256) of the least rounds x (T +
-// 0.8 m).  FHT_T_FIGURES
+// 0.8 m).
 int fht_columns(int m, int wout, int subs) {
     const int sms = device_sms();
     int best = 16;

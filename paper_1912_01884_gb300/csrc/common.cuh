@@ -29,7 +29,7 @@ struct Dead<float> {
 struct Shape {
     int h, w, k, n, W, D;  // D = 2n - 1 displacement values
     int log2n;
-    // Vertex domain [0, vw) of the standalone DP and read-back: w, or W when
+    // Vertex domain [0, vw) of the band chain and the read-back: w, or W when
     // vertices may lie in the zero padding right of the image (Sec. 2.2).
     int vw;
 };

