@@ -2657,8 +2657,8 @@ void set_point(ImgPlan &p, int j, int xp) {
 }
 
 // One image takes the chain (chain.cu): the engine's 128-column tiles leave
-// most of the chip idle on one image (2048 x 2048 uint8: 249 us, 115 on the
-// chain; 256 x 256: 67 and 34).  The engine needs a sixth of the workspace, and
+// most of the chip idle on one image (2048 x 2048 uint8: 249 us, 110 on the
+// chain; 256 x 256: 67 and 33).  The engine needs a sixth of the workspace, and
 // takes uint8 images whose workspace is too small for the chain (the built-in
 // scratch of the no-allocation call).
 int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
