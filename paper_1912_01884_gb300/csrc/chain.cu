@@ -80,14 +80,17 @@ struct BandFht {
     // Pixels c .. c + 3, c a multiple of 4; kInside: all in the image and
     // aligned.  Elsewhere a predicated load (one launch of one image waits for
     // its edge blocks), or four in unaligned rows and where the four straddle
-    // the image's edge; columns past W (of the padding's outputs) wrap around.
+    // the image's edge; columns past W wrap around (bands of 1 or 2 rows: also
+    // in the four that straddle the edge).
     __device__ bool inside4(int c) const { return aligned && c >= 0 && c + 4 <= im.w; }
     template <bool kInside>
     __device__ uint32_t quad8(const In *row, int c) const {
         if (kInside) return __ldg((const uint32_t *)(row + c));
         const bool ok = inside4(c);
         uint32_t v = ld_nc_if(row + c, ok);
-        if (!ok && c >= 0 && c < im.w) {
+        if (c + 3 >= im.W) {
+            for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
+        } else if (!ok && c >= 0 && c < im.w) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 uint32_t b = 0;
@@ -97,8 +100,6 @@ struct BandFht {
                     : "l"(row + c + j), "r"((uint32_t)(c + j < im.w)));
                 v |= b << (8 * j);
             }
-        } else if (c + 3 >= im.W) {
-            for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)px(row, c + j) << (8 * j);
         }
         return v;
     }
@@ -116,13 +117,13 @@ struct BandFht {
             : "+r"(q.x), "+r"(q.y), "+r"(q.z), "+r"(q.w)
             : "l"(row + c), "r"((uint32_t)ok));
         unpack4(q, v);
-        if (!ok && c >= 0 && c < im.w) {
+        if (c + 3 >= im.W) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = px(row, c + j);
+        } else if (!ok && c >= 0 && c < im.w) {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 v[j] = word_from<Acc>(ld_nc_if(row + c + j, c + j < im.w));
-        } else if (c + 3 >= im.W) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] = px(row, c + j);
         }
     }
     // Words u .. u + N - 1 (u a multiple of 4) of sub-band row y; kSign 1: of

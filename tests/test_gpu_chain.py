@@ -71,6 +71,21 @@ def test_fht_block_widths_match_oracle(lib, n, w):
             assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, 2))
 
 
+# Bands so short that the four pixels at the image's right edge reach past the
+# cyclic width (n = 2, w = 1 mod 4: column w - 1 + 3 is column 0 again).
+@pytest.mark.parametrize("n", [1, 2])
+@pytest.mark.parametrize("w", [1, 2, 3, 4, 5, 8, 33, 34, 255, 257])
+def test_fht_of_short_bands_wraps_at_the_padded_width(lib, n, w):
+    for dtype in ("u8", "i32", "f32"):
+        img = _img(6 * n, w, dtype, 7 * n + w)
+        H = lib.fht_bands(to_device(img), 6).cpu().numpy()
+        if dtype == "f32":
+            want = hough_from_oracle(img, 6, float32=True)
+            assert np.array_equal(H.view(np.uint32), want.view(np.uint32))
+        else:
+            assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, 6))
+
+
 @pytest.mark.parametrize("dtype", ["i32", "f32"])
 def test_batch_of_every_band_height(lib, dtype):
     shapes = [(256, 333, 128, 16), (512, 70, 128, 40), (256, 500, 64, 3), (320, 201, 32, 5),
