@@ -318,7 +318,9 @@ int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, i
  * (the single-channel first layer: [16][32], taps 9..15 zero), FP32
  * accumulation on the tensor cores, FP32 master weights.  All pointers are
  * device memory owned by the caller; w must be a multiple of 64 and the
- * dilation at most 8.
+ * dilation at most 8.  The 32-channel convolutions take x, y, dz and dx from a
+ * 16-byte boundary (FHTDP_EINVAL otherwise); weights and every other array
+ * only need the alignment of their values.
  * ---------------------------------------------------------------------- */
 /* uint8 [n][h][w] -> bf16 [n][h/4][w/4], the 4x4 mean divided by 255. */
 int fhtdp_cnn_downsample4(const uint8_t *img, int n, int h, int w, void *out, cudaStream_t stream);

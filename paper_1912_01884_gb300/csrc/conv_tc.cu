@@ -272,13 +272,25 @@ __global__ void __launch_bounds__(kFwThreads, 2) conv3x3_rows_kernel(
     // 2 - ky; flipped and transposed (W'[t][ci][co] = W[8-t][co][ci]) for the
     // data gradient.
     {
-        // 8-byte loads, all of a thread's in flight together
+        // 8-byte loads, all of a thread's in flight together; weights that do not
+        // begin on 8 bytes (any 2-byte address is taken) one value at a time
         constexpr int kLoads = 9 * kTcC * kTcC / 4, kPer = (kLoads + kFwThreads - 1) / kFwThreads;
         uint2 wv[kPer];
+        if ((uintptr_t)Wt % 8 == 0) {
 #pragma unroll
-        for (int m = 0; m < kPer; ++m)
-            if (tid + m * kFwThreads < kLoads)
-                wv[m] = __ldg((const uint2 *)Wt + tid + m * kFwThreads);
+            for (int m = 0; m < kPer; ++m)
+                if (tid + m * kFwThreads < kLoads)
+                    wv[m] = __ldg((const uint2 *)Wt + tid + m * kFwThreads);
+        } else {
+#pragma unroll
+            for (int m = 0; m < kPer; ++m)
+                if (tid + m * kFwThreads < kLoads) {
+                    const unsigned short *q =
+                        (const unsigned short *)Wt + 4 * (tid + m * kFwThreads);
+                    wv[m] = make_uint2(__ldg(q) | (uint32_t)__ldg(q + 1) << 16,
+                                       __ldg(q + 2) | (uint32_t)__ldg(q + 3) << 16);
+                }
+        }
 #pragma unroll
         for (int m = 0; m < kPer; ++m) {
             if (tid + m * kFwThreads >= kLoads) break;
@@ -710,6 +722,8 @@ int cnn_wgrad_tc(const void *X, int N, int H, int W, int dil, const void *dZ, fl
                  float *db, cudaStream_t stream, float *part) {
     if (dil < 1 || dil > kTcHalo || W < 1 || H < 1 || N < 1)
         return set_error(FHTDP_EINVAL, "conv3x3 wgrad: dilation 1..8 and a non-empty image");
+    if (((uintptr_t)X | (uintptr_t)dZ) % 16)
+        return set_error(FHTDP_EINVAL, "conv3x3 wgrad: x and dz must be 16-byte aligned");
     // set on every call: the attribute belongs to the current device
     int st = cuda_status(cudaFuncSetAttribute(conv3x3_wgrad_rows_kernel,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -718,7 +732,7 @@ int cnn_wgrad_tc(const void *X, int N, int H, int W, int dil, const void *dZ, fl
     if (st) return st;
     CUtensorMap xmap, zmap;
     if (!encode_px_map(&xmap, X, N, H, W, kTcPix) || !encode_px_map(&zmap, dZ, N, H, W, kTcM))
-        return set_error(FHTDP_EINVAL, "conv3x3 wgrad: x and dz must be 16-byte aligned");
+        return set_error(FHTDP_ECUDA, "conv3x3 wgrad: no tensor map of x or dz");
     const long long rows = (long long)N * H * ((W + kTcM - 1) / kTcM);
     unsigned grid = row_grid(rows);
     if (part) grid = std::min<unsigned>(grid, kWgradParts);
@@ -736,6 +750,9 @@ int cnn_conv3x3_tc(const void *X, int N, int H, int W, int dil, const void *Wt,
                    const void *mask) {
     if (dil < 1 || dil > kTcHalo || W < 1 || H < 1 || N < 1)
         return set_error(FHTDP_EINVAL, "conv3x3: dilation 1..8 and a non-empty image");
+    // (x: the tensor map; y and the mask: 16-byte accesses)
+    if (((uintptr_t)X | (uintptr_t)Y | (uintptr_t)mask) % 16)
+        return set_error(FHTDP_EINVAL, "conv3x3: x and y must be 16-byte aligned");
     auto kern = mask ? conv3x3_rows_kernel<false, true>
                 : relu ? conv3x3_rows_kernel<true, false>
                        : conv3x3_rows_kernel<false, false>;
@@ -746,7 +763,7 @@ int cnn_conv3x3_tc(const void *X, int N, int H, int W, int dil, const void *Wt,
     if (st) return st;
     CUtensorMap xmap;
     if (!encode_px_map(&xmap, X, N, H, W, kTcPix))
-        return set_error(FHTDP_EINVAL, "conv3x3: x must be 16-byte aligned");
+        return set_error(FHTDP_ECUDA, "conv3x3: no tensor map of x");
     const long long rows = (long long)N * H * ((W + kTcM - 1) / kTcM);
     kern<<<row_grid(rows), kFwThreads, kFwSmem, stream>>>(
         xmap, N, H, W, dil, (const __nv_bfloat16 *)Wt, flip ? 1 : 0, bias,

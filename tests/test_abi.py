@@ -244,3 +244,24 @@ def test_cnn_and_learned_entries_reject_bad_arguments_before_launch(lib):
     out = ctypes.c_void_p()
     assert L.fhtdp_learned_plan_create(None, 0, 6, ctypes.byref(out)) == 1
     assert not out.value
+
+
+def test_cnn_32_channel_layers_reject_unaligned_activations_before_launch(lib):
+    """x, y, dz and dx of the 32-channel layers are read and written 16 bytes at
+    a time; nothing is launched (fake pointers, never dereferenced)."""
+    L = lib.lib()
+    at = ctypes.c_void_p
+    f = at(1 << 12)
+    for off in (2, 4, 8):
+        g = at((1 << 12) + off)
+        calls = [
+            lambda: L.fhtdp_cnn_conv3x3(g, 32, 1, 6, 192, 2, f, None, 1, f, None),
+            lambda: L.fhtdp_cnn_conv3x3(f, 32, 1, 6, 192, 2, f, None, 1, g, None),
+            lambda: L.fhtdp_cnn_conv3x3_dgrad(g, 1, 6, 192, 2, f, f, f, None),
+            lambda: L.fhtdp_cnn_conv3x3_dgrad(f, 1, 6, 192, 2, f, f, g, None),
+            lambda: L.fhtdp_cnn_conv3x3_wgrad(g, 32, 1, 6, 192, 2, f, f, None, None),
+            lambda: L.fhtdp_cnn_conv3x3_wgrad(f, 32, 1, 6, 192, 2, g, f, None, None),
+        ]
+        for i, call in enumerate(calls):
+            assert call() == 1, (off, i)
+            assert "16-byte" in L.fhtdp_last_error().decode()

@@ -98,3 +98,32 @@ def test_first_layer_and_head_on_any_alignment(lib, N, H, W, dil, shift):
     assert np.array_equal(pred.cpu().numpy(), np.asarray(rpred).reshape(-1))
     assert abs(float(loss) - rl) <= 1e-4 * abs(rl)
     assert np.all(np.abs(_np(dl) - rdz) <= 2.0 ** -7 * np.abs(rdz) + 1e-6)
+
+
+# Weights at any 2-byte address (a view into a flat parameter buffer), `shift`
+# bf16 values past a 16-byte boundary: the same sums, so the same bits.
+@pytest.mark.parametrize("shift", [1, 2, 3, 4, 6, 7])
+def test_row_chains_take_weights_at_any_address(lib, shift):
+    import torch
+    L = lib.lib()
+    N, H, W, dil = 1, 9, 128, 2
+    rng = np.random.default_rng(shift)
+    x, w = _bf16(rng.standard_normal((N, H, W, 32))).cuda(), _bf16(rng.standard_normal(9216) * 0.1)
+    b = torch.from_numpy(rng.standard_normal(32).astype(np.float32)).cuda()
+    flat = torch.zeros(9216 + 8, dtype=torch.bfloat16, device="cuda")
+    wf = torch.empty(9216, dtype=torch.bfloat16, device="cuda")
+    got = []
+    for at in (0, shift):
+        wd = flat[at:at + 9216]
+        wd.copy_(w)
+        y, dx = torch.empty_like(x), torch.empty_like(x)
+        assert L.fhtdp_cnn_conv3x3(x.data_ptr(), 32, N, H, W, dil, wd.data_ptr(), b.data_ptr(), 1,
+                                   y.data_ptr(), _stream()) == 0
+        assert L.fhtdp_cnn_conv3x3_dgrad(x.data_ptr(), N, H, W, dil, wd.data_ptr(), wf.data_ptr(),
+                                         dx.data_ptr(), _stream()) == 0
+        got.append((y.view(torch.int16).cpu(), dx.view(torch.int16).cpu()))
+    w64 = _np(w).reshape(9, 32, 32)
+    _close(_np(got[0][0].view(torch.bfloat16)),
+           np.maximum(cnn_ref.conv3x3(_np(x), w64, _np(b), dil), 0))
+    for p, q in zip(*got):
+        assert torch.equal(p, q)
