@@ -13,6 +13,7 @@
 // 16: engine 249 us, chain 110 (FHT 34); 8192 x 8192 float, 64 bands: 1842 ->
 // 969; two polylines 281 -> 128; 24 ragged int32 images in a batch 1406 -> 629.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <new>
 #include <type_traits>
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
 // its tiles reads the polyline back (Eq. 5).
 // Bound by latency: one flag and one load round trip through L2 per band level.
 constexpr int kDpNT = 512;
+constexpr int kDpPerSm = 2;     // blocks an SM: all its registers at 64 a thread
 constexpr int kRun = 8;         // displacements of a thread's run
 constexpr int kPadB = 32;       // bend limits up to this read past the range unchecked
 constexpr int kMinLen = kRun + 1;   // windows from this length on span two runs
@@ -482,16 +484,16 @@ __host__ __device__ constexpr int row_words(int cols) { return cols == 16 ? 18 :
 // dead rows around the range (bend limits up to kPadB), or from S and P with the
 // windows clipped to the range (tables, longer limits).
 enum { kScan, kPadded, kClipped };
-__host__ __device__ inline int window_mode(int use_table, int minlen, int B) {
+__host__ __device__ constexpr int window_mode(int use_table, int minlen, int B) {
     if (use_table) return minlen >= kMinLen ? kClipped : kScan;
     return 2 * B + 1 < kMinLen ? kScan : B <= kPadB ? kPadded : kClipped;
 }
 // Dead rows above and below the range, whole runs.
-__host__ __device__ inline int window_pad(int mode, int use_table, int B) {
+__host__ __device__ constexpr int window_pad(int mode, int use_table, int B) {
     if (mode == kScan && !use_table) return kRun;
     return mode == kPadded ? (B + kRun - 1) / kRun * kRun : 0;
 }
-__host__ __device__ inline int range_rows(int n) {
+__host__ __device__ constexpr int range_rows(int n) {
     return (2 * n - 1 + kRun - 1) / kRun * kRun;
 }
 
@@ -778,7 +780,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
 
 // kC: the tile width when all images share it, or 0.
 template <typename Acc, int kC>
-__global__ void __launch_bounds__(kDpNT, 2) dp_chain_kernel(const __grid_constant__ ChainArgs args) {
+__global__ void __launch_bounds__(kDpNT, kDpPerSm) dp_chain_kernel(const __grid_constant__ ChainArgs args) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
     auto item = [&](const ChainImg &im, int band, int tile) {
@@ -926,15 +928,21 @@ __global__ void __cluster_dims__(kBtBlocks, 1, 1) __launch_bounds__(kBtNT)
 // ---------------------------------------------------------------------------
 // Host side.
 int device_sms() {
-    int dev = 0, v = 0;
+    static std::atomic<int> cached[64];
+    int dev = 0;
     cudaGetDevice(&dev);
+    const bool known = dev >= 0 && dev < 64;
+    int v = known ? cached[dev].load(std::memory_order_relaxed) : 0;
+    if (v > 0) return v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 152;
+    if (v < 1) v = 152;
+    if (known) cached[dev].store(v, std::memory_order_relaxed);
+    return v;
 }
 
 // Columns of a DP item: 2048 / n, so that 512 threads cover its displacements
 // in runs of 8.
-int chain_cols(int n) { return n >= 128 ? 16 : n <= 8 ? 256 : 2048 / n; }
+constexpr int chain_cols(int n) { return n >= 128 ? 16 : n <= 8 ? 256 : 2048 / n; }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -962,11 +970,37 @@ void chain_table(ChainArgs &a, const WindowTable &t) {
     }
 }
 
-// Shared memory of one image's items.
+// Shared memory of an item of bands of n rows.
+constexpr size_t item_bytes(int n, int cols, int use_table, int minlen, int B) {
+    const int pad = window_pad(window_mode(use_table, minlen, B), use_table, B);
+    return (size_t)(range_rows(n) + 2 * pad) * row_words(cols) * 4 * 2;
+}
 size_t item_smem(const ChainArgs &a, const ChainImg &im) {
-    const int mode = window_mode(a.use_table, a.minlen, im.B);
-    const int rows = range_rows(im.n) + 2 * window_pad(mode, a.use_table, im.B);
-    return (size_t)rows * row_words(im.cols) * 4 * 2;
+    return item_bytes(im.n, im.cols, a.use_table, a.minlen, im.B);
+}
+
+// The dynamic shared memory that every launch allows its kernel: the largest
+// that any image asks for.  The limit belongs to the kernel, not to a launch:
+// were it set to a launch's own size, a host thread with a smaller image could
+// lower it between another thread's call and launch, which is then refused.
+// (What a block occupies is the launch's own size.)
+constexpr int kFhtSmemMax = 226 * 1024, kDpSmemMax = 96 * 1024;
+constexpr size_t most_item_bytes() {
+    size_t most = 0;
+    for (int n = 1; n <= 256; n *= 2)
+        for (int B = 0; B <= 2 * n - 2; ++B)
+            for (int table = 0; table < 2; ++table) {
+                const size_t v = item_bytes(n, chain_cols(n), table, B + 1, B);
+                most = v > most ? v : most;
+            }
+    return most;
+}
+static_assert(most_item_bytes() <= kDpSmemMax, "every item fits the limit");
+template <typename Kernel>
+int allow_smem(Kernel kern, int bytes) {
+    return cuda_status(
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+        "cudaFuncSetAttribute");
 }
 
 // Blocks for one image whose band levels have t tiles.  A level can only use t,
@@ -990,16 +1024,11 @@ int one_image_blocks(int t) {
 template <typename Acc, int kC>
 int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cudaStream_t stream) {
     auto kern = dp_chain_kernel<Acc, kC>;
-    int st = cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem),
-                         "cudaFuncSetAttribute");
+    int st = dependent ? FHTDP_OK : allow_smem(kern, kDpSmemMax);   // once a call
     if (st) return st;
     if (a.band < 0) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kDpNT, smem);
-        const int most = device_sms() * (per_sm < 1 ? 1 : per_sm);
         if (a.one.tiles) blocks = std::min(blocks, one_image_blocks(a.one.tiles));
-        blocks = std::min(blocks, most);
+        blocks = std::min(blocks, kDpPerSm * device_sms());
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -1042,7 +1071,7 @@ int fht_columns(int m, int wout, int subs) {
     double least = 1e30;
     for (int T = 256; T >= 16; T -= 16) {
         const size_t smem = fht_smem_bytes(m, T);
-        if (smem > 227 * 1024 - 1024) continue;
+        if (smem > kFhtSmemMax) continue;
         const int per_sm = smem <= 112 * 1024 ? 2 : 1;   // 1,024 threads a block
         const long long blocks = (long long)((wout + T - 1) / T) * subs;
         const long long each = (blocks + sms - 1) / sms;   // on the busiest SM
@@ -1076,10 +1105,7 @@ FhtImg fht_img(const void *img, long long pitch, const Shape &s, int wout, void 
 template <typename In, typename Acc>
 int launch_fht_img(const FhtImg &f, cudaStream_t stream) {
     const size_t smem = fht_smem_bytes(f.m, f.T);
-    int st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<In, Acc>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem),
-                         "cudaFuncSetAttribute");
+    int st = allow_smem(fht_band_kernel<In, Acc>, kFhtSmemMax);
     if (st) return st;
     fht_band_kernel<In, Acc><<<(unsigned)(f.tiles * f.subs), kFhtNT, smem, stream>>>(f, nullptr, 1);
     return launched("fht_band_kernel");
@@ -1350,10 +1376,7 @@ int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream) {
 namespace {
 template <typename Acc>
 int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaStream_t stream) {
-    int st = cuda_status(cudaFuncSetAttribute(fht_band_kernel<Acc, Acc>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)b->fht_smem),
-                         "cudaFuncSetAttribute");
+    int st = allow_smem(fht_band_kernel<Acc, Acc>, kFhtSmemMax);
     if (st) return st;
     fht_band_kernel<Acc, Acc><<<(unsigned)b->fht_blocks, kFhtNT, b->fht_smem, stream>>>(
         b->fht[0], (const FhtImg *)(ws + b->fht_off), (int)b->fht.size());
