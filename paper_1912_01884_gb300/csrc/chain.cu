@@ -306,6 +306,72 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
     }
 }
 
+// Bands of at most 16 rows: a strip of so few rows leaves most of a block of
+// fht_band_kernel idle, so a thread takes one column of one band here and adds
+// up its sums of both signs in registers, straight from the image (L1 serves the
+// overlapping reads).  Bound by the stores of the rows (1 to 4 rows: 4 TB/s and
+// more) and from there on by the loads' issue.  2048 x 2048 uint8, n = 1, 2, 4, 8,
+// 16: a pass a level 17, 15, 33, 40, 58 us; fht_band_kernel 261, 232, 89, 62, 50;
+// this 13, 10, 10, 13, 23.  8192 x 8192 float, n = 8: 620, 1362, 143.  (32 rows
+// would need some 270 registers; fht_band_kernel takes 29 us for 2048 x 2048 uint8.)
+constexpr int kShortRows = 16;
+template <typename In, typename Acc, int kSign, bool kInside>
+struct ShortBand {
+    const In *base;      // first row of the band
+    long long pitch;
+    int x, w, W;
+    // Column x + j (sign "-": x - j) of a row of the cyclic band.
+    __device__ Acc px(const In *row, int j) const {
+        int c = kSign == 0 ? x + j : x - j;
+        if (!kInside) {
+            if (c >= W) c -= W;
+            if (c < 0 || c >= w) return Acc(0);   // (left of the image: padding)
+        }
+        return (Acc)__ldg(row + c);
+    }
+    // Shifts 0 .. R - 1 of the R rows from row y, words 0 .. M - 1.
+    template <int R, int M>
+    __device__ void sums(int y, Acc (&o)[R][M]) const {
+        if constexpr (R == 1) {
+            const In *row = base + y * pitch;
+#pragma unroll
+            for (int j = 0; j < M; ++j) o[0][j] = px(row, j);
+        } else {
+            Acc a[R / 2][M], b[R / 2][M + R / 2];
+            sums<R / 2, M>(y, a);
+            sums<R / 2, M + R / 2>(y + R / 2, b);
+#pragma unroll
+            for (int s = 0; s < R; ++s)
+#pragma unroll
+                for (int j = 0; j < M; ++j) o[s][j] = a[s / 2][j] + b[s / 2][j + (s + 1) / 2];
+        }
+    }
+};
+
+// A block: blockDim.x columns of blockDim.y bands.
+template <typename In, typename Acc, int N>
+__global__ void __launch_bounds__(256) fht_short_kernel(const __grid_constant__ FhtImg im) {
+    const int tile = blockIdx.x % im.tiles, x0 = tile * blockDim.x, x = x0 + threadIdx.x;
+    const int band = blockIdx.x / im.tiles * blockDim.y + threadIdx.y;
+    if (band >= im.subs || x >= im.wout) return;
+    const In *base = (const In *)im.img + (size_t)band * N * im.pitch;
+    Acc *out = (Acc *)im.out + (size_t)band * 2 * N * im.opitch + x;
+    const bool inside = x0 >= N && x0 + (int)blockDim.x + N <= im.w;
+    auto one_sign = [&](auto rows, int sign) {
+        Acc o[N][1];
+        rows.template sums<N, 1>(0, o);
+#pragma unroll
+        for (int s = 0; s < N; ++s) out[(size_t)(sign * N + s) * im.opitch] = o[s][0];
+    };
+    if (inside) {
+        one_sign(ShortBand<In, Acc, 0, true>{base, im.pitch, x, im.w, im.W}, 0);
+        one_sign(ShortBand<In, Acc, 1, true>{base, im.pitch, x, im.w, im.W}, 1);
+    } else {
+        one_sign(ShortBand<In, Acc, 0, false>{base, im.pitch, x, im.w, im.W}, 0);
+        one_sign(ShortBand<In, Acc, 1, false>{base, im.pitch, x, im.w, im.W}, 1);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // The DP chain (Sec. 2.2-2.3, Eqs. 3-4).  An item is one band b and `cols`
 // continuation columns xn: with V_{b+1}(xn, e) of all displacements e in
@@ -1097,13 +1163,33 @@ FhtImg fht_img(const void *img, long long pitch, const Shape &s, int wout, void 
     f.out = out;
     f.opitch = opitch;
     f.subs = s.h / f.m;
-    f.T = fht_columns(f.m, wout, f.subs);
-    f.tiles = (wout + f.T - 1) / f.T;
     return f;
+}
+void set_columns(FhtImg &f, int T) {
+    f.T = T;
+    f.tiles = (f.wout + T - 1) / T;
 }
 
 template <typename In, typename Acc>
-int launch_fht_img(const FhtImg &f, cudaStream_t stream) {
+int launch_fht_short(FhtImg f, cudaStream_t stream) {
+    int bx = 32;   // columns of a block; narrow images: several bands
+    while (bx < 256 && bx < f.wout) bx *= 2;
+    set_columns(f, bx);
+    const int by = 256 / bx;
+    const unsigned grid = (unsigned)f.tiles * (unsigned)((f.subs + by - 1) / by);
+    auto kern = f.m == 1   ? fht_short_kernel<In, Acc, 1>
+                : f.m == 2 ? fht_short_kernel<In, Acc, 2>
+                : f.m == 4 ? fht_short_kernel<In, Acc, 4>
+                : f.m == 8 ? fht_short_kernel<In, Acc, 8>
+                           : fht_short_kernel<In, Acc, 16>;
+    kern<<<grid, dim3(bx, by), 0, stream>>>(f);
+    return launched("fht_short_kernel");
+}
+
+template <typename In, typename Acc>
+int launch_fht_img(FhtImg f, cudaStream_t stream) {
+    if (f.m <= kShortRows) return launch_fht_short<In, Acc>(f, stream);
+    set_columns(f, fht_columns(f.m, f.wout, f.subs));
     const size_t smem = fht_smem_bytes(f.m, f.T);
     int st = allow_smem(fht_band_kernel<In, Acc>, kFhtSmemMax);
     if (st) return st;
@@ -1317,8 +1403,7 @@ ChainBatch *chain_batch_create(const std::vector<ChainImage> &images, int dtype)
         b->flags.push_back(o);
         o = (o + (size_t)im.k * im.tiles * 4 + 15) & ~(size_t)15;
         FhtImg f = fht_img(c.img, c.pitch, c.s, c.s.vw, nullptr, im.pitch);
-        f.T = std::min(256, (c.s.vw + 15) & ~15);   // the least work a column
-        f.tiles = (c.s.vw + f.T - 1) / f.T;
+        set_columns(f, std::min(256, (c.s.vw + 15) & ~15));   // the least work a column
         f.item0 = b->fht_blocks;
         b->fht_blocks += f.tiles * f.subs;
         b->fht_smem = std::max(b->fht_smem, fht_smem_bytes(f.m, f.T));

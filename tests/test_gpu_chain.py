@@ -86,6 +86,22 @@ def test_fht_of_short_bands_wraps_at_the_padded_width(lib, n, w):
             assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, 6))
 
 
+# Bands of at most 16 rows: blocks of several bands (narrow images), bands left
+# over, blocks inside the image and at its edges, rows of a wider array.
+@pytest.mark.parametrize("n", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("k,w", [(1, 1), (3, 5), (37, 7), (9, 33), (5, 131), (2, 1030)])
+def test_fht_of_short_bands_matches_oracle(lib, n, k, w):
+    for dtype in ("u8", "i32", "f32"):
+        wide = _img(k * n, w + 3, dtype, n + k + w)
+        H = lib.fht_bands(to_device(wide)[:, 1:w + 1], k).cpu().numpy()
+        img = np.ascontiguousarray(wide[:, 1:w + 1])
+        if dtype == "f32":
+            want = hough_from_oracle(img, k, float32=True)
+            assert np.array_equal(H.view(np.uint32), want.view(np.uint32))
+        else:
+            assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, k))
+
+
 @pytest.mark.parametrize("dtype", ["i32", "f32"])
 def test_batch_of_every_band_height(lib, dtype):
     shapes = [(256, 333, 128, 16), (512, 70, 128, 40), (256, 500, 64, 3), (320, 201, 32, 5),
