@@ -355,10 +355,7 @@ int fhtdp_detect_through_point(const void *img, int dtype, int h, int w, int pit
         return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
                          ws ? ws_bytes : (size_t)0);
     const PointMask pm{j, xp};
-    ChainQuery q;
-    q.B = B;
-    q.point = &pm;
-    return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
+    return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, ws_bytes, stream, &pm);
 }
 
 // ---------------------------------------------------------------------------

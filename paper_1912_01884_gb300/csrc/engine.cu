@@ -2656,28 +2656,76 @@ void set_point(ImgPlan &p, int j, int xp) {
     p.mask_end = j == p.s.k ? 1 : 0;
 }
 
-// One image takes the chain (chain.cu): the engine's 128-column tiles leave
-// most of the chip idle on one image (2048 x 2048 uint8: 249 us, 110 on the
-// chain; 256 x 256: 67 and 33).  The engine needs a sixth of the workspace, and
-// takes uint8 images whose workspace is too small for the chain (the built-in
-// scratch of the no-allocation call).
+// Whether the engine runs this image, and with a point: it masks the point's
+// band in V after forming it, which band 0 never stores.
+bool engine_takes(int dtype, const Shape &s, int B, const void *img, int pitch,
+                  const PointMask *pm) {
+    if (dtype != FHTDP_U8) return false;
+    if (pm) return s.n <= kMaxBandFused && s.k >= 2 && pm->j >= 1;
+    const int Bc = B < 2 * s.n - 2 ? B : 2 * s.n - 2;
+    return s.n <= kMaxBandFused || fused_256(dtype, s, Bc, img, pitch);
+}
+
+// One image: the engine or the chain (chain.cu), by the sizes.
+//
+// The engine's tiles of 128 columns leave most of the chip idle on an image of
+// ordinary width, at about 15.7 us a band level (128-row bands) up to 152 tiles;
+// the chain's levels take 5 us and more with the width, and its FHT is a pass of
+// its own over the image.  So the chain runs all but two kinds (uint8, us, engine
+// and chain):
+//  - one band, where the engine needs one launch and stores no rows: 300 to
+//    49,152 columns of 128 rows 21 -> 44 and 25 -> 97; 2048 columns of 16 rows 14
+//    and 19.  Up to 8 rows the chain's stores are short, and it wins from 65,536
+//    columns on; from 64 rows on rows that TMA cannot copy cost the engine more
+//    than that on narrow images (300 columns 25 and 22).
+//  - wide images, from the widths of the table on (columns where the two cross):
+//    8 bands of 128 rows: 8192 columns 135 and 116, 12,288: 140 and 159, 65,536:
+//    399 and 709; 8 bands of 64 rows: 24,576: 146 and 154, 65,536: 197 and 344; 8
+//    bands of 256 rows: 6160: 231 and 230, 16,400: 397 and 525.  Few bands leave
+//    the chain less time to win back its FHT's.  (16 rows: no crossing.)
+// The table holds for the bend limits whose windows the engine unrolls; the
+// other ones up to 16 cross at about twice the width (128 rows, B = 1: 24,576:
+// 461 and 529; 16,384: 422 and 358), longer ones not at all, nor 64-bit keys
+// (128 rows, B = 32: 49,152: 1206 and 1114).  Rows that TMA cannot copy: twice the
+// width for 128 rows (B = 1, 49,153: 1321 and 1247), the same for less.
+bool engine_faster(const Shape &s, int B, const void *img, int pitch) {
+    if (256LL * s.h >= (1LL << 22)) return false;   // 64-bit keys, see dispatch
+    const bool tma = (uintptr_t)img % 16 == 0 && pitch % 16 == 0;
+    if (s.k == 1) return s.n <= 8 ? s.w < 65536 : s.n <= 32 || tma;
+    if (s.n < 32) return false;
+    static const int kWide[4][3] = {   // 32, 64, 128, 256 rows; 2, 3, 4 and more bands
+        {10240, 19456, 36864}, {14336, 19456, 24576}, {6656, 9216, 11264}, {3072, 5120, 7168}};
+    long long w = kWide[s.log2n - 5][s.k < 4 ? s.k - 2 : 2];
+    if (s.n == 256) return B >= 16 && B <= 32 && s.w >= w;
+    if (B > kFastB) return false;
+    if (B < 4 || B % 4) w *= 2;
+    if (s.n == 128 && !tma) w *= 2;
+    return s.w >= w;
+}
+
 int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-               int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream) {
+               int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream,
+               const PointMask *pm) {
     const bool room = ws_bytes >= chain_layout(s, false).total;
-    if (room || dtype != FHTDP_U8 || s.n > kMaxBandFused) {
+    if ((room && !engine_faster(s, B, img, pitch)) || !engine_takes(dtype, s, B, img, pitch, pm) ||
+        ws_bytes < engine_one_bytes(dtype, s, B)) {
         hand_injection();
         ChainQuery q;
         q.tight = !room;
         q.B = B;
+        q.point = pm;
         return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
     }
     std::vector<ImgPlan> one{single_plan(dtype, img, pitch, s, B, x_out, d_out, score_out)};
+    if (pm) set_point(one[0], pm->j, pm->xp);
     RunLayout L = plan_layout(one, false);
     char *base = (char *)ws;
     int st = cuda_status(cudaMemsetAsync(base, 0, L.zero_bytes, stream), "cudaMemsetAsync");
     if (st) return st;
     LaunchArgs args = base_args(L, base, 1);
     args.one = make_desc(one[0], L, base, dtype);
+    if (one[0].kind == 1 && (!args.one.use_tma || !args.one.use_mtma))
+        return set_error(FHTDP_ECUDA, "tensor maps of a 256-row-band image could not be encoded");
     args.many = nullptr;
     args.order = nullptr;
     return dispatch(L.max_h, args, L.multi_tile, stream);

@@ -12,7 +12,8 @@ struct BatchPlan;
 size_t detect_workspace_bytes(int dtype, const Shape &s, int B);
 size_t detect_least_bytes(int dtype, const Shape &s, int B);
 int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-               int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream);
+               int32_t *d_out, void *score_out, void *ws, size_t ws_bytes, cudaStream_t stream,
+               const PointMask *pm = nullptr);
 int engine_status(const void *ws, cudaStream_t stream);
 int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **out);
 size_t batch_workspace_bytes(const BatchPlan *plan);
