@@ -727,36 +727,58 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 M[i] = vmax(vmax(a[i * R], z[i * R]), between);
             }
         } else if (mode == kClipped) {
+            // Both ends of a window grow with the displacement, so the runs between
+            // the last window's first one (ja) and the first window's last one (jz)
+            // lie inside all eight: their maximum once.  Each window adds its own
+            // few at both ends.  polyline_dp of 2048 x 2048, unrestricted, n = 128:
+            // every window's runs by itself 155 us, this 99 (n = 256: 190, 88).
+            auto first = [&](int c) -> int {
+                return (args.use_table ? args.tab.lo[c - lo] : max(c - B, lo)) - lo;
+            };
+            auto final = [&](int c) -> int {
+                return (args.use_table ? args.tab.hi[c - lo] : min(c + B, hi)) - lo;
+            };
+            const int ja = first(min(c0 + kRun - 1, hi)) >> 3, jz = final(c0) >> 3;
+            Acc mid = dead;
+#pragma unroll 1
+            for (int j = ja + 1; j < jz; j += 4) {   // four loads in flight
+                const int e = jz - 1;
+                const Acc x0 = run_of(j), x1 = run_of(min(j + 1, e));
+                const Acc x2 = run_of(min(j + 2, e)), x3 = run_of(min(j + 3, e));
+                mid = vmax(vmax(mid, vmax(x0, x1)), vmax(x2, x3));
+            }
 #pragma unroll
             for (int i = 0; i < kRun; ++i) {
-                const int c = min(c0 + i, hi);
-                const int a = (args.use_table ? args.tab.lo[c - lo] : max(c - B, lo)) - lo;
-                const int z = (args.use_table ? args.tab.hi[c - lo] : min(c + B, hi)) - lo;
-                Acc m = vmax(Su[a * R], Pu[z * R]);
-                const int e = (z >> 3) - 1;   // the last run inside
+                const int c = min(c0 + i, hi), a = first(c), z = final(c), e = z >> 3;
+                Acc m = vmax(vmax(Su[a * R], Pu[z * R]), mid);
 #pragma unroll 1
-                for (int j = (a >> 3) + 1; j <= e; j += 4) {   // four loads in flight
-                    const Acc x0 = run_of(j), x1 = run_of(min(j + 1, e));
-                    const Acc x2 = run_of(min(j + 2, e)), x3 = run_of(min(j + 3, e));
-                    m = vmax(vmax(m, vmax(x0, x1)), vmax(x2, x3));
-                }
+                for (int j = (a >> 3) + 1; j <= min(ja, e - 1); ++j) m = vmax(m, run_of(j));
+#pragma unroll 1
+                for (int j = max(jz, ja + 1); j < e; ++j) m = vmax(m, run_of(j));
                 M[i] = m;
             }
         } else if (args.use_table) {
+            // short windows, value by value: four of each of two outputs in flight (a
+            // window that has ended repeats its last value).  polyline_dp_angle of
+            // 2048 x 2048, n = 32, 0.05 rad: one output's four 286 us, this 270.
 #pragma unroll
-            for (int i = 0; i < kRun; ++i) {
-                const int c = min(c0 + i, hi);
+            for (int i = 0; i < kRun; i += 2) {
+                const int c = min(c0 + i, hi), d = min(c0 + i + 1, hi);
                 const int a = args.tab.lo[c - lo] - lo, z = args.tab.hi[c - lo] - lo;
-                Acc m = dead;
-                // four loads in flight (the last ones twice): 1120 x 603 float, n = 32,
-                // bends of 0.1 rad, whole call 232 -> 197 us
+                const int f = args.tab.lo[d - lo] - lo, g = args.tab.hi[d - lo] - lo;
+                const int most = max(z - a, g - f);
+                Acc m = dead, o = dead;
 #pragma unroll 1
-                for (int r = a; r <= z; r += 4) {
-                    const Acc x0 = Su[r * R], x1 = Su[min(r + 1, z) * R];
-                    const Acc x2 = Su[min(r + 2, z) * R], x3 = Su[min(r + 3, z) * R];
+                for (int t = 0; t <= most; t += 4) {
+                    const Acc x0 = Su[min(a + t, z) * R], x1 = Su[min(a + t + 1, z) * R];
+                    const Acc x2 = Su[min(a + t + 2, z) * R], x3 = Su[min(a + t + 3, z) * R];
+                    const Acc y0 = Su[min(f + t, g) * R], y1 = Su[min(f + t + 1, g) * R];
+                    const Acc y2 = Su[min(f + t + 2, g) * R], y3 = Su[min(f + t + 3, g) * R];
                     m = vmax(vmax(m, vmax(x0, x1)), vmax(x2, x3));
+                    o = vmax(vmax(o, vmax(y0, y1)), vmax(y2, y3));
                 }
                 M[i] = m;
+                M[i + 1] = o;
             }
         } else {
             // B <= 3: the run and three values either side, widened B times
