@@ -102,6 +102,18 @@ def test_fht_of_short_bands_matches_oracle(lib, n, k, w):
             assert np.array_equal(H.astype(np.float64), hough_from_oracle(img, k))
 
 
+# Rows split among the warps that search V_0 (fewer rows than 256), parts of odd
+# lengths and parts past the last column.
+@pytest.mark.parametrize("n,k,w", [(1, 3, 1), (1, 2, 5000), (2, 3, 77), (2, 2, 9001), (16, 2, 2049),
+                                   (64, 2, 700), (128, 2, 259), (256, 2, 65)])
+def test_backtrack_of_split_rows_matches_oracle(lib, n, k, w):
+    for dtype in ("i32", "f32"):
+        img = _img(n * k, w, dtype, n + w)
+        B = max(1, n // 4)
+        V = lib.polyline_dp(lib.fht_bands(to_device(img), k), n * k, w, k, B)
+        _same(lib.backtrack(V, n * k, w, k, B), _detect(img, k, B))
+
+
 @pytest.mark.parametrize("dtype", ["i32", "f32"])
 def test_batch_of_every_band_height(lib, dtype):
     shapes = [(256, 333, 128, 16), (512, 70, 128, 40), (256, 500, 64, 3), (320, 201, 32, 5),
