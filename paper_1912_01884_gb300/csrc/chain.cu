@@ -487,11 +487,13 @@ __device__ __forceinline__ int state_at(const ChainImg &im, int x, int d) {
 
 // One warp: the polyline from the argmax key (Eq. 5); every band's window is
 // scanned by the lanes, the smallest displacement of the largest value kept.
+// (args.band >= 0: the caller's array, whose d = 0 is read in the "+" half.)
 // Key 0 (no admissible polyline): x = -1 everywhere and a dead score.
 template <typename Acc>
 __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsigned long long key,
                                int32_t *x_out, int32_t *d_out, Acc *score_out) {
     const int lane = threadIdx.x & 31, n = im.n, D = 2 * n - 1;
+    const int zero = args.band >= 0 ? 0 : n;   // row of d = 0
     if (key == 0) {
         if (lane == 0) *score_out = Dead<Acc>::value();
         for (int i = lane; i <= im.k; i += 32) x_out[i] = -1;
@@ -510,27 +512,34 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
         const int lo = args.use_table ? args.tab.lo[d + n - 1] : max(d - im.B, -(n - 1));
         const int hi = args.use_table ? args.tab.hi[d + n - 1] : min(d + im.B, n - 1);
         const Acc *V = band_rows<Acc>(im, i);
-        unsigned best = 0;     // order image of the value (0: none)
-        unsigned be = INT_MAX; // its displacement index
+        Acc top = Dead<Acc>::value();   // (no comparison finds NaN to be the larger)
+        unsigned be = INT_MAX;          // its displacement index
+        auto value = [&](int e) {
+            const int row = e < 0 ? n - e : e > 0 ? e : zero;
+            return ld_if(V + row * im.pitch + x, e <= hi && alive(im, i, x, e),
+                         Dead<Acc>::value());
+        };
         for (int e0 = lo + lane; e0 <= hi; e0 += 128) {   // four loads in flight
             Acc v[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int e = e0 + 32 * j;
-                v[j] = ld_if(V + state_at(im, x, e), e <= hi && alive(im, i, x, e),
-                             Dead<Acc>::value());
-            }
+            for (int j = 0; j < 4; ++j) v[j] = value(e0 + 32 * j);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned o = v[j] == Dead<Acc>::value() ? 0 : vord(v[j]);
-                if (o > best) {
-                    best = o;
+            for (int j = 0; j < 4; ++j)
+                if (v[j] > top) {
+                    top = v[j];
                     be = e0 + 32 * j + n - 1;
                 }
-            }
         }
-        const unsigned top = __reduce_max_sync(0xffffffffu, best);
-        const unsigned at = __reduce_min_sync(0xffffffffu, best == top && top ? be : INT_MAX);
+        const unsigned mine = top == Dead<Acc>::value() ? 0 : vord(top);
+        const unsigned most = __reduce_max_sync(0xffffffffu, mine);
+        unsigned at = __reduce_min_sync(0xffffffffu, mine == most && most ? be : INT_MAX);
+        if (at >= (unsigned)D) {   // a window of nothing but NaN: its first one
+            for (int e = lo + lane; e <= hi; e += 32) {
+                const Acc v = value(e);
+                if (v != v) be = min(be, (unsigned)(e + n - 1));
+            }
+            at = __reduce_min_sync(0xffffffffu, be);
+        }
         if (at >= (unsigned)D) {   // only with inconsistent values (a wait gave up)
             if (lane == 0 && args.ctl) gave_up(args);
             return;
@@ -900,10 +909,26 @@ __global__ void __launch_bounds__(kDpNT, kDpPerSm) dp_chain_kernel(const __grid_
 }
 
 // fhtdp_polyline_dp stores dead states: every state of every band whose link
-// leaves [0, vw), and the padding columns.
+// leaves [0, vw), and the padding columns.  Its input's d = 0 is the row of the
+// "+" half; the chain works on the one of the "-" half, which further blocks
+// (kDeadCols columns of a band each) make equal to it.
+constexpr int kDeadNT = 128, kDeadCols = 8 * kDeadNT;
 template <typename Acc>
-__global__ void dp_dead_kernel(Acc *hv, Shape s) {
+__global__ void __launch_bounds__(kDeadNT) dp_dead_kernel(Acc *hv, Shape s) {
     const int row = blockIdx.x;   // [k][2][n]
+    if (row >= s.k * 2 * s.n) {
+        const int chunks = (s.vw + kDeadCols - 1) / kDeadCols, i = row - s.k * 2 * s.n;
+        const int band = i / chunks, x0 = (i - band * chunks) * kDeadCols + threadIdx.x;
+        const Acc *plus = hv + (size_t)band * 2 * s.n * s.W;
+        Acc *minus = hv + ((size_t)band * 2 + 1) * s.n * s.W, v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            v[e] = ld_if(plus + x0 + e * kDeadNT, x0 + e * kDeadNT < s.vw, Acc(0));
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            st_if(minus + x0 + e * kDeadNT, x0 + e * kDeadNT < s.vw, v[e]);
+        return;
+    }
     const int r = row % (2 * s.n), d = r < s.n ? r : s.n - r;
     Acc *v = hv + (size_t)row * s.W;
     const int from = max(0, -d), to = min(s.vw, s.vw - d);   // live columns
@@ -975,7 +1000,8 @@ __global__ void __cluster_dims__(kBtBlocks, 1, 1) __launch_bounds__(kBtNT)
     };
     cluster_sync();
     const Acc *V = band_rows<Acc>(im, 0);
-    unsigned long long best = 0;
+    Acc top = Dead<Acc>::value();   // largest value, and the smallest index that holds it
+    unsigned at = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // A warp takes a row, or a part of one where the rows are fewer than the warps,
     // with eight loads in flight.  300,000 columns, n = 2: a warp a row 1443 us
@@ -985,22 +1011,26 @@ __global__ void __cluster_dims__(kBtBlocks, 1, 1) __launch_bounds__(kBtNT)
     const int parts = max(kWarps / D, 1), len = (im.vw + parts - 1) / parts;
     for (int u = blockIdx.x * (kBtNT / 32) + warp; u < D * parts; u += kWarps) {
         const int e = u / parts, from = (u - e * parts) * len, to = min(from + len, im.vw);
-        const Acc *row = V + state_at(im, 0, e - (im.n - 1));
+        const int d = e - (im.n - 1);
+        const Acc *row = V + (size_t)(d < 0 ? im.n - d : d) * im.pitch;
         for (int x0 = from + lane; x0 < to; x0 += 32 * kFlight) {
             Acc v[kFlight];
 #pragma unroll
             for (int i = 0; i < kFlight; ++i)
                 v[i] = ld_if(row + x0 + 32 * i, x0 + 32 * i < to, Dead<Acc>::value());
 #pragma unroll
-            for (int i = 0; i < kFlight; ++i) {
-                if (v[i] == Dead<Acc>::value()) continue;
-                const unsigned long long k =
-                    ((unsigned long long)vord(v[i]) << 32) |
-                    (0xffffffffu - (unsigned)((x0 + 32 * i) * D + e));
-                best = best > k ? best : k;
+            for (int i = 0; i < kFlight; ++i) {   // (NaN loses every comparison)
+                const unsigned k = (unsigned)((x0 + 32 * i) * D + e);
+                if (v[i] > top || (v[i] == top && k < at)) {
+                    top = v[i];
+                    at = k;
+                }
             }
         }
     }
+    unsigned long long best = 0;
+    if (top != Dead<Acc>::value())
+        best = ((unsigned long long)vord(top) << 32) | (0xffffffffu - at);
     auto warp_max = [](unsigned long long k) {
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
@@ -1262,7 +1292,8 @@ template int launch_band_fht<float, float>(const float *, long long, const Shape
 
 template <typename Acc>
 int launch_dp_window(Acc *hv, const Shape &s, int B, const WindowTable *t, cudaStream_t stream) {
-    dp_dead_kernel<Acc><<<(unsigned)(s.k * 2 * s.n), 128, 0, stream>>>(hv, s);
+    const int copies = s.k * ((s.vw + kDeadCols - 1) / kDeadCols);
+    dp_dead_kernel<Acc><<<(unsigned)(s.k * 2 * s.n + copies), kDeadNT, 0, stream>>>(hv, s);
     int st = launched("dp_dead_kernel");
     ChainArgs a{};
     a.one.hv = hv;

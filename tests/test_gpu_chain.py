@@ -114,6 +114,59 @@ def test_backtrack_of_split_rows_matches_oracle(lib, n, k, w):
         _same(lib.backtrack(V, n * k, w, k, B), _detect(img, k, B))
 
 
+# The layer calls on arrays of the caller's own: d = 0 is read in the "+" half,
+# whatever the copy in the "-" half holds.
+@pytest.mark.parametrize("n,k,w", [(1, 3, 40), (4, 3, 1100), (64, 3, 90), (128, 2, 2050)])
+def test_layer_calls_read_d0_in_the_plus_half(lib, n, k, w):
+    for dtype in ("i32", "f32"):
+        img = _img(n * k, w, dtype, n + w + 2)
+        B = n // 2
+        H = lib.fht_bands(to_device(img), k)
+        H[:, 1, 0, :] = 1 << 20
+        V = lib.polyline_dp(H, n * k, w, k, B)
+        if k > 1:
+            import torch
+            assert torch.equal(V[:, 0, 0, :w], V[:, 1, 0, :w])
+        V[:, 1, 0, :] = 1 << 20
+        _same(lib.backtrack(V, n * k, w, k, B), _detect(img, k, B))
+
+
+def test_backtrack_passes_over_nan(lib):
+    """NaN values lose against every number, in the top band and in the windows;
+    a window of nothing but NaN is followed at its first value."""
+    import torch
+    n, k, w, B = 8, 3, 50, 2
+    rng = np.random.default_rng(0)
+    V = rng.standard_normal((k, 2, n, w + n)).astype(np.float32)
+    V[:, 1, 0] = V[:, 0, 0]
+    x = np.arange(w)
+    for s in range(n):
+        V[:, 0, s, :w][:, x + s >= w] = -np.inf
+        V[:, 1, s, :w][:, x - s < 0] = -np.inf
+    V[..., w:] = -np.inf
+    dead = np.isneginf(V)
+    V[rng.random(V.shape) < 0.3] = np.nan
+    V[1, :, :, 20:30] = np.nan          # whole windows
+    V[dead] = -np.inf
+    V[0, 0, 3, 22] = 9.0                # the optimum's link leads there
+    at = lambda b, x, d: V[b, 0, d, x] if d >= 0 else V[b, 1, -d, x]
+    best, xs, ds = None, [], []
+    for xx in range(w):
+        for d in range(-(n - 1), n):
+            v = at(0, xx, d)
+            if v == v and not np.isneginf(v) and (best is None or v > best):
+                best, xs, ds = v, [xx], [d]
+    for b in range(1, k):
+        xs.append(xs[-1] + ds[-1])
+        win = [d for d in range(max(ds[-1] - B, 1 - n), min(ds[-1] + B, n - 1) + 1)
+               if not np.isneginf(at(b, xs[-1], d))]
+        real = [d for d in win if at(b, xs[-1], d) == at(b, xs[-1], d)]
+        ds.append(max(real, key=lambda d: (at(b, xs[-1], d), -d)) if real else win[0])
+    xs.append(xs[-1] + ds[-1])
+    gx, gd, gs = lib.backtrack(torch.from_numpy(V).cuda(), n * k, w, k, B)
+    assert gx.tolist() == xs and gd.tolist() == ds and gs.item() == best
+
+
 @pytest.mark.parametrize("dtype", ["i32", "f32"])
 def test_batch_of_every_band_height(lib, dtype):
     shapes = [(256, 333, 128, 16), (512, 70, 128, 40), (256, 500, 64, 3), (320, 201, 32, 5),
