@@ -340,11 +340,12 @@ class BatchPlan:
         self._plan = handle
         need = lib().fhtdp_batch_workspace_bytes(handle)
         self.ws = ws if ws is not None else torch.empty(need, dtype=torch.uint8, device=dev)
-        if self.ws.numel() < need:
-            raise ValueError("workspace too small")
         self.items = lib().fhtdp_batch_items(handle)
-        _check(lib().fhtdp_batch_upload(handle, self.ws.data_ptr(), self.ws.numel(),
-                                        _stream(stream)))
+        code = lib().fhtdp_batch_upload(handle, self.ws.data_ptr(), self.ws.numel(),
+                                        _stream(stream))
+        if code == 2:   # (a little less than `need` is accepted)
+            raise ValueError("workspace too small")
+        _check(code)
 
     def run(self, stream=None):
         _check(lib().fhtdp_batch_run(self._plan, self.ws.data_ptr(), _stream(stream)))

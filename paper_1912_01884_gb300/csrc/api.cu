@@ -186,6 +186,19 @@ int fhtdp_detect_polyline(const void *img, int dtype, int h, int w, int pitch, i
 }
 
 // ---------------------------------------------------------------------------
+// A query's workspace: the size that its *_workspace_bytes call offers, or any
+// from the tight layout on.
+namespace {
+int check_workspace(const Shape &s, bool smooth, const void *ws, size_t bytes, bool *tight) {
+    const size_t least = chain_layout(s, smooth, true).total;
+    if (!ws || bytes < least)
+        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", least,
+                         ws ? bytes : (size_t)0);
+    *tight = bytes < chain_layout(s, smooth).total;
+    return FHTDP_OK;
+}
+}  // namespace
+
 // The main problem (Sec. 2.3): smoothing and bend-angle windows.
 namespace {
 int check_angle_common(int dtype, int h, int w, int k, double gamma, Shape *s) {
@@ -286,13 +299,11 @@ int fhtdp_detect_polyline_angle(const void *img, int dtype, int h, int w, int pi
     if (st) return st;
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = angle_workspace_bytes(s);
-    if (!ws || ws_bytes < need)
-        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
-                         ws ? ws_bytes : (size_t)0);
+    ChainQuery q;
+    st = check_workspace(s, r > 0, ws, ws_bytes, &q.tight);
+    if (st) return st;
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
-    ChainQuery q;
     q.r = r;
     q.table = &t;
     return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
@@ -314,14 +325,12 @@ int fhtdp_detect_through_point_angle(const void *img, int dtype, int h, int w, i
                          w, k);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = angle_workspace_bytes(s);
-    if (!ws || ws_bytes < need)
-        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
-                         ws ? ws_bytes : (size_t)0);
+    ChainQuery q;
+    st = check_workspace(s, r > 0, ws, ws_bytes, &q.tight);
+    if (st) return st;
     WindowTable t;
     make_angle_table(s.n, gamma, &t);
     const PointMask pm{j, xp};
-    ChainQuery q;
     q.r = r;
     q.table = &t;
     q.point = &pm;
@@ -350,10 +359,9 @@ int fhtdp_detect_through_point(const void *img, int dtype, int h, int w, int pit
                          w, k);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = through_workspace_bytes(s);
-    if (!ws || ws_bytes < need)
-        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
-                         ws ? ws_bytes : (size_t)0);
+    bool tight;
+    int st = check_workspace(s, false, ws, ws_bytes, &tight);   // (detect_one looks again)
+    if (st) return st;
     const PointMask pm{j, xp};
     return detect_one(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, ws_bytes, stream, &pm);
 }
@@ -371,12 +379,11 @@ int fhtdp_detect_polyline_padded(const void *img, int dtype, int h, int w, int p
     if (B < 0) return set_error(FHTDP_EINVAL, "bend limit B=%d < 0", B);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = through_workspace_bytes(s);
-    if (!ws || ws_bytes < need)
-        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
-                         ws ? ws_bytes : (size_t)0);
     s.vw = s.W;
-    return detect_padded(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, stream);
+    bool tight;
+    int st = check_workspace(s, false, ws, ws_bytes, &tight);
+    if (st) return st;
+    return detect_padded(img, dtype, pitch, s, B, x_out, d_out, score_out, ws, tight, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -397,11 +404,10 @@ int fhtdp_detect_two_polylines(const void *img, int dtype, int h, int w, int pit
     if (sep < 1) return set_error(FHTDP_EINVAL, "separation %d < 1", sep);
     if (!img || !x_out || !d_out || !score_out)
         return set_error(FHTDP_EINVAL, "null image or output pointer");
-    size_t need = through_workspace_bytes(s);
-    if (!ws || ws_bytes < need)
-        return set_error(FHTDP_EWORKSPACE, "workspace needs %zu bytes, got %zu", need,
-                         ws ? ws_bytes : (size_t)0);
-    return detect_two(img, dtype, pitch, s, B, sep, x_out, d_out, score_out, ws, stream);
+    bool tight;
+    int st = check_workspace(s, false, ws, ws_bytes, &tight);
+    if (st) return st;
+    return detect_two(img, dtype, pitch, s, B, sep, x_out, d_out, score_out, ws, tight, stream);
 }
 
 // ---------------------------------------------------------------------------

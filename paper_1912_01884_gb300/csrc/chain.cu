@@ -1352,21 +1352,27 @@ ChainLayout chain_layout(const Shape &s, bool smooth, bool tight) {
     L.cols = chain_cols(s.n);
     L.tiles = (s.vw + L.cols - 1) / L.cols;
     // rows a multiple of 128 bytes apart; those of 256-row bands hold the cyclic
-    // width (tight: and no more, where the workspace is short)
+    // width.  Tight: no padding, the keys in the head, and with 256-row bands the
+    // flags in `second`, which the FHT leaves free: no more than the method's own
+    // two arrays, which every call accepted before its rows were padded.
     L.pitch = s.n > 128 ? s.W : s.vw;
-    if (!tight || s.n <= 128) L.pitch = (L.pitch + 31) & ~31;
+    if (!tight) L.pitch = (L.pitch + 31) & ~31;
+    auto up = [tight](size_t v) { return tight ? (v + 15) & ~(size_t)15 : up256(v); };
     size_t o = sizeof(ChainCtl);
-    L.key = o;   // key, done; key, done of the second polyline
-    o += 256;
+    L.key = tight ? o - 64 : o;   // key, done; key, done of the second polyline
+    if (!tight) o += 256;
+    L.late = tight && s.n > 128;
+    L.flag_bytes = (size_t)s.k * L.tiles * 4;
     L.flags = o;
-    o = up256(o + (size_t)s.k * L.tiles * 4);
+    if (!L.late) o = up(o + L.flag_bytes);
     L.zero = o;
-    const size_t rows = up256((size_t)s.k * 2 * s.n * L.pitch * 4);
+    const size_t rows = up((size_t)s.k * 2 * s.n * L.pitch * 4);
     L.rows = o;
     o += rows;
     L.second = o;
+    if (L.late) L.flags = o;
     if (s.n > 128) o += rows;
-    else if (smooth) o = up256(o + (size_t)s.h * s.w * 4);
+    else if (smooth) o = up(o + (size_t)s.h * s.w * 4);
     L.total = o;
     return L;
 }
@@ -1389,6 +1395,8 @@ int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q
     } else {
         st = launch_band_fht<In, Acc>(img, pitch, s, s.vw, rows, second, L.pitch, stream);
     }
+    if (!st && L.late)
+        st = cuda_status(cudaMemsetAsync(ws + L.flags, 0, L.flag_bytes, stream), "cudaMemsetAsync");
     if (st) return st;
     ChainArgs a{};
     ChainImg &im = a.one;

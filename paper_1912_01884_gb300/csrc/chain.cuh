@@ -11,7 +11,7 @@ namespace fhtdp {
 // the status that fhtdp_workspace_status reads.
 struct ChainCtl {
     int queue, status;
-    int pad[62];
+    int pad[62];   // (the last 64 bytes: the keys of a tight layout)
 };
 
 // One image: its Hough rows / DP values and its outputs.
@@ -44,10 +44,12 @@ struct FhtImg {
 
 // Workspace of a single-image run: [head][key, done][flags][rows][second].
 struct ChainLayout {
-    size_t key, flags, rows, second, zero, total;
+    size_t key, flags, rows, second, zero, total, flag_bytes;
     int pitch, cols, tiles;
+    bool late;   // the flags lie in `second` and are cleared after the FHT
 };
-// smooth: the image is smoothed first (angle queries, r > 0).
+// smooth: the image is smoothed first (angle queries, r > 0).  tight: the least
+// workspace that is accepted.
 ChainLayout chain_layout(const Shape &s, bool smooth, bool tight = false);
 
 struct ChainQuery {

@@ -98,11 +98,12 @@ size_t angle_workspace_bytes(const Shape &s);
 size_t through_workspace_bytes(const Shape &s);
 // The method with vertices anywhere in [0, W) (s.vw = W).
 int detect_padded(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-                  int32_t *d_out, void *score_out, void *ws, cudaStream_t stream);
+                  int32_t *d_out, void *score_out, void *ws, bool tight, cudaStream_t stream);
 // Two different extreme polylines: the optimum and the best one whose top
 // vertex is at least sep columns from the optimum's (outputs [2][...]).
 int detect_two(const void *img, int dtype, int pitch, const Shape &s, int B, int sep,
-               int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream);
+               int32_t *x_out, int32_t *d_out, void *score_out, void *ws, bool tight,
+               cudaStream_t stream);
 // dst[x][y] = src[y][x] (Sec. 3, Fig. 7: mostly horizontal curves).
 template <typename T>
 int launch_transpose(const T *src, int h, int w, int pitch, T *dst, int dpitch,

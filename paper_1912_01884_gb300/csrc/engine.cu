@@ -2454,7 +2454,8 @@ struct BatchPlan {
     std::vector<ImgPlan> imgs;      // images of the fused launch
     std::vector<ImgPlan> separate;  // 256-row bands: run one by one on the band chain
     size_t separate_off = 0;        // their scratch: `lanes` slices of sep_bytes
-    size_t sep_bytes = 0;
+    size_t sep_bytes = 0;           // (full: the layout offered, or the tight one)
+    size_t sep_full = 0, sep_tight = 0;
     int lanes = 0;                  // streams the separate images are spread over
     std::vector<cudaStream_t> side; // one non-blocking stream per lane
     std::vector<cudaEvent_t> ev;    // fork + one join per lane
@@ -2472,6 +2473,7 @@ struct BatchPlan {
     WindowTable tab{};
     size_t reserve = 0;             // bytes of the fused part for any tile-width choice
     size_t ws_total = 0;            // workspace bytes (the reserve and the side lanes)
+    size_t ws_least = 0;            // the least accepted: side lanes with tight layouts
     ~BatchPlan() {
         if (chain) chain_batch_destroy(chain);
         for (cudaStream_t st : side) cudaStreamDestroy(st);
@@ -2639,8 +2641,7 @@ size_t detect_workspace_bytes(int dtype, const Shape &s, int B) {
 }
 
 // uint8 images with bands of at most 128 rows run on the engine where the
-// workspace is too small for the chain, the others with rows that are not padded
-// to whole lines.
+// workspace is too small for the chain, the others with the tight layout.
 size_t detect_least_bytes(int dtype, const Shape &s, int B) {
     const size_t chain = chain_layout(s, false, true).total;
     return dtype == FHTDP_U8 && s.n <= kMaxBandFused
@@ -2788,12 +2789,19 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
     }
     // Scratch of the images that run by themselves: up to kSideLanes lanes, each a stream
     // that runs its images one after the other on its own slice.
-    size_t sep = 0;
-    for (auto &p : plan->separate) sep = std::max(sep, chain_layout(p.s, false).total);
-    plan->sep_bytes = align_up(sep, 256);
+    for (auto &p : plan->separate) {
+        plan->sep_full = std::max(plan->sep_full, align_up(chain_layout(p.s, false).total, 256));
+        plan->sep_tight =
+            std::max(plan->sep_tight, align_up(chain_layout(p.s, false, true).total, 256));
+    }
+    plan->sep_bytes = plan->sep_full;
     plan->lanes = (int)std::min<size_t>(kSideLanes, plan->separate.size());
     plan->separate_off = align_up(plan->reserve, 256);
-    plan->ws_total = sep ? plan->separate_off + plan->sep_bytes * plan->lanes : plan->reserve;
+    plan->ws_total = plan->ws_least = plan->reserve;
+    if (plan->lanes) {
+        plan->ws_total = plan->separate_off + plan->sep_full * plan->lanes;
+        plan->ws_least = plan->separate_off + plan->sep_tight * plan->lanes;
+    }
     for (int l = 0; l < plan->lanes; ++l) {
         cudaStream_t st = nullptr;
         if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
@@ -2855,9 +2863,10 @@ int upload_tables(BatchPlan *plan, void *ws, cudaStream_t stream) {
 
 int batch_upload(BatchPlan *plan, void *ws, size_t ws_bytes, cudaStream_t stream) {
     if (!plan || !ws) return set_error(FHTDP_EINVAL, "null plan or workspace");
-    if (ws_bytes < plan->ws_total)
+    if (ws_bytes < plan->ws_least)
         return set_error(FHTDP_EWORKSPACE, "batch workspace needs %zu bytes, got %zu",
-                         plan->ws_total, ws_bytes);
+                         plan->ws_least, ws_bytes);
+    plan->sep_bytes = ws_bytes < plan->ws_total ? plan->sep_tight : plan->sep_full;
     plan->bound_ws = ws;
     return upload_tables(plan, ws, stream);
 }
@@ -2885,6 +2894,7 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
             const ImgPlan &p = plan->separate[i];
             const int l = (int)(i % plan->lanes);
             ChainQuery q;
+            q.tight = plan->sep_bytes != plan->sep_full;
             q.B = p.io.B;
             q.report = (int *)(base + offsetof(Ctl, status));
             st = chain_detect(p.io.img, plan->dtype, p.io.pitch, p.s, q, p.io.x_out, p.io.d_out,

@@ -61,7 +61,8 @@ size_t param_bytes() {
 
 // CNN workspace for n images of h x w pixels (low-resolution ho x wo): the
 // input, the four layer outputs, two gradient buffers, the FP32 gradients of
-// every layer, the loss and the CTAs' sums of a weight gradient.
+// every layer, the loss and, from `part` on, the CTAs' sums of a weight gradient
+// (a workspace without them is accepted).
 struct CnnWs {
     size_t x0, act[kLayers], g0, g1, grads[kLayers], loss, part, total;
 };
@@ -231,8 +232,8 @@ int fhtdp_cnn_forward(const void *params, const uint8_t *imgs, int n, int h, int
         return set_error(FHTDP_EINVAL, "unsupported CNN shape n=%d h=%d w=%d bands=%d", n, h, w,
                          bands);
     const CnnWs c = cnn_ws(n, h, w);
-    if (ws_bytes < c.total)
-        return set_error(FHTDP_EWORKSPACE, "CNN workspace needs %zu bytes, got %zu", c.total,
+    if (ws_bytes < c.part)
+        return set_error(FHTDP_EWORKSPACE, "CNN workspace needs %zu bytes, got %zu", c.part,
                          ws_bytes);
     return forward((const char *)params, imgs, n, h, w, bands, (char *)ws, c, pred, conf, true,
                    stream);
@@ -246,8 +247,8 @@ int fhtdp_cnn_backward(const void *params, const int32_t *labels, int n, int h, 
         return set_error(FHTDP_EINVAL, "unsupported CNN shape n=%d h=%d w=%d bands=%d", n, h, w,
                          bands);
     const CnnWs c = cnn_ws(n, h, w);
-    if (ws_bytes < c.total)
-        return set_error(FHTDP_EWORKSPACE, "CNN workspace needs %zu bytes, got %zu", c.total,
+    if (ws_bytes < c.part)
+        return set_error(FHTDP_EWORKSPACE, "CNN workspace needs %zu bytes, got %zu", c.part,
                          ws_bytes);
     const char *P = (const char *)params;
     char *W = (char *)ws;
@@ -263,8 +264,14 @@ int fhtdp_cnn_backward(const void *params, const int32_t *labels, int n, int h, 
         const LayerOff o = layer_off(l);
         float *dw = (float *)(W + c.grads[l]);
         const void *xin = l == 0 ? (const void *)(W + c.x0) : (const void *)(W + c.act[l - 1]);
-        st = cnn_wgrad(xin, l == 0 ? 1 : kC, n, ho, wo, kDil[l], dz, dw,
-                       dw + (size_t)taps_rows(l) * kC, stream, (float *)(W + c.part));
+        // the CTAs' sums in `part`, or without room for it added up by atomics
+        float *part = ws_bytes >= c.total ? (float *)(W + c.part) : nullptr;
+        if (!part)
+            st = cuda_status(cudaMemsetAsync(dw, 0, ((size_t)taps_rows(l) * kC + kC) * 4, stream),
+                             "cudaMemsetAsync");
+        if (!st)
+            st = cnn_wgrad(xin, l == 0 ? 1 : kC, n, ho, wo, kDil[l], dz, dw,
+                           dw + (size_t)taps_rows(l) * kC, stream, part);
         if (l == 0 || st) break;
         // input gradient: the forward of the flipped and transposed weights,
         // masked by the ReLU of the layer below

@@ -26,8 +26,9 @@ size_t through_workspace_bytes(const Shape &s) {
 // in [0, W), so its values are the plain sums with zeros right of the image;
 // the DP and the read-back run over the vertex domain s.vw = W.
 int detect_padded(const void *img, int dtype, int pitch, const Shape &s, int B, int32_t *x_out,
-                  int32_t *d_out, void *score_out, void *ws, cudaStream_t stream) {
+                  int32_t *d_out, void *score_out, void *ws, bool tight, cudaStream_t stream) {
     ChainQuery q;
+    q.tight = tight;
     q.B = B;
     return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);
 }
@@ -36,8 +37,10 @@ int detect_padded(const void *img, int dtype, int pitch, const Shape &s, int B, 
 // no rule): the optimum, then the best polyline whose top vertex lies at
 // least sep columns from the optimum's, both read back from the same V.
 int detect_two(const void *img, int dtype, int pitch, const Shape &s, int B, int sep,
-               int32_t *x_out, int32_t *d_out, void *score_out, void *ws, cudaStream_t stream) {
+               int32_t *x_out, int32_t *d_out, void *score_out, void *ws, bool tight,
+               cudaStream_t stream) {
     ChainQuery q;
+    q.tight = tight;
     q.B = B;
     q.sep = sep;
     return chain_detect(img, dtype, pitch, s, q, x_out, d_out, score_out, ws, stream);

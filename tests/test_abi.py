@@ -265,3 +265,60 @@ def test_cnn_32_channel_layers_reject_unaligned_activations_before_launch(lib):
         for i, call in enumerate(calls):
             assert call() == 1, (off, i)
             assert "16-byte" in L.fhtdp_last_error().decode()
+
+
+def _needs(lib, call):
+    """The least workspace of a call, from its message for one of a single byte."""
+    assert call(1) == 2
+    return int(lib.lib().fhtdp_last_error().decode().split("needs ")[1].split()[0])
+
+
+@pytest.mark.parametrize("n", [1, 2, 8, 16, 64, 128, 256])
+@pytest.mark.parametrize("k", [1, 3, 128])
+@pytest.mark.parametrize("w", [1, 2, 31, 33, 257, 4097])
+def test_workspaces_of_two_hough_arrays_are_accepted(lib, n, k, w):
+    """Every single-image call runs in a head and the method's own two Hough
+    arrays (for one-row bands and smoothing the image too); the size that the
+    *_workspace_bytes calls offer may be larger.  Nothing is launched."""
+    L = lib.lib()
+    p = ctypes.c_void_p(1 << 12)
+    h = n * k
+    up = lambda v: (v + 255) // 256 * 256
+    two = 256 + 2 * up(k * 2 * n * (w + n) * 4)
+    smooth = up(h * w * 4) if n == 1 else 0
+    outs = (p, p, p, p)
+    for dt in (0, 1, 2):
+        calls = {
+            "through": (two, lambda b: L.fhtdp_detect_through_point(p, dt, h, w, w, k, 2, 0, 0,
+                                                                    *outs, b, None)),
+            "padded": (two, lambda b: L.fhtdp_detect_polyline_padded(p, dt, h, w, w, k, 2, *outs, b,
+                                                                     None)),
+            "two": (two, lambda b: L.fhtdp_detect_two_polylines(p, dt, h, w, w, k, 2, 1, *outs, b,
+                                                                None)),
+        }
+        for r in (0, 2):
+            calls["angle", r] = (two + smooth,
+                                 lambda b, r=r: L.fhtdp_detect_polyline_angle(
+                                     p, dt, h, w, w, k, r, 0.1, *outs, b, None))
+            calls["through angle", r] = (two + smooth,
+                                         lambda b, r=r: L.fhtdp_detect_through_point_angle(
+                                             p, dt, h, w, w, k, r, 0.1, 0, 0, *outs, b, None))
+        if n == 256:
+            calls["detect"] = (two, lambda b: L.fhtdp_detect_polyline(p, dt, h, w, w, k, 2, *outs,
+                                                                      b, None))
+        for name, (size, call) in calls.items():
+            assert _needs(lib, call) <= size, (name, dt)
+
+
+def test_cnn_workspace_without_the_partial_sums_is_accepted(lib):
+    """Activations, gradients and the loss are enough for the network's calls."""
+    L = lib.lib()
+    p = ctypes.c_void_p(1 << 12)
+    for n, h, w in ((1, 64, 256), (4, 128, 512)):
+        px = n * (h // 4) * (w // 4)
+        a = lambda v: (v + 255) // 256 * 256
+        size = a(px * 2) + 6 * a(px * 64) + a(9 * 32 * 32 * 2) + a(17 * 32 * 4) \
+            + 3 * a((288 + 1) * 32 * 4) + 256
+        for call in (lambda b: L.fhtdp_cnn_forward(p, p, n, h, w, 8, p, b, p, None, None),
+                     lambda b: L.fhtdp_cnn_backward(p, p, n, h, w, 8, p, b, None, None)):
+            assert _needs(lib, call) <= size

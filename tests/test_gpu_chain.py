@@ -258,3 +258,67 @@ def test_batch_status_reports_a_wait_of_a_256_row_image_that_gave_up(lib):
     assert plan.status() == 0
     for i in range(2):
         _same((plan.x[i], plan.d[i], plan.score[i]), oracle.detect(img, 4, 9))
+
+
+# Every single-image call in the least workspace that it accepts (one byte less is
+# refused), the bytes after it untouched.
+@pytest.mark.parametrize("n,k,w", [(1, 5, 9), (2, 3, 1), (8, 4, 33), (64, 3, 101), (128, 2, 257),
+                                   (256, 1, 65), (256, 3, 130)])
+def test_calls_in_the_least_workspace(lib, n, k, w):
+    import torch
+    L = lib.lib()
+    for dtype, code in (("u8", 0), ("i32", 1), ("f32", 2)):
+        img = _img(n * k, w, dtype, n + k + w)
+        dev, h, B = to_device(img), n * k, max(1, n // 8)
+        f = dtype == "f32"
+        at = lambda t: t.data_ptr()
+        cases = [
+            (L.fhtdp_detect_polyline, (B,), 1, [_detect(img, k, B)]),
+            (L.fhtdp_detect_through_point, (B, 0, w // 2), 1,
+             [(oracle.detect_through_f32 if f else oracle.detect_through)(img, k, B, 0, w // 2)]),
+            (L.fhtdp_detect_polyline_padded, (B,), 1,
+             [(oracle.detect_padded_f32 if f else oracle.detect_padded)(img, k, B)]),
+            (L.fhtdp_detect_two_polylines, (B, 2), 2,
+             list(zip(*(oracle.detect_two_f32 if f else oracle.detect_two)(img, k, B, 2)))),
+        ]
+        for r in (0, 2):
+            cases.append((L.fhtdp_detect_polyline_angle, (r, 0.3), 1,
+                          [(oracle.detect_angle_f32 if f else oracle.detect_angle)(img, k, r, 0.3)]))
+        for fn, args, count, want in cases:
+            x = torch.empty((count, k + 1), dtype=torch.int32, device="cuda")
+            d = torch.empty((count, k), dtype=torch.int32, device="cuda")
+            s = torch.empty(count, dtype=torch.float32 if f else torch.int32, device="cuda")
+            ws = torch.full((1 << 22,), 0x5a, dtype=torch.uint8, device="cuda")
+            call = lambda b: fn(at(dev), code, h, w, w, k, *args, at(x), at(d), at(s), at(ws), b,
+                                torch.cuda.current_stream().cuda_stream)
+            assert call(1) == 2
+            need = int(L.fhtdp_last_error().decode().split("needs ")[1].split()[0])
+            assert call(need - 1) == 2 and call(need) == 0
+            for i in range(count):
+                _same((x[i], d[i], s[i]), want[i])
+            assert bool((ws[need:] == 0x5a).all())
+
+
+def test_batch_of_256_row_bands_in_the_least_workspace(lib):
+    """int32 images that run one by one: the workspace that the plan offers, and
+    the smaller one of their two Hough arrays each."""
+    import torch
+    L = lib.lib()
+    shapes = [(256, 65, 1), (512, 130, 2), (768, 33, 3), (256, 64, 1), (512, 31, 2)]
+    imgs = [_img(h, w, "i32", w) for h, w, _ in shapes]
+    dev = [to_device(i) for i in imgs]
+    ks, Bs = [k for _, _, k in shapes], [20] * len(shapes)
+    plan = lib.BatchPlan(dev, ks, Bs)
+    least = 4 * max(256 + 2 * (k * 2 * 256 * (w + 256) * 4) for _, w, k in shapes) + 4096
+    offered = plan.ws.numel()
+    assert least < offered
+    for size in (offered, least):
+        ws = torch.full((offered + 4096,), 0x5a, dtype=torch.uint8, device="cuda")
+        small = lib.BatchPlan(dev, ks, Bs, ws=ws[:size])
+        small.run()
+        assert small.status() == 0
+        for i, img in enumerate(imgs):
+            _same((small.x[i], small.d[i], small.score[i]), _detect(img, ks[i], Bs[i]))
+        assert bool((ws[size:] == 0x5a).all())
+    with pytest.raises(ValueError):
+        lib.BatchPlan(dev, ks, Bs, ws=ws[:4096])
