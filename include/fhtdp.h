@@ -444,22 +444,25 @@ long long fhtdp_batch_items(const fhtdp_batch_plan *plan);
  * It uploads the chosen layout and queue, and writes the width to
  * *target_out (may be NULL); fhtdp_batch_choice reports the rest.  The
  * outputs are those of an ordinary run.  Batches of int32 and float images
- * have one schedule and nothing to tune: the call runs them and leaves the
- * plan as it is.  It synchronises `stream` (not for use under stream capture).  The paper has no counterpart: this tunes the GPU
- * schedule of its method, not the method. */
+ * have one schedule and nothing to tune: the call runs them once and leaves the
+ * plan as it is.  It synchronises `stream` (not for use under stream capture).
+ * The paper has no counterpart: this tunes the GPU schedule of its method, not
+ * the method. */
 int fhtdp_batch_autotune(fhtdp_batch_plan *plan, void *ws, int reps, cudaStream_t stream,
                          long long *target_out);
 /* The plan's current choices: the queue schedule (*mode: 0 groups, 1 band
  * chains, 2 band chains with the 256-row-band images spread, 3 band chains
- * with 256-row bands every second step, 4 both) and width, and for its images of band height n the column tile
- * width and register FHT depth (0 and 0 when it has none).  Any pointer may
- * be NULL.  The paper has no counterpart (see fhtdp_batch_autotune). */
+ * with 256-row bands every second step, 4 both) and width, and for its images of
+ * band height n the column tile width and register FHT depth (0 and 0 when it has
+ * none).  int32 and float batches: 0 and the column tiles of a band level of the
+ * whole batch, which advances together.  Any pointer may be NULL.  The paper has
+ * no counterpart (see fhtdp_batch_autotune). */
 int fhtdp_batch_choice(const fhtdp_batch_plan *plan, int n, int *mode, long long *target,
                        int *tile, int *depth);
 /* Sets, by hand, the column tile width and register FHT depth of the plan's
- * uint8 images of band height n (the choices of step 2 of
- * fhtdp_batch_autotune; FHTDP_EINVAL for one that band height does not
- * allow) and enqueues the upload of the new layout and queue into the bound
+ * images of band height n (uint8: the choices of step 2 of
+ * fhtdp_batch_autotune; int32 and float images have one; FHTDP_EINVAL for one
+ * that band height does not allow) and enqueues the upload of the new layout and queue into the bound
  * workspace `ws`.  The paper has no counterpart (see fhtdp_batch_autotune). */
 int fhtdp_batch_configure(fhtdp_batch_plan *plan, void *ws, int n, int tile, int depth,
                           cudaStream_t stream);

@@ -1519,6 +1519,16 @@ ChainBatch *chain_batch_create(const std::vector<ChainImage> &images, int dtype)
 void chain_batch_destroy(ChainBatch *b) { delete b; }
 size_t chain_batch_bytes(const ChainBatch *b) { return b->total; }
 long long chain_batch_items(const ChainBatch *b) { return (long long)b->order.size(); }
+long long chain_batch_width(const ChainBatch *b) {
+    long long tiles = 0;
+    for (const ChainImg &im : b->imgs) tiles += im.tiles;
+    return tiles;
+}
+int chain_batch_tile(const ChainBatch *b, int n) {
+    for (const ChainImg &im : b->imgs)
+        if (im.n == n) return im.cols;
+    return 0;
+}
 
 int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream) {
     char *W = (char *)ws;

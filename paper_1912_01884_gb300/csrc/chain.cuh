@@ -81,6 +81,10 @@ ChainBatch *chain_batch_create(const std::vector<ChainImage> &images, int dtype)
 void chain_batch_destroy(ChainBatch *b);
 size_t chain_batch_bytes(const ChainBatch *b);
 long long chain_batch_items(const ChainBatch *b);
+// The tiles of a band level over all images, and the columns of the DP items of
+// band height n (0: no such image).
+long long chain_batch_width(const ChainBatch *b);
+int chain_batch_tile(const ChainBatch *b, int n);
 // The batch's tables for workspace ws (from host memory held by the batch).
 int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream);
 // A run: the clearing of its head, then the launches.  t (optional): bend-angle

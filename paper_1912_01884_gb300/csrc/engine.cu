@@ -2818,7 +2818,8 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
         }
         plan->ev.push_back(e);
     }
-    plan->target = num_sms();
+    // (the chain's queue: all images of the batch advance together)
+    plan->target = plan->chain ? chain_batch_width(plan->chain) : num_sms();
     plan->order = queue_order(plan->imgs, plan->target, plan->mode);
     *out = plan;
     return FHTDP_OK;
@@ -2940,9 +2941,11 @@ int batch_autotune(BatchPlan *plan, void *ws, int reps, cudaStream_t stream, lon
     if (ws != plan->bound_ws)
         return set_error(FHTDP_EINVAL, "workspace differs from the one given to fhtdp_batch_upload");
     if (reps < 1) reps = 1;
-    if (plan->imgs.empty()) {
+    if (plan->imgs.empty()) {   // one schedule: the run that every tuning ends with
+        int st = batch_run(plan, ws, stream);
+        if (!st) st = cuda_status(cudaStreamSynchronize(stream), "cudaStreamSynchronize");
         if (chosen) *chosen = plan->target;
-        return FHTDP_OK;
+        return st;
     }
     const long long sms = num_sms();
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -3070,6 +3073,17 @@ int batch_configure(BatchPlan *plan, void *ws, int n, int tile, int depth, cudaS
     if (!plan || !ws) return set_error(FHTDP_EINVAL, "null plan or workspace");
     if (ws != plan->bound_ws)
         return set_error(FHTDP_EINVAL, "workspace differs from the one given to fhtdp_batch_upload");
+    if (const int own = plan->chain ? chain_batch_tile(plan->chain, n) : 0) {
+        // int32 and float images have one width and depth (16 columns is taken for
+        // every band height, for choices stored when it was theirs)
+        if (tile != own && tile != 16)
+            return set_error(FHTDP_EINVAL, "tile width %d not available for band height %d",
+                             tile, n);
+        if (depth < 2 || depth > 3 || (depth == 3 && n < 8))
+            return set_error(FHTDP_EINVAL, "register depth %d not available for band height %d",
+                             depth, n);
+        return upload_tables(plan, ws, stream);
+    }
     bool any = false;
     for (const ImgPlan &p : plan->imgs) {
         if (p.s.n != n) continue;
@@ -3098,7 +3112,7 @@ void batch_choice(const BatchPlan *plan, int n, int *mode, long long *target, in
                   int *depth) {
     if (mode) *mode = plan->mode;
     if (target) *target = plan->target;
-    int T = 0, dd = 0;
+    int T = plan->chain ? chain_batch_tile(plan->chain, n) : 0, dd = T ? 2 : 0;
     for (const ImgPlan &p : plan->imgs)
         if (p.s.n == n) {
             T = p.T;

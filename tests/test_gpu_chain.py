@@ -322,3 +322,34 @@ def test_batch_of_256_row_bands_in_the_least_workspace(lib):
         assert bool((ws[size:] == 0x5a).all())
     with pytest.raises(ValueError):
         lib.BatchPlan(dev, ks, Bs, ws=ws[:4096])
+
+
+@pytest.mark.parametrize("dtype", ["i32", "f32"])
+def test_tuning_calls_on_int32_and_float_batches(lib, dtype):
+    """autotune leaves the outputs of a run, choice reports what the queue is, and
+    configure takes the one width that there is."""
+    shapes = [(256, 300, 64), (64, 90, 8), (256, 41, 128)]
+    imgs = [_img(h, w, dtype, w) for h, w, _ in shapes]
+    ks, Bs = [h // n for h, _, n in shapes], [n // 8 for _, _, n in shapes]
+    plan = lib.BatchPlan([to_device(i) for i in imgs], ks, Bs)
+    tiles = {64: 32, 8: 256, 128: 16}
+    width = sum(-(-w // tiles[n]) for _, w, n in shapes)
+    assert plan.autotune(reps=1) == width
+
+    def right():
+        for i, img in enumerate(imgs):
+            _same((plan.x[i], plan.d[i], plan.score[i]), _detect(img, ks[i], Bs[i]))
+            plan.x[i].fill_(-7)
+    right()
+    for n, tile in tiles.items():
+        c = plan.choice(n)
+        assert c["schedule"] == "groups" and c["width"] == width and c["tile"] == tile
+        plan.configure(n, tile, c["depth"])
+        plan.configure(n, 16, 2)
+        for bad in ((tile + 1, 2), (tile, 4), (tile, 1)):
+            with pytest.raises(lib.FhtdpError):
+                plan.configure(n, *bad)
+    with pytest.raises(lib.FhtdpError):
+        plan.configure(32, 16, 2)          # no image of 32-row bands
+    plan.run()
+    right()
