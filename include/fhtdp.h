@@ -403,8 +403,8 @@ typedef struct fhtdp_image {
      * [lo_i, hi_i] of each band's link.  With it the DP searches only those
      * links (the pruned DP of the learned proposal, which the paper does not
      * have) and returns the best polyline inside the windows; if there is none,
-     * the score is INT32_MIN / -infinity and every vertex -1.  Bands of at most
-     * 128 rows. */
+     * the score is INT32_MIN and every vertex -1.  uint8 images with bands of
+     * at most 128 rows (FHTDP_EINVAL otherwise). */
     const int32_t *d_window;
 } fhtdp_image;
 

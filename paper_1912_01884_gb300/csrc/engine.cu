@@ -2761,11 +2761,12 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
         }
         ImgPlan p = single_plan(dtype, io.img, io.pitch, s, io.B, io.x_out, io.d_out, io.score_out);
         p.io.d_window = io.d_window;
-        if (io.d_window && s.n > kMaxBandFused) {
+        if (io.d_window && (s.n > kMaxBandFused || dtype != FHTDP_U8)) {
             delete plan;
             return set_error(FHTDP_EINVAL,
-                             "image %d: displacement windows need bands of at most %d rows", i,
-                             kMaxBandFused);
+                             "image %d: displacement windows need uint8 images with bands of at "
+                             "most %d rows",
+                             i, kMaxBandFused);
         }
         if (s.n > kMaxBandFused && p.kind != 1)
             plan->separate.push_back(p);

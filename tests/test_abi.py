@@ -322,3 +322,17 @@ def test_cnn_workspace_without_the_partial_sums_is_accepted(lib):
         for call in (lambda b: L.fhtdp_cnn_forward(p, p, n, h, w, 8, p, b, p, None, None),
                      lambda b: L.fhtdp_cnn_backward(p, p, n, h, w, 8, p, b, None, None)):
             assert _needs(lib, call) <= size
+
+
+def test_displacement_windows_are_for_uint8_images(lib):
+    """The pruned DP runs in the uint8 engine; a window that another pixel type's
+    batch could not honour is refused when the plan is made."""
+    L = lib.lib()
+    plan = ctypes.c_void_p()
+    for dtype, want in ((0, 0), (1, 1), (2, 1)):
+        img = lib.Image(16, 64, 40, 40, 4, 2, 16, 16, 16, 16)   # never dereferenced
+        assert L.fhtdp_batch_plan_create(ctypes.byref(img), 1, dtype, ctypes.byref(plan)) == want
+        if want:
+            assert "windows" in L.fhtdp_last_error().decode()
+        else:
+            L.fhtdp_batch_plan_destroy(plan)
