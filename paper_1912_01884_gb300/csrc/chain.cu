@@ -1193,22 +1193,21 @@ int launch_chain_cols(const ChainArgs &a, int cols, size_t smem, int blocks, boo
 size_t fht_smem_bytes(int m, int T) { return (size_t)m * fht_pitch(m, T) * 4; }
 
 // Columns of an FHT block: a block's time grows as T + 0.8 m (the passes sweep
-// T + m - 4, T + m - 16, ... columns), two on an SM take about 0.85 of their sum,
-// and the SM with the most blocks decides, so the T (a multiple of 16, at most
-// 256) of the least product.  2048 x 2048 uint8, n = 128: T = 64, 128, 192, 256
-// take 46, 34, 44, 33 us; 1024 x 512, n = 64: T = 32, 64, 128, 256 17, 11.5, 15, 21;
-// 8192 x 8192, n = 128: T = 128, 192, 256 296, 272, 243.
+// T + m - 4, T + m - 16, ... columns), one fits an SM (1,024 threads of 64
+// registers), and the SM with the most blocks decides, so the T (a multiple of
+// 16, at most 256) of the least product.  2048 x 2048 uint8, n = 128: T = 64, 128,
+// 192, 256 take 46, 34, 44, 33 us; 1024 x 512, n = 64: T = 32, 64, 128, 256 17,
+// 11.5, 15, 21; 512 x 2016, n = 32: T = 112, 240 15.8, 10.2; 8192 x 8192, n = 128:
+// T = 128, 192, 256 296, 272, 243.  (Those registers are a few
+// too few: 32 to 64 bytes a thread spill.)
 int fht_columns(int m, int wout, int subs) {
     const int sms = device_sms();
     int best = 16;
     double least = 1e30;
     for (int T = 256; T >= 16; T -= 16) {
-        const size_t smem = fht_smem_bytes(m, T);
-        if (smem > kFhtSmemMax) continue;
-        const int per_sm = smem <= 112 * 1024 ? 2 : 1;   // 1,024 threads a block
+        if (fht_smem_bytes(m, T) > kFhtSmemMax) continue;
         const long long blocks = (long long)((wout + T - 1) / T) * subs;
-        const long long each = (blocks + sms - 1) / sms;   // on the busiest SM
-        const double cost = each * (each > 1 && per_sm > 1 ? 0.85 : 1.0) * (T + 0.8 * m);
+        const double cost = (blocks + sms - 1) / sms * (T + 0.8 * m);   // on the busiest SM
         if (cost < least) {
             least = cost;
             best = T;
