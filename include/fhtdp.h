@@ -97,7 +97,7 @@ size_t fhtdp_hough_bytes(int dtype, int h, int w, int k);
  *          moving left; columns are taken modulo W (cyclic FHT), so for
  *          x in [0, w) and an end column inside the image it is the plain sum.
  *   ws     device workspace of at least fhtdp_fht_workspace_bytes() bytes
- *          (stage ping-pong buffer), overwritten.
+ *          (the halves' level of 256-row bands), overwritten.
  */
 size_t fhtdp_fht_workspace_bytes(int dtype, int h, int w, int k);
 int fhtdp_fht_bands(const void *img, int dtype, int h, int w, int pitch, int k,
@@ -125,9 +125,13 @@ int fhtdp_backtrack(const void *V, int dtype, int h, int w, int k, int B,
                     int32_t *x_out, int32_t *d_out, void *score_out, cudaStream_t stream);
 
 /* The whole method on one image (Sec. 2.1-2.3 and the main problem): the
- * band FHTs, the bend-limited DP and the read-back, through the fused engine
- * (the Hough images never reach global memory).
- *   ws     device workspace of at least fhtdp_workspace_bytes() bytes.
+ * band FHTs, the bend-limited DP and the read-back.  Two paths give the same
+ * result: an FHT launch that stores the Hough images in the workspace and a DP
+ * launch over them, and for uint8 images one fused launch whose Hough images
+ * never reach global memory (wide images, single bands, short workspaces).
+ *   ws     device workspace of fhtdp_workspace_bytes() bytes.  Less is taken
+ *          while a layout fits (uint8 images with bands of at most 128 rows: that of
+ *          the fused launch; others: rows without padding); FHTDP_EWORKSPACE names the least size.
  *   Outputs as for fhtdp_backtrack.  Returns FHTDP_ETIMEOUT if a device-side
  *   dependency wait gave up (the outputs are then undefined).
  */
@@ -144,9 +148,10 @@ int fhtdp_detect_polyline(const void *img, int dtype, int h, int w, int pitch, i
  * FHTDP_NOALLOC_SCRATCH_BYTES inside the library, which every GPU that loads
  * the library holds until the process exits.  Arguments, outputs and results
  * are those of fhtdp_detect_polyline.
- *   - Images whose scratch (fhtdp_workspace_bytes) exceeds the array are
- *     rejected with FHTDP_EWORKSPACE before anything is enqueued (a 2048x2048
- *     uint8 image with 128-row bands needs about 12.5 MiB).
+ *   - Images whose least scratch exceeds the array are rejected with
+ *     FHTDP_EWORKSPACE before anything is enqueued.  That is the least size that
+ *     fhtdp_detect_polyline accepts, below fhtdp_workspace_bytes (a 2048x2048
+ *     uint8 image with 128-row bands needs about 12.5 MiB and is offered 32).
  *   - The first call on a device looks up the array's device address (with
  *     that device current); make that first call before any stream capture.
  *   - All calls share the one array, and it keeps the last call's contents;
@@ -292,9 +297,9 @@ int fhtdp_detect_two_polylines(const void *img, int dtype, int h, int w, int pit
  * image.  The bands are the image's k vertical strips of n = w/k columns (n a
  * power of two, 1 <= n <= 256); link i joins row y_i on the strip's first
  * column to row y_{i+1} = y_i + d_i on its last column, |d_i| <= n-1, every
- * y_i in [0, h).  The image is transposed into the workspace and run through
- * the fused engine, so results, ties and errors are those of
- * fhtdp_detect_polyline on the transposed image (dtype any of the three).
+ * y_i in [0, h).  The image is transposed into the workspace and run as in
+ * fhtdp_detect_polyline, so results, ties and errors are those of that call on
+ * the transposed image (dtype any of the three).
  *   y_out [k+1], d_out [k], score_out [1] (device).
  *   ws     device workspace of at least fhtdp_horizontal_workspace_bytes();
  *          fhtdp_workspace_status is not available for these calls.
@@ -326,7 +331,7 @@ int fhtdp_detect_polyline_horizontal(const void *img, int dtype, int h, int w, i
 int fhtdp_cnn_downsample4(const uint8_t *img, int n, int h, int w, void *out, cudaStream_t stream);
 /* y = act(conv3x3_dil(x, wt) + bias), act = ReLU when relu != 0; cin 1 or 32,
  * cout 32, zero padding ("same").  32 input channels run on tcgen05.mma
- * (persistent CTAs down columns of 256 pixels, an input row meeting the nine
+ * (persistent CTAs down columns of 128 pixels, an input row meeting the nine
  * taps of the three output rows that it feeds, FP32 accumulators in tensor
  * memory); a bounded wait that gives up records FHTDP_ETIMEOUT for
  * fhtdp_cnn_status. */
@@ -377,9 +382,9 @@ int fhtdp_cnn_bin_windows(const int32_t *pred, int count, int n, int margin, int
 int fhtdp_workspace_status(const void *ws, cudaStream_t stream);
 
 /* Test hook for failure detection (no counterpart in the paper): the next
- * fused-engine run started from this host thread (fhtdp_detect_polyline or
- * fhtdp_batch_run) never publishes the window maxima of column tile `tile` of
- * band `band` of its first image, and its device-side waits give up after
+ * detection run started from this host thread (fhtdp_detect_polyline or
+ * fhtdp_batch_run) never publishes column tile `tile` of band `band` of its
+ * first image, and its device-side waits give up after
  * `wait_cycles` SM cycles instead of about two seconds.  The run then ends with
  * FHTDP_ETIMEOUT in fhtdp_workspace_status and undefined outputs; the CUDA
  * context stays usable.  Nothing faults or hangs. */

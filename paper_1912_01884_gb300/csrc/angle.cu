@@ -16,18 +16,16 @@ bool make_angle_table(int n, double gamma, WindowTable *t) {
     const int D = 2 * n - 1;
     double a[kMaxD];
     for (int i = 0; i < D; ++i) a[i] = std::atan((double)(i - (n - 1)) / n);
-    int lo = 0, hi = 0, maxlen = 1;
+    int lo = 0, hi = 0;
     for (int i = 0; i < D; ++i) {
         while (a[i] - a[lo] > gamma) ++lo;
         if (hi < i) hi = i;
         while (hi + 1 < D && a[hi + 1] - a[i] <= gamma) ++hi;
         t->lo[i] = (int16_t)(lo - (n - 1));
         t->hi[i] = (int16_t)(hi - (n - 1));
-        if (hi - lo + 1 > maxlen) maxlen = hi - lo + 1;
     }
     for (int i = D; i < kMaxD; ++i) t->lo[i] = t->hi[i] = 0;
     t->n = n;
-    t->maxlen = maxlen;
     return true;
 }
 

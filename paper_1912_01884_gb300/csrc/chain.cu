@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
                 fht_two_levels<Wd, kFhtNT, true>(F, pitch, m, l, T, out);
                 l += 2;
             } else {
-                fht_level<Wd, kFhtNT, true>(F, pitch, m, l + 1, T, out);
+                fht_level<Wd, kFhtNT>(F, pitch, m, l + 1, T, out);
                 l += 1;
             }
             __syncthreads();

@@ -43,7 +43,6 @@ constexpr int kMaxD = 511;
 struct WindowTable {
     int16_t lo[kMaxD], hi[kMaxD];
     int n;
-    int maxlen;  // the longest window, hi - lo + 1
 };
 // Fills *t for bands of n rows; false if gamma is negative or not finite.
 bool make_angle_table(int n, double gamma, WindowTable *t);
@@ -108,11 +107,5 @@ int detect_two(const void *img, int dtype, int pitch, const Shape &s, int B, int
 template <typename T>
 int launch_transpose(const T *src, int h, int w, int pitch, T *dst, int dpitch,
                      cudaStream_t stream);
-int detect_through(const void *img, int dtype, int pitch, const Shape &s, int B,
-                   const PointMask &pm, int32_t *x_out, int32_t *d_out, void *score_out,
-                   void *ws, cudaStream_t stream);
-int detect_angle(const void *img, int dtype, int pitch, const Shape &s, int r,
-                 const WindowTable &t, int32_t *x_out, int32_t *d_out, void *score_out,
-                 void *ws, cudaStream_t stream, const PointMask *pm = nullptr);
 
 }  // namespace fhtdp

@@ -75,7 +75,7 @@ struct ImgDesc {
     const void *img;
     long long pitch;          // row stride in elements
     int h, w, k, n, log2n, B, tiles;
-    int tw;                   // column tile width of its work items (uint8: 64, 128 or 256)
+    int tw;                   // column tile width of its work items (64, 128 or 256)
     int depth;                // uint8: FHT levels done in registers before the merges (2 or 3)
     long long item0;          // first work item of this image
     void *mbuf[2];            // ping-pong window maxima, [D][mpitch] of Acc
@@ -2176,10 +2176,10 @@ struct RunLayout {
     bool multi_tile;     // some image's tiles are not kTile wide
 };
 
-// Column tile width of an image's work items: uint8 images with bands of at
+// Column tile width of an image's work items: images with bands of at
 // most 64 rows take 256 columns (more work per item and fewer items for the
 // short bands), the others 128.
-int default_tile(int dtype, int n) { return dtype == FHTDP_U8 && n <= 64 ? 256 : kTile; }
+int default_tile(int n) { return n <= 64 ? 256 : kTile; }
 
 int tiles_of(const Shape &s, int T) { return (s.w + T - 1) / T; }
 
@@ -2196,24 +2196,23 @@ int tile_code(int T) { return T == 256 ? 2 : T == 64 ? 0 : 1; }
 
 // Tile widths a uint8 image's items may take (the tuner's choices): bands of
 // at most 64 rows 128 or 256, 128-row bands 128, 256-row bands 64.
-bool tile_choice(int dtype, const ImgPlan &p, int T) {
-    if (dtype != FHTDP_U8 || p.kind == 1) return T == p.T;
+bool tile_choice(const ImgPlan &p, int T) {
+    if (p.kind == 1) return T == p.T;
     return T == kTile || (T == 2 * kTile && p.s.n <= max_band<2 * kTile>());
 }
 
 // With `reserve`, every image's counters and buffers are sized for the
 // largest of its tile-width choices (most tiles, widest M rows), so that the
 // workspace fits any choice the tuner makes.
-RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve = false,
-                      int dtype = FHTDP_U8) {
+RunLayout plan_layout(std::vector<ImgPlan> &imgs, bool with_table, bool reserve = false) {
     RunLayout L{};
     size_t off = sizeof(Ctl);
     long long items = 0;
     for (auto &p : imgs) {
         const int T0 = p.T;
-        if (reserve && tile_choice(dtype, p, kTile)) p.T = kTile;   // the most tiles
+        if (reserve && tile_choice(p, kTile)) p.T = kTile;   // the most tiles
         p.tiles = tiles_of(p.s, p.T);
-        if (reserve && tile_choice(dtype, p, 2 * kTile)) p.T = 2 * kTile;   // the widest rows
+        if (reserve && tile_choice(p, 2 * kTile)) p.T = 2 * kTile;   // the widest rows
         p.item0 = items;
         items += (long long)p.s.k * p.tiles;
         if (p.kind == 1) {
@@ -2300,15 +2299,14 @@ bool encode_m_map(CUtensorMap *map, void *m0, int D, int mpitch, int bw, int bh)
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws, int dtype) {
+ImgDesc make_desc(const ImgPlan &p, const RunLayout &L, char *ws) {
     ImgDesc im{};
-    im.use_tma = dtype == FHTDP_U8 &&
-                 encode_strip_map(&im.tmap, p.io.img, p.s.h, p.s.w, p.io.pitch, p.s.n);
+    im.use_tma = encode_strip_map(&im.tmap, p.io.img, p.s.h, p.s.w, p.io.pitch, p.s.n);
     if (p.kind == 1)
         im.use_mtma = ws && encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch,
                                          kTile256, kMBox256);
     else
-        im.use_mtma = dtype == FHTDP_U8 && p.s.n <= kMaxBandFused && ws &&
+        im.use_mtma = p.s.n <= kMaxBandFused && ws &&
                       encode_m_map(&im.mtmap, ws + L.data_off + p.m0, p.s.D, p.mpitch, kTile,
                                    p.s.D);
     im.img = p.io.img;
@@ -2423,7 +2421,7 @@ LaunchArgs base_args(const RunLayout &L, char *ws, int count) {
 ImgPlan single_plan(int dtype, const void *img, int pitch, const Shape &s, int B,
                     int32_t *x_out, int32_t *d_out, void *score_out) {
     ImgPlan p{};
-    p.T = default_tile(dtype, s.n);
+    p.T = default_tile(s.n);
     p.depth = 3;
     p.io.img = img;
     p.io.h = s.h;
@@ -2724,7 +2722,7 @@ int detect_one(const void *img, int dtype, int pitch, const Shape &s, int B, int
     int st = cuda_status(cudaMemsetAsync(base, 0, L.zero_bytes, stream), "cudaMemsetAsync");
     if (st) return st;
     LaunchArgs args = base_args(L, base, 1);
-    args.one = make_desc(one[0], L, base, dtype);
+    args.one = make_desc(one[0], L, base);
     if (one[0].kind == 1 && (!args.one.use_tma || !args.one.use_mtma))
         return set_error(FHTDP_ECUDA, "tensor maps of a 256-row-band image could not be encoded");
     args.many = nullptr;
@@ -2786,7 +2784,7 @@ int batch_create(const fhtdp_image *images, int count, int dtype, BatchPlan **ou
         plan->reserve = chain_batch_bytes(plan->chain);
     } else {
         std::vector<ImgPlan> any = plan->imgs;
-        plan->reserve = plan_layout(any, true, true, dtype).total;
+        plan->reserve = plan_layout(any, true, true).total;
     }
     // Scratch of the images that run by themselves: up to kSideLanes lanes, each a stream
     // that runs its images one after the other on its own slice.
@@ -2845,7 +2843,7 @@ int upload_tables(BatchPlan *plan, void *ws, cudaStream_t stream) {
     if (plan->chain) return chain_batch_upload(plan->chain, ws, stream);
     plan->staging.clear();
     for (auto &p : plan->imgs) {
-        plan->staging.push_back(make_desc(p, plan->L, (char *)ws, plan->dtype));
+        plan->staging.push_back(make_desc(p, plan->L, (char *)ws));
         const ImgDesc &im = plan->staging.back();
         if (p.kind == 1 && (!im.use_tma || !im.use_mtma))
             return set_error(FHTDP_ECUDA,
@@ -2931,7 +2929,7 @@ int batch_run(const BatchPlan *plan, void *ws, cudaStream_t stream) {
 //   1. the queue schedule (groups or band chains) and its width, from half a
 //      wave to the whole batch at once (wider steps wait less for
 //      dependencies but keep more window-maximum buffers in flight in L2);
-//   2. for each band height of the uint8 images, the column tile width of
+//   2. for each band height of the images, the column tile width of
 //      its items (128 or 256 columns where shared memory allows) and the
 //      number of FHT levels done in registers before the shared-memory merges
 //      (2 or 3), applied to every image of that height;
@@ -3012,7 +3010,7 @@ int batch_autotune(BatchPlan *plan, void *ws, int reps, cudaStream_t stream, lon
         return r;
     };
     if (!st) st = tune_schedule();
-    if (!st && plan->dtype == FHTDP_U8) {
+    if (!st) {
         std::vector<int> heights;
         for (const ImgPlan &p : plan->imgs)
             if (std::find(heights.begin(), heights.end(), p.s.n) == heights.end())
@@ -3033,7 +3031,7 @@ int batch_autotune(BatchPlan *plan, void *ws, int reps, cudaStream_t stream, lon
                 for (int depth = 2; depth <= 3 && !st; ++depth) {
                     const int T = first->kind == 1 ? T0 : Ts[ti];
                     if (ti == 1 && first->kind == 1) continue;
-                    if (!tile_choice(plan->dtype, *first, T)) continue;
+                    if (!tile_choice(*first, T)) continue;
                     if (depth == 3 && n < 8) continue;
                     if (T == T0 && depth == D0) continue;   // timed already
                     for (ImgPlan &p : plan->imgs)
@@ -3089,7 +3087,7 @@ int batch_configure(BatchPlan *plan, void *ws, int n, int tile, int depth, cudaS
     for (const ImgPlan &p : plan->imgs) {
         if (p.s.n != n) continue;
         any = true;
-        if (!tile_choice(plan->dtype, p, tile))
+        if (!tile_choice(p, tile))
             return set_error(FHTDP_EINVAL, "tile width %d not available for band height %d",
                              tile, n);
         if (depth < 2 || depth > 3 || (depth == 3 && n < 8))
@@ -3144,7 +3142,7 @@ int batch_points(BatchPlan *plan, void *ws, const int32_t *points, cudaStream_t 
         const ImgPlan &p = plan->imgs[i];
         if (j < 0) continue;
         if (j > p.s.k || xp < 0 || xp >= p.s.w || p.kind != 0 ||
-            plan->dtype != FHTDP_U8 || p.s.n > kMaxBandFused || p.s.k < 2 || j < 1)
+            p.s.n > kMaxBandFused || p.s.k < 2 || j < 1)
             return set_error(FHTDP_EINVAL,
                              "point %zu: border 1..k, column 0..w-1, uint8, 2+ bands of <= 128 rows",
                              i);

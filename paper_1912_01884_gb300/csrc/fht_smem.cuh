@@ -2,9 +2,9 @@
 // that store the Hough rows (chain.cu).
 //
 // F holds m rows of `pitch` words; after the level of 2^l-row sub-bands, row
-// j * 2^l + brev(s) holds shift s of sub-band j.  The first three levels are
-// done in registers straight from the image (bands of at least 8 rows); the
-// rest in shared memory, two levels a pass where possible, in place: a warp
+// j * 2^l + brev(s) holds shift s of sub-band j.  The first two levels are done
+// in registers straight from the image (sub-bands of at least 4 rows, chain.cu);
+// the rest in shared memory, two levels a pass where possible, in place: a warp
 // owns a set of rows and sweeps their columns left to right, and column u is
 // only read by columns <= u.  The last level hands its values to `out(s, u,
 // four words)` instead of storing them.  Every value is (top half) + (bottom
@@ -93,49 +93,35 @@ __device__ __forceinline__ void fht_quad(const uint4 &j0, const uint4 *j1, const
     for (int k = 0; k < 4; ++k) o[k] = pack4(r[k]);
 }
 
-// Level l (sub-bands of 2^(l-1) rows merged) in place, or into `out` (kOut,
-// the last level).  T output columns, m rows, NT threads; no barrier.
-template <typename W, int NT, bool kOut, typename Out>
-__device__ void fht_level(W *F, int pitch, int m, int l, int T, Out out) {
+// The last level, l (sub-bands of 2^(l-1) rows merged), into `out`.  T output
+// columns, m rows, NT threads; no barrier.
+template <typename W, int NT, typename Out>
+__device__ void fht_level(const W *F, int pitch, int m, int l, int T, Out out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int half = 1 << (l - 1), width = T + m - 2 * half;
     for (int p = warp; p < m / 2; p += NT / 32) {
         const int j = p >> (l - 1), r = p & (half - 1);
         const int q = bit_reverse(r, l - 1);
-        W *A = F + (size_t)(2 * j * half + r) * pitch, *B = A + (size_t)half * pitch;
+        const W *A = F + (size_t)(2 * j * half + r) * pitch, *B = A + (size_t)half * pitch;
         const W *Bq = B + (q & ~3);
-        for (int u0 = 0; u0 < width; u0 += 128) {
-            const int u = u0 + 4 * lane;
-            const bool live = u < width;
+        for (int u = 4 * lane; u < width; u += 128) {
             uint4 o[2];
-            if (live) {
-                const uint4 a4 = *(const uint4 *)&A[u];
-                const uint4 b4[2] = {*(const uint4 *)&Bq[u], *(const uint4 *)&Bq[u + 4]};
-                switch (q & 3) {   // warp-uniform
-                    case 0: fht_pair<W, 0>(a4, b4, o); break;
-                    case 1: fht_pair<W, 1>(a4, b4, o); break;
-                    case 2: fht_pair<W, 2>(a4, b4, o); break;
-                    default: fht_pair<W, 3>(a4, b4, o); break;
-                }
+            const uint4 a4 = *(const uint4 *)&A[u];
+            const uint4 b4[2] = {*(const uint4 *)&Bq[u], *(const uint4 *)&Bq[u + 4]};
+            switch (q & 3) {   // warp-uniform
+                case 0: fht_pair<W, 0>(a4, b4, o); break;
+                case 1: fht_pair<W, 1>(a4, b4, o); break;
+                case 2: fht_pair<W, 2>(a4, b4, o); break;
+                default: fht_pair<W, 3>(a4, b4, o); break;
             }
-            if (kOut) {
-                if (live) {
-                    out(2 * q, u, o[0]);
-                    out(2 * q + 1, u, o[1]);
-                }
-                continue;
-            }
-            __syncwarp();
-            if (live) {
-                *(uint4 *)&A[u] = o[0];
-                *(uint4 *)&B[u] = o[1];
-            }
-            __syncwarp();
+            out(2 * q, u, o[0]);
+            out(2 * q + 1, u, o[1]);
         }
     }
 }
 
-// Levels l + 1 and l + 2 (sub-bands of 2^l rows merged into 4 * 2^l).
+// Levels l + 1 and l + 2 (sub-bands of 2^l rows merged into 4 * 2^l) in place, or
+// into `out` (kOut, the last ones).
 template <typename W, int NT, bool kOut, typename Out>
 __device__ void fht_two_levels(W *F, int pitch, int m, int l, int T, Out out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
