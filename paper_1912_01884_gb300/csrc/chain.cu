@@ -202,7 +202,8 @@ struct BandFht {
     }
 };
 
-template <typename In, typename Acc>
+// kSplit: a block makes one slope sign, two blocks a tile (int32 and float).
+template <typename In, typename Acc, bool kSplit>
 __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_constant__ FhtImg one,
                                                              const FhtImg *__restrict__ many,
                                                              int count) {
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
         }
     }
     const FhtImg &im = many ? many[i] : one;
-    const int block = blockIdx.x - (many ? im.item0 : 0), item = block >> im.split;
+    const int item = (blockIdx.x - (many ? im.item0 : 0)) >> (kSplit ? 1 : 0);
     const int sub = item / im.tiles, T = im.T, x0 = (item - sub * im.tiles) * T;
     const int m = im.m, pitch = fht_pitch(m, T), per_band = im.n / m;
     const int band = sub / per_band, j = sub - band * per_band;
@@ -241,9 +242,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
                 if (x + e < im.wout) dst[e] = v[e];
         }
     };
-    const int sign0 = im.split ? block & 1 : 0;
-    const int signs = Tile::kPacked ? 1 : im.split ? sign0 + 1 : 2;
-    for (int sign = sign0; sign < signs; ++sign) {
+    for (int sign = kSplit ? blockIdx.x & 1 : 0; sign < (Tile::kPacked ? 1 : 2); ++sign) {
         auto out = [&](int s, int u, const uint4 &q) {
             Acc v[4];
             if constexpr (Tile::kPacked) {
@@ -304,6 +303,7 @@ __global__ void __launch_bounds__(kFhtNT, 1) fht_band_kernel(const __grid_consta
             }
             __syncthreads();
         }
+        if (kSplit) break;
         __syncthreads();   // F is rewritten for the other sign
     }
 }
@@ -1257,13 +1257,20 @@ int launch_fht_img(FhtImg f, cudaStream_t stream) {
     if (f.m <= kShortRows) return launch_fht_short<In, Acc>(f, stream);
     set_columns(f, fht_columns(f.m, f.wout, f.subs));
     const long long blocks = (long long)f.tiles * f.subs;
-    // int32 and float: a block a sign while there is an SM for each (256 x 256
-    // float, n = 128: 20.8 -> 14.6 us; the passes over whole arrays took 16.7)
-    f.split = sizeof(In) > 1 && 2 * blocks <= device_sms();
     const size_t smem = fht_smem_bytes(f.m, f.T);
-    int st = allow_smem(fht_band_kernel<In, Acc>, kFhtSmemMax);
+    auto kern = fht_band_kernel<In, Acc, false>;
+    unsigned grid = (unsigned)blocks;
+    if constexpr (sizeof(In) > 1) {
+        // a block a sign while there is an SM for each (256 x 256 float, n = 128:
+        // 20.8 -> 14.6 us; the passes over whole arrays took 16.7)
+        if (2 * blocks <= device_sms()) {
+            kern = fht_band_kernel<In, Acc, true>;
+            grid *= 2;
+        }
+    }
+    int st = allow_smem(kern, kFhtSmemMax);
     if (st) return st;
-    fht_band_kernel<In, Acc><<<(unsigned)(blocks << f.split), kFhtNT, smem, stream>>>(f, nullptr, 1);
+    kern<<<grid, kFhtNT, smem, stream>>>(f, nullptr, 1);
     return launched("fht_band_kernel");
 }
 
@@ -1550,9 +1557,9 @@ int chain_batch_upload(ChainBatch *b, void *ws, cudaStream_t stream) {
 namespace {
 template <typename Acc>
 int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaStream_t stream) {
-    int st = allow_smem(fht_band_kernel<Acc, Acc>, kFhtSmemMax);
+    int st = allow_smem(fht_band_kernel<Acc, Acc, false>, kFhtSmemMax);
     if (st) return st;
-    fht_band_kernel<Acc, Acc><<<(unsigned)b->fht_blocks, kFhtNT, b->fht_smem, stream>>>(
+    fht_band_kernel<Acc, Acc, false><<<(unsigned)b->fht_blocks, kFhtNT, b->fht_smem, stream>>>(
         b->fht[0], (const FhtImg *)(ws + b->fht_off), (int)b->fht.size());
     st = launched("fht_band_kernel");
     if (st) return st;

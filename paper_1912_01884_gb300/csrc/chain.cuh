@@ -38,7 +38,6 @@ struct FhtImg {
     int n, m, log2m;     // band height; sub-bands of m = min(n, 128) rows are merged
     void *out;           // [k][2][n][opitch], row j * m + s for sub-band j, shift s
     int opitch, T, tiles, subs;   // T columns a block (a multiple of 16)
-    int split;           // 1: a block makes one slope sign, 2 tiles blocks a sub-band
     int item0;           // first block of this image in a launch of several
 };
 

@@ -104,18 +104,21 @@ __device__ void fht_level(const W *F, int pitch, int m, int l, int T, Out out) {
         const int q = bit_reverse(r, l - 1);
         const W *A = F + (size_t)(2 * j * half + r) * pitch, *B = A + (size_t)half * pitch;
         const W *Bq = B + (q & ~3);
-        for (int u = 4 * lane; u < width; u += 128) {
-            uint4 o[2];
-            const uint4 a4 = *(const uint4 *)&A[u];
-            const uint4 b4[2] = {*(const uint4 *)&Bq[u], *(const uint4 *)&Bq[u + 4]};
-            switch (q & 3) {   // warp-uniform
-                case 0: fht_pair<W, 0>(a4, b4, o); break;
-                case 1: fht_pair<W, 1>(a4, b4, o); break;
-                case 2: fht_pair<W, 2>(a4, b4, o); break;
-                default: fht_pair<W, 3>(a4, b4, o); break;
+        for (int u0 = 0; u0 < width; u0 += 128) {
+            const int u = u0 + 4 * lane;
+            if (u < width) {
+                uint4 o[2];
+                const uint4 a4 = *(const uint4 *)&A[u];
+                const uint4 b4[2] = {*(const uint4 *)&Bq[u], *(const uint4 *)&Bq[u + 4]};
+                switch (q & 3) {   // warp-uniform
+                    case 0: fht_pair<W, 0>(a4, b4, o); break;
+                    case 1: fht_pair<W, 1>(a4, b4, o); break;
+                    case 2: fht_pair<W, 2>(a4, b4, o); break;
+                    default: fht_pair<W, 3>(a4, b4, o); break;
+                }
+                out(2 * q, u, o[0]);
+                out(2 * q + 1, u, o[1]);
             }
-            out(2 * q, u, o[0]);
-            out(2 * q + 1, u, o[1]);
         }
     }
 }
