@@ -400,7 +400,11 @@ __global__ void __launch_bounds__(256) fht_short_kernel(const __grid_constant__ 
 constexpr int kDpNT = 512;
 constexpr int kDpPerSm = 2;     // blocks an SM: all its registers at 64 a thread
 constexpr int kRun = 8;         // displacements of a thread's run
-constexpr int kPadB = 32;       // bend limits up to this read past the range unchecked
+// Bend limits up to this read past the range unchecked: 2048 x 2048 uint8, n = 64,
+// B = 20, 32: 156 and 161 us the call, clipped 175 and 172 (n = 128, B = 32: 103,
+// 108).  B = 40 would still gain, 174 -> 162 us (n = 128: 109 -> 105), for twice the
+// dead rows in shared memory.
+constexpr int kPadB = 32;
 constexpr int kMinLen = kRun + 1;   // windows from this length on span two runs
 
 struct ChainItem {
@@ -487,13 +491,12 @@ __device__ __forceinline__ int state_at(const ChainImg &im, int x, int d) {
 
 // One warp: the polyline from the argmax key (Eq. 5); every band's window is
 // scanned by the lanes, the smallest displacement of the largest value kept.
-// (args.band >= 0: the caller's array, whose d = 0 is read in the "+" half.)
+// kCaller: a caller's array, whose d = 0 is read in the "+" half.
 // Key 0 (no admissible polyline): x = -1 everywhere and a dead score.
-template <typename Acc>
+template <typename Acc, bool kCaller = false>
 __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsigned long long key,
                                int32_t *x_out, int32_t *d_out, Acc *score_out) {
     const int lane = threadIdx.x & 31, n = im.n, D = 2 * n - 1;
-    const int zero = args.band >= 0 ? 0 : n;   // row of d = 0
     if (key == 0) {
         if (lane == 0) *score_out = Dead<Acc>::value();
         for (int i = lane; i <= im.k; i += 32) x_out[i] = -1;
@@ -512,28 +515,30 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
         const int lo = args.use_table ? args.tab.lo[d + n - 1] : max(d - im.B, -(n - 1));
         const int hi = args.use_table ? args.tab.hi[d + n - 1] : min(d + im.B, n - 1);
         const Acc *V = band_rows<Acc>(im, i);
-        Acc top = Dead<Acc>::value();   // (no comparison finds NaN to be the larger)
-        unsigned be = INT_MAX;          // its displacement index
-        auto value = [&](int e) {
-            const int row = e < 0 ? n - e : e > 0 ? e : zero;
-            return ld_if(V + row * im.pitch + x, e <= hi && alive(im, i, x, e),
-                         Dead<Acc>::value());
+        unsigned best = 0;     // order image of the value (0: none)
+        unsigned be = INT_MAX; // its displacement index
+        auto value = [&](int e) -> Acc {
+            const int at = kCaller && e == 0 ? x : state_at(im, x, e);
+            return ld_if(V + at, e <= hi && alive(im, i, x, e), Dead<Acc>::value());
         };
         for (int e0 = lo + lane; e0 <= hi; e0 += 128) {   // four loads in flight
             Acc v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) v[j] = value(e0 + 32 * j);
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (v[j] > top) {
-                    top = v[j];
+            for (int j = 0; j < 4; ++j) {
+                v[j] = vmax(v[j], Dead<Acc>::value());   // (NaN loses against every number)
+                const unsigned o = v[j] == Dead<Acc>::value() ? 0 : vord(v[j]);
+                if (o > best) {
+                    best = o;
                     be = e0 + 32 * j + n - 1;
                 }
+            }
         }
-        const unsigned mine = top == Dead<Acc>::value() ? 0 : vord(top);
-        const unsigned most = __reduce_max_sync(0xffffffffu, mine);
-        unsigned at = __reduce_min_sync(0xffffffffu, mine == most && most ? be : INT_MAX);
-        if (at >= (unsigned)D) {   // a window of nothing but NaN: its first one
+        const unsigned top = __reduce_max_sync(0xffffffffu, best);
+        unsigned at = __reduce_min_sync(0xffffffffu, best == top && top ? be : INT_MAX);
+        if (std::is_same<Acc, float>::value && top == 0) {   // nothing but NaN: the first one
+            be = INT_MAX;
             for (int e = lo + lane; e <= hi; e += 32) {
                 const Acc v = value(e);
                 if (v != v) be = min(be, (unsigned)(e + n - 1));
@@ -579,8 +584,11 @@ __host__ __device__ constexpr int range_rows(int n) {
 }
 
 // kC: the image's tile width, or 0 to take it from the image (a batch of several
-// widths: five copies of the code for one kernel spill).
-template <typename Acc, int kC>
+// widths: five copies of the code for one kernel spill).  kLong: the code of
+// kShared and of scanned tables alone, in a kernel of its own (beside the other
+// modes' it cost those 0.2 us a band level: 2048 x 2048 uint8, n = 128, 105.6 ->
+// 108.6 us the call); without it kShared runs as kClipped.
+template <typename Acc, int kC, bool kLong>
 __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char *smem,
                            const ChainArgs &args) {
     const int C = kC ? kC : im.cols, lg = 31 - __clz(C);
@@ -588,7 +596,8 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     const int n = im.n, D = 2 * n - 1, lo = -(n - 1), hi = n - 1, xn0 = tile * C;
     const int u = threadIdx.x & (C - 1), q = threadIdx.x >> lg, xn = xn0 + u;
     const bool last = band == im.k - 1;   // (only one-band images: V = H)
-    const int B = im.B, mode = window_mode(args.use_table, args.minlen, B);
+    const int B = im.B, asked = window_mode(args.use_table, args.minlen, B);
+    const int mode = !kLong && asked == kShared ? kClipped : asked;
     const int pad = window_pad(mode, args.use_table, B), rows = range_rows(n);
     const Acc dead = Dead<Acc>::value();
     // S (or the values), then P: row e - lo + pad of displacement e
@@ -720,7 +729,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         const int r0 = c0 - lo + pad;   // the run's first row
         auto run_of = [&](int j) -> Acc { return Su[j * kRun * R]; };   // maximum of run j
         if (last) {
-        } else if (mode == kPadded) {
+        } else if (!kLong && mode == kPadded) {
             // windows [r - B, r + B]: their first run is j0 or, from row 8 - ol
             // on, j0 + 1; their last one z0 or, from row 8 - oz on, z0 + 1
             const int j0 = (r0 - B) >> 3, z0 = (r0 + B) >> 3;
@@ -739,7 +748,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 const Acc between = la ? (lz ? m11 : mid) : (lz ? m01 : m00);
                 M[i] = vmax(vmax(a[i * R], z[i * R]), between);
             }
-        } else if (mode == kShared) {
+        } else if (kLong && mode == kShared) {
             // Both ends of a window grow with the displacement, so the runs between
             // the last window's first one (ja) and the first window's last one (jz)
             // lie inside all eight: their maximum once.  Each window adds its own
@@ -770,7 +779,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 for (int j = max(jz, ja + 1); j < e; ++j) m = vmax(m, run_of(j));
                 M[i] = m;
             }
-        } else if (mode == kClipped) {
+        } else if (!kLong && mode == kClipped) {
 #pragma unroll
             for (int i = 0; i < kRun; ++i) {
                 const int c = min(c0 + i, hi);
@@ -786,7 +795,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
                 }
                 M[i] = m;
             }
-        } else if (args.use_table) {
+        } else if (kLong) {
             // short windows, value by value: four of each of two outputs in flight (a
             // window that has ended repeats its last value).  polyline_dp_angle of
             // 2048 x 2048, n = 32, 0.05 rad: one output's four 286 us, this 270.
@@ -898,12 +907,12 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
 }
 
 // kC: the tile width when all images share it, or 0.
-template <typename Acc, int kC>
+template <typename Acc, int kC, bool kLong>
 __global__ void __launch_bounds__(kDpNT, kDpPerSm) dp_chain_kernel(const __grid_constant__ ChainArgs args) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
     auto item = [&](const ChainImg &im, int band, int tile) {
-        chain_item<Acc, kC>(im, band, tile, smem, args);
+        chain_item<Acc, kC, kLong>(im, band, tile, smem, args);
     };
     if (args.band >= 0) {
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1074,8 +1083,8 @@ __global__ void __cluster_dims__(kBtBlocks, 1, 1) __launch_bounds__(kBtNT)
     __syncthreads();
     cluster_sync();
     if (blockIdx.x == 0 && warp == 0)
-        chain_readback<Acc>(im, args, warp_max(lane < kBtBlocks ? s_block[lane] : 0ull), im.x_out,
-                            im.d_out, (Acc *)im.score_out);
+        chain_readback<Acc, true>(im, args, warp_max(lane < kBtBlocks ? s_block[lane] : 0ull),
+                                  im.x_out, im.d_out, (Acc *)im.score_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1174,9 +1183,9 @@ int one_image_blocks(int t) {
     return t / half * half;
 }
 
-template <typename Acc, int kC>
+template <typename Acc, int kC, bool kLong>
 int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cudaStream_t stream) {
-    auto kern = dp_chain_kernel<Acc, kC>;
+    auto kern = dp_chain_kernel<Acc, kC, kLong>;
     int st = dependent ? FHTDP_OK : allow_smem(kern, kDpSmemMax);   // once a call
     if (st) return st;
     if (a.band < 0) {
@@ -1197,17 +1206,28 @@ int launch_chain(const ChainArgs &a, size_t smem, int blocks, bool dependent, cu
     if (st) return st;
     return launched("dp_chain_kernel");
 }
-template <typename Acc>
+template <typename Acc, bool kLong>
 int launch_chain_cols(const ChainArgs &a, int cols, size_t smem, int blocks, bool dependent,
                       cudaStream_t stream) {
     switch (cols) {
-        case 0: return launch_chain<Acc, 0>(a, smem, blocks, dependent, stream);
-        case 16: return launch_chain<Acc, 16>(a, smem, blocks, dependent, stream);
-        case 32: return launch_chain<Acc, 32>(a, smem, blocks, dependent, stream);
-        case 64: return launch_chain<Acc, 64>(a, smem, blocks, dependent, stream);
-        case 128: return launch_chain<Acc, 128>(a, smem, blocks, dependent, stream);
-        default: return launch_chain<Acc, 256>(a, smem, blocks, dependent, stream);
+        case 0: return launch_chain<Acc, 0, kLong>(a, smem, blocks, dependent, stream);
+        case 16: return launch_chain<Acc, 16, kLong>(a, smem, blocks, dependent, stream);
+        case 32: return launch_chain<Acc, 32, kLong>(a, smem, blocks, dependent, stream);
+        case 64: return launch_chain<Acc, 64, kLong>(a, smem, blocks, dependent, stream);
+        case 128: return launch_chain<Acc, 128, kLong>(a, smem, blocks, dependent, stream);
+        default: return launch_chain<Acc, 256, kLong>(a, smem, blocks, dependent, stream);
     }
+}
+// Whether kLong's kernel runs an image's windows.
+bool long_windows(const ChainArgs &a, const ChainImg &im) {
+    const int mode = window_mode(a.use_table, a.minlen, im.B);
+    return mode == kShared || (a.use_table && mode == kScan);
+}
+template <typename Acc>
+int launch_chain_cols(const ChainArgs &a, bool longw, int cols, size_t smem, int blocks,
+                      bool dependent, cudaStream_t stream) {
+    return longw ? launch_chain_cols<Acc, true>(a, cols, smem, blocks, dependent, stream)
+                 : launch_chain_cols<Acc, false>(a, cols, smem, blocks, dependent, stream);
 }
 
 size_t fht_smem_bytes(int m, int T) { return (size_t)m * fht_pitch(m, T) * 4; }
@@ -1336,7 +1356,8 @@ int launch_dp_window(Acc *hv, const Shape &s, int B, const WindowTable *t, cudaS
     const size_t smem = item_smem(a, a.one);
     for (int b = s.k - 2; b >= 0 && !st; --b) {
         a.band = b;
-        st = launch_chain_cols<Acc>(a, a.one.cols, smem, a.one.tiles, b != s.k - 2, stream);
+        st = launch_chain_cols<Acc>(a, long_windows(a, a.one), a.one.cols, smem, a.one.tiles,
+                                    b != s.k - 2, stream);
     }
     return st;
 }
@@ -1452,7 +1473,8 @@ int chain_detect_t(const In *img, int pitch, const Shape &s, const ChainQuery &q
     a.band = -1;
     a.store0 = q.sep > 0;
     if (q.table) chain_table(a, *q.table);
-    st = launch_chain_cols<Acc>(a, im.cols, item_smem(a, im), a.items, false, stream);
+    st = launch_chain_cols<Acc>(a, long_windows(a, im), im.cols, item_smem(a, im), a.items, false,
+                                stream);
     if (!st && q.sep > 0) {
         const int D = 2 * s.n - 1;
         second_kernel<Acc><<<D, 256, 0, stream>>>(
@@ -1592,8 +1614,12 @@ int chain_batch_run_t(const ChainBatch *b, char *ws, const WindowTable *t, cudaS
     a.band = -1;
     if (t) chain_table(a, *t);
     size_t smem = 0;
-    for (const ChainImg &im : b->imgs) smem = std::max(smem, item_smem(a, im));
-    return launch_chain_cols<Acc>(a, b->cols, smem, a.items, false, stream);
+    bool longw = true;   // all images alike
+    for (const ChainImg &im : b->imgs) {
+        smem = std::max(smem, item_smem(a, im));
+        longw = longw && long_windows(a, im);
+    }
+    return launch_chain_cols<Acc>(a, longw, b->cols, smem, a.items, false, stream);
 }
 }  // namespace
 
