@@ -10,8 +10,9 @@
 // chip and the chain advances at the latency of one exchange through L2.
 // Bound by that latency, about 5 us a level (poll, V_{b+1} from L2, windows in
 // shared memory, store, release).  One call on 2048 x 2048 uint8, n = 128, B =
-// 16: engine 249 us, chain 110 (FHT 34); 8192 x 8192 float, 64 bands: 1842 ->
-// 969; two polylines 281 -> 128; 24 ragged int32 images in a batch 1406 -> 629.
+// 16: engine 249 us, chain 108 (FHT 26); 8192 x 8192 float, 64 bands: 1842 ->
+// 977; two polylines 281 -> 124; 24 ragged int32 images in a batch 1406 -> 625.
+// Wide uint8 images run on the engine (detect_one).
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -59,8 +60,9 @@ __device__ __forceinline__ void st_if(Acc *p, bool ok, Acc v) {
 // float images run the signs one after the other, the "-" sign on the mirrored
 // strip; uint8 images both at once (fht_smem.cuh).  Bound by shared memory
 // (about 28 bytes a word and sign) and the stores of the rows.
-// 2048 x 2048 uint8, n = 128: four passes over the whole arrays 102 us, this 34
-// (three register levels and 768 threads: 43).
+// 2048 x 2048 uint8, n = 128, a call of fhtdp_fht_bands: four passes over the whole
+// arrays 93 us, this 31 (the kernel 26).  Three register levels and 768 threads
+// took a quarter more.
 constexpr int kFhtNT = 1024;
 
 template <typename In, typename Acc>
@@ -1236,7 +1238,7 @@ size_t fht_smem_bytes(int m, int T) { return (size_t)m * fht_pitch(m, T) * 4; }
 // T + m - 4, T + m - 16, ... columns), one fits an SM (1,024 threads of 64
 // registers), and the SM with the most blocks decides, so the T (a multiple of
 // 16, at most 256) of the least product.  2048 x 2048 uint8, n = 128: T = 64, 128,
-// 192, 256 take 46, 34, 44, 33 us; 1024 x 512, n = 64: T = 32, 64, 128, 256 17,
+// 192, 256 took 46, 34, 44, 33 us (31 now); 1024 x 512, n = 64: T = 32, 64, 128, 256 17,
 // 11.5, 15, 21; 512 x 2016, n = 32: T = 112, 240 15.8, 10.2; 8192 x 8192, n = 128:
 // T = 128, 192, 256 296, 272, 243.  (Those registers are a few
 // too few: 32 to 64 bytes a thread spill.)
