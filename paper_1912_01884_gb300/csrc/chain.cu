@@ -11,7 +11,7 @@
 // Bound by that latency, about 5 us a level (poll, V_{b+1} from L2, windows in
 // shared memory, store, release).  One call on 2048 x 2048 uint8, n = 128, B =
 // 16: engine 249 us, chain 108 (FHT 26); 8192 x 8192 float, 64 bands: 1842 ->
-// 977; two polylines 281 -> 124; 24 ragged int32 images in a batch 1406 -> 625.
+// 974; two polylines 281 -> 124; 24 ragged int32 images in a batch 1406 -> 625.
 // Wide uint8 images run on the engine (detect_one).
 #include <algorithm>
 #include <atomic>
@@ -529,8 +529,8 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
             for (int j = 0; j < 4; ++j) v[j] = value(e0 + 32 * j);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                v[j] = vmax(v[j], Dead<Acc>::value());   // (NaN loses against every number)
-                const unsigned o = v[j] == Dead<Acc>::value() ? 0 : vord(v[j]);
+                // (NaN, whose comparisons are false, counts as dead)
+                const unsigned o = v[j] > Dead<Acc>::value() ? vord(v[j]) : 0;
                 if (o > best) {
                     best = o;
                     be = e0 + 32 * j + n - 1;
@@ -539,17 +539,20 @@ __device__ void chain_readback(const ChainImg &im, const ChainArgs &args, unsign
         }
         const unsigned top = __reduce_max_sync(0xffffffffu, best);
         unsigned at = __reduce_min_sync(0xffffffffu, best == top && top ? be : INT_MAX);
-        if (std::is_same<Acc, float>::value && top == 0) {   // nothing but NaN: the first one
-            be = INT_MAX;
-            for (int e = lo + lane; e <= hi; e += 32) {
-                const Acc v = value(e);
-                if (v != v) be = min(be, (unsigned)(e + n - 1));
+        if (at >= (unsigned)D) {
+            if (std::is_same<Acc, float>::value) {   // nothing but NaN: the first one
+                be = INT_MAX;
+#pragma unroll 1
+                for (int e = lo + lane; e <= hi; e += 32) {
+                    const Acc v = value(e);
+                    if (v != v) be = min(be, (unsigned)(e + n - 1));
+                }
+                at = __reduce_min_sync(0xffffffffu, be);
             }
-            at = __reduce_min_sync(0xffffffffu, be);
-        }
-        if (at >= (unsigned)D) {   // only with inconsistent values (a wait gave up)
-            if (lane == 0 && args.ctl) gave_up(args);
-            return;
+            if (at >= (unsigned)D) {   // only with inconsistent values (a wait gave up)
+                if (lane == 0 && args.ctl) gave_up(args);
+                return;
+            }
         }
         d = (int)at - (n - 1);
         if (lane == 0) {
@@ -599,7 +602,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
     const int u = threadIdx.x & (C - 1), q = threadIdx.x >> lg, xn = xn0 + u;
     const bool last = band == im.k - 1;   // (only one-band images: V = H)
     const int B = im.B, asked = window_mode(args.use_table, args.minlen, B);
-    const int mode = !kLong && asked == kShared ? kClipped : asked;
+    const int mode = kLong ? asked : min(asked, (int)kClipped);
     const int pad = window_pad(mode, args.use_table, B), rows = range_rows(n);
     const Acc dead = Dead<Acc>::value();
     // S (or the values), then P: row e - lo + pad of displacement e
@@ -731,7 +734,7 @@ __device__ void chain_item(const ChainImg &im, int band, int tile, unsigned char
         const int r0 = c0 - lo + pad;   // the run's first row
         auto run_of = [&](int j) -> Acc { return Su[j * kRun * R]; };   // maximum of run j
         if (last) {
-        } else if (!kLong && mode == kPadded) {
+        } else if (mode == kPadded && !kLong) {
             // windows [r - B, r + B]: their first run is j0 or, from row 8 - ol
             // on, j0 + 1; their last one z0 or, from row 8 - oz on, z0 + 1
             const int j0 = (r0 - B) >> 3, z0 = (r0 + B) >> 3;
